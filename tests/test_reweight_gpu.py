@@ -63,3 +63,35 @@ def test_reweight_argument_errors():
     w = torch.ones((4, 4, 1, 1, 1), device="cuda")
     with pytest.raises(rt3d.Rt3dError):
         rt3d.rt3d_kgs_group_norms(w, 4, 4, 3, torch.empty((1, 1, 1), device="cuda"))
+
+
+@pytest.mark.parametrize("M,N,k,g_m,g_n,byte", [
+    (4, 4, (1, 1, 1), 4, 4, 0), (5, 3, (3, 1, 1), 4, 4, 1), (9, 37, (3, 3, 3), 8, 4, 3),      # rows at odd bytes, ragged groups
+    (8, 152, (3, 3, 3), 4, 4, 0), (12, 151, (3, 3, 3), 4, 4, 5),                              # a mask chunk and a few bytes
+    (16, 76, (3, 3, 3), 4, 4, 0), (7, 80, (3, 3, 3), 8, 8, 2), (6, 20, (5, 7, 7), 4, 16, 0)])  # run ends; groups beyond a chunk
+def test_pruning_step_at_run_and_word_edges(M, N, k, g_m, g_n, byte):
+    """Rows and buffers that start at any byte / float, runs and chunks that end inside a word, groups too long for a run."""
+    rng = np.random.default_rng(M * 1000 + N)
+    Ks = k[0] * k[1] * k[2]
+    P, Q = synth.n_groups(M, N, g_m, g_n)
+    w = rng.standard_normal((M, N) + k).astype(np.float32)
+    for shift in (0, 1):                                          # weights 16-byte aligned, and 4 bytes further
+        buf = torch.zeros(w.size + 1, device="cuda")
+        wd = buf[shift:shift + w.size].view(w.shape)
+        wd.copy_(torch.from_numpy(w))
+        norms = torch.zeros(P * Q * Ks + 1, device="cuda")[shift:shift + P * Q * Ks]
+        for norm in (1, 2):
+            rt3d.rt3d_kgs_group_norms(wd, g_m, g_n, norm, norms)
+            np.testing.assert_allclose(norms.cpu().numpy().reshape(P, Q, Ks), oracle.group_norms(w, g_m, g_n, norm), rtol=1e-5)
+        pen = torch.zeros(P * Q * Ks + 1, device="cuda")[shift:shift + P * Q * Ks]
+        keep = torch.zeros(P * Q * Ks + 4, dtype=torch.uint8, device="cuda")[shift:shift + P * Q * Ks]
+        rt3d.rt3d_kgs_reweight(norms, 1e-3, float(norms.median()) * 1.0001, pen, keep)
+        got = norms.double().cpu().numpy()
+        np.testing.assert_allclose(pen.cpu().numpy(), 1.0 / (got * got + 1e-3), rtol=1e-5)
+        np.testing.assert_array_equal(keep.cpu().numpy(), (norms > float(norms.median()) * 1.0001).cpu().numpy())
+    gm = torch.from_numpy((rng.random((P, Q, Ks)) < 0.4).astype(np.uint8)).cuda()
+    out = torch.full((M * N * Ks + 64,), 7, dtype=torch.uint8, device="cuda")
+    mask = out[16 + byte:16 + byte + M * N * Ks]
+    rt3d.rt3d_kgs_expand_mask(gm, M, N, *k, g_m, g_n, mask)
+    np.testing.assert_array_equal(mask.cpu().numpy().reshape((M, N) + k), synth.expand_group_mask(gm.cpu().numpy(), M, N, g_m, g_n, *k))
+    assert bool((out[:16 + byte] == 7).all()) and bool((out[16 + byte + M * N * Ks:] == 7).all())     # neighbours untouched
