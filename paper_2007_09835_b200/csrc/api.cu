@@ -154,7 +154,7 @@ DeviceBlob* find_blob(rt3d_packed* h, int dev) {
   return nullptr;
 }
 
-// Returns the blob of the current device, creating and uploading the canonical arrays on first use.
+// Returns the blob of the current device, creating it on first use.
 rt3d_status get_blob(rt3d_packed* h, DeviceBlob** out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return RT3D_ERR_CUDA;
@@ -164,27 +164,54 @@ rt3d_status get_blob(rt3d_packed* h, DeviceBlob** out) {
     b = new (std::nothrow) DeviceBlob;
     if (!b) return RT3D_ERR_ALLOC;
     b->device = dev;
-    rt3d_status s = RT3D_OK;
-    if (dev_malloc(&b->group_ptr, h->group_ptr.size() * 4) != cudaSuccess ||
-        dev_malloc(&b->pos_idx, h->pos_idx.size() * 2 + 16) != cudaSuccess ||
-        dev_malloc(&b->tiles, h->tiles.size() + 16) != cudaSuccess)
-      s = RT3D_ERR_ALLOC;
-    if (s == RT3D_OK &&
-        (cudaMemcpy(b->group_ptr, h->group_ptr.data(), h->group_ptr.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-         (h->nnz && cudaMemcpy(b->pos_idx, h->pos_idx.data(), h->pos_idx.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess) ||
-         (h->nnz && cudaMemcpy(b->tiles, h->tiles.data(), h->tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess)))
-      s = RT3D_ERR_CUDA;
-    if (s != RT3D_OK) {
-      cudaFree(b->group_ptr); cudaFree(b->pos_idx); cudaFree(b->tiles);
-      delete b;
-      return s;
-    }
     h->blobs.push_back(b);
     std::lock_guard<std::mutex> reg(g_blobs_mu);
     g_blobs.push_back(b);
   }
   *out = b;
   return RT3D_OK;
+}
+
+// Host arrays that become one device allocation: a cudaMalloc costs more than the copy of a small layer's index, so the
+// arrays of a layout share one.  `add` remembers an array and the pointer that will refer to its device copy.
+class Upload {
+ public:
+  template <typename T, typename V>
+  void add(T** dst, const V& v) {
+    items_[n_++] = Item{reinterpret_cast<void**>(dst), v.data(), v.size() * sizeof(v[0]), bytes_};
+    bytes_ += (v.size() * sizeof(v[0]) + 16 + 255) & ~size_t(255);       // 256-byte aligned parts, readable 16 bytes on
+  }
+  // Allocates, copies and sets the pointers; *base owns the memory.  Nothing is kept on failure.
+  rt3d_status run(void** base) {
+    if (dev_malloc(base, bytes_) != cudaSuccess) { *base = nullptr; return RT3D_ERR_ALLOC; }
+    for (int i = 0; i < n_; ++i) {
+      char* d = static_cast<char*>(*base) + items_[i].off;
+      if (items_[i].bytes && cudaMemcpy(d, items_[i].src, items_[i].bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaFree(*base);
+        *base = nullptr;
+        return RT3D_ERR_CUDA;
+      }
+      *items_[i].dst = d;
+    }
+    return RT3D_OK;
+  }
+
+ private:
+  struct Item { void** dst; const void* src; size_t bytes, off; };
+  Item items_[8];
+  int n_ = 0;
+  size_t bytes_ = 0;
+};
+
+// Device copies of the canonical arrays: only the index-driven CUDA-core kernel reads them.
+rt3d_status get_canonical(rt3d_packed* h, DeviceBlob* b) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  if (b->canonical) return RT3D_OK;
+  Upload up;
+  up.add(&b->group_ptr, h->group_ptr);
+  up.add(&b->pos_idx, h->pos_idx);
+  up.add(&b->tiles, h->tiles);
+  return up.run(&b->canonical);
 }
 
 rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, DeviceBlob::Umma** out) {
@@ -660,6 +687,63 @@ rt3d_status try_sub(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   return RT3D_OK;
 }
 
+// Device copy of the register-blocked fp32 kernel's layout.
+rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, DeviceBlob::F32** out) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  DeviceBlob::F32& u = blob->f32;
+  if (!u.base) {
+    Upload up;
+    up.add(&u.entry_ptr, L->entry_ptr);
+    up.add(&u.tile_ptr, L->tile_ptr);
+    up.add(&u.counts, L->counts);
+    up.add(&u.entries, L->entries);
+    up.add(&u.tiles, L->tiles);
+    const rt3d_status s = up.run(&u.base);
+    if (s != RT3D_OK) return s;
+  }
+  *out = &u;
+  return RT3D_OK;
+}
+
+// Register-blocked fp32 kernel: every fp32 call whose kernel groups are whole 4 x 4 tiles.
+// *launched = false (and RT3D_OK) when the handle or the shape cannot use it.
+rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
+                    const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, cudaStream_t st, bool* launched) {
+  *launched = false;
+  if (!f32_layout_possible(w)) return RT3D_OK;
+  struct Entry { ConvGeom g; int64_t nnz; int n; F32Plan plans[kF32MaxPlans]; };     // as in choose_box
+  thread_local Entry cache[16];
+  thread_local int used = 0, next = 0;
+  Entry* e = nullptr;
+  for (int i = 0; i < used && !e; ++i)
+    if (memcmp(&cache[i].g, &g, sizeof(g)) == 0 && cache[i].nnz == w->nnz) e = &cache[i];
+  if (!e) {
+    e = &cache[next];
+    next = (next + 1) % 16;
+    if (used < 16) ++used;
+    e->g = g; e->nnz = w->nnz;
+    e->n = conv_f32_plans(g, double(w->nnz) / (double(w->P) * w->Q * w->Ks), d->sm_count, e->plans);
+  }
+  F32Args a;
+  a.g = g;
+  for (int i = 0; i < e->n; ++i) {
+    const F32Layout* L = get_f32_layout(w);
+    if (!L || !conv_f32_fill(e->plans[i], *L, &a)) continue;
+    DeviceBlob::F32* u = nullptr;
+    rt3d_status s = get_f32_blob(w, blob, L, &u);
+    if (s != RT3D_OK) return s;
+    a.entry_ptr = u->entry_ptr; a.tile_ptr = u->tile_ptr; a.counts = u->counts; a.entries = u->entries; a.tiles = u->tiles;
+    a.x = static_cast<const float*>(x->data); a.y = static_cast<float*>(y->data);
+    a.bias = bias; a.residual = static_cast<const float*>(res_data); a.rcs = res_pitch;
+    *launched = true;
+    if (t_plan_only) return RT3D_OK;
+    if (launch_conv_f32(a, e->plans[i], st) != cudaSuccess) return RT3D_ERR_CUDA;
+    g_launches.fetch_add(1);
+    return RT3D_OK;
+  }
+  return RT3D_OK;
+}
+
 rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
                       rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz = nullptr) {
   ConvGeom g;
@@ -708,6 +792,10 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   if (!use_umma) {
     if (pooled) return RT3D_ERR_UNSUPPORTED;
     t_last_plan = rt3d_plan_info{0, 0, 1, 0, 0};
+    bool launched = false;
+    s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, st, &launched);
+    if (s != RT3D_OK || launched) return s;
+    if ((s = get_canonical(w, blob)) != RT3D_OK) return s;
     if (t_plan_only) return RT3D_OK;
     cudaError_t e = launch_conv_simt(w->dtype, g, x->data, y->data, blob->group_ptr, blob->pos_idx, blob->tiles, bias,
                                      w->g_m, w->g_n, w->P, w->Q, dense_entry, res_data, res_pitch, st);
@@ -1093,6 +1181,11 @@ rt3d_status rt3d_packed_prepare(rt3d_packed* p) {
     const UmmaLayout* L = get_umma_layout(p, 0);
     DeviceBlob::Umma* u = nullptr;
     if (L && (s = get_umma_blob(p, blob, L, &u)) != RT3D_OK) return s;
+  } else if (const F32Layout* L = get_f32_layout(p)) {
+    DeviceBlob::F32* u = nullptr;
+    if ((s = get_f32_blob(p, blob, L, &u)) != RT3D_OK) return s;
+  } else if ((s = get_canonical(p, blob)) != RT3D_OK) {
+    return s;
   }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return RT3D_ERR_CUDA;
@@ -1111,7 +1204,7 @@ void rt3d_packed_free(rt3d_packed* p) {
   }
   for (DeviceBlob* b : p->blobs) {
     if (have_dev) cudaSetDevice(b->device);
-    cudaFree(b->group_ptr); cudaFree(b->pos_idx); cudaFree(b->tiles);
+    cudaFree(b->canonical);
     for (auto& kv : b->umma) {
       cudaFree(kv.second.wtiles); cudaFree(kv.second.step_ptr); cudaFree(kv.second.steps);
       cudaFree(kv.second.grp_ptr); cudaFree(kv.second.grp_first);
@@ -1120,6 +1213,7 @@ void rt3d_packed_free(rt3d_packed* p) {
     for (void* hs : b->host_streams) if (hs) cudaStreamDestroy(static_cast<cudaStream_t>(hs));
     for (void* he : b->host_events) if (he) cudaEventDestroy(static_cast<cudaEvent_t>(he));
     for (auto& kv : b->smallc) { cudaFree(kv.second.wimg); cudaFree(kv.second.pairs); }
+    cudaFree(b->f32.base);
     for (auto& kv : b->sub) { cudaFree(kv.second.steps); cudaFree(kv.second.step_ptr); cudaFree(kv.second.blocks); }
     cudaFree(b->splitk); cudaFree(b->splitk_cnt);
     delete b;

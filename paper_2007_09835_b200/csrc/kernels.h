@@ -24,6 +24,37 @@ cudaError_t launch_conv_simt(int dtype, const ConvGeom& g, const void* x, void* 
                              const float* bias, int g_m, int g_n, int P, int Q, bool dense,
                              const void* residual, int rcs, cudaStream_t stream);
 
+// Register-blocked fp32 kernel (simt_conv_f32.cu).
+struct F32Args {
+  ConvGeom g;
+  int bt, bh, bw;                     // output box of a block: at most (8 / sets) * 16 lanes' positions times vt * vh voxels
+  int vt, vh;                         // a thread's voxels: vt along t times vh along h, bt / vt and bh / vh apart
+  int tiles_t, tiles_h, tiles_w;
+  int ht, hh, hw;                     // staged input box
+  int ht_step, hh_step, hw_step;      // input voxels between neighbouring staged voxels (the stride where the kernel is 1 wide)
+  int n_sets, n_stages, quads;
+  int sets;                           // row sets per block: 1, 2, 4 or 8
+  int max_entries, max_tiles;         // of one stage of a block
+  const int32_t* entry_ptr;           // device arrays of the layout
+  const int32_t* tile_ptr;
+  const int32_t* counts;
+  const uint32_t* entries;
+  const float* tiles;
+  const float* x;
+  float* y;
+  const float* bias;                  // or nullptr
+  const float* residual;              // or nullptr, pitch rcs
+  int rcs;
+};
+struct F32Plan { int voxels, sets; int bt, bh, bw, vt, vh; };
+struct F32Layout;
+// Candidate (voxels per thread, row sets per block, output box) for a call, best first (density = kept
+// share of the (group, location) places); conv_f32_fill says whether one's staging fits shared memory.
+constexpr int kF32MaxPlans = 16;
+int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]);
+bool conv_f32_fill(const F32Plan& plan, const F32Layout& L, F32Args* a);
+cudaError_t launch_conv_f32(const F32Args& a, const F32Plan& plan, cudaStream_t stream);
+
 cudaError_t launch_maxpool3d(int dtype, const void* x, int n, int t, int h, int w, int c, int xcs,
                              int kt, int kh, int kw, int st, int sh, int sw, int pt, int ph, int pw,
                              void* y, int To, int Ho, int Wo, int ycs, cudaStream_t stream);

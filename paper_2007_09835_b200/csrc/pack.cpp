@@ -268,6 +268,75 @@ const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw) {
   return &res.first->second;
 }
 
+constexpr int kF32MaxKs = 512;      // kernel locations the fp32 kernel's offset table holds
+
+bool f32_layout_possible(const rt3d_packed* p) {
+  return p->dtype == RT3D_F32 && p->g_m % 4 == 0 && p->g_n % 4 == 0 && p->Ks <= kF32MaxKs;
+}
+
+const F32Layout* get_f32_layout(rt3d_packed* p) {
+  if (!f32_layout_possible(p)) return nullptr;
+  std::lock_guard<std::mutex> lock(p->mu);
+  if (p->f32_layout) return p->f32_layout.get();
+  std::unique_ptr<F32Layout> layout(new F32Layout);
+  F32Layout& L = *layout;
+  L.quads = f32_stage_quads(p->Ks);
+  const int n_rows = ceil_div(p->M, 4), n_quads = ceil_div(p->N, 4);
+  L.n_sets = ceil_div(n_rows, 2);
+  L.n_stages = ceil_div(n_quads, L.quads);
+  const int Ks = p->Ks, rm = p->g_m / 4, rn = p->g_n / 4;
+  const float* tiles = reinterpret_cast<const float*>(p->tiles.data());
+  std::vector<int32_t> kept(size_t(2) * L.quads * Ks);   // packed entry that holds (row, quad, location), or -1
+  const size_t n_lists = size_t(L.n_stages) * L.n_sets;
+  L.entry_ptr.reserve(n_lists + 1);
+  L.tile_ptr.reserve(n_lists + 1);
+  L.counts.reserve(n_lists);
+  L.entries.reserve(size_t(p->nnz) * rm * rn);           // at most one entry per 4 x 4 tile
+  L.tiles.resize(size_t(p->nnz) * rm * rn * 16);
+  float* out = L.tiles.data();
+  L.entry_ptr.push_back(0);
+  L.tile_ptr.push_back(0);
+  for (int st = 0; st < L.n_stages; ++st)
+    for (int s = 0; s < L.n_sets; ++s) {
+      std::fill(kept.begin(), kept.end(), -1);
+      for (int r = 0; r < 2 && s * 2 + r < n_rows; ++r)
+        for (int ql = 0; ql < L.quads && st * L.quads + ql < n_quads; ++ql) {
+          const size_t grp = size_t((s * 2 + r) / rm) * p->Q + (st * L.quads + ql) / rn;
+          for (int32_t e = p->group_ptr[grp]; e < p->group_ptr[grp + 1]; ++e)
+            kept[size_t(r * L.quads + ql) * Ks + p->pos_idx[e]] = e;
+        }
+      int count[3] = {0, 0, 0};
+      for (int list = 0; list < 3; ++list)
+        for (int ql = 0; ql < L.quads; ++ql)
+          for (int k = 0; k < Ks; ++k) {
+            const int32_t e[2] = {kept[size_t(ql) * Ks + k], kept[size_t(L.quads + ql) * Ks + k]};
+            const int which = e[0] >= 0 ? (e[1] >= 0 ? 0 : 1) : (e[1] >= 0 ? 2 : -1);
+            if (which != list) continue;
+            ++count[list];
+            L.entries.push_back(uint32_t(k) | uint32_t(ql) << 16);
+            for (int r = 0; r < 2; ++r) {
+              if (e[r] < 0) continue;
+              const int ib = ((s * 2 + r) % rm) * 4, jb = ((st * L.quads + ql) % rn) * 4;
+              for (int i = 0; i < 4; ++i, out += 4)
+                std::memcpy(out, tiles + (int64_t(e[r]) * p->g_m + ib + i) * p->g_n + jb, 16);
+            }
+          }
+      L.counts.push_back(count[0] | count[1] << 16);
+      L.entry_ptr.push_back(int32_t(L.entries.size()));
+      L.tile_ptr.push_back(int32_t((out - L.tiles.data()) / 16));
+    }
+  L.tiles.resize(size_t(out - L.tiles.data()));
+  for (int lg = 0; lg < 4; ++lg)
+    for (int st = 0; st < L.n_stages; ++st)
+      for (int s = 0; s < L.n_sets; s += 1 << lg) {
+        const size_t a = size_t(st) * L.n_sets + s, b = size_t(st) * L.n_sets + std::min(L.n_sets, s + (1 << lg));
+        L.max_entries[lg] = std::max(L.max_entries[lg], L.entry_ptr[b] - L.entry_ptr[a]);
+        L.max_tiles[lg] = std::max(L.max_tiles[lg], L.tile_ptr[b] - L.tile_ptr[a]);
+      }
+  p->f32_layout = std::move(layout);
+  return p->f32_layout.get();
+}
+
 static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, int Kt, int Kh, int Kw,
                              int g_m, int g_n, int dtype, int is_dense, rt3d_packed** out) {
   if (!w || !out) return RT3D_ERR_INVALID_ARG;

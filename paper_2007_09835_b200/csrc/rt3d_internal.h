@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cstddef>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -79,10 +80,26 @@ struct SubLayout {
   int max_steps = 0;                 // longest bundle list
 };
 
+// Layout of the register-blocked fp32 kernel (simt_conv_f32.cu).  Kernel groups are cut into 4 x 4 tiles; a "row set" is
+// two consecutive rows of four output channels, a stage is `quads` consecutive quads of input channels.  For each
+// (stage, row set), stage-major, three lists of entries, one after the other: the (quad, kernel location) places that
+// both rows keep, that only the first and that only the second keeps, each with one tile per row that keeps it.
+struct F32Layout {
+  int quads = 0, n_sets = 0, n_stages = 0;
+  std::vector<int32_t> entry_ptr;    // [n_stages * n_sets + 1]
+  std::vector<int32_t> tile_ptr;     // [n_stages * n_sets + 1]
+  std::vector<int32_t> counts;       // [n_stages * n_sets] entries of the first list | of the second << 16
+  std::vector<uint32_t> entries;     // kernel location | quad inside the stage << 16
+  std::vector<float> tiles;          // [tile][16]: [output pair][output][input]
+  int max_entries[4] = {0, 0, 0, 0}; // most entries / tiles of a stage in 1, 2, 4, 8 aligned consecutive row sets
+  int max_tiles[4] = {0, 0, 0, 0};
+};
+
 // Per-device copies of a handle's arrays.
 struct DeviceBlob {
   int device = -1;
-  int32_t* group_ptr = nullptr;      // canonical arrays (CUDA-core kernel)
+  void* canonical = nullptr;         // owns the canonical arrays (CUDA-core kernel), uploaded on its first use
+  int32_t* group_ptr = nullptr;
   uint16_t* pos_idx = nullptr;
   void* tiles = nullptr;
   struct Umma {
@@ -100,6 +117,8 @@ struct DeviceBlob {
   std::map<int, Sub> sub;            // sub-tile kernel, keyed by n_tile
   struct SmallC { void* wimg = nullptr; int32_t* pairs = nullptr; };
   std::map<int, SmallC> smallc;      // small-C_in kernel: weight image and pair offsets, keyed by sh*16+sw
+  struct F32 { void* base = nullptr; int32_t* entry_ptr = nullptr; int32_t* tile_ptr = nullptr; int32_t* counts = nullptr; uint32_t* entries = nullptr; float* tiles = nullptr; };
+  F32 f32;                           // register-blocked fp32 kernel
   float* splitk = nullptr; size_t splitk_bytes = 0;            // split-K partial tiles (grown on demand)
   int32_t* splitk_cnt = nullptr; size_t splitk_cnt_bytes = 0;  // split-K arrival counters, zero between launches
   void* stage_x = nullptr; size_t stage_x_bytes = 0;   // staging for rt3d_conv3d_host
@@ -124,6 +143,7 @@ struct rt3d_packed {
   std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by n_tile (+ 4096: the t-grouped order)
   std::map<int, rt3d::SubLayout> sub_layouts;     // keyed by n_tile
   std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw, built on first use
+  std::unique_ptr<rt3d::F32Layout> f32_layout;        // built on first use
   std::vector<rt3d::DeviceBlob*> blobs;
 };
 
@@ -139,5 +159,9 @@ const SubLayout* get_sub_layout(rt3d_packed* p, int n_tile);
 
 // Small-C_in layout (nullptr if the handle does not qualify: needs bf16, N <= 8, M <= 256).
 const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw);
+
+// Layout of the register-blocked fp32 kernel (nullptr unless fp32 with group sizes that are multiples of four).
+bool f32_layout_possible(const rt3d_packed* p);
+const F32Layout* get_f32_layout(rt3d_packed* p);
 
 }  // namespace rt3d

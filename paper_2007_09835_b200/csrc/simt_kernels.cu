@@ -5,8 +5,8 @@
 // one output voxel and one row of kernel groups (g_m output channels); for every kernel
 // group of that row it walks the kept kernel locations of the packed index and applies the
 // group's g_m x g_n weight tile to the g_n input channels at the shifted voxel.  Pruned
-// locations are never visited.  It is the cross-check for the tensor-core kernel and the
-// production path for shapes that kernel does not take.
+// locations are never visited.  It is the cross-check for the tensor-core kernel and takes what neither that nor the
+// register-blocked fp32 kernel (simt_conv_f32.cu) does: kernel groups that are not whole 4 x 4 tiles, mostly.
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -29,7 +29,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
 // staged once per block in shared memory (in pieces of kStageEntries kept entries across the row's Q groups, which
 // are contiguous in the packed arrays), with each kept location
 // decoded to its (kt, kh, kw) there: the inner loop then has no integer division and no dependent global load
-// besides the input voxel itself, which is fetched with one 16-byte load when the group is four channels wide.
+// besides the input voxel itself.
 constexpr int kStageEntries = 64;
 
 template <typename T, int GM, int GN, bool DENSE>
@@ -62,7 +62,6 @@ conv3d_kgs_simt_kernel(ConvGeom g, const T* __restrict__ x, T* __restrict__ y,
   for (int i = 0; i < MAXM; ++i) acc[i] = 0.f;
 
   const int tile_elems = g_m * g_n;
-  const bool vec4 = GN == 4 && sizeof(T) == 4 && (g.xcs & 3) == 0 && (g.c & 3) == 0;
   // the kept entries of all Q groups of row p are one contiguous range of the packed arrays
   const int row0 = group_ptr[p * Q], row1 = group_ptr[p * Q + Q];
   for (int eb = row0; eb < row1; eb += kStageEntries) {
@@ -87,15 +86,8 @@ conv3d_kgs_simt_kernel(ConvGeom g, const T* __restrict__ x, T* __restrict__ y,
       const bool inb = valid && unsigned(ti) < unsigned(g.t) && unsigned(hi) < unsigned(g.h) && unsigned(wi) < unsigned(g.w);
       const T* xp = x + ((((long long)nn * g.t + (inb ? ti : 0)) * g.h + (inb ? hi : 0)) * g.w + (inb ? wi : 0)) * g.xcs + c0;
       float xv[MAXN];
-      if (vec4) {
-        const float4 t4 = inb ? __ldg(reinterpret_cast<const float4*>(xp)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        xv[0] = t4.x; xv[1] = t4.y; xv[2] = t4.z; xv[3] = t4.w;
 #pragma unroll
-        for (int j = 4; j < MAXN; ++j) xv[j] = 0.f;
-      } else {
-#pragma unroll
-        for (int j = 0; j < MAXN; ++j) xv[j] = (inb && j < g_n && c0 + j < g.c) ? to_f32<T>(xp[j]) : 0.f;
-      }
+      for (int j = 0; j < MAXN; ++j) xv[j] = (inb && j < g_n && c0 + j < g.c) ? to_f32<T>(xp[j]) : 0.f;
       const float* tp = w_s + e * (MAXM * MAXN);
 #pragma unroll
       for (int i = 0; i < MAXM; ++i) {
@@ -136,7 +128,9 @@ cudaError_t launch_conv_t(const ConvGeom& g, const void* x, void* y, const int32
   cudaError_t le = cudaSuccess;
 #define RT3D_LAUNCH(GM_, GN_) \
   le = cudaLaunchKernelEx(&ls.cfg, conv3d_kgs_simt_kernel<T, GM_, GN_, DENSE>, g, xt, yt, group_ptr, pos_idx, tt, bias, g_m, g_n, Q, total, rt, rcs)
-  if (g_m == 4 && g_n == 4) RT3D_LAUNCH(4, 4);
+  // fp32 calls on whole 4 x 4 tiles run on the register-blocked kernel: here fp32 needs the run-time group size only
+  if constexpr (sizeof(T) == 4) RT3D_LAUNCH(0, 0);
+  else if (g_m == 4 && g_n == 4) RT3D_LAUNCH(4, 4);
   else if (g_m == 8 && g_n == 4) RT3D_LAUNCH(8, 4);
   else if (g_m == 8 && g_n == 8) RT3D_LAUNCH(8, 8);
   else RT3D_LAUNCH(0, 0);

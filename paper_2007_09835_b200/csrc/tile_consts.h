@@ -21,4 +21,8 @@ struct SubStep {
   int nblk;
   int pad;
 };
+
+// Register-blocked fp32 kernel (simt_conv_f32.cu): quads of input channels per stage.  A stage should hold some fifty
+// (quad, location) entries, so that its arithmetic covers the latency of staging the next one.
+constexpr int f32_stage_quads(int Ks) { return Ks >= 9 ? 2 : Ks >= 3 ? 4 : 8; }
 }  // namespace rt3d
