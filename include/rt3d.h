@@ -324,6 +324,26 @@ rt3d_status rt3d_kgs_reweight(const float* norms, int64_t count, float eps, floa
 rt3d_status rt3d_kgs_expand_mask(const uint8_t* group_mask, int M, int N, int Kt, int Kh, int Kw, int g_m, int g_n,
                                  uint8_t* mask, void* stream);
 
+/* rt3d_run_calls - a sequence of the compute calls above, e.g. one forward pass of a network, issued in one go: what each
+ * call enqueues and returns is what the single call would, in the order given, without the caller's language between
+ * them.  Stops at the first call that fails and returns its status, its index in *failed (may be NULL).
+ *   lane      index into `streams`: the stream the call goes to
+ *   RECORD / WAIT  k[0] = slot: the slot takes the lane's work so far / the lane waits for what the slot took last
+ * Calls:  SPARSE, DENSE (x, w, bias, p, y); FUSED (and r = residual or data NULL, k[0..2] = pool_t/h/w); PAIR (x, w, bias,
+ * p, w2, bias2, p2, r, y); MAXPOOL (x, k[0..8] = kt kh kw st sh sw pt ph pw, y); ADD (x, r = second addend, k[0] = relu, y). */
+enum { RT3D_CALL_SPARSE = 0, RT3D_CALL_DENSE = 1, RT3D_CALL_FUSED = 2, RT3D_CALL_PAIR = 3, RT3D_CALL_MAXPOOL = 4,
+       RT3D_CALL_ADD = 5, RT3D_CALL_RECORD = 6, RT3D_CALL_WAIT = 7 };
+#define RT3D_CALL_SLOTS 8
+typedef struct {
+  int32_t kind, lane;
+  rt3d_tensor x, y, r;
+  const rt3d_packed *w, *w2;
+  const float *bias, *bias2;
+  rt3d_conv_params p, p2;
+  int32_t k[9];
+} rt3d_call;
+rt3d_status rt3d_run_calls(const rt3d_call* calls, int32_t n, void* const* streams, int32_t n_streams, int32_t* failed);
+
 /* Work and traffic the method itself requires for one call (Section 3 cost model):
  * kept multiply-accumulates, dense multiply-accumulates, and algorithmic bytes
  * (input once + output once + packed weights and index once + bias). */

@@ -42,6 +42,16 @@ class ConvParams(ctypes.Structure):
                 ("concurrent", ctypes.c_int32)]
 
 
+class Call(ctypes.Structure):
+    """One step of rt3d_run_calls."""
+    _fields_ = [("kind", ctypes.c_int32), ("lane", ctypes.c_int32), ("x", Tensor), ("y", Tensor), ("r", Tensor),
+                ("w", ctypes.c_void_p), ("w2", ctypes.c_void_p), ("bias", ctypes.c_void_p), ("bias2", ctypes.c_void_p),
+                ("p", ConvParams), ("p2", ConvParams), ("k", ctypes.c_int32 * 9)]
+
+
+(CALL_SPARSE, CALL_DENSE, CALL_FUSED, CALL_PAIR, CALL_MAXPOOL, CALL_ADD, CALL_RECORD, CALL_WAIT), CALL_SLOTS = range(8), 8
+
+
 class Fusion(ctypes.Structure):
     _fields_ = [("residual", ctypes.POINTER(Tensor)), ("pool_t", ctypes.c_int32), ("pool_h", ctypes.c_int32),
                 ("pool_w", ctypes.c_int32)]
@@ -82,6 +92,8 @@ def _load():
     lib.rt3d_kgs_group_norms.argtypes = [vp, i, i, i, i, i, i, i, i, vp, vp]
     lib.rt3d_kgs_reweight.argtypes = [vp, ctypes.c_int64, ctypes.c_float, ctypes.c_float, vp, vp, vp]
     lib.rt3d_kgs_expand_mask.argtypes = [vp, i, i, i, i, i, i, i, vp, vp]
+    lib.rt3d_run_calls.argtypes = [ctypes.POINTER(Call), ctypes.c_int32, ctypes.POINTER(vp), ctypes.c_int32,
+                                   ctypes.POINTER(ctypes.c_int32)]
     lib.rt3d_maxpool3d.argtypes = [TP] + [i] * 9 + [TP, vp]
     lib.rt3d_add_relu.argtypes = [TP, TP, i, TP, vp]
     i64p = ctypes.POINTER(ctypes.c_int64)
@@ -247,10 +259,19 @@ def planning():
     """Planning mode (rt3d_plan_begin / rt3d_plan_end): compute calls inside the block choose their kernels, upload
     their weight layouts and size their workspaces but launch nothing."""
     _lib.rt3d_plan_begin()
+    _planning.on = True
     try:
         yield
     finally:
+        _planning.on = False
         _lib.rt3d_plan_end()
+
+
+_planning = threading.local()
+
+
+def is_planning() -> bool:
+    return getattr(_planning, "on", False)
 
 
 def _params(stride, pad, relu, algo, x_pad_zero=False) -> ConvParams:
@@ -258,23 +279,118 @@ def _params(stride, pad, relu, algo, x_pad_zero=False) -> ConvParams:
                       int(bool(relu)), int(algo), int(bool(x_pad_zero)), int(getattr(_concurrent, "on", False)))
 
 
-def _stream_ptr(stream):
-    if stream is None:
+def concurrent() -> bool:
+    """Whether this thread is inside concurrent_kernels()."""
+    return getattr(_concurrent, "on", False)
+
+
+_torch_cuda = None      # torch's current-device and current-raw-stream functions, fetched on the first call that needs them
+
+
+def current_stream_ptr() -> int:
+    """Handle of the current device's current torch stream (the Stream object around it costs ten times as much)."""
+    global _torch_cuda
+    if _torch_cuda is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        torch.cuda.init()
+        _torch_cuda = (torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    return _torch_cuda[1](_torch_cuda[0]())
+
+
+def _stream_ptr(stream):
+    return ctypes.c_void_p(current_stream_ptr() if stream is None else int(stream))
 
 
 def _bias_ptr(bias):
     return None if bias is None else ctypes.c_void_p(bias.data_ptr())
 
 
+# ------------------------------------------------------------------------------------ sequences of calls
+_recording = threading.local()      # .seq: the CallSequence that this thread's calls are noted in
+
+
+class CallSequence:
+    """The compute calls of one forward pass, noted while they are made for the first time and then issued by one library
+    call (rt3d_run_calls).  Holds what it was noted from: the descriptors, and references that keep handles, biases and
+    buffers alive.  `x_ptr` is the address of the pass's input while noting: later runs may bring their input elsewhere."""
+
+    def __init__(self, x_ptr: int, stream_ptr: int):
+        self.x_ptr, self.calls, self.keep, self.lanes, self.slots = x_ptr, [], [], [stream_ptr], {}
+        self.array = None
+
+    @contextlib.contextmanager
+    def noting(self):
+        prev = getattr(_recording, "seq", None)
+        _recording.seq = self
+        try:
+            yield self
+        finally:
+            _recording.seq = prev
+
+    def _lane(self, stream) -> int:
+        ptr = current_stream_ptr() if stream is None else int(stream)
+        if ptr not in self.lanes:
+            self.lanes.append(ptr)
+        return self.lanes.index(ptr)
+
+    def note(self, kind, stream, x, y, r=None, w=None, bias=None, p=None, w2=None, bias2=None, p2=None, k=()):
+        c = Call(kind=kind, lane=self._lane(stream), x=x, y=y)
+        if r is not None:
+            c.r = r
+        for h, b, q, names in ((w, bias, p, ("w", "bias", "p")), (w2, bias2, p2, ("w2", "bias2", "p2"))):
+            if h is not None:
+                setattr(c, names[0], h.handle)
+                setattr(c, names[2], q)
+            if b is not None:
+                setattr(c, names[1], b.data_ptr())
+            self.keep.append((h, b))
+        for i, v in enumerate(k):
+            c.k[i] = int(v)
+        self.calls.append(c)
+
+    def note_event(self, kind, stream, event):
+        """Work recorded into / waited for through a torch event, on a torch stream."""
+        if kind == CALL_RECORD:
+            self.slots[id(event)] = len(self.slots) % CALL_SLOTS
+            self.keep.append(event)
+        c = Call(kind=kind, lane=self._lane(stream.cuda_stream))
+        c.k[0] = self.slots[id(event)]
+        self.calls.append(c)
+
+    def finish(self):
+        self.array = (Call * len(self.calls))(*self.calls)
+        self.inputs = [t for c in self.array for t in (c.x, c.r) if t.data == self.x_ptr]
+        self.streams = (ctypes.c_void_p * len(self.lanes))(*self.lanes)
+        self.calls = None
+
+    def run(self, x_ptr: int, stream_ptr: int) -> int:
+        """Status of the run; the side streams are the ones of the first pass."""
+        if x_ptr != self.x_ptr:
+            for t in self.inputs:
+                t.data = x_ptr
+            self.x_ptr = x_ptr
+        self.streams[0] = stream_ptr
+        return _lib.rt3d_run_calls(self.array, len(self.array), self.streams, len(self.streams), None)
+
+
+def noting():
+    """The CallSequence in which this thread's calls are being noted, or None."""
+    return getattr(_recording, "seq", None)
+
+
+def _note(kind, stream, *args, **kw):
+    seq = getattr(_recording, "seq", None)
+    if seq is not None:
+        seq.note(kind, stream, *args, **kw)
+
+
 def rt3d_conv3d_sparse(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1, 1), pad=(0, 0, 0), relu=False,
                        algo=ALGO_AUTO, stream=None, x_pad_zero=False):
     """x, y: Tensor descriptors (device); bias: torch float32 device tensor [M] or None."""
-    _check(_lib.rt3d_conv3d_sparse(ctypes.byref(x), w.handle, _bias_ptr(bias),
-                                   ctypes.byref(_params(stride, pad, relu, algo, x_pad_zero)), ctypes.byref(y),
+    p = _params(stride, pad, relu, algo, x_pad_zero)
+    _check(_lib.rt3d_conv3d_sparse(ctypes.byref(x), w.handle, _bias_ptr(bias), ctypes.byref(p), ctypes.byref(y),
                                    _stream_ptr(stream)), "rt3d_conv3d_sparse")
+    _note(CALL_SPARSE, stream, x, y, None, w, bias, p)
 
 
 def rt3d_conv3d_sparse_noalloc(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1, 1), pad=(0, 0, 0), relu=False,
@@ -294,9 +410,10 @@ def rt3d_conv3d_sparse_fused(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1
     """y = pool(act(bias + conv(x) + residual)); residual: descriptor of a device tensor with the un-pooled
     output's extents or None; pool: (1|2, 1|2, 1|2) max-pool window = stride applied after the activation."""
     fz = Fusion(ctypes.pointer(residual) if residual is not None else None, int(pool[0]), int(pool[1]), int(pool[2]))
-    _check(_lib.rt3d_conv3d_sparse_fused(ctypes.byref(x), w.handle, _bias_ptr(bias),
-                                         ctypes.byref(_params(stride, pad, relu, algo, x_pad_zero)), ctypes.byref(fz),
+    p = _params(stride, pad, relu, algo, x_pad_zero)
+    _check(_lib.rt3d_conv3d_sparse_fused(ctypes.byref(x), w.handle, _bias_ptr(bias), ctypes.byref(p), ctypes.byref(fz),
                                          ctypes.byref(y), _stream_ptr(stream)), "rt3d_conv3d_sparse_fused")
+    _note(CALL_FUSED, stream, x, y, residual, w, bias, p, k=pool)
 
 
 def rt3d_conv2plus1d_fused(x: Tensor, w_s: Packed, bias_s, pad_s, relu_s, w_t: Packed, bias_t, pad_t, relu_t,
@@ -304,17 +421,19 @@ def rt3d_conv2plus1d_fused(x: Tensor, w_s: Packed, bias_s, pad_s, relu_s, w_t: P
     """Spatial 1xKhxKw conv then temporal 3x1x1 conv in one launch (all strides 1); Rt3dError with status
     ERR_UNSUPPORTED when the pair does not fit the fused kernel (run the two layers separately then)."""
     res = ctypes.pointer(residual) if residual is not None else None
-    _check(_lib.rt3d_conv2plus1d_fused(ctypes.byref(x), w_s.handle, _bias_ptr(bias_s),
-                                       ctypes.byref(_params((1, 1, 1), pad_s, relu_s, ALGO_AUTO)), w_t.handle,
-                                       _bias_ptr(bias_t), ctypes.byref(_params((1, 1, 1), pad_t, relu_t, ALGO_AUTO)),
-                                       res, ctypes.byref(y), _stream_ptr(stream)), "rt3d_conv2plus1d_fused")
+    ps, pt = _params((1, 1, 1), pad_s, relu_s, ALGO_AUTO), _params((1, 1, 1), pad_t, relu_t, ALGO_AUTO)
+    _check(_lib.rt3d_conv2plus1d_fused(ctypes.byref(x), w_s.handle, _bias_ptr(bias_s), ctypes.byref(ps), w_t.handle,
+                                       _bias_ptr(bias_t), ctypes.byref(pt), res, ctypes.byref(y), _stream_ptr(stream)),
+           "rt3d_conv2plus1d_fused")
+    _note(CALL_PAIR, stream, x, y, residual, w_s, bias_s, ps, w_t, bias_t, pt)
 
 
 def rt3d_conv3d_dense(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1, 1), pad=(0, 0, 0), relu=False,
                        algo=ALGO_AUTO, stream=None, x_pad_zero=False):
-    _check(_lib.rt3d_conv3d_dense(ctypes.byref(x), w.handle, _bias_ptr(bias),
-                                  ctypes.byref(_params(stride, pad, relu, algo, x_pad_zero)), ctypes.byref(y),
+    p = _params(stride, pad, relu, algo, x_pad_zero)
+    _check(_lib.rt3d_conv3d_dense(ctypes.byref(x), w.handle, _bias_ptr(bias), ctypes.byref(p), ctypes.byref(y),
                                   _stream_ptr(stream)), "rt3d_conv3d_dense")
+    _note(CALL_DENSE, stream, x, y, None, w, bias, p)
 
 
 def rt3d_conv3d_host(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1, 1), pad=(0, 0, 0), relu=False,
@@ -328,11 +447,13 @@ def rt3d_conv3d_host(x: Tensor, w: Packed, bias, y: Tensor, stride=(1, 1, 1), pa
 def rt3d_maxpool3d(x: Tensor, k, stride, pad, y: Tensor, stream=None):
     _check(_lib.rt3d_maxpool3d(ctypes.byref(x), *map(int, k), *map(int, stride), *map(int, pad), ctypes.byref(y),
                                _stream_ptr(stream)), "rt3d_maxpool3d")
+    _note(CALL_MAXPOOL, stream, x, y, k=(*k, *stride, *pad))
 
 
 def rt3d_add_relu(a: Tensor, b: Tensor, relu: bool, y: Tensor, stream=None):
     _check(_lib.rt3d_add_relu(ctypes.byref(a), ctypes.byref(b), int(bool(relu)), ctypes.byref(y),
                               _stream_ptr(stream)), "rt3d_add_relu")
+    _note(CALL_ADD, stream, a, y, b, k=(bool(relu),))
 
 
 def rt3d_kgs_group_norms(w, g_m: int, g_n: int, norm: int, norms, stream=None):

@@ -8,6 +8,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -15,6 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librt3d.so")
 SOURCES = ["api.cu", "pack.cpp", "simt_kernels.cu", "simt_conv_f32.cu", "umma_conv.cu", "umma_conv_pair.cu", "umma_conv_halo.cu", "umma_conv_st.cu", "umma_conv_sub.cu", "umma_smallc.cu", "reweight.cu", "debug_poison.cu"]
 HEADERS = ["kernels.h", "rt3d_internal.h", "umma_common.cuh", "umma_pair.cuh", "pdl.cuh", "tile_consts.h"]
+PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))   # extension module of the binding
 MICROBENCH = os.path.join(HERE, "rt3d_microbench")       # stand-alone instruction-rate microbenchmarks
 
 
@@ -31,7 +33,21 @@ def needs_build() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_pycall(force: bool = False) -> str:
+    """Compiles csrc/pycall.cpp, the extension module through which the layers of `nets` call the library."""
+    src = os.path.join(CSRC, "pycall.cpp")
+    deps = [src, os.path.join(ROOT, "include", "rt3d.h")]
+    if not force and os.path.exists(PYCALL) and all(os.path.getmtime(d) <= os.path.getmtime(PYCALL) for d in deps):
+        return PYCALL
+    tmp = PYCALL + f".tmp{os.getpid()}"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                           "-I", os.path.join(ROOT, "include"), "-o", tmp, src])
+    os.replace(tmp, PYCALL)
+    return PYCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_pycall(force)
     if not force and not needs_build():
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"

@@ -8,6 +8,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -146,6 +148,97 @@ bool overlaps(const rt3d_tensor* a, const rt3d_tensor* b) {
   const char* b0 = static_cast<const char*>(b->data);
   return a0 < b0 + tensor_span_bytes(b) && b0 < a0 + tensor_span_bytes(a);
 }
+
+// ------------------------------------------------------------------------ prepared calls
+thread_local rt3d_plan_info t_last_plan = {-1, 0, 0, 0, 0};
+std::atomic<int> g_plan_epoch{0};              // advanced by rt3d_debug_set: calls prepared before it are prepared again
+
+}  // namespace
+
+namespace rt3d {
+// Everything a convolution call is determined by.
+struct CallKey {
+  const void *x, *y, *res, *bias, *bias2;
+  uint64_t w2;                                 // the second handle, by its id: its address may be another handle's later
+  int32_t geo[24];                             // extents, pitches and dtypes of x, y and the residual
+  int32_t p[20];                               // both convolutions' parameters
+  int32_t misc[6];                             // device, entry point, fused pool, epoch
+};
+// One call of a handle, ready to launch: a user runs a layer on the same few buffers again and again, and validating,
+// choosing the kernel and encoding two or three tensor maps cost 1 to 2 us of the host's time for each call.
+struct PreparedCall {
+  CallKey key;
+  rt3d_plan_info info;
+  std::function<cudaError_t(cudaStream_t)> launch;
+};
+}  // namespace rt3d
+
+namespace {
+
+constexpr size_t kPreparedCalls = 8;           // per handle
+
+void put_tensor(const rt3d_tensor* t, int32_t* at) {
+  const int32_t v[8] = {1, t->n, t->t, t->h, t->w, t->c, t->c_stride, t->dtype};
+  memcpy(at, v, sizeof(v));
+}
+void put_params(const rt3d_conv_params* p, int32_t* at) {
+  const int32_t v[10] = {p->st, p->sh, p->sw, p->pt, p->ph, p->pw, p->relu, p->algo, p->x_pad_zero, p->concurrent};
+  memcpy(at, v, sizeof(v));
+}
+// False for arguments that the call will refuse anyway.
+bool make_key(CallKey* k, const rt3d_tensor* x, const rt3d_packed* w, const float* bias, const rt3d_conv_params* p,
+              const rt3d_tensor* y, const rt3d_tensor* res, int entry) {
+  int dev = 0;
+  if (!x || !w || !p || !y || cudaGetDevice(&dev) != cudaSuccess) return false;
+  memset(k, 0, sizeof(*k));
+  k->x = x->data; k->y = y->data; k->bias = bias;
+  put_tensor(x, k->geo);
+  put_tensor(y, k->geo + 8);
+  if (res) { k->res = res->data; put_tensor(res, k->geo + 16); }
+  put_params(p, k->p);
+  k->misc[0] = dev; k->misc[1] = entry; k->misc[5] = g_plan_epoch.load();
+  return true;
+}
+
+// Runs one call of a handle: from its prepared calls, or prepared now and kept.
+class Submit {
+ public:
+  Submit(rt3d_packed* w, const CallKey& key, cudaStream_t st) : w_(w), key_(key), st_(st) {}
+  // true: the call was found and has been run (or only planned), with *status as its result
+  bool again(rt3d_status* status) {
+    std::shared_ptr<PreparedCall> c;
+    {
+      std::lock_guard<std::mutex> lock(w_->mu);
+      for (const auto& e : w_->calls)
+        if (memcmp(&e->key, &key_, sizeof(key_)) == 0) { c = e; break; }
+    }
+    if (!c) return false;
+    *status = run(*c);
+    return true;
+  }
+  // A kernel launch chosen for this call.  `launch` must hold by value whatever it needs besides the handle's own memory.
+  rt3d_status operator()(const rt3d_plan_info& info, std::function<cudaError_t(cudaStream_t)> launch) {
+    auto c = std::make_shared<PreparedCall>(PreparedCall{key_, info, std::move(launch)});
+    {
+      std::lock_guard<std::mutex> lock(w_->mu);
+      if (w_->calls.size() < kPreparedCalls) w_->calls.push_back(c);
+      else w_->calls[w_->next_call++ % kPreparedCalls] = c;
+    }
+    return run(*c);
+  }
+
+ private:
+  rt3d_status run(const PreparedCall& c) {
+    t_last_plan = c.info;
+    if (t_plan_only) return RT3D_OK;
+    if (c.launch(st_) != cudaSuccess) return RT3D_ERR_CUDA;
+    g_launches.fetch_add(1);
+    return RT3D_OK;
+  }
+  rt3d_packed* w_;
+  const CallKey& key_;
+  cudaStream_t st_;
+};
 
 // ------------------------------------------------------------------------- device blobs
 DeviceBlob* find_blob(rt3d_packed* h, int dev) {
@@ -495,7 +588,7 @@ bool smallc_eligible(const DeviceState* d, rt3d_packed* w, const rt3d_tensor* x,
 }
 
 rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d, const SmallCLayout* L,
-                          const rt3d_tensor* x, const ConvGeom& g, const float* bias, rt3d_tensor* y, cudaStream_t st,
+                          const rt3d_tensor* x, const ConvGeom& g, const float* bias, rt3d_tensor* y, Submit& submit,
                           const void* residual, int rcs, int pool_h, int pool_w, bool x_pad_zero) {
   // pooled rows leave as whole 32-channel pieces through the bulk-store epilogue; a trailing 16-channel piece is
   // written by plain per-voxel stores, which know nothing of pooling
@@ -555,13 +648,11 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   const int sb[4] = {kSmallCTileW, 4, 1, 1};          // a warp owns 4 rows of 8 voxels of the 16 x 8 tile
   a.store_tma = encode_ymap(y, sb, pool_w, pool_h, 1, &ymap) ? 1 : 0;
   if (!a.store_tma && pool_h * pool_w > 1) return RT3D_ERR_UNSUPPORTED;
-  if (t_plan_only) return RT3D_OK;
-  if (launch_conv_umma_smallc(a, &xmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return RT3D_OK;
+  const int sms = d->sm_count;
+  return submit(rt3d_plan_info{3, L->n_pad, 1, 0, pool_h * pool_w > 1 ? 1 : 0}, [=](cudaStream_t st) {
+    return launch_conv_umma_smallc(a, &xmap, a.store_tma ? &ymap : nullptr, sms, st);
+  });
 }
-
-thread_local rt3d_plan_info t_last_plan = {-1, 0, 0, 0, 0};
 
 // Grows the handle's K-split workspace on this device: `bytes` of partial tiles and `cnt_bytes` of
 // counters / flags, which every kernel that uses them leaves zeroed.
@@ -587,7 +678,7 @@ rt3d_status ensure_splitk(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t
 // at least one tile per SM.  *launched = false (and RT3D_OK) when the caller should take another kernel.
 rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
                      const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, bool dense_entry,
-                     bool forced, cudaStream_t st, bool* launched) {
+                     bool forced, Submit& submit, bool* launched) {
   *launched = false;
   if (g.st != 1 || g.sh != 1 || g.sw != 1 || w->M > 256) return RT3D_OK;
   const int n_tile = round_up(w->M, 16);
@@ -639,13 +730,12 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   const bool rect = warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb);
   a.sbw = sb[0]; a.sbh = sb[1];
   a.store_tma = (rect && encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
-  t_last_plan = rt3d_plan_info{4, a.n_tile, 1, 0, 0};
   *launched = true;
-  if (t_plan_only) return RT3D_OK;
-  cudaError_t e = launch_conv_umma_halo(h, &xmap, u->wmap_half, a.store_tma ? &ymap : nullptr, d->sm_count, st);
-  if (e != cudaSuccess) return RT3D_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return RT3D_OK;
+  const int sms = d->sm_count;
+  const void* wmap = u->wmap_half;
+  return submit(rt3d_plan_info{4, a.n_tile, 1, 0, 0}, [=](cudaStream_t st) {
+    return launch_conv_umma_halo(h, &xmap, wmap, h.u.store_tma ? &ymap : nullptr, sms, st);
+  });
 }
 
 // Sub-tile kernel: blocks of 16 x 16 channels in which no kernel group keeps the step's location are skipped.
@@ -654,7 +744,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
 // tensor memory costs about as much as the dense MMAs of that step.
 // *launched = false (and RT3D_OK) when the handle cannot use it.
 rt3d_status try_sub(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
-                    const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, cudaStream_t st, bool* launched) {
+                    const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, Submit& submit, bool* launched) {
   *launched = false;
   if (w->is_dense) return RT3D_OK;
   SubArgs a;
@@ -679,12 +769,11 @@ rt3d_status try_sub(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   int sb[4] = {1, 1, 1, 1};
   const bool rect = warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb);
   a.store_tma = (rect && encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
-  t_last_plan = rt3d_plan_info{6, a.n_tile, 1, 0, 0};
   *launched = true;
-  if (t_plan_only) return RT3D_OK;
-  if (launch_conv_umma_sub(a, &xmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return RT3D_OK;
+  const int sms = d->sm_count;
+  return submit(rt3d_plan_info{6, a.n_tile, 1, 0, 0}, [=](cudaStream_t st) {
+    return launch_conv_umma_sub(a, &xmap, a.store_tma ? &ymap : nullptr, sms, st);
+  });
 }
 
 // Device copy of the register-blocked fp32 kernel's layout.
@@ -708,27 +797,16 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
 // Register-blocked fp32 kernel: every fp32 call whose kernel groups are whole 4 x 4 tiles.
 // *launched = false (and RT3D_OK) when the handle or the shape cannot use it.
 rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
-                    const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, cudaStream_t st, bool* launched) {
+                    const float* bias, rt3d_tensor* y, const void* res_data, int res_pitch, Submit& submit, bool* launched) {
   *launched = false;
   if (!f32_layout_possible(w)) return RT3D_OK;
-  struct Entry { ConvGeom g; int64_t nnz; int n; F32Plan plans[kF32MaxPlans]; };     // as in choose_box
-  thread_local Entry cache[16];
-  thread_local int used = 0, next = 0;
-  Entry* e = nullptr;
-  for (int i = 0; i < used && !e; ++i)
-    if (memcmp(&cache[i].g, &g, sizeof(g)) == 0 && cache[i].nnz == w->nnz) e = &cache[i];
-  if (!e) {
-    e = &cache[next];
-    next = (next + 1) % 16;
-    if (used < 16) ++used;
-    e->g = g; e->nnz = w->nnz;
-    e->n = conv_f32_plans(g, double(w->nnz) / (double(w->P) * w->Q * w->Ks), d->sm_count, e->plans);
-  }
+  F32Plan plans[kF32MaxPlans];
+  const int n_plans = conv_f32_plans(g, double(w->nnz) / (double(w->P) * w->Q * w->Ks), d->sm_count, plans);
   F32Args a;
   a.g = g;
-  for (int i = 0; i < e->n; ++i) {
+  for (int i = 0; i < n_plans; ++i) {
     const F32Layout* L = get_f32_layout(w);
-    if (!L || !conv_f32_fill(e->plans[i], *L, &a)) continue;
+    if (!L || !conv_f32_fill(plans[i], *L, &a)) continue;
     DeviceBlob::F32* u = nullptr;
     rt3d_status s = get_f32_blob(w, blob, L, &u);
     if (s != RT3D_OK) return s;
@@ -736,16 +814,20 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
     a.x = static_cast<const float*>(x->data); a.y = static_cast<float*>(y->data);
     a.bias = bias; a.residual = static_cast<const float*>(res_data); a.rcs = res_pitch;
     *launched = true;
-    if (t_plan_only) return RT3D_OK;
-    if (launch_conv_f32(a, e->plans[i], st) != cudaSuccess) return RT3D_ERR_CUDA;
-    g_launches.fetch_add(1);
-    return RT3D_OK;
+    const F32Plan plan = plans[i];
+    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](cudaStream_t st) { return launch_conv_f32(a, plan, st); });
   }
   return RT3D_OK;
 }
 
 rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
                       rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz = nullptr) {
+  CallKey key;
+  if (make_key(&key, x, wc, bias, p, y, fz ? fz->residual : nullptr, dense_entry ? 1 : 0)) {
+    if (fz) { key.misc[2] = fz->pool_t; key.misc[3] = fz->pool_h; key.misc[4] = fz->pool_w; }
+    rt3d_status found;
+    if (Submit(const_cast<rt3d_packed*>(wc), key, static_cast<cudaStream_t>(stream)).again(&found)) return found;
+  }
   ConvGeom g;
   if (!y) return RT3D_ERR_INVALID_ARG;
   const bool pooled = fz && (fz->pool_t != 1 || fz->pool_h != 1 || fz->pool_w != 1);
@@ -779,7 +861,7 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   if ((s = get_device_state(&d)) != RT3D_OK) return s;
   DeviceBlob* blob = nullptr;
   if ((s = get_blob(w, &blob)) != RT3D_OK) return s;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  Submit submit(w, key, static_cast<cudaStream_t>(stream));
 
   const bool can_umma = umma_eligible(d, w, x, y, p);
   const bool can_simt = w->g_m <= kMaxGroupSimt && w->g_n <= kMaxGroupSimt;
@@ -791,38 +873,34 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   const bool use_umma = want_umma || (p->algo == RT3D_ALGO_AUTO && can_umma);
   if (!use_umma) {
     if (pooled) return RT3D_ERR_UNSUPPORTED;
-    t_last_plan = rt3d_plan_info{0, 0, 1, 0, 0};
     bool launched = false;
-    s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, st, &launched);
+    s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
     if (s != RT3D_OK || launched) return s;
     if ((s = get_canonical(w, blob)) != RT3D_OK) return s;
-    if (t_plan_only) return RT3D_OK;
-    cudaError_t e = launch_conv_simt(w->dtype, g, x->data, y->data, blob->group_ptr, blob->pos_idx, blob->tiles, bias,
-                                     w->g_m, w->g_n, w->P, w->Q, dense_entry, res_data, res_pitch, st);
-    if (e != cudaSuccess) return RT3D_ERR_CUDA;
-    g_launches.fetch_add(1);
-    t_last_plan = rt3d_plan_info{0, 0, 1, 0, 0};
-    return RT3D_OK;
+    const void *xdata = x->data;
+    void* ydata = y->data;
+    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](cudaStream_t st) {
+      return launch_conv_simt(w->dtype, g, xdata, ydata, blob->group_ptr, blob->pos_idx, blob->tiles, bias, w->g_m, w->g_n,
+                              w->P, w->Q, dense_entry, res_data, res_pitch, st);
+    });
   }
 
   const SmallCLayout* SL = nullptr;
   if (p->algo != RT3D_ALGO_UMMA_PAIR && p->algo != RT3D_ALGO_UMMA_HALO && p->algo != RT3D_ALGO_UMMA_SUB && (!pooled || pl_t == 1) &&
       smallc_eligible(d, w, x, y, p, &SL)) {
-    s = launch_smallc(w, blob, d, SL, x, g, bias, y, st, res_data, res_pitch, pl_h, pl_w, p->x_pad_zero != 0);
-    if (s == RT3D_OK) t_last_plan = rt3d_plan_info{3, SL->n_pad, 1, 0, pooled ? 1 : 0};
-    return s;
+    return launch_smallc(w, blob, d, SL, x, g, bias, y, submit, res_data, res_pitch, pl_h, pl_w, p->x_pad_zero != 0);
   }
 
   if ((p->algo == RT3D_ALGO_AUTO || p->algo == RT3D_ALGO_UMMA_HALO) && !pooled) {
     bool launched = false;
-    s = try_halo(w, blob, d, x, g, bias, y, res_data, res_pitch, dense_entry, p->algo == RT3D_ALGO_UMMA_HALO, st, &launched);
+    s = try_halo(w, blob, d, x, g, bias, y, res_data, res_pitch, dense_entry, p->algo == RT3D_ALGO_UMMA_HALO, submit, &launched);
     if (s != RT3D_OK || launched) return s;
   }
   if (p->algo == RT3D_ALGO_UMMA_HALO) return RT3D_ERR_UNSUPPORTED;
   if (p->algo == RT3D_ALGO_UMMA_SUB) {
     bool launched = false;
     if (!pooled && !dense_entry) {
-      s = try_sub(w, blob, d, x, g, bias, y, res_data, res_pitch, st, &launched);
+      s = try_sub(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
       if (s != RT3D_OK || launched) return s;
     }
     return RT3D_ERR_UNSUPPORTED;
@@ -930,14 +1008,16 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
       a.tail_scratch = blob->splitk; a.tail_flags = blob->splitk_cnt;
     }
   }
-  const void* ym = a.store_tma ? &ymap : nullptr;
-  t_last_plan = rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0};
-  if (t_plan_only) return RT3D_OK;
-  cudaError_t e = use_pair ? launch_conv_umma_pair(a, &xmap, u->wmap_half, ym, d->sm_count, st)
-                           : launch_conv_umma(a, &xmap, u->wmap, ym, d->sm_count, st);
-  if (e != cudaSuccess) return RT3D_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return RT3D_OK;
+  const int sms = d->sm_count;
+  const void* wmap = use_pair ? u->wmap_half : u->wmap;
+  return submit(rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0},
+                [=](cudaStream_t st) {
+    UmmaArgs now = a;                              // a later call of another shape may have moved the handle's workspace
+    if (a.n_splits > 1) { now.scratch = blob->splitk; now.counters = blob->splitk_cnt; }
+    if (a.tail_workers > 0) { now.tail_scratch = blob->splitk; now.tail_flags = blob->splitk_cnt; }
+    const void* ym = a.store_tma ? &ymap : nullptr;
+    return use_pair ? launch_conv_umma_pair(now, &xmap, wmap, ym, sms, st) : launch_conv_umma(now, &xmap, wmap, ym, sms, st);
+  });
 }
 
 
@@ -947,6 +1027,13 @@ rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* wsc, const
                              const rt3d_packed* wtc, const float* bias_t, const rt3d_conv_params* pt,
                              const rt3d_tensor* res, rt3d_tensor* y, void* stream) {
   if (!wsc || !wtc || !ps || !pt || !y) return RT3D_ERR_INVALID_ARG;
+  CallKey key;
+  if (make_key(&key, x, wsc, bias_s, ps, y, res, 2)) {
+    key.w2 = wtc->id; key.bias2 = bias_t;
+    put_params(pt, key.p + 10);
+    rt3d_status found;
+    if (Submit(const_cast<rt3d_packed*>(wsc), key, static_cast<cudaStream_t>(stream)).again(&found)) return found;
+  }
   ConvGeom g;
   rt3d_status s = make_geom(x, wsc, ps, nullptr, &g);
   if (s != RT3D_OK) return s;
@@ -1000,12 +1087,11 @@ rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* wsc, const
   CUtensorMap xmap;
   ConvGeom unit = g;
   if ((s = encode_xmap(x, unit, TileBox{1, 1, a.hh, a.hw}, &xmap)) != RT3D_OK) return s;
-  t_last_plan = rt3d_plan_info{5, a.n1, 1, 0, 0};
-  if (t_plan_only) return RT3D_OK;
-  cudaError_t e = launch_conv_umma_st(a, &xmap, u1->wmap_half, u2->wmap_half, d->sm_count, static_cast<cudaStream_t>(stream));
-  if (e != cudaSuccess) return RT3D_ERR_CUDA;
-  g_launches.fetch_add(1);
-  return RT3D_OK;
+  const int sms = d->sm_count;
+  const void *m1 = u1->wmap_half, *m2 = u2->wmap_half;
+  return Submit(ws, key, static_cast<cudaStream_t>(stream))(rt3d_plan_info{5, a.n1, 1, 0, 0}, [=](cudaStream_t st) {
+    return launch_conv_umma_st(a, &xmap, m1, m2, sms, st);
+  });
 }
 
 }  // namespace
@@ -1258,6 +1344,77 @@ rt3d_status rt3d_add_relu(const rt3d_tensor* a, const rt3d_tensor* b, int relu, 
   return RT3D_OK;
 }
 
+rt3d_status rt3d_run_calls(const rt3d_call* calls, int32_t n, void* const* streams, int32_t n_streams, int32_t* failed) {
+  if (failed) *failed = -1;
+  if (!calls || n < 0 || !streams || n_streams < 1) return RT3D_ERR_INVALID_ARG;
+  // Events of the record / wait steps: one set per host thread and device.  A wait refers to the record issued last before
+  // it, so a set serves one run after the other.
+  struct Events {
+    int device = -1;
+    cudaEvent_t slot[RT3D_CALL_SLOTS] = {};
+  };
+  struct EventSets {
+    std::vector<Events> sets;
+    ~EventSets() {
+      for (Events& e : sets)
+        for (cudaEvent_t ev : e.slot)
+          if (ev) cudaEventDestroy(ev);
+    }
+  };
+  thread_local EventSets own;
+  Events* events = nullptr;
+  for (int32_t i = 0; i < n; ++i) {
+    const rt3d_call& c = calls[i];
+    rt3d_status s = RT3D_ERR_INVALID_ARG;
+    if (c.lane >= 0 && c.lane < n_streams) {
+      void* st = streams[c.lane];
+      rt3d_tensor y = c.y;
+      switch (c.kind) {
+        case RT3D_CALL_SPARSE: s = conv_impl(&c.x, c.w, c.bias, &c.p, &y, st, false); break;
+        case RT3D_CALL_DENSE: s = conv_impl(&c.x, c.w, c.bias, &c.p, &y, st, true); break;
+        case RT3D_CALL_FUSED: {
+          const rt3d_fusion fz{c.r.data ? &c.r : nullptr, c.k[0], c.k[1], c.k[2]};
+          s = rt3d_conv3d_sparse_fused(&c.x, c.w, c.bias, &c.p, &fz, &y, st);
+          break;
+        }
+        case RT3D_CALL_PAIR:
+          s = conv2plus1d_impl(&c.x, c.w, c.bias, &c.p, c.w2, c.bias2, &c.p2, c.r.data ? &c.r : nullptr, &y, st);
+          break;
+        case RT3D_CALL_MAXPOOL:
+          s = rt3d_maxpool3d(&c.x, c.k[0], c.k[1], c.k[2], c.k[3], c.k[4], c.k[5], c.k[6], c.k[7], c.k[8], &y, st);
+          break;
+        case RT3D_CALL_ADD: s = rt3d_add_relu(&c.x, &c.r, c.k[0], &y, st); break;
+        case RT3D_CALL_RECORD:
+        case RT3D_CALL_WAIT: {
+          if (c.k[0] < 0 || c.k[0] >= RT3D_CALL_SLOTS) break;
+          if (!events) {
+            int dev = 0;
+            if (cudaGetDevice(&dev) != cudaSuccess) { s = RT3D_ERR_CUDA; break; }
+            for (Events& e : own.sets)
+              if (e.device == dev) events = &e;
+            if (!events) {
+              own.sets.emplace_back();
+              events = &own.sets.back();
+              events->device = dev;
+            }
+          }
+          cudaEvent_t& ev = events->slot[c.k[0]];
+          if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) { s = RT3D_ERR_CUDA; break; }
+          const cudaError_t e = c.kind == RT3D_CALL_RECORD ? cudaEventRecord(ev, static_cast<cudaStream_t>(st))
+                                                           : cudaStreamWaitEvent(static_cast<cudaStream_t>(st), ev, 0);
+          s = e == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
+          break;
+        }
+      }
+    }
+    if (s != RT3D_OK) {
+      if (failed) *failed = i;
+      return s;
+    }
+  }
+  return RT3D_OK;
+}
+
 rt3d_status rt3d_conv3d_cost(const rt3d_tensor* x, const rt3d_packed* w, const rt3d_conv_params* p,
                              int64_t* kept_macs, int64_t* dense_macs, int64_t* alg_bytes) {
   ConvGeom g;
@@ -1430,6 +1587,7 @@ void rt3d_plan_begin(void) { t_plan_only = true; }
 void rt3d_plan_end(void) { t_plan_only = false; }
 
 rt3d_status rt3d_debug_set(int what, long long value) {
+  g_plan_epoch.fetch_add(1);
   if (what == RT3D_DEBUG_WAIT_CYCLES) { if (value < 0) return RT3D_ERR_INVALID_ARG; g_debug_wait_cycles.store(value); return RT3D_OK; }
   if (what == RT3D_DEBUG_DROP_LAST_LOAD) { g_debug_drop_last_load.store(value != 0); return RT3D_OK; }
   if (what == RT3D_DEBUG_T_GROUPS) { g_ts_enabled.store(value != 0); return RT3D_OK; }

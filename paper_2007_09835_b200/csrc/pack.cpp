@@ -2,6 +2,7 @@
 // inverse, and the derivation of the tensor-core weight layout from the canonical arrays.
 // Pure host code: no CUDA calls, usable without a GPU.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <new>
 #include <utility>
@@ -348,6 +349,8 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
   if (Ks64 > 65535) return RT3D_ERR_INVALID_ARG;
   rt3d_packed* h = new (std::nothrow) rt3d_packed;
   if (!h) return RT3D_ERR_ALLOC;
+  static std::atomic<uint64_t> next_id{1};
+  h->id = next_id.fetch_add(1);
   try {
     h->M = M; h->N = N; h->Kt = Kt; h->Kh = Kh; h->Kw = Kw; h->g_m = g_m; h->g_n = g_n;
     h->P = ceil_div(M, g_m); h->Q = ceil_div(N, g_n); h->Ks = int(Ks64);

@@ -132,7 +132,10 @@ struct DeviceBlob {
 
 }  // namespace rt3d
 
+namespace rt3d { struct PreparedCall; }
+
 struct rt3d_packed {
+  uint64_t id = 0;                   // never used twice in a process
   int M = 0, N = 0, Kt = 0, Kh = 0, Kw = 0, g_m = 0, g_n = 0, P = 0, Q = 0, Ks = 0;
   int dtype = 0, is_vanilla = 0, is_dense = 0;
   int64_t nnz = 0;
@@ -145,6 +148,9 @@ struct rt3d_packed {
   std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw, built on first use
   std::unique_ptr<rt3d::F32Layout> f32_layout;        // built on first use
   std::vector<rt3d::DeviceBlob*> blobs;
+  // The last few calls made with this handle, ready to launch again (api.cu); the oldest one gives way.
+  std::vector<std::shared_ptr<rt3d::PreparedCall>> calls;
+  size_t next_call = 0;
 };
 
 namespace rt3d {
