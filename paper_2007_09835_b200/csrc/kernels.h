@@ -62,6 +62,12 @@ cudaError_t launch_maxpool3d(int dtype, const void* x, int n, int t, int h, int 
 cudaError_t launch_add_relu(int dtype, const void* a, int acs, const void* b, int bcs, void* y, int ycs,
                             int64_t voxels, int c, int relu, cudaStream_t stream);
 
+// Fills the zeroed tiles [steps][n_tile][64] of a tensor-core layout from the canonical arrays (layout.cu), on the legacy
+// default stream.
+cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const void* tiles, const int32_t* slots,
+                                   int M, int N, int Ks, int g_m, int g_n, int Q, int n_groups, int64_t nnz, int n_tile,
+                                   int n_chunks, void* wtiles, size_t bytes);
+
 // Output-voxel box of one tensor-core tile: bn*bt*bh*bw <= 128 voxels.
 struct TileBox { int bn, bt, bh, bw; };
 

@@ -5,6 +5,8 @@
 #include <atomic>
 #include <cstring>
 #include <new>
+#include <system_error>
+#include <thread>
 #include <utility>
 
 #include "rt3d_internal.h"
@@ -41,10 +43,33 @@ static float tile_value(const rt3d_packed* p, int64_t e, int i, int j) {
   return reinterpret_cast<const float*>(p->tiles.data())[o];
 }
 
+// Runs fn(i) for i in [0, n), on up to eight threads if each gets at least `grain` units of work in all.
+template <typename F>
+static void parallel_for(int n, int64_t work, int64_t grain, const F& fn) {
+  int threads = int(std::min<int64_t>(std::min<int64_t>(work / grain, n), std::min(8u, std::thread::hardware_concurrency())));
+  if (threads <= 1) {
+    for (int i = 0; i < n; ++i) fn(i);
+    return;
+  }
+  std::atomic<int> next{0};
+  const int step = std::max(1, n / (threads * 8));       // pieces small enough to even out, large enough to be few
+  auto worker = [&] {
+    for (int i0 = next.fetch_add(step); i0 < n; i0 = next.fetch_add(step))
+      for (int i = i0; i < std::min(n, i0 + step); ++i) fn(i);
+  };
+  std::vector<std::thread> pool;
+  try {
+    for (int t = 1; t < threads; ++t) pool.emplace_back(worker);
+  } catch (const std::system_error&) {                   // no more threads to be had: the others do the work
+  }
+  worker();
+  for (std::thread& t : pool) t.join();
+}
+
 // For each bundle of n_tile output channels, list the (kernel location, 64-channel chunk)
-// steps in which at least one kernel group of the bundle keeps that location, and build the
-// matching [n_tile][64] weight tiles (zeros where a group prunes the location).  Steps are
-// ordered by location, then chunk.
+// steps in which at least one kernel group of the bundle keeps that location; each step has an [n_tile][64]
+// weight tile (zeros where a group prunes the location), which the device fills in (fill_umma_tiles does it
+// here, for checks).  Steps are ordered by location, then chunk.
 // `t_groups`: the order is (kh, kw), chunk, kt instead, and the steps that differ only in kt form a
 // group (grp_ptr / grp_first): the CTA-pair kernel stages one input tile, Kt - 1 frames deeper, per group.
 const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
@@ -103,26 +128,27 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
     }
     L.step_ptr[b + 1] = base + cnt;
     L.max_steps = std::max(L.max_steps, int(cnt));
-    L.wtiles.resize(size_t(base + cnt) * n_tile * kChunk, 0);
-    // pass 2: scatter the kept tiles
-    for (int pr = p_lo; pr < p_hi; ++pr)
-      for (int q = 0; q < p->Q; ++q)
-        for (int32_t e = p->group_ptr[pr * p->Q + q]; e < p->group_ptr[pr * p->Q + q + 1]; ++e)
-          for (int i = 0; i < p->g_m; ++i) {
-            const int m = pr * p->g_m + i;
-            if (m < m_lo || m >= m_hi) continue;
-            for (int j = 0; j < p->g_n; ++j) {
-              const int c = q * p->g_n + j;
-              if (c >= p->N) continue;
-              const int32_t s = slot[size_t(p->pos_idx[e]) * L.n_chunks + c / kChunk];
-              L.wtiles[(size_t(s) * n_tile + (m - m_lo)) * kChunk + c % kChunk] =
-                  reinterpret_cast<const uint16_t*>(p->tiles.data())[(int64_t(e) * p->g_m + i) * p->g_n + j];
-            }
-          }
+    L.slots.insert(L.slots.end(), slot.begin(), slot.end());
   }
   if (t_groups) L.grp_first.push_back(int32_t(L.steps.size()));     // sentinel: end of the last group
   auto res = p->umma_layouts.emplace(key, std::move(L));
   return &res.first->second;
+}
+
+// The weight tiles of a layout, as the device kernel builds them.
+std::vector<uint16_t> fill_umma_tiles(const rt3d_packed* p, const UmmaLayout& L) {
+  std::vector<uint16_t> wtiles(L.steps.size() * size_t(L.n_tile) * kChunk, 0);
+  for (int pr = 0; pr < p->P; ++pr)
+    for (int q = 0; q < p->Q; ++q)
+      for (int32_t e = p->group_ptr[size_t(pr) * p->Q + q]; e < p->group_ptr[size_t(pr) * p->Q + q + 1]; ++e)
+        for (int i = 0; i < p->g_m && pr * p->g_m + i < p->M; ++i)
+          for (int j = 0; j < p->g_n && q * p->g_n + j < p->N; ++j) {
+            const int m = pr * p->g_m + i, c = q * p->g_n + j, b = m / L.n_tile;
+            const int32_t s = L.slots[(size_t(b) * p->Ks + p->pos_idx[e]) * L.n_chunks + c / kChunk];
+            wtiles[(size_t(s) * L.n_tile + (m - b * L.n_tile)) * kChunk + c % kChunk] =
+                reinterpret_cast<const uint16_t*>(p->tiles.data())[(int64_t(e) * p->g_m + i) * p->g_n + j];
+          }
+  return wtiles;
 }
 
 // Layout of the sub-tile kernel (see SubLayout and SubStep).
@@ -287,34 +313,53 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
   L.n_stages = ceil_div(n_quads, L.quads);
   const int Ks = p->Ks, rm = p->g_m / 4, rn = p->g_n / 4;
   const float* tiles = reinterpret_cast<const float*>(p->tiles.data());
-  std::vector<int32_t> kept(size_t(2) * L.quads * Ks);   // packed entry that holds (row, quad, location), or -1
+  const int64_t work = int64_t(p->M) * p->N * Ks, grain = int64_t(1) << 18;
   const size_t n_lists = size_t(L.n_stages) * L.n_sets;
-  L.entry_ptr.reserve(n_lists + 1);
-  L.tile_ptr.reserve(n_lists + 1);
-  L.counts.reserve(n_lists);
-  L.entries.reserve(size_t(p->nnz) * rm * rn);           // at most one entry per 4 x 4 tile
-  L.tiles.resize(size_t(p->nnz) * rm * rn * 16);
-  float* out = L.tiles.data();
-  L.entry_ptr.push_back(0);
-  L.tile_ptr.push_back(0);
-  for (int st = 0; st < L.n_stages; ++st)
+  L.entry_ptr.assign(n_lists + 1, 0);
+  L.tile_ptr.assign(n_lists + 1, 0);
+  L.counts.assign(n_lists, 0);
+  // Packed entry that holds (row, quad, location) of one (stage, row set), or -1.
+  auto find_kept = [&](int st, int s, std::vector<int32_t>& kept) {
+    kept.assign(size_t(2) * L.quads * Ks, -1);
+    for (int r = 0; r < 2 && s * 2 + r < n_rows; ++r)
+      for (int ql = 0; ql < L.quads && st * L.quads + ql < n_quads; ++ql) {
+        const size_t grp = size_t((s * 2 + r) / rm) * p->Q + (st * L.quads + ql) / rn;
+        int32_t* at = kept.data() + size_t(r * L.quads + ql) * Ks;
+        for (int32_t e = p->group_ptr[grp]; e < p->group_ptr[grp + 1]; ++e) at[p->pos_idx[e]] = e;
+      }
+  };
+  parallel_for(L.n_stages, work, grain, [&](int st) {
+    std::vector<int32_t> kept;
     for (int s = 0; s < L.n_sets; ++s) {
-      std::fill(kept.begin(), kept.end(), -1);
-      for (int r = 0; r < 2 && s * 2 + r < n_rows; ++r)
-        for (int ql = 0; ql < L.quads && st * L.quads + ql < n_quads; ++ql) {
-          const size_t grp = size_t((s * 2 + r) / rm) * p->Q + (st * L.quads + ql) / rn;
-          for (int32_t e = p->group_ptr[grp]; e < p->group_ptr[grp + 1]; ++e)
-            kept[size_t(r * L.quads + ql) * Ks + p->pos_idx[e]] = e;
-        }
+      find_kept(st, s, kept);
       int count[3] = {0, 0, 0};
+      for (int v = 0; v < L.quads * Ks; ++v) {
+        const bool e0 = kept[size_t(v)] >= 0, e1 = kept[size_t(L.quads) * Ks + v] >= 0;
+        count[0] += e0 && e1; count[1] += e0 && !e1; count[2] += !e0 && e1;
+      }
+      const size_t at = size_t(st) * L.n_sets + s;
+      L.counts[at] = count[0] | count[1] << 16;
+      L.entry_ptr[at + 1] = count[0] + count[1] + count[2];
+      L.tile_ptr[at + 1] = 2 * count[0] + count[1] + count[2];
+    }
+  });
+  for (size_t i = 0; i < n_lists; ++i) { L.entry_ptr[i + 1] += L.entry_ptr[i]; L.tile_ptr[i + 1] += L.tile_ptr[i]; }
+  L.entries.resize(size_t(L.entry_ptr[n_lists]));
+  L.tiles.allocate(size_t(L.tile_ptr[n_lists]) * 64);
+  parallel_for(L.n_stages, work, grain, [&](int st) {
+    std::vector<int32_t> kept;
+    for (int s = 0; s < L.n_sets; ++s) {
+      find_kept(st, s, kept);
+      const size_t at = size_t(st) * L.n_sets + s;
+      uint32_t* entry = L.entries.data() + L.entry_ptr[at];
+      float* out = reinterpret_cast<float*>(L.tiles.data()) + size_t(L.tile_ptr[at]) * 16;
       for (int list = 0; list < 3; ++list)
         for (int ql = 0; ql < L.quads; ++ql)
           for (int k = 0; k < Ks; ++k) {
             const int32_t e[2] = {kept[size_t(ql) * Ks + k], kept[size_t(L.quads + ql) * Ks + k]};
             const int which = e[0] >= 0 ? (e[1] >= 0 ? 0 : 1) : (e[1] >= 0 ? 2 : -1);
             if (which != list) continue;
-            ++count[list];
-            L.entries.push_back(uint32_t(k) | uint32_t(ql) << 16);
+            *entry++ = uint32_t(k) | uint32_t(ql) << 16;
             for (int r = 0; r < 2; ++r) {
               if (e[r] < 0) continue;
               const int ib = ((s * 2 + r) % rm) * 4, jb = ((st * L.quads + ql) % rn) * 4;
@@ -322,11 +367,8 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
                 std::memcpy(out, tiles + (int64_t(e[r]) * p->g_m + ib + i) * p->g_n + jb, 16);
             }
           }
-      L.counts.push_back(count[0] | count[1] << 16);
-      L.entry_ptr.push_back(int32_t(L.entries.size()));
-      L.tile_ptr.push_back(int32_t((out - L.tiles.data()) / 16));
     }
-  L.tiles.resize(size_t(out - L.tiles.data()));
+  });
   for (int lg = 0; lg < 4; ++lg)
     for (int st = 0; st < L.n_stages; ++st)
       for (int s = 0; s < L.n_sets; s += 1 << lg) {
@@ -357,54 +399,75 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
     h->dtype = dtype; h->is_dense = is_dense;
     const int Ks = h->Ks;
     const size_t esz = dtype == RT3D_BF16 ? 2 : 4;
-    h->group_ptr.resize(size_t(h->P) * h->Q + 1);
+    const size_t n_groups = size_t(h->P) * h->Q;
+    h->group_ptr.resize(n_groups + 1);
+    // Both passes walk the weights and the mask in memory order, the Ks values of one kernel at a time, and are shared
+    // between threads by rows of groups.
+    const int64_t work = int64_t(M) * N * Ks, grain = int64_t(1) << 18;
     // pass 1: group-level decisions with the uniformity check of the KGS definition
-    std::vector<uint8_t> keep(size_t(h->P) * h->Q * Ks);
-    int64_t nnz = 0;
-    bool vanilla = true;
-    for (int pr = 0; pr < h->P; ++pr)
+    std::vector<uint8_t> keep(mask ? n_groups * Ks : 0);
+    std::atomic<bool> uniform{true}, vanilla{true};
+    parallel_for(h->P, work, grain, [&](int pr) {
       for (int q = 0; q < h->Q; ++q) {
+        const size_t grp = size_t(pr) * h->Q + q;
+        if (!mask) { h->group_ptr[grp + 1] = Ks; continue; }
+        uint8_t* kp = keep.data() + grp * Ks;
+        uint8_t differs = 0;
+        for (int i = 0; i < g_m && pr * g_m + i < M; ++i)
+          for (int j = 0; j < g_n && q * g_n + j < N; ++j) {
+            const uint8_t* row = mask + (int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks;
+            if (i == 0 && j == 0) {
+              for (int k = 0; k < Ks; ++k) kp[k] = row[k] != 0;
+            } else {
+              for (int k = 0; k < Ks; ++k) differs |= uint8_t(kp[k] ^ uint8_t(row[k] != 0));
+            }
+          }
+        if (differs) uniform = false;
         int kept_here = 0;
-        for (int k = 0; k < Ks; ++k) {
-          int decided = -1;
-          if (!mask) decided = 1;
-          else
-            for (int i = 0; i < g_m && pr * g_m + i < M; ++i)
-              for (int j = 0; j < g_n && q * g_n + j < N; ++j) {
-                const int bit = mask[(int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks + k] ? 1 : 0;
-                if (decided < 0) decided = bit;
-                else if (decided != bit) { delete h; return RT3D_ERR_MASK_NOT_GROUP_UNIFORM; }
-              }
-          keep[(size_t(pr) * h->Q + q) * Ks + k] = uint8_t(decided > 0);
-          kept_here += decided > 0;
-        }
+        for (int k = 0; k < Ks; ++k) kept_here += kp[k];
         if (kept_here != 0 && kept_here != Ks) vanilla = false;
-        nnz += kept_here;
+        h->group_ptr[grp + 1] = kept_here;
       }
-    if (nnz > 0x7FFFFFFF) { delete h; return RT3D_ERR_UNSUPPORTED; }
+    });
+    if (!uniform) { delete h; return RT3D_ERR_MASK_NOT_GROUP_UNIFORM; }
+    int64_t nnz = 0;
+    for (size_t grp = 0; grp < n_groups; ++grp) {
+      nnz += h->group_ptr[grp + 1];
+      if (nnz > 0x7FFFFFFF) { delete h; return RT3D_ERR_UNSUPPORTED; }
+      h->group_ptr[grp + 1] = int32_t(nnz);
+    }
+    h->group_ptr[0] = 0;
     h->nnz = nnz;
     h->is_vanilla = vanilla;
     h->pos_idx.resize(size_t(nnz));
-    h->tiles.assign(size_t(nnz) * g_m * g_n * esz, 0);
+    h->tiles.allocate(size_t(nnz) * g_m * g_n * esz);
     // pass 2: emit index and tiles
-    int64_t e = 0;
-    for (int pr = 0; pr < h->P; ++pr)
+    parallel_for(h->P, work, grain, [&](int pr) {
+      const int rows = std::min(g_m, M - pr * g_m);
       for (int q = 0; q < h->Q; ++q) {
-        h->group_ptr[size_t(pr) * h->Q + q] = int32_t(e);
-        for (int k = 0; k < Ks; ++k) {
-          if (!keep[(size_t(pr) * h->Q + q) * Ks + k]) continue;
-          h->pos_idx[size_t(e)] = uint16_t(k);
-          for (int i = 0; i < g_m && pr * g_m + i < M; ++i)
-            for (int j = 0; j < g_n && q * g_n + j < N; ++j) {
-              const float v = w[(int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks + k];
-              const size_t o = (size_t(e) * g_m + i) * g_n + j;
-              if (dtype == RT3D_BF16) reinterpret_cast<uint16_t*>(h->tiles.data())[o] = f32_to_bf16_bits(v);
-              else reinterpret_cast<float*>(h->tiles.data())[o] = v;
+        const size_t grp = size_t(pr) * h->Q + q;
+        const int32_t e0 = h->group_ptr[grp], n_e = h->group_ptr[grp + 1] - e0;
+        const int cols = std::min(g_n, N - q * g_n);
+        uint16_t* pos = h->pos_idx.data() + e0;
+        int n = 0;
+        for (int k = 0; k < Ks; ++k)
+          if (!mask || keep[grp * Ks + k]) pos[n++] = uint16_t(k);
+        unsigned char* out = h->tiles.data() + size_t(e0) * g_m * g_n * esz;
+        if (rows < g_m || cols < g_n) std::memset(out, 0, size_t(n_e) * g_m * g_n * esz);    // kernels that do not exist
+        for (int i = 0; i < rows; ++i)
+          for (int j = 0; j < cols; ++j) {
+            const float* row = w + (int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks;
+            const size_t at = size_t(i) * g_n + j, step = size_t(g_m) * g_n;
+            if (dtype == RT3D_BF16) {
+              uint16_t* o = reinterpret_cast<uint16_t*>(out) + at;
+              for (int e = 0; e < n_e; ++e) o[e * step] = f32_to_bf16_bits(row[pos[e]]);
+            } else {
+              float* o = reinterpret_cast<float*>(out) + at;
+              for (int e = 0; e < n_e; ++e) o[e * step] = row[pos[e]];
             }
-          ++e;
-        }
+          }
       }
-    h->group_ptr[size_t(h->P) * h->Q] = int32_t(e);
+    });
   } catch (const std::bad_alloc&) {
     delete h;
     return RT3D_ERR_ALLOC;
@@ -467,6 +530,7 @@ rt3d_status unpack_device_layout(const rt3d_packed* p, int n_tile, bool t_groups
   if (!p || !w_out) return RT3D_ERR_INVALID_ARG;
   const UmmaLayout* L = get_umma_layout(const_cast<rt3d_packed*>(p), n_tile, t_groups);
   if (!L) return RT3D_ERR_UNSUPPORTED;
+  const std::vector<uint16_t> wtiles = fill_umma_tiles(p, *L);
   if (t_groups) {
     // groups tile each bundle's list exactly; inside a group only kt changes, upwards
     if (int(L->grp_ptr.size()) != L->n_bundles + 1 || L->grp_first.size() != size_t(L->grp_ptr.back()) + 1 ||
@@ -499,7 +563,7 @@ rt3d_status unpack_device_layout(const rt3d_packed* p, int n_tile, bool t_groups
       for (int r = 0; r < L->n_tile && b * L->n_tile + r < p->M; ++r)
         for (int j = 0; j < kChunk && ch * kChunk + j < p->N; ++j)
           w_out[(int64_t(b * L->n_tile + r) * p->N + (ch * kChunk + j)) * p->Ks + kpos] =
-              bf16_bits_to_f32(L->wtiles[(size_t(s) * L->n_tile + r) * kChunk + j]);
+              bf16_bits_to_f32(wtiles[(size_t(s) * L->n_tile + r) * kChunk + j]);
     }
   return RT3D_OK;
 }

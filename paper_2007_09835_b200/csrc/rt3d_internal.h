@@ -42,7 +42,7 @@ struct UmmaLayout {
   int n_chunks = 0;                  // ceil(N / 64)
   std::vector<int32_t> step_ptr;     // [n_bundles + 1] offsets into steps / weight tiles
   std::vector<int32_t> steps;        // encoded (kt,kh,kw,chunk), only non-empty steps of each bundle
-  std::vector<uint16_t> wtiles;      // [steps.size()][n_tile][64] bf16 bits, zero where pruned / absent
+  std::vector<int32_t> slots;        // [n_bundles][Ks][n_chunks] index of that (location, chunk)'s step, -1 if it has none
   int max_steps = 0;                 // longest bundle list
   bool t_groups = false;             // steps ordered (kh, kw), chunk, kt; groups = runs that differ only in kt
   std::vector<int32_t> grp_ptr;      // [n_bundles + 1] offsets into grp_first            (t_groups only)
@@ -80,6 +80,20 @@ struct SubLayout {
   int max_steps = 0;                 // longest bundle list
 };
 
+// Bytes that are written once, without the zeros a vector would fill them with first.
+class RawBytes {
+ public:
+  void allocate(size_t n) { data_.reset(new unsigned char[n]); size_ = n; }
+  unsigned char* data() { return data_.get(); }
+  const unsigned char* data() const { return data_.get(); }
+  size_t size() const { return size_; }
+  unsigned char operator[](size_t i) const { return data_[i]; }
+
+ private:
+  std::unique_ptr<unsigned char[]> data_;
+  size_t size_ = 0;
+};
+
 // Layout of the register-blocked fp32 kernel (simt_conv_f32.cu).  Kernel groups are cut into 4 x 4 tiles; a "row set" is
 // two consecutive rows of four output channels, a stage is `quads` consecutive quads of input channels.  For each
 // (stage, row set), stage-major, three lists of entries, one after the other: the (quad, kernel location) places that
@@ -90,7 +104,7 @@ struct F32Layout {
   std::vector<int32_t> tile_ptr;     // [n_stages * n_sets + 1]
   std::vector<int32_t> counts;       // [n_stages * n_sets] entries of the first list | of the second << 16
   std::vector<uint32_t> entries;     // kernel location | quad inside the stage << 16
-  std::vector<float> tiles;          // [tile][16]: [output pair][output][input]
+  RawBytes tiles;                    // float [tile][4 outputs][4 inputs]
   int max_entries[4] = {0, 0, 0, 0}; // most entries / tiles of a stage in 1, 2, 4, 8 aligned consecutive row sets
   int max_tiles[4] = {0, 0, 0, 0};
 };
@@ -103,6 +117,7 @@ struct DeviceBlob {
   uint16_t* pos_idx = nullptr;
   void* tiles = nullptr;
   struct Umma {
+    void* base = nullptr;                       // owns the index arrays
     void* wtiles = nullptr;
     int32_t* step_ptr = nullptr;
     int32_t* steps = nullptr;
@@ -141,7 +156,7 @@ struct rt3d_packed {
   int64_t nnz = 0;
   std::vector<int32_t> group_ptr;
   std::vector<uint16_t> pos_idx;
-  std::vector<unsigned char> tiles;  // nnz * g_m * g_n elements of float or bf16 bits
+  rt3d::RawBytes tiles;              // nnz * g_m * g_n elements of float or bf16 bits
   std::mutex mu;                     // guards the lazily built members below
   std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by n_tile (+ 4096: the t-grouped order)
   std::map<int, rt3d::SubLayout> sub_layouts;     // keyed by n_tile
@@ -154,6 +169,9 @@ struct rt3d_packed {
 };
 
 namespace rt3d {
+
+// The weight tiles [steps.size()][n_tile][64] of a layout on the host (checks; the device fills its own).
+std::vector<uint16_t> fill_umma_tiles(const rt3d_packed* p, const UmmaLayout& L);
 
 // Default bundle width for M output channels: as few bundles as possible with n_tile <= 256.
 int default_n_tile(int M);

@@ -19,7 +19,9 @@
 // 524 us (7.2 -> 34 TFLOP/s kept); 16 -> 32 channels, 8 x 28 x 28 voxels 27.4 -> 9.6 us, half of it launch and latency.
 //
 // Two buffers; the copies of stage s + 1 (cp.async) run while stage s is multiplied.
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "kernels.h"
 #include "pdl.cuh"
@@ -257,7 +259,7 @@ double choose_box_f32(const ConvGeom& g, int lanes, int voxels, double weight, F
   for (int vh = 1; vh <= voxels; vh *= 2) {
     const int vt = voxels / vh;
     for (int bw = 1; bw <= g.Wo && bw <= lanes; ++bw) {
-      if (bw < g.Wo && bw % 4) continue;               // whole rows, or runs of 64 bytes
+      if (bw < g.Wo && bw % 8 && bw != 4) continue;    // whole rows, or runs of 64 bytes and more
       for (int lh = 1; lh <= ceil_div(g.Ho, vh) && bw * lh <= lanes; ++lh) {
         const int most_t = ceil_div(g.To, vt), lt = lanes / (bw * lh) < most_t ? lanes / (bw * lh) : most_t;
         const int bt = lt * vt, bh = lh * vh;
@@ -277,7 +279,7 @@ double choose_box_f32(const ConvGeom& g, int lanes, int voxels, double weight, F
 
 // Cycles of the busiest SM for every variant, fitted to timings on B200: an entry costs a scheduler 25 + V (4 + 10 h) with
 // four warps at work (h = tiles per entry) and a warp by itself 45 + V (12 + 30 h); a stage costs its copies and barriers.
-int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
+static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
   const int Ks = g.Kt * g.Kh * g.Kw, n_rows = ceil_div(g.M, 4), n_quads = ceil_div(g.c, 4), quads = f32_stage_quads(Ks);
   const int n_stages = ceil_div(n_quads, quads);
   double cost[kF32MaxPlans];
@@ -309,6 +311,24 @@ int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plan
       ++n;
     }
   return n;
+}
+
+int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
+  // The search takes 0.1 ms; a call in chunks asks for the same shape for every chunk.
+  struct Entry { ConvGeom g; double density; int n; F32Plan plans[kF32MaxPlans]; };
+  thread_local Entry cache[4];
+  thread_local int next = 0;
+  for (const Entry& e : cache)
+    if (e.n > 0 && memcmp(&e.g, &g, sizeof(g)) == 0 && e.density == density) {
+      std::copy(e.plans, e.plans + e.n, plans);
+      return e.n;
+    }
+  Entry& e = cache[next];
+  next = (next + 1) % 4;
+  e.g = g; e.density = density;
+  e.n = search_plans(g, density, sm_count, e.plans);
+  std::copy(e.plans, e.plans + e.n, plans);
+  return e.n;
 }
 
 bool conv_f32_fill(const F32Plan& p, const F32Layout& L, F32Args* a) {
