@@ -234,24 +234,33 @@ __device__ __forceinline__ void epilogue_cols(const uint32_t* v, const float* bi
       }
     }
   }
-  if (valid >= NC) {
 #pragma unroll
-    for (int q = 0; q < NC / 8; ++q) {
-      uint4 o;
-      if (relu) {                                  // activation and rounding in one instruction per pair
-        o.x = cvt_relu_bf16x2(f[8 * q], f[8 * q + 1]); o.y = cvt_relu_bf16x2(f[8 * q + 2], f[8 * q + 3]);
-        o.z = cvt_relu_bf16x2(f[8 * q + 4], f[8 * q + 5]); o.w = cvt_relu_bf16x2(f[8 * q + 6], f[8 * q + 7]);
-      } else {
-        __nv_bfloat162* po = reinterpret_cast<__nv_bfloat162*>(&o);
+  for (int q = 0; q < NC / 8; ++q) {
+    if (8 * q >= valid) break;
+    uint4 o;
+    if (relu) {                                  // activation and rounding in one instruction per pair
+      o.x = cvt_relu_bf16x2(f[8 * q], f[8 * q + 1]); o.y = cvt_relu_bf16x2(f[8 * q + 2], f[8 * q + 3]);
+      o.z = cvt_relu_bf16x2(f[8 * q + 4], f[8 * q + 5]); o.w = cvt_relu_bf16x2(f[8 * q + 6], f[8 * q + 7]);
+    } else {
+      __nv_bfloat162* po = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) po[e] = __floats2bfloat162_rn(f[8 * q + 2 * e], f[8 * q + 2 * e + 1]);
-      }
-      reinterpret_cast<uint4*>(dst)[q] = o;
+      for (int e = 0; e < 4; ++e) po[e] = __floats2bfloat162_rn(f[8 * q + 2 * e], f[8 * q + 2 * e + 1]);
     }
-  } else {
-#pragma unroll
-    for (int q = 0; q < NC; ++q)                 // static indices: f stays in registers
-      if (q < valid) dst[q] = __float2bfloat16_rn(relu ? fmaxf(f[q], 0.f) : f[q]);
+    // A row's last 16-byte unit may hold fewer than eight channels: 8, 4 and 2 bytes as needed, the padding behind them is
+    // left alone.  (Channel by channel, the 13 two-byte stores of a thread's second piece made the 45 outputs of the
+    // R(2+1)D stem cost twice what 48 do: 74 -> 38 us.)
+    const int left = valid - 8 * q;
+    if (left >= 8) {
+      reinterpret_cast<uint4*>(dst)[q] = o;
+    } else {
+      __nv_bfloat16* d = dst + 8 * q;
+      if (left & 4) *reinterpret_cast<uint2*>(d) = make_uint2(o.x, o.y);
+      if (left & 2) *reinterpret_cast<uint32_t*>(d + (left & 4)) = (left & 4) ? o.z : o.x;
+      if (left & 1) {
+        const uint32_t w = (left & 4) ? ((left & 2) ? o.w : o.z) : ((left & 2) ? o.y : o.x);
+        *reinterpret_cast<uint16_t*>(d + (left & 6)) = uint16_t(w);
+      }
+    }
   }
 }
 
@@ -287,11 +296,10 @@ __device__ __forceinline__ void add_partials(uint32_t (&v)[32], bool wide, int c
 // One voxel row of a finished accumulator tile: columns [0, n_cols) of the TMEM buffer at `taddr`
 // hold output channels m_base.. ; channels >= M are dropped.  Warp-uniform control flow around the
 // TMEM loads (.sync.aligned); `in_range` may differ per lane.
-// `res_row`: the voxel's residual row at channel m_base (nullptr: none); `res_pitch_left` = channels from
-// m_base to the end of the residual tensor's channel pitch.
+// `res_row`: the voxel's residual row at channel m_base (nullptr: none); `res_left` = channels from m_base to M.
 __device__ __forceinline__ void epilogue_row(uint32_t taddr, int n_cols, bool has_acc, bool in_range,
                                              const float* bias_s, int relu, __nv_bfloat16* dst, int m_base, int M,
-                                             const __nv_bfloat16* res_row = nullptr, int res_pitch_left = 0,
+                                             const __nv_bfloat16* res_row = nullptr, int res_left = 0,
                                              int col0 = 0, int col_step = 32, const float* extra_first = nullptr,
                                              const float* extra = nullptr, size_t extra_stride = 0, int n_extra = 0,
                                              uint32_t acc2_off = 0) {
@@ -310,8 +318,8 @@ __device__ __forceinline__ void epilogue_row(uint32_t taddr, int n_cols, bool ha
     if (extra_first != nullptr) add_partials(v, wide, col, extra_first, extra, extra_stride, n_extra);
     const __nv_bfloat16* res = res_row ? res_row + col : nullptr;
     const float* bs = bias_s ? bias_s + m0 : nullptr;
-    if (wide) epilogue_cols<32>(v, bs, relu, dst + col, M - m0, res, res_pitch_left - col);
-    else epilogue_cols<16>(v, bs, relu, dst + col, M - m0, res, res_pitch_left - col);
+    if (wide) epilogue_cols<32>(v, bs, relu, dst + col, M - m0, res, res_left - col);
+    else epilogue_cols<16>(v, bs, relu, dst + col, M - m0, res, res_left - col);
   }
 }
 
@@ -405,7 +413,8 @@ __device__ __forceinline__ void epilogue_piece_tma(const uint32_t* v, const floa
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float2 t = __bfloat1622float2(pr[e]);
-          f[8 * k + 2 * e] += t.x; f[8 * k + 2 * e + 1] += t.y;
+          // channels beyond the last: whatever the residual's padding holds must not reach the output's
+          f[8 * k + 2 * e] += 8 * k + 2 * e < res_avail ? t.x : 0.f; f[8 * k + 2 * e + 1] += 8 * k + 2 * e + 1 < res_avail ? t.y : 0.f;
         }
       }
     }
@@ -477,7 +486,7 @@ __device__ __forceinline__ void epilogue_piece_tma(const uint32_t* v, const floa
 __device__ __forceinline__ void epilogue_row_tma(uint32_t taddr, int n_cols, bool has_acc, bool warp_rows_valid,
                                                  bool in_range, const float* bias_s, int relu, __nv_bfloat16* dst,
                                                  int m_base, int M, int lane, TmaStore& ts,
-                                                 const __nv_bfloat16* res_row = nullptr, int res_pitch_left = 0,
+                                                 const __nv_bfloat16* res_row = nullptr, int res_left = 0,
                                                  const PoolLanes* pool = nullptr, const float* extra_first = nullptr,
                                                  const float* extra = nullptr, size_t extra_stride = 0,
                                                  int n_extra = 0, int col0 = 0, int col_step = 32,
@@ -497,9 +506,9 @@ __device__ __forceinline__ void epilogue_row_tma(uint32_t taddr, int n_cols, boo
     if (extra_first != nullptr) add_partials(v, wide, col, extra_first, extra, extra_stride, n_extra);
     const __nv_bfloat16* res = (res_row && in_range) ? res_row + col : nullptr;
     if (wide) {
-      if (warp_rows_valid) epilogue_piece_tma(v, bias_s ? bias_s + m0 : nullptr, relu, m0, lane, ts, res, res_pitch_left - col, pool);
+      if (warp_rows_valid) epilogue_piece_tma(v, bias_s ? bias_s + m0 : nullptr, relu, m0, lane, ts, res, res_left - col, pool);
     } else if (in_range) {
-      epilogue_cols<16>(v, bias_s ? bias_s + m0 : nullptr, relu, dst + col, M - m0, res, res_pitch_left - col);
+      epilogue_cols<16>(v, bias_s ? bias_s + m0 : nullptr, relu, dst + col, M - m0, res, res_left - col);
     }
   }
 }

@@ -346,7 +346,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
       const uint32_t taddr = tmem_base + (uint32_t(quad * 32) << 16) + buf * uint32_t(a.n_tile);
       __nv_bfloat16* dst = yb + vox * a.g.ycs + m_base;
       const __nv_bfloat16* res = (rb != nullptr && in_range) ? rb + vox * a.rcs + m_base : nullptr;
-      const int res_left = a.rcs - m_base;
+      const int res_left = a.g.M - m_base;
       if (two_sets) {
         ts.c1 = c.w0 + bw_0; ts.c2 = c.h0 + bh_0; ts.c3 = c.t0 + bt_0; ts.c4 = c.n0 + bn_0;
         for (int col = half * 32; col < a.n_tile; col += 64) {

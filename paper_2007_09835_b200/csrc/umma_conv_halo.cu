@@ -242,10 +242,10 @@ conv3d_umma_halo_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
         }
         const __nv_bfloat16* res = res_row ? res_row + col : nullptr;
         if (wide && a.store_tma) {
-          if (quad * 32 < box_rows) epilogue_piece_tma(v, bias_s + col, a.g.relu, col, lane, ts, res, a.rcs - col, nullptr);
+          if (quad * 32 < box_rows) epilogue_piece_tma(v, bias_s + col, a.g.relu, col, lane, ts, res, a.g.M - col, nullptr);
         } else if (in_range) {
-          if (wide) epilogue_cols<32>(v, bias_s + col, a.g.relu, dst + col, a.g.M - col, res, a.rcs - col);
-          else epilogue_cols<16>(v, bias_s + col, a.g.relu, dst + col, a.g.M - col, res, a.rcs - col);
+          if (wide) epilogue_cols<32>(v, bias_s + col, a.g.relu, dst + col, a.g.M - col, res, a.g.M - col);
+          else epilogue_cols<16>(v, bias_s + col, a.g.relu, dst + col, a.g.M - col, res, a.g.M - col);
         }
       }
       tc_fence_before();

@@ -440,7 +440,7 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
       if (kDual && units_here == 1 && (gg & 1u)) taddr += uint32_t(a.n_tile);
       gg += uint32_t(units_here > 0 ? units_here : 0);
       const __nv_bfloat16* res = (rb != nullptr && in_range) ? rb + vox * a.rcs + m_base : nullptr;
-      const int res_left = a.rcs - m_base;
+      const int res_left = a.g.M - m_base;
       if (wk.nparts > 1 && wk.part != 0) {
         // A share of a tile another pair owns: leave the raw partial sums in scratch and raise this warp's flag.
         // It is the first segment of this pair's range.

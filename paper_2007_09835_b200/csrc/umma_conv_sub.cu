@@ -234,7 +234,7 @@ conv3d_umma_sub_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
         const uint32_t taddr = tmem_base + (uint32_t(quad * 32) << 16) + uint32_t(col0);
         __nv_bfloat16* dst = yb + vox * a.g.ycs + m_base;
         const __nv_bfloat16* res = (rb != nullptr && in_range) ? rb + vox * a.rcs + m_base : nullptr;
-        const int res_left = a.rcs - m_base;
+        const int res_left = a.g.M - m_base;
         if (a.store_tma) {
           ts.c1 = c.w0 + bw_0; ts.c2 = c.h0 + bh_0; ts.c3 = c.t0 + bt_0; ts.c4 = c.n0 + bn_0;
           epilogue_row_tma(taddr, n_cols, c.nsteps > 0, quad * 32 < box_rows, in_range, bias_s, a.g.relu, dst, m_base,

@@ -195,9 +195,9 @@ conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid
         // pooling windows are 1 or 2 wide: the division is a shift
         ts.c1 = (iw * kSmallCTileW) >> (a.pool_w - 1); ts.c2 = (ih * kSmallCTileH + quad * 4) >> (a.pool_h - 1); ts.c3 = to; ts.c4 = nn;
         epilogue_row_tma(taddr, a.n_pad, a.n_pairs > 0, true, in_range, bias_e, a.g.relu, yb + vox * a.g.ycs, 0, a.g.M,
-                         lane, ts, res, a.rcs, pool);
+                         lane, ts, res, a.g.M, pool);
       } else {
-        epilogue_row(taddr, a.n_pad, a.n_pairs > 0, in_range, bias_e, a.g.relu, yb + vox * a.g.ycs, 0, a.g.M, res, a.rcs);
+        epilogue_row(taddr, a.n_pad, a.n_pairs > 0, in_range, bias_e, a.g.relu, yb + vox * a.g.ycs, 0, a.g.M, res, a.g.M);
       }
       tc_fence_before();
       __syncwarp();

@@ -500,3 +500,30 @@ def test_padding_channels_of_the_output(algo):
     assert ((unit == 9.0) | (unit == 0.0)).all()
     if algo == "simt":
         assert (unit == 9.0).all()
+
+
+@pytest.mark.parametrize("cin,cout,k,x", [(3, 45, (1, 7, 7), (1, 2, 33, 18)), (3, 9, (3, 3, 3), (1, 2, 17, 9)),         # small C_in
+                                          (64, 1, (1, 3, 3), (8, 8, 24, 24)), (24, 29, (3, 1, 1), (8, 8, 24, 24)),      # halo
+                                          (96, 150, (3, 3, 3), (1, 3, 9, 9)), (256, 71, (1, 1, 1), (1, 3, 9, 9)),       # single CTA
+                                          (96, 23, (3, 3, 3), (16, 4, 28, 28)), (130, 267, (3, 3, 3), (8, 4, 28, 28))])  # CTA pairs
+def test_last_unit_of_ragged_output_channels(cin, cout, k, x):
+    """Output channels that end inside a 16-byte unit, on every tensor-core kernel, with and without a residual whose own
+    padding holds NaNs: right values, zeros (or nothing) in the unit's padding channels, the next unit untouched."""
+    spec = synth.ConvSpec("unit", cin, cout, k, (1, 1, 1), tuple(v // 2 for v in k), True)
+    L = synth.make_layer(spec, 52, cout, 4, 4, "bernoulli", 0.5)
+    xs = synth.make_input(6200, x + (cin,))
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.bfloat16)
+    xd = nets.to_device(xs)
+    shape = lay.out_shape(xd)
+    res = synth.uniform_pm1(9, shape[:4] + (cout,))
+    rd = nets.to_device(res)
+    rd[..., cout:] = float("nan")
+    for residual in (False, True):
+        y = torch.full(shape[:4] + (shape[4] + 8,), 9.0, dtype=torch.bfloat16, device="cuda")
+        lay.fused(xd, y, residual=rd if residual else None)
+        assert rt3d.rt3d_last_device_status() == rt3d.OK and rt3d.rt3d_last_plan()["kernel"] != 0
+        ref = oracle.conv3d(xs, L["w"], L["mask"], L["bias"], spec.stride, spec.pad, False)
+        ref = np.maximum(ref + (oracle.bf16_round(res) if residual else 0.0), 0.0)
+        check(nets.to_numpy(y, cout), ref, torch.bfloat16, "unit")
+        unit = y[..., cout:shape[4]]
+        assert ((unit == 9.0) | (unit == 0.0)).all() and (y[..., shape[4]:] == 9.0).all()
