@@ -164,10 +164,7 @@ rt3d_status rt3d_unpack_device_layout_tgroups(const rt3d_packed* p, int n_tile, 
 rt3d_status rt3d_unpack_sub_layout(const rt3d_packed* p, int n_tile, float* w_out);
 
 /* Upload the handle's device blobs to the current CUDA device now (otherwise done by the
- * first compute call), and look up, once per device, the device address of the fixed workspace of
- * rt3d_conv3d_sparse_noalloc (that look-up may make the CUDA runtime load this library's module on the
- * device, which is when the driver sets the workspace's memory aside).  Call it before any stream capture.
- * Synchronises the device. */
+ * first compute call).  Call it before any stream capture.  Synchronises the device. */
 rt3d_status rt3d_packed_prepare(rt3d_packed* p);
 
 void rt3d_packed_free(rt3d_packed* p);
@@ -256,10 +253,8 @@ rt3d_status rt3d_conv2plus1d_fused(const rt3d_tensor* x, const rt3d_packed* w_s,
  * Some callers cannot call cudaMalloc at the point where they run a layer: code inside a
  * real-time or latency-critical loop, code that runs while another component owns the device's
  * memory budget, or a host thread that must never block on the allocator's device-wide
- * synchronisation.  For them this entry point runs the same tensor-core convolution, including its
- * K-split variant whose fp32 partial tiles need scratch memory, without any allocation: the scratch
- * is a fixed array inside the library (16 MiB of partial tiles plus 4 KiB of counters, resident on
- * every GPU that loads the library until the process exits).
+ * synchronisation.  For them this entry point runs the single-CTA tensor-core convolution, whose K
+ * splits exchange their fp32 partial tiles through the SMs' shared memory, without any allocation.
  *   - Same arguments, layouts and alignment rules as rt3d_conv3d_sparse (device x, y, bias); bf16 only.
  *   - Everything that does need an allocation must exist already: call rt3d_packed_prepare(w) on this
  *     device beforehand, else RT3D_ERR_NOT_PREPARED.  Shapes the tensor-core kernel does not take
@@ -269,13 +264,6 @@ rt3d_status rt3d_conv2plus1d_fused(const rt3d_tensor* x, const rt3d_packed* w_s,
  *     channels that some kernel group of the tile's channels keeps (the longest such list counts).  If S > 1 and (output tiles x S) partial tiles of 128 x n_tile floats exceed
  *     16 MiB, or there are more than 128 output tiles, the call is rejected with
  *     RT3D_ERR_WORKSPACE and nothing is launched (rt3d_conv3d_sparse has no such limit).
- *   - The device address of the workspace is looked up by rt3d_packed_prepare (once per device, with that
- *     device current; do it before any stream capture begins).  This entry point itself never allocates
- *     or frees device or pinned memory and never triggers that look-up: without a prepared handle on the
- *     device it returns RT3D_ERR_NOT_PREPARED.
- *   - All calls on a device share the one workspace, which keeps the previous call's contents; the
- *     entry point clears the counters it needs on `stream` before the kernel.  Two calls whose
- *     kernels may overlap on the GPU (different streams) race on it: serialise them.
  *   - Results agree with rt3d_conv3d_sparse within the library's tolerance (the split count, and so
  *     the fp32 summation order, may differ); repeated calls give identical bits.
  */

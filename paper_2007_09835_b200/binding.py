@@ -397,8 +397,7 @@ def rt3d_conv3d_sparse_noalloc(x: Tensor, w: Packed, bias, y: Tensor, stride=(1,
                                algo=ALGO_AUTO, stream=None):
     """rt3d_conv3d_sparse for callers that must not allocate device memory at call time (a real-time
     loop, a thread that may not block on the allocator): the handle must have been prepared on this
-    device (`w.prepare()`), the K-split scratch is a fixed 16 MiB array inside the library, and a call
-    that would need more raises Rt3dError with status ERR_WORKSPACE."""
+    device (`w.prepare()`), and a K-split call with more than 16 MiB of partial tiles raises Rt3dError with status ERR_WORKSPACE."""
     _check(_lib.rt3d_conv3d_sparse_noalloc(ctypes.byref(x), w.handle, _bias_ptr(bias),
                                            ctypes.byref(_params(stride, pad, relu, algo)), ctypes.byref(y),
                                            _stream_ptr(stream)), "rt3d_conv3d_sparse_noalloc")

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -51,7 +52,7 @@ long long debug_wait_cycles() {
   return v;
 }
 
-// All device blobs of live handles: their K-split counters are cleared when a kernel reported a timeout.
+// All device blobs of live handles: their tail-split flags are cleared when a kernel reported a timeout.
 std::mutex g_blobs_mu;
 std::vector<DeviceBlob*> g_blobs;
 
@@ -431,43 +432,63 @@ TileBox choose_box_search(const ConvGeom& g, bool prefer_deep) {
   return best;
 }
 
-// Bundle width and number of K splits for a call.  Model (fitted to timings on B200): a K step costs
-// the issuing thread about 175 ns of barrier hand-shake plus 4 MMA issues, or the tensor time of the
-// step if that is longer; a layer with few output tiles runs as many serial steps per CTA as its
-// step list is long, so it is split along K (at the price of writing and re-reading fp32 partial
-// tiles) until the SMs are occupied.  The step count of each candidate bundle width comes from the
-// handle's real step lists: with kernel groups as wide as a bundle, pruned (location, chunk) steps
-// vanish and a narrower bundle that matches the group height can win.
-struct UmmaPlan { int n_tile, n_splits; };
+// Bundle width, number of K splits and kernel (single CTAs or CTA pairs) for a call.  Model, fitted to timings on B200:
+//  - A K step takes its tensor time or the time its operands need from L2, 65 bytes per clock and SM whatever the kernel
+//    (at 128 columns 32 KB for a CTA, 24 KB for one of a pair, 14 KB where the kt steps share an input tile): this bounds
+//    nearly every layer with few tiles.
+//  - A launch has 5 us around its steps, one of CTA pairs 6.9 us (cluster set-up, its tables).
+//  - A split costs the shares' way through shared memory and the wait for a cluster's SMs, growing with its size.
+// Measured against it: 128 -> 256 at 8 x 28 x 28 (49 tiles, 54 steps) single 18.5 us, pairs 16.0 us; 256 -> 512 at 4 x 14 x 14
+// (7 tiles, 108 steps) S = 4: 14.5 us, pairs 19 us; 512 -> 1152 1x3x3 at 8 x 2 x 7 x 7: 192 columns S = 3 16.5 us, 64 columns
+// unsplit 21.8 us.  The step count of each candidate width comes from the handle's real step lists where kernel groups
+// are tall enough for whole steps to vanish; a narrower bundle that matches the group height can win there.
+struct UmmaPlan { int n_tile, n_splits; bool pair; };
 
-UmmaPlan pick_plan(rt3d_packed* w, long long m_tiles, int sm_count) {
+UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_count) {
   const int M = w->M;
   const int widest = default_n_tile(M);
-  UmmaPlan best{widest, 1};
+  const bool tall = w->g_m >= 16 && !w->is_dense;
+  UmmaPlan best{widest, 1, false};
   double best_ns = -1.0;
-  static const int kSplits[] = {1, 2, 3, 4, 6, 8};
-  for (int n = widest; n >= 32; n = (n > 128 ? 128 : n / 2)) {
+  int last = 0;
+  for (int b = ceil_div(M, widest);; ++b) {
+    // widths that cut M evenly, in whole 32-column pieces below the widest (odd ones for splits only: a layer with enough
+    // tiles takes the widest); tall groups: halves, which match their heights
+    int n = tall ? (b == ceil_div(M, widest) ? widest : last > 128 ? 128 : last / 2) : round_up(ceil_div(M, b), b == ceil_div(M, widest) ? 16 : 32);
+    if (last && (n >= last || n < 32)) {
+      if (n < 32 || n <= 32) break;
+      continue;
+    }
+    last = n;
     if (n % 16) break;
-    // narrower bundles only pay when they let pruned steps drop out (groups at least 16 rows high)
-    // or when the layer has too few tiles; for the paper's 4..8-row groups the lists are full anyway
     const int bundles = ceil_div(M, n);
+    if (n != widest && !tall && n != 128 && n != 64 && bundles * n * 14 > round_up(M, 16) * 15) continue;   // padding columns
     const long long items = m_tiles * bundles;
     double steps = double(w->Ks) * ceil_div(w->N, kChunk);      // full lists: true for groups a few rows high
-    if (w->g_m >= 16 && !w->is_dense) {
+    if (tall) {
       const UmmaLayout* L = get_umma_layout(w, n);
       if (!L) break;
       steps = items < sm_count ? double(L->max_steps) : double(L->steps.size()) / bundles;
     }
-    const double issue = 175.0 + 4.0 * (25.0 + 0.06 * n), tensor = 1.4 * n;
-    const double step_ns = issue > tensor ? issue : tensor;
-    for (int S : kSplits) {
-      if (S > 1 && (steps / S < 8 || items >= 2LL * sm_count)) continue;
-      const double waves = double(ceil_div64(items * S, sm_count));
-      double ns = waves * (steps / S) * step_ns;
-      // partial tile out (every split) and S partial tiles back in (the CTA that arrives last), plus the
-      // traffic of all partials (written once, read once) at about 2.5 TB/s
-      if (S > 1) ns += 3000.0 + (1.0 + S) * n * 4.0 + double(items) * S * (kTileM * n * 4.0 * 2.0) / 2500.0;
-      if (best_ns < 0 || ns < best_ns * 0.97) { best = UmmaPlan{n, S}; best_ns = ns; }
+    constexpr double kByteNs = 1.0 / (65.0 * 1.85);
+    const double step_ns = std::max({1.08 * n, (kTileM * 128.0 + 128.0 * n) * kByteNs, 204.0});
+    for (int S = 1; S <= 8; ++S) {
+      const int capacity = umma_split_capacity(S, sm_count);
+      if (capacity == 0 || (S > 1 && (steps / S < 4 || items >= 2LL * sm_count))) continue;
+      if (S == 1 && n != widest && (n & (n - 1))) continue;
+      const double waves = double(ceil_div64(items * S, capacity));
+      const double ns = S == 1 ? 5000.0 + waves * steps * step_ns : waves * (7100.0 + 0.32 * n * S * S + steps / S * step_ns);
+      if (best_ns < 0 || ns < best_ns * 0.98) { best = UmmaPlan{n, S, false}; best_ns = ns; }
+    }
+    if (umma_pair_supported(n, bundles) && (n == widest || (n & (n - 1)) == 0)) {
+      const bool ts = g.Kt >= 2 && g.Kt <= 8 && g.st == 1 && g.To >= 4 && (n <= 128 || g.Kh * g.Kw >= 4);
+      const double a_bytes = kTileM * 128.0 * (ts ? 1.25 / g.Kt : 1.0);
+      const double pair_ns = std::max({(n <= 128 ? 1.3 : 1.1) * n, (a_bytes + 64.0 * n) * kByteNs, 165.0});
+      // a last round that is not full is shared out along K where the items are long enough
+      const double rounds = double((m_tiles + 1) / 2 * bundles) / (sm_count / 2);
+      const double whole = std::ceil(rounds) * steps * pair_ns, shared = 5000.0 + rounds * steps * pair_ns;
+      const double ns = 6900.0 + (rounds <= 1.0 || whole < shared ? whole : shared);
+      if (ns < best_ns * 0.97) { best = UmmaPlan{n, 1, true}; best_ns = ns; }
     }
     if (n == 32) break;
   }
@@ -663,8 +684,8 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   });
 }
 
-// Grows the handle's K-split workspace on this device: `bytes` of partial tiles and `cnt_bytes` of
-// counters / flags, which every kernel that uses them leaves zeroed.
+// Grows the handle's tail-split workspace on this device: `bytes` of partial tiles and `cnt_bytes` of
+// flags, which every kernel that uses them leaves zeroed.
 rt3d_status ensure_splitk(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t cnt_bytes) {
   std::lock_guard<std::mutex> lock(w->mu);
   if (blob->splitk_bytes < bytes) {
@@ -728,7 +749,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   a.bias = bias; a.y = y->data; a.sched = d->sched;
   a.residual = res_data; a.rcs = res_pitch;
   a.pool_t = a.pool_h = a.pool_w = 1;
-  a.n_splits = 1; a.scratch = nullptr; a.counters = nullptr;
+  a.n_splits = 1;
   a.tail_workers = 0; a.tail_scratch = nullptr; a.tail_flags = nullptr;
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = 0; a.debug_drop_last_load = 0;
@@ -930,7 +951,7 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
   a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
   const long long m_tiles = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
-  UmmaPlan plan = pick_plan(w, m_tiles, d->sm_count);
+  UmmaPlan plan = pick_plan(w, g, m_tiles, d->sm_count);
   if (pooled) {                     // pooling lives in the TMA-store epilogue, which a K split does not use
     // A layer this small is faster split over K and pooled by a second launch: AUTO declines the fusion.
     if (p->algo == RT3D_ALGO_AUTO && plan.n_splits > 1) return RT3D_ERR_UNSUPPORTED;
@@ -939,12 +960,12 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   // CTA pairs: two tiles per MMA.  Worth it when every pair has work; forced by RT3D_ALGO_UMMA_PAIR.
   bool use_pair = false;
   if (p->algo == RT3D_ALGO_UMMA_PAIR) {
-    plan = UmmaPlan{default_n_tile(w->M), 1};
+    plan = UmmaPlan{default_n_tile(w->M), 1, true};
     if (!umma_pair_supported(plan.n_tile, ceil_div(w->M, plan.n_tile))) return RT3D_ERR_UNSUPPORTED;
     use_pair = true;
   } else if (p->algo == RT3D_ALGO_AUTO && plan.n_splits == 1 &&
              umma_pair_supported(plan.n_tile, ceil_div(w->M, plan.n_tile)) &&
-             m_tiles * ceil_div(w->M, plan.n_tile) >= d->sm_count) {
+             (plan.pair || m_tiles * ceil_div(w->M, plan.n_tile) >= d->sm_count)) {
     use_pair = true;
   }
   if (pooled && plan.n_tile % 32) return RT3D_ERR_UNSUPPORTED;      // pooled rows leave as whole 32-channel pieces
@@ -984,17 +1005,10 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.step_ptr = u->step_ptr; a.steps = u->steps;
   a.bias = bias; a.y = y->data; a.sched = d->sched;
   a.residual = res_data; a.rcs = res_pitch;
-  a.n_splits = plan.n_splits; a.scratch = nullptr; a.counters = nullptr;
+  a.n_splits = plan.n_splits;
   a.tail_workers = 0; a.tail_scratch = nullptr; a.tail_flags = nullptr;
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = debug_wait_cycles(); a.debug_drop_last_load = g_debug_drop_last_load.load();
-  if (a.n_splits > 1) {
-    // split-K workspace of this handle on this device: partial tiles + per-warp arrival counters
-    const long long tiles = m_tiles * L->n_bundles;
-    if ((s = ensure_splitk(w, blob, size_t(tiles) * a.n_splits * kTileM * L->n_tile * sizeof(float),
-                           size_t(tiles) * 8 * sizeof(int32_t))) != RT3D_OK) return s;
-    a.scratch = blob->splitk; a.counters = blob->splitk_cnt;
-  }
   if (use_ts) {
     a.ts = 1; a.grp_ptr = u->grp_ptr; a.grp_first = u->grp_first;
     a.ts_a_bytes = probe.ts_a_bytes; a.ts_frame_bytes = probe.ts_frame_bytes; a.ts_table = probe.ts_table;
@@ -1006,11 +1020,13 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.store_tma = (a.n_splits == 1 && rect && encode_ymap(y, sb, pl_w, pl_h, pl_t, &ymap)) ? 1 : 0;
   if (pooled && !a.store_tma) return RT3D_ERR_UNSUPPORTED;
   if (use_pair) {
-    // items that do not fill a last round of CTA pairs are cut along K and shared (same workspace as split-K)
+    // items that do not fill a last round of CTA pairs are cut along K and shared
     // (its CTA pairs wait for one another, which needs the whole grid resident at once: not used when the caller
     // says that other kernels may run beside this call)
     size_t tail_bytes = 0, flag_bytes = 0;
-    if (!p->concurrent)
+    // (nor for AUTO when there are fewer items than pairs: what it would gain there, the cluster split gains with less)
+    const long long pairs = (m_tiles + 1) / 2 * L->n_bundles;
+    if (!p->concurrent && (p->algo != RT3D_ALGO_AUTO || pairs >= d->sm_count / 2))
       umma_pair_tail_plan(&a, L->step_ptr.data(), d->sm_count, &tail_bytes, &flag_bytes, use_ts ? L->grp_ptr.data() : nullptr);
     if (a.tail_workers > 0) {
       if ((s = ensure_splitk(w, blob, tail_bytes, flag_bytes)) != RT3D_OK) return s;
@@ -1022,7 +1038,6 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   return submit(rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0},
                 [=](cudaStream_t st) {
     UmmaArgs now = a;                              // a later call of another shape may have moved the handle's workspace
-    if (a.n_splits > 1) { now.scratch = blob->splitk; now.counters = blob->splitk_cnt; }
     if (a.tail_workers > 0) { now.tail_scratch = blob->splitk; now.tail_flags = blob->splitk_cnt; }
     const void* ym = a.store_tma ? &ymap : nullptr;
     return use_pair ? launch_conv_umma_pair(now, &xmap, wmap, ym, sms, st) : launch_conv_umma(now, &xmap, wmap, ym, sms, st);
@@ -1106,40 +1121,9 @@ rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* wsc, const
 }  // namespace
 
 // ------------------------------------------------------------------ entry point without allocation
-// Fixed workspace for rt3d_conv3d_sparse_noalloc: split-K partial tiles followed by the per-warp
-// arrival counters.  It lives in every GPU context that loads this library, for the life of the
-// process.  In host code `g_noalloc_ws` is only a handle for the runtime, never a device address:
-// the address is looked up per device with cudaGetSymbolAddress below.
+// Size limit of rt3d_conv3d_sparse_noalloc's K split: output tiles and fp32 partial tiles of a call.
 #define RT3D_NOALLOC_PARTIAL_TILES 128                                   /* 128 x 256 fp32 each */
 #define RT3D_NOALLOC_PARTIAL_BYTES (RT3D_NOALLOC_PARTIAL_TILES * 128 * 256 * 4)   /* 16 MiB */
-#define RT3D_NOALLOC_COUNTER_BYTES (RT3D_NOALLOC_PARTIAL_TILES * 8 * 4)  /* 8 counters (epilogue warps) per output tile */
-static __device__ __align__(256) unsigned char g_noalloc_ws[RT3D_NOALLOC_PARTIAL_BYTES + RT3D_NOALLOC_COUNTER_BYTES];
-
-namespace {
-struct NoAllocState { bool ready = false; unsigned char* ws = nullptr; };
-NoAllocState g_noalloc[64];
-std::mutex g_noalloc_mu;
-
-// Once per device, with that device current: resolve the device address of the workspace.  Called from
-// rt3d_packed_prepare, the documented set-up point: the first look-up may make the CUDA runtime load this
-// module on the device, which is when the driver sets the array's memory aside.
-rt3d_status noalloc_workspace_setup(int dev) {
-  std::lock_guard<std::mutex> lock(g_noalloc_mu);
-  NoAllocState& st = g_noalloc[dev];
-  if (!st.ready) {
-    void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_noalloc_ws) != cudaSuccess || p == nullptr) return RT3D_ERR_CUDA;
-    st.ws = static_cast<unsigned char*>(p);
-    st.ready = true;
-  }
-  return RT3D_OK;
-}
-// The cached address, or nullptr if no handle has been prepared on this device yet.
-unsigned char* noalloc_workspace(int dev) {
-  std::lock_guard<std::mutex> lock(g_noalloc_mu);
-  return g_noalloc[dev].ready ? g_noalloc[dev].ws : nullptr;
-}
-}  // namespace
 
 extern "C" {
 
@@ -1284,9 +1268,7 @@ rt3d_status rt3d_packed_prepare(rt3d_packed* p) {
   } else if ((s = get_canonical(p, blob)) != RT3D_OK) {
     return s;
   }
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return RT3D_ERR_CUDA;
-  if ((s = noalloc_workspace_setup(dev)) != RT3D_OK) return s;
+  for (int S = 2; S <= 8; ++S) umma_split_capacity(S, d->sm_count);      // what the K splits ask the runtime, once per device
   return cudaDeviceSynchronize() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
 }
 
@@ -1490,9 +1472,8 @@ rt3d_status rt3d_last_device_status(void* stream) {
   if (cudaMemcpy(&word, d->sched + 2, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return RT3D_ERR_CUDA;
   if (word != 0) {
     cudaMemset(d->sched + 2, 0, 4);
-    // A kernel that gave up may have left K-split arrival counters and tail-split flags non-zero (they are
-    // cleared by the CTA that finishes a tile): clear them for every handle on this device, so that later
-    // calls do not take a stale count for "all other splits have arrived".
+    // A kernel that gave up may have left tail-split flags non-zero (they are cleared by the pair that finishes a tile):
+    // clear them for every handle on this device, so that later calls do not take a stale flag for a share that is there.
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) {
       cudaDeviceSynchronize();
@@ -1540,8 +1521,6 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
     if (li != w->umma_layouts.end()) L = &li->second;
   }
   if (!blob || !u || !L) return RT3D_ERR_NOT_PREPARED;
-  unsigned char* ws = noalloc_workspace(dev);
-  if (!ws) return RT3D_ERR_NOT_PREPARED;
 
   UmmaArgs a;
   a.g = g;
@@ -1559,20 +1538,13 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
   long long splits = tiles > 0 ? d->sm_count / tiles : 1;
   if (splits > 8) splits = 8;
   if (splits > L->max_steps / 8) splits = L->max_steps / 8;
+  while (splits > 1 && umma_split_capacity(int(splits), d->sm_count) == 0) --splits;
   if (splits < 1) splits = 1;
   a.n_splits = int(splits);
   a.residual = nullptr; a.rcs = 0;
-  a.scratch = nullptr; a.counters = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (a.n_splits > 1) {
-    const long long partial_bytes = tiles * a.n_splits * kTileM * L->n_tile * 4LL;
-    if (partial_bytes > RT3D_NOALLOC_PARTIAL_BYTES || tiles * 32 > RT3D_NOALLOC_COUNTER_BYTES)
-      return RT3D_ERR_WORKSPACE;
-    a.scratch = reinterpret_cast<float*>(ws);
-    a.counters = reinterpret_cast<int32_t*>(ws + RT3D_NOALLOC_PARTIAL_BYTES);
-    // the counters must start at zero; the workspace keeps whatever the last call left behind
-    if (cudaMemsetAsync(a.counters, 0, size_t(tiles) * 32, st) != cudaSuccess) return RT3D_ERR_CUDA;
-  }
+  if (a.n_splits > 1 && (tiles * a.n_splits * kTileM * L->n_tile * 4LL > RT3D_NOALLOC_PARTIAL_BYTES || tiles > RT3D_NOALLOC_PARTIAL_TILES))
+    return RT3D_ERR_WORKSPACE;
   CUtensorMap xmap;
   if ((s = encode_xmap(x, g, a.box, &xmap)) != RT3D_OK) return s;
   CUtensorMap ymap;
@@ -1608,7 +1580,7 @@ rt3d_status rt3d_debug_set(int what, long long value) {
     if (d->cc_major != 10) return RT3D_ERR_UNSUPPORTED;
     if (launch_debug_poison(uint32_t(value), d->sm_count, d->sched + 8, nullptr) != cudaSuccess) return RT3D_ERR_CUDA;
     if (cudaDeviceSynchronize() != cudaSuccess) return RT3D_ERR_CUDA;
-    // the K splits' partial tiles in global memory too (all ones: NaNs as fp32); their counters and flags stay zero
+    // the tail splits' partial tiles in global memory too (all ones: NaNs as fp32); their flags stay zero
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return RT3D_ERR_CUDA;
     std::lock_guard<std::mutex> reg(g_blobs_mu);

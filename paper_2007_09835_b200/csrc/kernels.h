@@ -89,9 +89,7 @@ struct UmmaArgs {
   int rcs;                                  // its channel pitch
   int pool_t, pool_h, pool_w;               // fused max-pool window (1,1,1 = none); needs store_tma, ymap over the pooled tensor
   int sbw, sbh;                             // extents along w, h of the block of 32 voxels an epilogue warp owns
-  int n_splits;                             // K splits per output tile (1 = none)
-  float* scratch;                           // device, split-K partial tiles [tile][split][128][n_tile] (n_splits > 1)
-  int32_t* counters;                        // device, [tiles * 8] arrival counters (one per epilogue warp), zero between launches
+  int n_splits;                             // K splits per output tile (1 = none): the CTAs of one cluster
   int tail_workers;                         // CTA-pair kernel: pairs sharing the left-over items of the last round (0 = off)
   float* tail_scratch;                      // device, [tail_workers][2 shares][2 CTAs][n_tile][128] fp32 partial tiles
   int32_t* tail_flags;                      // device, [tail_workers][2][2][4 warps] "partial written" flags, zero between launches
@@ -111,6 +109,8 @@ struct UmmaArgs {
 // xmap / wmap point to 128-byte CUtensorMap objects in host memory.
 // ymap: tensor map of the output for the TMA-store epilogue (box = 32 channels x one warp's 32 voxels,
 // 64-byte swizzle); used when a.store_tma != 0, may be nullptr otherwise.
+// CTAs that can be resident at once when every tile is split `n_splits` ways; 0: no such clusters on this device.
+int umma_split_capacity(int n_splits, int sm_count);
 cudaError_t launch_conv_umma(const UmmaArgs& a, const void* xmap, const void* wmap, const void* ymap, int sm_count,
                              cudaStream_t stream);
 

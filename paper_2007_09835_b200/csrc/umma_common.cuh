@@ -14,6 +14,7 @@ constexpr int kMaxStages = 8;
 constexpr int kABytes = 128 * 128;                  // 128 voxel rows x 64 bf16
 constexpr long long kWaitCycles = 1ll << 31;        // about one second of SM clocks
 constexpr size_t kSmemBudget = 200 * 1024;
+constexpr int kMaxSplits = 8;                       // K splits = CTAs of a cluster, as many as any GPU of the architecture places
 
 struct __align__(8) Barriers {
   unsigned long long full[kMaxStages];
@@ -70,6 +71,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, Barrier
       return false;
     }
   }
+}
+
+// The same for a whole warp that must stay convergent: the answer is one the compiler knows to be uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, Barriers* bars, int32_t* err, int code) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, bars, err, code));
+}
+// A value that every lane holds, in a form the compiler knows to be uniform.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+// One lane of a convergent warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
 }
 
 // Walk over a 4-digit mixed-radix index (digits i0 fastest .. i3 slowest, radices r0, r1, r2) that advances by a
@@ -542,6 +558,57 @@ __device__ __forceinline__ void store_partial_row(uint32_t taddr, int n_cols, bo
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+
+// ------------------------------------------------------------------------------ K split over a thread-block cluster
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The CTAs of a cluster have each accumulated a share of one tile's K steps and left it in their own shared memory as
+// store_partial_row lays it out.  Between two cluster barriers each of them finishes a slice of the columns: for NC
+// columns at a time, units u0, u0 + 2, .. below u1, this thread adds its row's values of all shares in rank order (so the
+// result does not depend on timing), reading them straight from the other SMs' shared memory, and writes the output.
+// Against partial tiles in global memory which the last CTA to arrive adds up: no fences, no counters, no trips to L2,
+// and all CTAs share the additions.
+template <int NC>
+__device__ __forceinline__ void cluster_reduce_row(uint32_t part_smem, int row, int u0, int u1, int n_parts, bool in_range,
+                                                   const float* bias_s, int relu, __nv_bfloat16* dst, int m_base, int M,
+                                                   const __nv_bfloat16* res_row) {
+  if (!in_range) return;
+  for (int u = u0; u < u1; u += 2) {
+    const int col = u * NC, m0 = m_base + col;
+    if (m0 >= M) return;
+    const uint32_t local = part_smem + uint32_t(col * 128 + row * kPartRow) * 4u;
+    float acc[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) acc[q] = 0.f;
+#pragma unroll 4
+    for (int p = 0; p < n_parts; ++p) {
+      const uint32_t remote = mapa_shared(local, uint32_t(p));
+#pragma unroll
+      for (int q = 0; q < NC / 4; ++q) {
+        float4 t;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(remote + q * 2048u));
+        acc[4 * q] += t.x; acc[4 * q + 1] += t.y; acc[4 * q + 2] += t.z; acc[4 * q + 3] += t.w;
+      }
+    }
+    uint32_t v[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) v[q] = __float_as_uint(acc[q]);
+    epilogue_cols<NC>(v, bias_s + m0, relu, dst + col, M - m0, res_row ? res_row + col : nullptr, M - m0);
+  }
+}
 
 // Shared-memory matrix descriptor without swizzle: core matrices of 8 rows x 16 bytes stored
 // contiguously (rows 16 bytes apart); `lbo` = byte distance between the two core matrices along K,

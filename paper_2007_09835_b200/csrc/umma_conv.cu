@@ -14,13 +14,13 @@
 // owner), warps 2..5 = epilogue (TMEM -> registers -> +bias, ReLU, bf16 -> NDHWC stores).  Two
 // accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the next.
 //
-// Layers with few output tiles are split along K: each of `n_splits` CTAs accumulates a slice of
-// the step list and writes its fp32 partial tile to a scratch buffer; the CTA that arrives last
-// (a counter per output tile and warp) adds the partials in split order, so the result does not depend
-// on which CTA that is, applies the epilogue and resets the counter for the next launch.
+// Layers with few output tiles are split along K: the `n_splits` CTAs of a thread-block cluster accumulate a slice of the
+// step list each and finish the tile together through distributed shared memory (cluster_reduce_row).
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA records an error word in global
 // memory, all roles fall through, TMEM is released and the kernel returns.
+#include <atomic>
+
 #include "kernels.h"
 #include "umma_common.cuh"
 #include "pdl.cuh"
@@ -58,62 +58,6 @@ __device__ __forceinline__ void item_steps(const UmmaArgs& a, const ItemCoord& c
   nsteps = hi - local0;
 }
 
-// Sum of the partials of all splits (in split order, two splits' loads in flight at a time) + epilogue
-// for one output voxel; `part0` points at this thread's row of column 0 of split 0.
-template <int NC>
-__device__ __forceinline__ void reduce_partial_cols(const float* part0, size_t split_stride, int n_splits,
-                                                    const float* bias_s, int relu, __nv_bfloat16* dst, int valid,
-                                                    const __nv_bfloat16* res, int res_avail) {
-  float acc[NC];
-#pragma unroll
-  for (int q = 0; q < NC; ++q) acc[q] = 0.f;
-  int s = 0;
-  for (; s + 1 < n_splits; s += 2) {
-    float4 t0[NC / 4], t1[NC / 4];
-    const float* p0 = part0 + size_t(s) * split_stride;
-    const float* p1 = p0 + split_stride;
-#pragma unroll
-    for (int q = 0; q < NC / 4; ++q) {
-      t0[q] = __ldcg(reinterpret_cast<const float4*>(p0 + size_t(q) * 512));
-      t1[q] = __ldcg(reinterpret_cast<const float4*>(p1 + size_t(q) * 512));
-    }
-#pragma unroll
-    for (int q = 0; q < NC / 4; ++q) {
-      acc[4 * q] = (acc[4 * q] + t0[q].x) + t1[q].x;
-      acc[4 * q + 1] = (acc[4 * q + 1] + t0[q].y) + t1[q].y;
-      acc[4 * q + 2] = (acc[4 * q + 2] + t0[q].z) + t1[q].z;
-      acc[4 * q + 3] = (acc[4 * q + 3] + t0[q].w) + t1[q].w;
-    }
-  }
-  if (s < n_splits) {
-    const float* p0 = part0 + size_t(s) * split_stride;
-#pragma unroll
-    for (int q = 0; q < NC / 4; ++q) {
-      const float4 t = __ldcg(reinterpret_cast<const float4*>(p0 + size_t(q) * 512));
-      acc[4 * q] += t.x; acc[4 * q + 1] += t.y; acc[4 * q + 2] += t.z; acc[4 * q + 3] += t.w;
-    }
-  }
-  uint32_t v[NC];
-#pragma unroll
-  for (int q = 0; q < NC; ++q) v[q] = __float_as_uint(acc[q]);
-  epilogue_cols<NC>(v, bias_s, relu, dst, valid, res, res_avail);
-}
-
-__device__ __forceinline__ void reduce_partial_row(const float* part0, size_t split_stride, int n_splits, int n_cols,
-                                                   bool in_range, const float* bias_s, int relu, __nv_bfloat16* dst,
-                                                   int m_base, int M, const __nv_bfloat16* res_row, int res_left,
-                                                   int col0 = 0, int col_step = 32) {
-  if (!in_range) return;
-  for (int col = col0; col < n_cols; col += col_step) {
-    const int m0 = m_base + col;
-    if (m0 >= M) break;
-    const float* p = part0 + size_t(col) * 128;
-    const __nv_bfloat16* res = res_row ? res_row + col : nullptr;
-    if (col + 32 <= n_cols) reduce_partial_cols<32>(p, split_stride, n_splits, bias_s + m0, relu, dst + col, M - m0, res, res_left - col);
-    else reduce_partial_cols<16>(p, split_stride, n_splits, bias_s + m0, relu, dst + col, M - m0, res, res_left - col);
-  }
-}
-
 // kCps: K steps per pipeline stage (and per barrier hand-shake): 1, or 2 for narrow bundles, where the
 // issuing thread's hand-shake, not the tensor pipe, bounds a step.
 // Threads of the single-CTA kernel: producer warp, MMA warp, two sets of four epilogue warps.  The second set
@@ -139,7 +83,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   float* bias_s = align16_f32(bars + 1);                            // bias of all bundles (zeros if none), padded
   int32_t* err = a.sched + 2;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(int(threadIdx.x >> 5)), lane = threadIdx.x & 31;
   const int n_mtiles = a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
   const int n_items = n_mtiles * a.n_bundles * a.n_splits;
   const int box_rows = a.box.bn * a.box.bt * a.box.bh * a.box.bw;
@@ -173,7 +117,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = uniform(uint32_t(bars->tmem_base));
 
   // Everything above touched only shared memory, barriers and TMEM.  The successor may be scheduled now that
   // this CTA holds its TMEM columns (a successor CTA that shared the SM and allocated first could otherwise
@@ -269,46 +213,53 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc_bf16(a.n_tile);
-      uint32_t j = 0, phase = 0;
-      int stage = 0;
-      bool ok = true, ready = false;
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++j) {
-        const bool first_item = item == int(blockIdx.x);
-        const ItemCoord c = first_item ? pre_c : decode_item(a, item, n_mtiles);
-        int s_begin = pre_sbegin, nsteps = pre_nsteps, local0 = pre_local0;
-        if (!first_item) item_steps<kDense>(a, c, s_begin, nsteps, local0);
-        const uint32_t buf = j & 1u;
-        if (!mbar_wait(smem_u32(&bars->tmem_empty[buf]), ((j >> 1) & 1u) ^ 1u, bars, err, 2)) break;
+    // The whole warp walks the loop and one elected lane issues: control flow and operands are uniform, which the MMA
+    // and its descriptors need in uniform registers anyway (2 to 6 % of the layers that run here).
+    const bool elected = elect_one();
+    const uint32_t idesc = instr_desc_bf16(a.n_tile);
+    uint32_t j = 0, phase = 0;
+    int stage = 0;
+    bool ok = true, ready = false;
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++j) {
+      int nsteps = pre_nsteps;
+      if (item != int(blockIdx.x)) {
+        int s_begin, local0;
+        item_steps<kDense>(a, decode_item(a, item, n_mtiles), s_begin, nsteps, local0);
+      }
+      nsteps = uniform(nsteps);
+      const uint32_t buf = j & 1u;
+      if (!mbar_wait_warp(smem_u32(&bars->tmem_empty[buf]), ((j >> 1) & 1u) ^ 1u, bars, err, 2)) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + buf * uint32_t(a.n_tile);
+      for (int i = 0; i < nsteps; i += kCps) {
+        const int nload = nsteps - i < kCps ? nsteps - i : kCps;
+        if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(smem_u32(&bars->full[stage]), phase, bars, err, 3)) { ok = false; break; }
+        // poll the next stage's barrier now: its answer arrives while this stage's MMAs are issued (not behind the last
+        // step, where a load that is never issued keeps the poll waiting for microseconds)
+        const int stage_n = stage + 1 == stages ? 0 : stage + 1;
+        const uint32_t phase_n = stage + 1 == stages ? phase ^ 1u : phase;
+        ready = i + kCps < nsteps && mbar_try_wait(smem_u32(&bars->full[stage_n]), phase_n);
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * uint32_t(a.n_tile);
-        for (int i = 0; i < nsteps; i += kCps) {
-          const int nload = nsteps - i < kCps ? nsteps - i : kCps;
-          if (!ready && !mbar_wait(smem_u32(&bars->full[stage]), phase, bars, err, 3)) { ok = false; break; }
-          // poll the next stage's barrier now: its answer arrives while this stage's MMAs are issued
-          const int stage_n = stage + 1 == stages ? 0 : stage + 1;
-          const uint32_t phase_n = stage + 1 == stages ? phase ^ 1u : phase;
-          ready = mbar_try_wait(smem_u32(&bars->full[stage_n]), phase_n);
-          tc_fence_after();
 #pragma unroll
-          for (int q = 0; q < kCps; ++q) {
-            if (q >= nload) break;
-            const uint32_t a_addr = tiles_base + stage * stage_bytes + q * chunk_bytes;
-            const uint64_t adesc = smem_desc_sw128(a_addr);
-            const uint64_t bdesc = smem_desc_sw128(a_addr + kABytes);
+        for (int q = 0; q < kCps; ++q) {
+          if (q >= nload) break;
+          const uint32_t a_addr = tiles_base + stage * stage_bytes + q * chunk_bytes;
+          const uint64_t adesc = smem_desc_sw128(a_addr);
+          const uint64_t bdesc = smem_desc_sw128(a_addr + kABytes);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)    // 4 x K=16 per 64-channel chunk: +32 bytes = +2 in descriptor units
-              umma_bf16(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, (i | q | kk) ? 1u : 0u);
-          }
-          umma_commit(smem_u32(&bars->empty[stage]));
-          stage = stage_n; phase = phase_n;
+          for (int kk = 0; kk < 4; ++kk)    // 4 x K=16 per 64-channel chunk: +32 bytes = +2 in descriptor units
+            if (elected) umma_bf16(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, (i | q | kk) ? 1u : 0u);
         }
-        if (!ok) break;
+        if (elected) umma_commit(smem_u32(&bars->empty[stage]));
+        stage = stage_n; phase = phase_n;
+      }
+      if (!ok) break;
+      if (elected) {
         if (nsteps > 0) umma_commit(smem_u32(&bars->tmem_full[buf]));
         else mbar_arrive(smem_u32(&bars->tmem_full[buf]));
       }
     }
+    __syncwarp();
   } else if (warp < 6 || two_sets || split_sets) {
     // ------------------------------------------------------------------ epilogue (warps 2..5, and 6..9 on plain calls)
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
@@ -329,7 +280,6 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
     const int bh_0 = r0 % a.box.bh; r0 /= a.box.bh;
     const int bt_0 = r0 % a.box.bt; r0 /= a.box.bt;
     const int bn_0 = r0;
-    const size_t part_tile = size_t(128) * a.n_tile;       // floats per partial tile
     uint32_t j = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++j) {
       const bool first_item = item == int(blockIdx.x);
@@ -384,28 +334,39 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[buf]));
       } else {
-        float* tile_part = a.scratch + size_t(c.tile_id) * a.n_splits * part_tile;
-        store_partial_row(taddr, a.n_tile, nsteps > 0, tile_part + size_t(c.split) * part_tile + row * kPartRow, half * 32, 64);
+        // This CTA's only item: its share goes into the stages, which every load has filled and every MMA has read.
+        store_partial_row(taddr, a.n_tile, nsteps > 0, reinterpret_cast<float*>(smem_raw + (tiles_base - raw)) + row * kPartRow,
+                          half * 32, 64);
         tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[buf]));    // accumulator consumed: MMAs may go on
-        // Each warp owns 32 rows of the tile in every split, so the hand-over is per warp: fence the
-        // partial, count this warp in, and the warp that counts last reduces those 32 rows.
-        __threadfence();
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) last = atomicAdd(a.counters + c.tile_id * 8 + half * 4 + quad, 1) == a.n_splits - 1;
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (last) {
-          __threadfence();
-          reduce_partial_row(tile_part + row * kPartRow, part_tile, a.n_splits, a.n_tile, in_range, bias_s,
-                             a.g.relu, dst, m_base, a.g.M, res, res_left, half * 32, 64);
-          __syncwarp();
-          if (lane == 0) a.counters[c.tile_id * 8 + half * 4 + quad] = 0;   // ready for the next launch
-        }
       }
     }
     if (lane == 0) tma_store_wait_all();         // all bulk stores done before shared memory goes away
+  }
+
+  if (split_sets) {                  // the CTAs of the cluster finish a slice of the tile's columns each
+    __syncwarp();
+    cluster_sync_all();
+    if (warp >= 2 && !bars->abort_flag) {
+      const int half = (warp - 2) >> 2, row = (warp & 3) * 32 + lane;
+      int r = row;
+      const int wo = pre_c.w0 + r % a.box.bw; r /= a.box.bw;
+      const int ho = pre_c.h0 + r % a.box.bh; r /= a.box.bh;
+      const int to = pre_c.t0 + r % a.box.bt; r /= a.box.bt;
+      const int nn = pre_c.n0 + r;
+      const bool in_range = row < box_rows && nn < a.g.n && to < a.g.To && ho < a.g.Ho && wo < a.g.Wo;
+      const long long vox = (((long long)nn * a.g.To + to) * a.g.Ho + ho) * a.g.Wo + wo;
+      const int m_base = pre_c.bundle * a.n_tile;
+      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.y) + vox * a.g.ycs + m_base;
+      const __nv_bfloat16* res = (a.residual != nullptr && in_range)
+                                     ? static_cast<const __nv_bfloat16*>(a.residual) + vox * a.rcs + m_base : nullptr;
+      // 16 columns at a time, or 8 where that would leave a set of warps without work
+      const int wide = a.n_tile >= 32 * a.n_splits ? 16 : 8, units = a.n_tile / wide;
+      const int u0 = pre_c.split * units / a.n_splits + half, u1 = (pre_c.split + 1) * units / a.n_splits;
+      if (wide == 16) cluster_reduce_row<16>(tiles_base, row, u0, u1, a.n_splits, in_range, bias_s, a.g.relu, dst, m_base, a.g.M, res);
+      else cluster_reduce_row<8>(tiles_base, row, u0, u1, a.n_splits, in_range, bias_s, a.g.relu, dst, m_base, a.g.M, res);
+    }
+    __syncwarp();
+    cluster_sync_all();              // nobody leaves while its share is still being read
   }
 
   // ---------------------------------------------------------------------- teardown
@@ -441,11 +402,33 @@ cudaError_t launch_single_t(const UmmaArgs& a, const CUtensorMap& xm, const CUte
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  LaunchSetup ls(dim3(grid), dim3(kThreadsSingle), smem, stream);
+  LaunchSetup ls(dim3(grid), dim3(kThreadsSingle), smem, stream, unsigned(a.n_splits));
   return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_kernel<kDense, kCps>, xm, wm, ym, a, stages, cols);
 }
 
 }  // namespace
+
+int umma_split_capacity(int n_splits, int sm_count) {
+  if (n_splits == 1) return sm_count;
+  if (n_splits < 1 || n_splits > kMaxSplits) return 0;
+  static std::atomic<int> known[kMaxDevices][kMaxSplits + 1];          // per device: capacity + 1
+  const int dev = current_device_index();
+  if (dev < 0) return 0;
+  int v = known[dev][n_splits].load();
+  if (v == 0) {
+    // any instantiation with one CTA per SM answers for all: the shared memory decides
+    const size_t smem = 227 * 1024;
+    int n = 0;
+    LaunchSetup ls(dim3(unsigned(sm_count / n_splits * n_splits)), dim3(kThreadsSingle), smem, nullptr, unsigned(n_splits));
+    ls.cfg.numAttrs = 1;                                               // the cluster dimension alone
+    if (cudaFuncSetAttribute(conv3d_umma_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, conv3d_umma_kernel<false, 2>, &ls.cfg) != cudaSuccess)
+      n = 0;
+    v = n * n_splits + 1;
+    known[dev][n_splits].store(v);
+  }
+  return v - 1;
+}
 
 size_t umma_smem_bytes(int n_tile, int n_bundles) {
   return size_t(pick_stages(n_tile)) * pick_cps_single(n_tile) * (kABytes + size_t(n_tile) * 128) + 1024 + 4 * kStoreWarpBytes + sizeof(Barriers) + 16 +
@@ -461,10 +444,11 @@ cudaError_t launch_conv_umma(const UmmaArgs& a, const void* xmap, const void* wm
   int cols = 32;
   while (cols < 2 * a.n_tile) cols *= 2;
   if (cols > 512) return cudaErrorInvalidValue;
-  if (a.n_splits < 1 || (a.n_splits > 1 && (a.scratch == nullptr || a.counters == nullptr))) return cudaErrorInvalidValue;
+  if (a.n_splits < 1 || a.n_splits > kMaxSplits) return cudaErrorInvalidValue;
   const long long n_items = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w * a.n_bundles * a.n_splits;
   if (n_items <= 0) return cudaSuccess;
-  const int grid = int(n_items < sm_count ? n_items : sm_count);
+  if (n_items > (1ll << 30)) return cudaErrorInvalidValue;
+  const int grid = int(a.n_splits > 1 || n_items < sm_count ? n_items : sm_count);     // split tiles: one share per CTA
   if (a.store_tma && ymap == nullptr) return cudaErrorInvalidValue;
   CUtensorMap xm, wm, ym;
   memcpy(&xm, xmap, sizeof(CUtensorMap));

@@ -18,6 +18,13 @@ from . import _pycall, binding as B
 _pycall.setup(torch.float32, torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
 _ADDRESS = {fn: ctypes.cast(getattr(B.lib(), fn), ctypes.c_void_p).value
             for fn in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_sparse_fused")}
+# The binding's compute functions as they are: calls go round them only while they are what the binding's module holds (a
+# tracer or a test that wraps them sees every call).
+_FUNCTIONS = {fn: getattr(B, fn) for fn in (*_ADDRESS, "rt3d_conv2plus1d_fused", "rt3d_maxpool3d", "rt3d_add_relu")}
+
+
+def _unwrapped(*names) -> bool:
+    return B.noting() is None and all(getattr(B, fn) is _FUNCTIONS[fn] for fn in names)
 
 
 def pitch_for(c: int, dtype) -> int:
@@ -82,12 +89,12 @@ class ConvLayer:
         `to_device`); lets the first-layer kernel fetch whole image rows per request."""
         if y is None:
             y = self.alloc_out(x)
-        if B.noting() is not None:
+        name = "rt3d_conv3d_dense" if self.dense else "rt3d_conv3d_sparse"
+        if not _unwrapped(name):
             fn = B.rt3d_conv3d_dense if self.dense else B.rt3d_conv3d_sparse
             fn(B.tensor_desc(x, self.spec.cin), self.packed, self.bias, B.tensor_desc(y, self.spec.cout), self.spec.stride,
                self.spec.pad, self.spec.relu if relu is None else relu, algo, stream, x_pad_zero)
             return y
-        name = "rt3d_conv3d_dense" if self.dense else "rt3d_conv3d_sparse"
         status = _pycall.conv(_ADDRESS[name], x, self.spec.cin, self.packed.handle.value, self.bias,
                               self._param_struct(relu, algo, x_pad_zero), y, self.spec.cout, stream)
         if status != B.OK:
@@ -102,7 +109,7 @@ class ConvLayer:
     def fused(self, x: torch.Tensor, y: torch.Tensor, residual: torch.Tensor | None = None, pool=(1, 1, 1),
               relu=None, algo=B.ALGO_AUTO, stream=None, x_pad_zero=False):
         """y = pool(act(conv(x) + bias + residual)) in one launch (rt3d_conv3d_sparse_fused)."""
-        if B.noting() is not None:
+        if not _unwrapped("rt3d_conv3d_sparse_fused"):
             res = None if residual is None else B.tensor_desc(residual, self.spec.cout)
             B.rt3d_conv3d_sparse_fused(B.tensor_desc(x, self.spec.cin), self.packed, self.bias,
                                        B.tensor_desc(y, self.spec.cout), self.spec.stride, self.spec.pad,
@@ -175,7 +182,7 @@ class _NotedForward:
         return [getattr(self, name) for name in self._SWITCHES]
 
     def forward(self, x: torch.Tensor, algo=B.ALGO_AUTO, keep=None, stream=None, **kw) -> torch.Tensor:
-        if keep is not None or any(v is not None for v in kw.values()) or B.is_planning() or B.noting() is not None:
+        if keep is not None or any(v is not None for v in kw.values()) or B.is_planning() or not _unwrapped(*_FUNCTIONS):
             return self._forward(x, algo, keep, stream, **kw)
         noted = self.__dict__.setdefault("_noted", {})
         # torch.Size, dtype and device hash by value; the current device and whether a stream is named decide the streams
