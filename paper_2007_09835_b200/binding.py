@@ -116,6 +116,23 @@ _lib = None
 _lib = _load()
 
 
+ADDRESS = {fn: ctypes.cast(getattr(_lib, fn), ctypes.c_void_p).value
+           for fn in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_sparse_fused", "rt3d_kgs_group_norms",
+                      "rt3d_kgs_reweight", "rt3d_kgs_expand_mask")}
+_pycall_module = None
+
+
+def pycall():
+    """The extension module that calls the library on torch tensors (csrc/pycall.cpp), ready to use."""
+    global _pycall_module
+    if _pycall_module is None:
+        import torch
+        from . import _pycall as m
+        m.setup(torch.float32, torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _pycall_module = m
+    return _pycall_module
+
+
 def lib():
     """The loaded ctypes library (for callers that want the raw C ABI)."""
     return _lib
@@ -457,23 +474,20 @@ def rt3d_add_relu(a: Tensor, b: Tensor, relu: bool, y: Tensor, stream=None):
 
 def rt3d_kgs_group_norms(w, g_m: int, g_n: int, norm: int, norms, stream=None):
     """w: torch float32 device tensor [M,N,Kt,Kh,Kw]; norms: torch float32 device tensor [P,Q,Kt*Kh*Kw] (output)."""
-    M, N, Kt, Kh, Kw = w.shape
-    _check(_lib.rt3d_kgs_group_norms(ctypes.c_void_p(w.data_ptr()), M, N, Kt, Kh, Kw, int(g_m), int(g_n), int(norm),
-                                     ctypes.c_void_p(norms.data_ptr()), _stream_ptr(stream)), "rt3d_kgs_group_norms")
+    _check((_pycall_module or pycall()).group_norms(ADDRESS["rt3d_kgs_group_norms"], w, int(g_m), int(g_n), int(norm), norms, stream),
+           "rt3d_kgs_group_norms")
 
 
 def rt3d_kgs_reweight(norms, eps: float, threshold: float, penalty=None, keep=None, stream=None):
     """norms: float32 device tensor; penalty (float32) / keep (uint8): device tensors of the same size or None."""
-    _check(_lib.rt3d_kgs_reweight(ctypes.c_void_p(norms.data_ptr()), norms.numel(), float(eps), float(threshold),
-                                  None if penalty is None else ctypes.c_void_p(penalty.data_ptr()),
-                                  None if keep is None else ctypes.c_void_p(keep.data_ptr()), _stream_ptr(stream)),
-           "rt3d_kgs_reweight")
+    _check((_pycall_module or pycall()).reweight(ADDRESS["rt3d_kgs_reweight"], norms, norms.numel(), float(eps), float(threshold),
+                                                 penalty, keep, stream), "rt3d_kgs_reweight")
 
 
 def rt3d_kgs_expand_mask(group_mask, M, N, Kt, Kh, Kw, g_m, g_n, mask, stream=None):
     """group_mask: uint8 device [P,Q,Ks]; mask: uint8 device [M,N,Kt,Kh,Kw] (output)."""
-    _check(_lib.rt3d_kgs_expand_mask(ctypes.c_void_p(group_mask.data_ptr()), M, N, Kt, Kh, Kw, int(g_m), int(g_n),
-                                     ctypes.c_void_p(mask.data_ptr()), _stream_ptr(stream)), "rt3d_kgs_expand_mask")
+    _check((_pycall_module or pycall()).expand_mask(ADDRESS["rt3d_kgs_expand_mask"], group_mask, int(M), int(N), int(Kt), int(Kh),
+                                                    int(Kw), int(g_m), int(g_n), mask, stream), "rt3d_kgs_expand_mask")
 
 
 def rt3d_conv3d_cost(x: Tensor, w: Packed, stride=(1, 1, 1), pad=(0, 0, 0)):

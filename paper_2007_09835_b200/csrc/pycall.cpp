@@ -90,6 +90,81 @@ bool describe(PyObject* t, PyObject* channels, rt3d_tensor* d) {
   return true;
 }
 
+bool stream_of(PyObject* v, uintptr_t* out) {
+  if (v != Py_None) return as_pointer(v, out);
+  PyObject* dev = PyObject_CallNoArgs(g_get_device);
+  if (!dev) return false;
+  PyObject* st = PyObject_CallOneArg(g_raw_stream, dev);
+  Py_DECREF(dev);
+  if (!st) return false;
+  const bool ok = as_pointer(st, out);
+  Py_DECREF(st);
+  return ok;
+}
+
+bool tensor_or_none(PyObject* t, uintptr_t* out) {
+  *out = 0;
+  return t == Py_None || data_ptr(t, out);
+}
+
+bool ints(PyObject* const* a, int n, int* out) {
+  for (int i = 0; i < n; ++i) {
+    const long v = PyLong_AsLong(a[i]);
+    if (v == -1 && PyErr_Occurred()) return false;
+    out[i] = int(v);
+  }
+  return true;
+}
+
+bool want(Py_ssize_t n, Py_ssize_t expected) {
+  if (n != expected) PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+  return n == expected;
+}
+
+// The three calls of the pruning step, with the arguments of their binding functions behind the library's address.
+PyObject* group_norms(PyObject*, PyObject* const* a, Py_ssize_t n) {   // address, w, g_m, g_n, norm, norms, stream
+  uintptr_t fn, w, norms, stream;
+  int v[3], e[5];
+  if (!want(n, 7) || !as_pointer(a[0], &fn) || !data_ptr(a[1], &w) || !ints(a + 2, 3, v) || !data_ptr(a[5], &norms) ||
+      !stream_of(a[6], &stream))
+    return nullptr;
+  PyObject* shape = PyObject_GetAttr(a[1], s_shape);
+  if (!shape) return nullptr;
+  bool ok = PyTuple_Check(shape) && PyTuple_GET_SIZE(shape) == 5;
+  if (!ok) PyErr_SetString(PyExc_ValueError, "expected a 5-D weight tensor");
+  for (int i = 0; ok && i < 5; ++i) {
+    PyObject* item = PyTuple_GET_ITEM(shape, i);
+    ok = ints(&item, 1, e + i);
+  }
+  Py_DECREF(shape);
+  if (!ok) return nullptr;
+  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_group_norms)>(fn)(
+      reinterpret_cast<const float*>(w), e[0], e[1], e[2], e[3], e[4], v[0], v[1], v[2], reinterpret_cast<float*>(norms),
+      reinterpret_cast<void*>(stream)));
+}
+
+PyObject* reweight(PyObject*, PyObject* const* a, Py_ssize_t n) {      // address, norms, count, eps, threshold, penalty, keep, stream
+  uintptr_t fn, norms, penalty, keep, stream;
+  if (!want(n, 8) || !as_pointer(a[0], &fn) || !data_ptr(a[1], &norms)) return nullptr;
+  const long long count = PyLong_AsLongLong(a[2]);
+  const double eps = PyFloat_AsDouble(a[3]), threshold = PyFloat_AsDouble(a[4]);
+  if (PyErr_Occurred() || !tensor_or_none(a[5], &penalty) || !tensor_or_none(a[6], &keep) || !stream_of(a[7], &stream)) return nullptr;
+  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_reweight)>(fn)(
+      reinterpret_cast<const float*>(norms), count, float(eps), float(threshold), reinterpret_cast<float*>(penalty),
+      reinterpret_cast<uint8_t*>(keep), reinterpret_cast<void*>(stream)));
+}
+
+PyObject* expand_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {   // address, group mask, M, N, Kt, Kh, Kw, g_m, g_n, mask, stream
+  uintptr_t fn, g, mask, stream;
+  int v[7];
+  if (!want(n, 11) || !as_pointer(a[0], &fn) || !data_ptr(a[1], &g) || !ints(a + 2, 7, v) || !data_ptr(a[9], &mask) ||
+      !stream_of(a[10], &stream))
+    return nullptr;
+  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_expand_mask)>(fn)(
+      reinterpret_cast<const uint8_t*>(g), v[0], v[1], v[2], v[3], v[4], v[5], v[6], reinterpret_cast<uint8_t*>(mask),
+      reinterpret_cast<void*>(stream)));
+}
+
 // conv(address, x, c_in, handle, bias, params, y, c_out, stream[, residual, (pool_t, pool_h, pool_w)]) -> status.
 // With the last two the address is rt3d_conv3d_sparse_fused's, else rt3d_conv3d_sparse's or _dense's.
 PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -102,18 +177,7 @@ PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!as_pointer(a[0], &fn) || !describe(a[1], a[2], &x) || !as_pointer(a[3], &handle)) return nullptr;
   if (a[4] != Py_None && !data_ptr(a[4], &bias)) return nullptr;
   if (!describe(a[6], a[7], &y)) return nullptr;
-  if (a[8] == Py_None) {
-    PyObject* dev = PyObject_CallNoArgs(g_get_device);
-    if (!dev) return nullptr;
-    PyObject* st = PyObject_CallOneArg(g_raw_stream, dev);
-    Py_DECREF(dev);
-    if (!st) return nullptr;
-    const bool ok = as_pointer(st, &stream);
-    Py_DECREF(st);
-    if (!ok) return nullptr;
-  } else if (!as_pointer(a[8], &stream)) {
-    return nullptr;
-  }
+  if (!stream_of(a[8], &stream)) return nullptr;
   rt3d_fusion fz{};
   if (n == 11) {
     if (a[9] != Py_None) {
@@ -154,6 +218,9 @@ PyMethodDef methods[] = {
     {"setup", setup, METH_VARARGS, "setup(float32, bfloat16, raw_stream, get_device): torch objects the calls need"},
     {"conv", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(conv)), METH_FASTCALL,
      "conv(address, x, c_in, handle, bias, params, y, c_out, stream[, residual, pool]) -> status"},
+    {"group_norms", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(group_norms)), METH_FASTCALL, ""},
+    {"reweight", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(reweight)), METH_FASTCALL, ""},
+    {"expand_mask", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(expand_mask)), METH_FASTCALL, ""},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

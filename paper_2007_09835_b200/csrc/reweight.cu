@@ -142,6 +142,7 @@ __global__ void reweight_kernel(const float* __restrict__ norms, long long count
 
 constexpr int kMaskThreads = 256;
 constexpr int kMaskChunk = 4096;      // bytes of one mask row that a block expands at a time
+constexpr int kMaskStage = 8192;      // decisions held in shared memory; one-channel groups of many locations may need more
 
 // The g_m mask rows of a row of kernel groups are the same N * Ks bytes: a block expands a chunk of them once into
 // shared memory and writes it to every row in 16-byte stores.  A row may start at any byte, so the words of each row
@@ -151,24 +152,43 @@ __global__ void __launch_bounds__(kMaskThreads)
 expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int n_chunks,
                    uint8_t* __restrict__ mask) {
   pdl_entry();
-  __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 8];       // [4] words of slack in front: shifts read from there
+  __shared__ uint8_t dec_s[kMaskStage];
+  __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 12];       // [4] words of slack in front: shifts read from there
   const int p = blockIdx.x / n_chunks;
   const long long row_len = (long long)N * Ks, c0 = (long long)(blockIdx.x - p * n_chunks) * kMaskChunk;
   const int len = int(min((long long)kMaskChunk, row_len - c0));
-  const uint8_t* g = gmask + (long long)p * Q * Ks;
   const int cs = int(c0 / Ks), ks = int(c0 - (long long)cs * Ks);    // input channel and location the chunk starts at
-  for (int o = threadIdx.x * 4; o < len; o += kMaskThreads * 4) {
-    const int dc = (ks + o) / Ks;
-    int k = ks + o - dc * Ks, q = (cs + dc) / g_n, j = cs + dc - q * g_n;
-    uint32_t word = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      if (o + b < len) word |= uint32_t(__ldg(g + (long long)q * Ks + k)) << (8 * b);
-      if (++k == Ks) { k = 0; if (++j == g_n) { j = 0; ++q; } }
-    }
-    row_s[4 + o / 4] = word;
+  // the decisions that the chunk covers, a contiguous run, come in at once
+  const int q0 = cs / g_n, n_dec = ((cs + (ks + len - 1) / Ks) / g_n + 1 - q0) * Ks;
+  const uint8_t* g = gmask + ((long long)p * Q + q0) * Ks;
+  const bool staged = n_dec <= kMaskStage;
+  if (staged) {
+    for (int i = threadIdx.x; i < n_dec; i += kMaskThreads) dec_s[i] = __ldg(g + i);
+    __syncthreads();
   }
-  if (threadIdx.x < 4) { row_s[threadIdx.x] = 0; row_s[4 + (len + 3) / 4 + threadIdx.x] = 0; }
+  // 16 bytes at a time: the divisions that find the first byte's decision cost more than the bytes themselves
+  for (int o = threadIdx.x * 16; o < len; o += kMaskThreads * 16) {
+    const int dc = (ks + o) / Ks;
+    int k = ks + o - dc * Ks, q = (cs + dc) / g_n - q0, j = cs + dc - (q + q0) * g_n;
+    int at = q * Ks + k;
+    uint32_t word[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      word[v] = 0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        if (o + 4 * v + b < len) word[v] |= uint32_t(staged ? dec_s[at] : __ldg(g + at)) << (8 * b);
+        ++at;
+        if (++k == Ks) {                                             // the next channel: the same decisions, or the next group's
+          k = 0;
+          if (++j == g_n) j = 0;
+          else at -= Ks;
+        }
+      }
+    }
+    *reinterpret_cast<uint4*>(row_s + 4 + o / 4) = make_uint4(word[0], word[1], word[2], word[3]);
+  }
+  if (threadIdx.x < 4) { row_s[threadIdx.x] = 0; row_s[4 + (len + 15) / 16 * 4 + threadIdx.x] = 0; }
   __syncthreads();
   const uint8_t* bytes = reinterpret_cast<const uint8_t*>(row_s + 4);
   const int rows = min(g_m, M - p * g_m);

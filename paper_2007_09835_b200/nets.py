@@ -8,19 +8,17 @@ step is a call into librt3d; torch provides device memory and streams.
 from __future__ import annotations
 
 import contextlib
-import ctypes
 
 import numpy as np
 import torch
 
-from . import _pycall, binding as B
+from . import binding as B
 
-_pycall.setup(torch.float32, torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
-_ADDRESS = {fn: ctypes.cast(getattr(B.lib(), fn), ctypes.c_void_p).value
-            for fn in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_sparse_fused")}
+_pycall, _ADDRESS = B.pycall(), B.ADDRESS
 # The binding's compute functions as they are: calls go round them only while they are what the binding's module holds (a
 # tracer or a test that wraps them sees every call).
-_FUNCTIONS = {fn: getattr(B, fn) for fn in (*_ADDRESS, "rt3d_conv2plus1d_fused", "rt3d_maxpool3d", "rt3d_add_relu")}
+_FUNCTIONS = {fn: getattr(B, fn) for fn in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_sparse_fused",
+                                            "rt3d_conv2plus1d_fused", "rt3d_maxpool3d", "rt3d_add_relu")}
 
 
 def _unwrapped(*names) -> bool:
