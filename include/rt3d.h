@@ -140,6 +140,12 @@ rt3d_status rt3d_pack_kgs(const float* w, const uint8_t* mask, int M, int N, int
 rt3d_status rt3d_pack_dense(const float* w, int M, int N, int Kt, int Kh, int Kw,
                             int compute_dtype, rt3d_packed** out);
 
+/* rt3d_pack_concat - handle whose filters are those of `parts` one after the other: layers that read the same tensor run as
+ * one convolution.  All parts have the same N, kernel extents, group size, dtype and kind (pruned or dense), and every
+ * part but the last a filter count that is a multiple of g_m; else RT3D_ERR_SHAPE.  The parts stay as they are.
+ * Pure host work. */
+rt3d_status rt3d_pack_concat(const rt3d_packed* const* parts, int n_parts, rt3d_packed** out);
+
 /* Read-only view of the canonical arrays (for bit-exact checks of the pack). */
 rt3d_status rt3d_packed_view_get(const rt3d_packed* p, rt3d_packed_view* view);
 

@@ -77,6 +77,7 @@ def _load():
     TP, CP = ctypes.POINTER(Tensor), ctypes.POINTER(ConvParams)
     lib.rt3d_pack_kgs.argtypes = [f32p, u8p, i, i, i, i, i, i, i, i, ctypes.POINTER(vp)]
     lib.rt3d_pack_dense.argtypes = [f32p, i, i, i, i, i, i, ctypes.POINTER(vp)]
+    lib.rt3d_pack_concat.argtypes = [ctypes.POINTER(vp), i, ctypes.POINTER(vp)]
     lib.rt3d_packed_view_get.argtypes = [vp, ctypes.POINTER(PackedView)]
     lib.rt3d_unpack_to_dense.argtypes = [vp, f32p]
     lib.rt3d_unpack_device_layout.argtypes = [vp, i, f32p]
@@ -229,6 +230,14 @@ def rt3d_pack_dense(w, compute_dtype: int) -> Packed:
     h = ctypes.c_void_p()
     _check(_lib.rt3d_pack_dense(w.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), M, N, Kt, Kh, Kw,
                                 int(compute_dtype), ctypes.byref(h)), "rt3d_pack_dense")
+    return Packed(h.value)
+
+
+def rt3d_pack_concat(parts) -> Packed:
+    """One handle with the filters of `parts` (Packed handles over the same input channels) one after the other."""
+    arr = (ctypes.c_void_p * len(parts))(*(p.handle for p in parts))
+    h = ctypes.c_void_p()
+    _check(_lib.rt3d_pack_concat(arr, len(parts), ctypes.byref(h)), "rt3d_pack_concat")
     return Packed(h.value)
 
 

@@ -380,6 +380,11 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
   return p->f32_layout.get();
 }
 
+static uint64_t next_handle_id() {
+  static std::atomic<uint64_t> next_id{1};
+  return next_id.fetch_add(1);
+}
+
 static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, int Kt, int Kh, int Kw,
                              int g_m, int g_n, int dtype, int is_dense, rt3d_packed** out) {
   if (!w || !out) return RT3D_ERR_INVALID_ARG;
@@ -391,8 +396,7 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
   if (Ks64 > 65535) return RT3D_ERR_INVALID_ARG;
   rt3d_packed* h = new (std::nothrow) rt3d_packed;
   if (!h) return RT3D_ERR_ALLOC;
-  static std::atomic<uint64_t> next_id{1};
-  h->id = next_id.fetch_add(1);
+  h->id = next_handle_id();
   try {
     h->M = M; h->N = N; h->Kt = Kt; h->Kh = Kh; h->Kw = Kw; h->g_m = g_m; h->g_n = g_n;
     h->P = ceil_div(M, g_m); h->Q = ceil_div(N, g_n); h->Ks = int(Ks64);
@@ -490,6 +494,48 @@ rt3d_status rt3d_pack_kgs(const float* w, const uint8_t* mask, int M, int N, int
 rt3d_status rt3d_pack_dense(const float* w, int M, int N, int Kt, int Kh, int Kw, int compute_dtype,
                             rt3d_packed** out) {
   return pack_impl(w, nullptr, M, N, Kt, Kh, Kw, 4, 4, compute_dtype, 1, out);
+}
+
+rt3d_status rt3d_pack_concat(const rt3d_packed* const* parts, int n_parts, rt3d_packed** out) {
+  if (!parts || n_parts < 1 || !out) return RT3D_ERR_INVALID_ARG;
+  *out = nullptr;
+  int64_t nnz = 0, bytes = 0;
+  for (int i = 0; i < n_parts; ++i) {
+    const rt3d_packed *a = parts[0], *p = parts[i];
+    if (!p) return RT3D_ERR_INVALID_ARG;
+    if (p->N != a->N || p->Kt != a->Kt || p->Kh != a->Kh || p->Kw != a->Kw || p->g_m != a->g_m || p->g_n != a->g_n ||
+        p->dtype != a->dtype || p->is_dense != a->is_dense || (i + 1 < n_parts && p->M % p->g_m))
+      return RT3D_ERR_SHAPE;
+    nnz += p->nnz;
+    bytes += int64_t(p->tiles.size());
+  }
+  if (nnz > 0x7FFFFFFF) return RT3D_ERR_UNSUPPORTED;
+  rt3d_packed* h = new (std::nothrow) rt3d_packed;
+  if (!h) return RT3D_ERR_ALLOC;
+  h->id = next_handle_id();
+  try {
+    const rt3d_packed* a = parts[0];
+    h->N = a->N; h->Kt = a->Kt; h->Kh = a->Kh; h->Kw = a->Kw; h->g_m = a->g_m; h->g_n = a->g_n; h->Q = a->Q; h->Ks = a->Ks;
+    h->dtype = a->dtype; h->is_dense = a->is_dense; h->is_vanilla = 1;
+    h->tiles.allocate(size_t(bytes));
+    h->group_ptr.push_back(0);
+    unsigned char* at = h->tiles.data();
+    for (int i = 0; i < n_parts; ++i) {
+      const rt3d_packed* p = parts[i];
+      h->M += p->M; h->P += p->P;
+      h->is_vanilla = h->is_vanilla && p->is_vanilla;
+      for (size_t g = 1; g < p->group_ptr.size(); ++g) h->group_ptr.push_back(int32_t(h->nnz) + p->group_ptr[g]);
+      h->pos_idx.insert(h->pos_idx.end(), p->pos_idx.begin(), p->pos_idx.end());
+      if (p->tiles.size()) std::memcpy(at, p->tiles.data(), p->tiles.size());
+      at += p->tiles.size();
+      h->nnz += p->nnz;
+    }
+  } catch (const std::bad_alloc&) {
+    delete h;
+    return RT3D_ERR_ALLOC;
+  }
+  *out = h;
+  return RT3D_OK;
 }
 
 rt3d_status rt3d_packed_view_get(const rt3d_packed* p, rt3d_packed_view* v) {

@@ -142,55 +142,36 @@ __global__ void reweight_kernel(const float* __restrict__ norms, long long count
 
 constexpr int kMaskThreads = 256;
 constexpr int kMaskChunk = 4096;      // bytes of one mask row that a block expands at a time
-constexpr int kMaskStage = 8192;      // decisions held in shared memory; one-channel groups of many locations may need more
 
 // The g_m mask rows of a row of kernel groups are the same N * Ks bytes: a block expands a chunk of them once into
-// shared memory and writes it to every row in 16-byte stores.  A row may start at any byte, so the words of each row
-// are cut out of the staged chunk at that row's shift (funnel shifts), and only a chunk's first and last partial word
-// go out byte by byte.  One thread per mask byte, as before, paid two 64-bit divisions for each.
+// shared memory (each decision goes to the g_n channels of its group) and writes it to every row in 16-byte stores.  A row
+// may start at any byte, so the words of a row that does not start on a 16-byte boundary are cut out of the staged chunk at
+// that row's shift (funnel shifts), and only a chunk's first and last partial word go out byte by byte.  Bound by its
+// instructions: one thread per mask byte paid two 64-bit divisions for each, and gathering the bytes of a word instead of
+// scattering the decisions still took 740 instructions a thread (1024 x 512 x 27: 9.7 us, scattering 7.3 us).
 __global__ void __launch_bounds__(kMaskThreads)
 expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int n_chunks,
                    uint8_t* __restrict__ mask) {
   pdl_entry();
-  __shared__ uint8_t dec_s[kMaskStage];
-  __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 12];       // [4] words of slack in front: shifts read from there
+  __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 12];      // [4] words of slack in front: shifts read from there
+  uint8_t* bytes = reinterpret_cast<uint8_t*>(row_s + 4);
   const int p = blockIdx.x / n_chunks;
   const long long row_len = (long long)N * Ks, c0 = (long long)(blockIdx.x - p * n_chunks) * kMaskChunk;
   const int len = int(min((long long)kMaskChunk, row_len - c0));
-  const int cs = int(c0 / Ks), ks = int(c0 - (long long)cs * Ks);    // input channel and location the chunk starts at
-  // the decisions that the chunk covers, a contiguous run, come in at once
-  const int q0 = cs / g_n, n_dec = ((cs + (ks + len - 1) / Ks) / g_n + 1 - q0) * Ks;
+  // the groups that the chunk touches, their decisions a contiguous run; first: where the first of them starts
+  const long long span = (long long)g_n * Ks;
+  const int q0 = int(c0 / span), q1 = int((c0 + len - 1) / span);
+  const int first = int(q0 * span - c0), n_dec = (q1 + 1 - q0) * Ks;
   const uint8_t* g = gmask + ((long long)p * Q + q0) * Ks;
-  const bool staged = n_dec <= kMaskStage;
-  if (staged) {
-    for (int i = threadIdx.x; i < n_dec; i += kMaskThreads) dec_s[i] = __ldg(g + i);
-    __syncthreads();
+  for (int i = threadIdx.x; i < n_dec; i += kMaskThreads) {
+    const uint8_t bit = __ldg(g + i);
+    const int q = i / Ks;
+    int o = first + q * int(span) + (i - q * Ks);
+#pragma unroll 4
+    for (int j = 0; j < g_n; ++j, o += Ks)
+      if (unsigned(o) < unsigned(len)) bytes[o] = bit;
   }
-  // 16 bytes at a time: the divisions that find the first byte's decision cost more than the bytes themselves
-  for (int o = threadIdx.x * 16; o < len; o += kMaskThreads * 16) {
-    const int dc = (ks + o) / Ks;
-    int k = ks + o - dc * Ks, q = (cs + dc) / g_n - q0, j = cs + dc - (q + q0) * g_n;
-    int at = q * Ks + k;
-    uint32_t word[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      word[v] = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        if (o + 4 * v + b < len) word[v] |= uint32_t(staged ? dec_s[at] : __ldg(g + at)) << (8 * b);
-        ++at;
-        if (++k == Ks) {                                             // the next channel: the same decisions, or the next group's
-          k = 0;
-          if (++j == g_n) j = 0;
-          else at -= Ks;
-        }
-      }
-    }
-    *reinterpret_cast<uint4*>(row_s + 4 + o / 4) = make_uint4(word[0], word[1], word[2], word[3]);
-  }
-  if (threadIdx.x < 4) { row_s[threadIdx.x] = 0; row_s[4 + (len + 15) / 16 * 4 + threadIdx.x] = 0; }
   __syncthreads();
-  const uint8_t* bytes = reinterpret_cast<const uint8_t*>(row_s + 4);
   const int rows = min(g_m, M - p * g_m);
   for (int i = 0; i < rows; ++i) {
     uint8_t* dst = mask + (long long)(p * g_m + i) * row_len + c0;
@@ -199,12 +180,16 @@ expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int 
     for (int u = threadIdx.x; u < n_words; u += kMaskThreads) {
       const int o = u * 16 - shift;                                  // first byte of the word inside the chunk
       if (o >= 0 && o + 16 <= len) {
-        const int w0 = (o >> 2) + 4, sh = (o & 3) * 8;
         uint4 v;
-        v.x = __funnelshift_r(row_s[w0], row_s[w0 + 1], sh);
-        v.y = __funnelshift_r(row_s[w0 + 1], row_s[w0 + 2], sh);
-        v.z = __funnelshift_r(row_s[w0 + 2], row_s[w0 + 3], sh);
-        v.w = __funnelshift_r(row_s[w0 + 3], row_s[w0 + 4], sh);
+        if (shift == 0) {
+          v = *reinterpret_cast<const uint4*>(bytes + o);
+        } else {
+          const int w0 = (o >> 2) + 4, sh = (o & 3) * 8;
+          v.x = __funnelshift_r(row_s[w0], row_s[w0 + 1], sh);
+          v.y = __funnelshift_r(row_s[w0 + 1], row_s[w0 + 2], sh);
+          v.z = __funnelshift_r(row_s[w0 + 2], row_s[w0 + 3], sh);
+          v.w = __funnelshift_r(row_s[w0 + 3], row_s[w0 + 4], sh);
+        }
         *reinterpret_cast<uint4*>(dst + o) = v;
       } else {
         for (int b = max(o, 0); b < min(o + 16, len); ++b) dst[b] = bytes[b];

@@ -8,6 +8,7 @@ step is a call into librt3d; torch provides device memory and streams.
 from __future__ import annotations
 
 import contextlib
+import dataclasses
 
 import numpy as np
 import torch
@@ -445,59 +446,125 @@ class S3DNet(_NotedForward):
         y = self.ws.get(spec.name, layer.out_shape(x), x.dtype, x.device)
         return layer(x, y, algo=algo, stream=stream, x_pad_zero=pad0)
 
-    def _pool(self, spec, x, c, stream):
-        n, t, h, w, cs = x.shape
-        ext = [(d + 2 * p - k) // s + 1 for d, p, k, s in zip((t, h, w), spec.pad, spec.k, spec.stride)]
-        y = self.ws.get(spec.name, (n, ext[0], ext[1], ext[2], cs), x.dtype, x.device)
-        return maxpool(x, c, spec, y, stream=stream)
+    def _concat(self, specs):
+        """The layers of `specs`, which read the same tensor, as one; None where their handles do not go together."""
+        parts = [self.layers[sp.name] for sp in specs]
+        made = self.__dict__.setdefault("_concats", {})
+        key = tuple(sp.name for sp in specs)
+        now = [(p.packed, p.bias) for p in parts]
+        if key not in made or any(a is not c or b is not d for (a, b), (c, d) in zip(made[key][0], now)):
+            layer = None
+            if all(sp.relu == specs[0].relu and sp.stride == specs[0].stride and sp.pad == specs[0].pad for sp in specs) and \
+                    len({p.dtype for p in parts}) == 1 and all(sp.cout % 8 == 0 for sp in specs):
+                try:
+                    packed = B.rt3d_pack_concat([p.packed for p in parts])
+                except B.Rt3dError as e:
+                    if e.status != B.ERR_SHAPE:
+                        raise
+                else:
+                    layer = object.__new__(ConvLayer)
+                    layer.spec = dataclasses.replace(specs[0], name="+".join(key), cout=sum(sp.cout for sp in specs))
+                    layer.dtype, layer.dense, layer.device = parts[0].dtype, parts[0].dense, parts[0].device
+                    layer.packed = packed
+                    layer.bias = None if all(p.bias is None for p in parts) else torch.cat(
+                        [torch.zeros(sp.cout, device=p.device) if p.bias is None else p.bias for sp, p in zip(specs, parts)])
+            made[key] = (now, layer)
+        return made[key][1]
+
+    def _block(self, op, x, off, last, algo, stream, merge):
+        """One Inception block on channels [off, off + cin) of x; returns (output tensor, first channel of the output in it).
+
+        The three 1x1x1 convolutions that read the block's input run as one where the layers allow it (`merge`): a third of
+        the reads of x and of the launches.  It writes [b1 reduction | b2 reduction | b0] side by side, so the block's output
+        then lies behind the reductions in one wide tensor, on a 128-byte boundary; the last block, whose output is the
+        network's, merges the two reductions only."""
+        n, t, h, w, _ = x.shape
+        xd = B.channel_slice_desc(x, off, op.cin)
+        r1, r2 = op.b1[0].cout, op.b2[0].cout
+        wide = self._concat((op.b1[0], op.b2[0], op.b0)) if merge and not last else None
+        both = self._concat((op.b1[0], op.b2[0])) if merge and last else None
+        if wide is not None:
+            start = -(-(r1 + r2) // 64) * 64                        # first channel of the output
+            out = self.ws.get(op.name + ".wide", (n, t, h, w, start + -(-op.cout // 64) * 64), x.dtype, x.device)
+            red, red_off = out, start - r1 - r2
+        else:
+            start, red_off = 0, 0
+            out = self.ws.get(op.name, (n, t, h, w, op.cout), x.dtype, x.device)
+            red = None if both is None else self.ws.get(op.name + ".reduce", (n, t, h, w, r1 + r2), x.dtype, x.device)
+        offs = [start, start + op.b0.cout, start + op.b0.cout + op.b1[2].cout, start + op.b0.cout + op.b1[2].cout + op.b2[2].cout]
+
+        def branch0():
+            self.layers[op.b0.name].run_desc(xd, B.channel_slice_desc(out, offs[0], op.b0.cout), algo, stream)
+
+        def sep(br, to, at):
+            if red is None:
+                a = self.ws.get(br[0].name, self.layers[br[0].name].out_shape(x), x.dtype, x.device)
+                ad = B.tensor_desc(a, br[0].cout)
+                self.layers[br[0].name].run_desc(xd, ad, algo, stream)
+            else:
+                ad = B.channel_slice_desc(red, at, br[0].cout)
+            b = self.ws.get(br[1].name, (n, t, h, w, pitch_for(br[1].cout, x.dtype)), x.dtype, x.device)
+            self.layers[br[1].name].run_desc(ad, B.tensor_desc(b, br[1].cout), algo, stream)
+            self.layers[br[2].name].run_desc(B.tensor_desc(b, br[2].cin), B.channel_slice_desc(out, to, br[2].cout), algo, stream)
+
+        def branch3():
+            p = self.ws.get(op.pool.name, (n, t, h, w, pitch_for(op.cin, x.dtype)), x.dtype, x.device)
+            B.rt3d_maxpool3d(xd, op.pool.k, op.pool.stride, op.pool.pad, B.tensor_desc(p, op.cin), stream)
+            self.layers[op.b3.name].run_desc(B.tensor_desc(p, op.cin), B.channel_slice_desc(out, offs[3], op.b3.cout), algo, stream)
+
+        def reduce():
+            layer = wide if wide is not None else both
+            if layer is not None:
+                layer.run_desc(xd, B.channel_slice_desc(red, red_off, layer.spec.cout), algo, stream)
+
+        seps = [lambda: sep(op.b1, offs[1], red_off), lambda: sep(op.b2, offs[2], red_off + r1)]
+        rest = branch0 if wide is None else None
+        if not (self.parallel_branches and stream is None):
+            reduce()
+            for fn in ([rest] if rest else []) + seps + [branch3]:
+                fn()
+            return out, start
+        # independent branches on streams of their own; the main stream takes the reductions and the longest branch
+        main, side = torch.cuda.current_stream(x.device), self._branch_streams(x.device)
+        joins = []
+        with B.concurrent_kernels():
+            def beside(s, fn, after):
+                _wait(s, after)
+                with torch.cuda.stream(s):
+                    fn()
+                    joins.append(_record(s))
+
+            fork = _record(main)
+            beside(side[2], branch3, fork)
+            if rest is not None:
+                beside(side[0], rest, fork)
+            reduce()
+            beside(side[1], seps[1], _record(main) if red is not None else fork)
+            seps[0]()
+        for ev in joins:
+            _wait(main, ev)
+        return out, start
 
     def _forward(self, x, algo, keep, stream):
-        c = self.plan[0].cin
+        c, off = self.plan[0].cin, 0
         for i, op in enumerate(self.plan):
             if hasattr(op, "b0"):                                   # Inception block
-                n, t, h, w, _ = x.shape
-                out = self.ws.get(op.name, (n, t, h, w, op.cout), x.dtype, x.device)
-                xd = B.tensor_desc(x, op.cin)
-                offs = [0, op.b0.cout, op.b0.cout + op.b1[2].cout, op.b0.cout + op.b1[2].cout + op.b2[2].cout]
-
-                def branch0(x=x, xd=xd, out=out, op=op):
-                    self.layers[op.b0.name].run_desc(xd, B.channel_slice_desc(out, offs[0], op.b0.cout), algo, stream)
-
-                def branch_sep(br, off, x=x, out=out):
-                    a = self._conv(br[0], x, algo, stream)
-                    b = self._conv(br[1], a, algo, stream)
-                    self.layers[br[2].name].run_desc(B.tensor_desc(b, br[2].cin), B.channel_slice_desc(out, off, br[2].cout),
-                                                     algo, stream)
-
-                def branch3(x=x, out=out, op=op):
-                    p = self._pool(op.pool, x, op.cin, stream)
-                    self.layers[op.b3.name].run_desc(B.tensor_desc(p, op.cin), B.channel_slice_desc(out, offs[3], op.b3.cout),
-                                                     algo, stream)
-
-                work = [lambda: branch_sep(op.b1, offs[1]), lambda: branch_sep(op.b2, offs[2]), branch3]
-                if self.parallel_branches and stream is None:
-                    main = torch.cuda.current_stream(x.device)
-                    fork = _record(main)
-                    joins = []
-                    with B.concurrent_kernels():
-                        for fn, side in zip(work, self._branch_streams(x.device)):
-                            _wait(side, fork)
-                            with torch.cuda.stream(side):
-                                fn()
-                                joins.append(_record(side))
-                        branch0()                                    # the main stream takes the 1x1x1 branch
-                    for ev in joins:
-                        _wait(main, ev)
-                else:
-                    branch0()
-                    for fn in work:
-                        fn()
-                x, c = out, op.cout
-            elif hasattr(op, "cout"):
-                x = self._conv(op, x, algo, stream, pad0=self.input_pad_zero and i == 0)
+                x, off = self._block(op, x, off, i + 1 == len(self.plan), algo, stream, keep is None)
                 c = op.cout
+            elif hasattr(op, "cout"):
+                if off:                                             # behind a wide block
+                    y = self.ws.get(op.name, self.layers[op.name].out_shape(x), x.dtype, x.device)
+                    self.layers[op.name].run_desc(B.channel_slice_desc(x, off, c), B.tensor_desc(y, op.cout), algo, stream)
+                    x = y
+                else:
+                    x = self._conv(op, x, algo, stream, pad0=self.input_pad_zero and i == 0)
+                c, off = op.cout, 0
             else:
-                x = self._pool(op, x, c, stream)
+                n, t, h, w, cs = x.shape
+                ext = [(d + 2 * p - k) // s + 1 for d, p, k, s in zip((t, h, w), op.pad, op.k, op.stride)]
+                y = self.ws.get(op.name, (n, ext[0], ext[1], ext[2], pitch_for(c, x.dtype)), x.dtype, x.device)
+                B.rt3d_maxpool3d(B.channel_slice_desc(x, off, c), op.k, op.stride, op.pad, B.tensor_desc(y, c), stream)
+                x, off = y, 0
             if keep is not None:
                 keep[op.name] = x
         return x

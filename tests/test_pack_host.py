@@ -108,3 +108,19 @@ def test_sub_tile_layout_holds_exactly_the_masked_weights(M, N, k, g_m, g_n, den
     L = _layer(M, N, k, g_m, g_n, density, 3)
     pk = rt3d.rt3d_pack_kgs(L["w"], L["mask"], g_m, g_n, rt3d.RT3D_BF16)
     np.testing.assert_array_equal(pk.unpack_sub_layout(0), oracle.bf16_round(L["w"] * L["mask"]))
+
+
+@pytest.mark.parametrize("dtype", [rt3d.RT3D_F32, rt3d.RT3D_BF16])
+def test_concatenated_handles_hold_the_filters_one_after_the_other(dtype):
+    layers = [synth.make_layer(synth.ConvSpec("c", 20, m, (1, 3, 3), (1, 1, 1), (0, 1, 1)), 7, i, 4, 4, "bernoulli", 0.3)
+              for i, m in enumerate((8, 16, 6))]                       # the last count need not be a multiple of the group's
+    parts = [rt3d.rt3d_pack_kgs(L["w"], L["mask"], 4, 4, dtype) for L in layers]
+    got = rt3d.rt3d_pack_concat(parts).view()
+    ref = rt3d.rt3d_pack_kgs(np.concatenate([L["w"] for L in layers]), np.concatenate([L["mask"] for L in layers]), 4, 4, dtype).view()
+    for k, v in ref.items():
+        assert np.array_equal(got[k], v), k
+    other = rt3d.rt3d_pack_dense(layers[0]["w"], dtype)
+    for bad in ([parts[2], parts[0]], [parts[0], other]):              # ragged rows in the middle; pruned with dense
+        with pytest.raises(rt3d.Rt3dError) as e:
+            rt3d.rt3d_pack_concat(bad)
+        assert e.value.status == rt3d.ERR_SHAPE
