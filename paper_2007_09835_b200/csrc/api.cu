@@ -611,6 +611,11 @@ bool smallc_eligible(const DeviceState* d, rt3d_packed* w, const rt3d_tensor* x,
   if (w->Kt > 16 || w->Kh > 32 || w->Kw > 32) return false;
   const SmallCLayout* L = get_smallc_layout(w, p->sh, p->sw);
   if (!L) return false;
+  const SmallCLayout* P = get_smallc_layout(w, p->sh, p->sw, true);
+  if (P && P->n_pairs < L->n_pairs && smallc_smem_bytes(P->n_pairs, P->n_pad, P->phase_stride, int(P->ops.size())) <= 227 * 1024) {
+    *out = P;
+    return true;
+  }
   if (L->img_w * p->sw > 256 || L->img_h * p->sh > 256) return false;
   if (smallc_smem_bytes(L->n_pairs, L->n_pad, L->n_phases * L->phase_stride) > 227 * 1024) return false;
   *out = L;
@@ -626,19 +631,14 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   DeviceBlob::SmallC* sc = nullptr;
   {
     std::lock_guard<std::mutex> lock(w->mu);
-    sc = &blob->smallc[L->sh * 16 + L->sw];
-    if (!sc->wimg) {
-      void* wi = nullptr;
-      int32_t* po = nullptr;
-      if (dev_malloc(&wi, L->wimg.size() * 2 + 16) != cudaSuccess ||
-          dev_malloc(&po, L->pair_off.size() * 4 + 16) != cudaSuccess)
-        return RT3D_ERR_ALLOC;
-      if ((!L->wimg.empty() && cudaMemcpy(wi, L->wimg.data(), L->wimg.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess) ||
-          (!L->pair_off.empty() &&
-           cudaMemcpy(po, L->pair_off.data(), L->pair_off.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess))
-        return RT3D_ERR_CUDA;
-      sc->pairs = po;
-      sc->wimg = wi;
+    sc = &blob->smallc[L->sh * 16 + L->sw + (L->packed ? 1024 : 0)];
+    if (!sc->base) {
+      Upload up;
+      up.add(&sc->wimg, L->wimg);
+      up.add(&sc->pairs, L->pair_off);
+      up.add(&sc->ops, L->ops);
+      const rt3d_status s = up.run(&sc->base);
+      if (s != RT3D_OK) return s;
     }
   }
   SmallCArgs a;
@@ -651,6 +651,7 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   a.residual = residual; a.rcs = rcs;
   a.pool_t = 1; a.pool_h = pool_h; a.pool_w = pool_w;
   a.wimg = sc->wimg; a.pair_off = sc->pairs;
+  a.ops = L->packed ? sc->ops : nullptr; a.n_ops = int(L->ops.size()); a.img_h = L->img_h; a.x = x->data;
   a.bias = bias; a.y = y->data; a.sched = d->sched;
   // input as [n][t][h][w][8]: one box = one phase image of a 1 x 16 x 8 output tile (every sh-th row and
   // sw-th column: a traversal stride s loads ceil(box / s) elements), no swizzle
@@ -664,14 +665,16 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   // image row as one contiguous run instead of one 16-byte request per voxel (the tile load was the
   // kernel's bottleneck).  Otherwise the separate channel axis stays: its out-of-range
   // fill is what zeroes the padding channels, whatever the caller's buffer holds there.
-  a.merged_cw = (g.sw == 1 && (x->c == 8 || x_pad_zero) && L->img_w * 8 <= 256) ? 1 : 0;
+  a.merged_cw = (!L->packed && g.sw == 1 && (x->c == 8 || x_pad_zero) && L->img_w * 8 <= 256) ? 1 : 0;
   if (a.merged_cw) {
     dims[0] = cuuint64_t(x->w) * 8; dims[1] = 1;
     strides[0] = cs;                                   // the unit axis never moves
     bx[0] = cuuint32_t(L->img_w * 8); bx[1] = 1;
     estr[1] = 1;
   }
-  if (g_encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, x->data, dims, strides, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  memset(&xmap, 0, sizeof(xmap));
+  if (!L->packed &&
+      g_encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, x->data, dims, strides, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return RT3D_ERR_CUDA;
   CUtensorMap ymap;
@@ -1290,7 +1293,7 @@ void rt3d_packed_free(rt3d_packed* p) {
     cudaFree(b->stage_x); cudaFree(b->stage_y); cudaFree(b->stage_bias);
     for (void* hs : b->host_streams) if (hs) cudaStreamDestroy(static_cast<cudaStream_t>(hs));
     for (void* he : b->host_events) if (he) cudaEventDestroy(static_cast<cudaEvent_t>(he));
-    for (auto& kv : b->smallc) { cudaFree(kv.second.wimg); cudaFree(kv.second.pairs); }
+    for (auto& kv : b->smallc) cudaFree(kv.second.base);
     cudaFree(b->f32.base);
     for (auto& kv : b->sub) { cudaFree(kv.second.steps); cudaFree(kv.second.step_ptr); cudaFree(kv.second.blocks); }
     cudaFree(b->splitk); cudaFree(b->splitk_cnt);

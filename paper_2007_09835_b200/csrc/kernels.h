@@ -214,6 +214,9 @@ struct SmallCArgs {
   const void* residual;               // device bf16 tensor added before the ReLU, or nullptr
   int rcs;                            // its channel pitch
   int pool_t, pool_h, pool_w;         // fused max-pool window (1,1,1 = none; pool_t must be 1); needs store_tma
+  const uint32_t* ops;                // device: the copies of the packed form, or nullptr
+  int n_ops, img_h;
+  const void* x;                      // input of the packed form, 16 bytes a voxel
   const void* wimg;                   // device: [n_pairs][2][n_pad/8][8][8] bf16
   const int32_t* pair_off;            // device: [n_pairs][2] byte offsets inside the staged images
   const float* bias;
@@ -222,7 +225,7 @@ struct SmallCArgs {
 };
 cudaError_t launch_conv_umma_smallc(const SmallCArgs& a, const void* xmap, const void* ymap, int sm_count,
                                     cudaStream_t stream);
-size_t smallc_smem_bytes(int n_pairs, int n_pad, int stage_bytes);
+size_t smallc_smem_bytes(int n_pairs, int n_pad, int stage_bytes, int n_ops = 0);
 
 // Test hook (debug_poison.cu): every SM's shared memory and tensor memory filled with `pattern`; `sink`: a device int.
 cudaError_t launch_debug_poison(uint32_t pattern, int sm_count, int* sink, cudaStream_t stream);

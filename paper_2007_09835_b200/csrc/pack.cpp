@@ -242,15 +242,21 @@ const SubLayout* get_sub_layout(rt3d_packed* p, int n_tile) {
 // sorted by the offset of their window inside the staged phase images and paired; each pair is one
 // K=16 MMA whose two K halves are the 8 (padded) channels at the two locations.  Operands use the
 // no-swizzle core-matrix layout (8 rows x 16 bytes).
-const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw) {
+static bool build_smallc_packed(rt3d_packed* p, SmallCLayout& L);
+const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw, bool packed) {
   if (p->dtype != RT3D_BF16 || p->N > 8 || p->M > 256 || sh < 1 || sw < 1 || sh > 4 || sw > 4) return nullptr;
   std::lock_guard<std::mutex> lock(p->mu);
-  const int key = sh * 16 + sw;
+  const int key = sh * 16 + sw + (packed ? 1024 : 0);
   auto it = p->smallc_layouts.find(key);
-  if (it != p->smallc_layouts.end()) return &it->second;
+  if (it != p->smallc_layouts.end()) return it->second.n_pad ? &it->second : nullptr;
   SmallCLayout L;
   L.sh = sh; L.sw = sw;
   L.n_pad = round_up(p->M, 16);
+  if (packed) {
+    if (!build_smallc_packed(p, L)) L.n_pad = 0;         // remembered as not to be had
+    auto res = p->smallc_layouts.emplace(key, std::move(L));
+    return res.first->second.n_pad ? &res.first->second : nullptr;
+  }
   L.n_phases = sh * sw;
   L.img_w = kSmallCTileW - 1 + ceil_div(p->Kw, sw);
   L.img_h = kSmallCTileH - 1 + ceil_div(p->Kh, sh);
@@ -378,6 +384,73 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
       }
   p->f32_layout = std::move(layout);
   return p->f32_layout.get();
+}
+
+// The packed form: entry e of a row holds columns (2e, 2e + 1), the kernel columns (2a, 2a + 1) read entries from a on; an
+// odd last kernel column has entries of its own, with zeros behind it (a column outside the window must not be read even
+// against zero weights: NaN x 0 is NaN).
+static bool build_smallc_packed(rt3d_packed* p, SmallCLayout& L) {
+  const int Kw = p->Kw, pairs = Kw / 2;
+  if (p->N > 4 || L.sw != 2 || Kw > 32 || p->Kt > 15) return false;
+  struct Entry { int lo, hi; };
+  std::vector<Entry> row;                               // the entries of an image row: input columns, -1 = zeros
+  struct Half { int slot, tap0, tap1; };
+  std::vector<Half> halves;                             // what a kernel row reads: first entry, its two kernel columns
+  if (pairs > 0)
+    for (int e = 0; e < kSmallCTileW - 1 + pairs; ++e) row.push_back({2 * e, 2 * e + 1});
+  for (int a = 0; a < pairs; ++a) halves.push_back({a, 2 * a, 2 * a + 1});
+  if (Kw % 2) {
+    halves.push_back({int(row.size()), Kw - 1, -1});
+    for (int e = 0; e < kSmallCTileW; ++e) row.push_back({2 * e + Kw - 1, -1});
+  }
+  L.packed = true;
+  L.n_phases = 1;
+  L.img_w = int(row.size());
+  L.img_h = (kSmallCTileH - 1) * L.sh + p->Kh;
+  L.img_t = p->Kt;
+  L.phase_stride = round_up(L.img_w * L.img_h * L.img_t * 16, 128);
+  if (L.img_h > 63 || L.phase_stride > (1 << 16) * 8) return false;
+  for (int t = 0; t < L.img_t; ++t)
+    for (int h = 0; h < L.img_h; ++h)
+      for (int e = 0; e < L.img_w; ++e)
+        for (int half = 0; half < 2; ++half) {
+          const int col = half ? row[size_t(e)].hi : row[size_t(e)].lo;
+          if (col < 0) continue;
+          if (col > 63) return false;
+          L.ops.push_back(uint32_t(((t * L.img_h + h) * L.img_w + e) * 2 + half) | uint32_t(col) << 16 | uint32_t(h) << 22 |
+                          uint32_t(t) << 28);
+        }
+  std::vector<uint8_t> used(size_t(p->Ks), 0);
+  for (int64_t e = 0; e < p->nnz; ++e) used[p->pos_idx[size_t(e)]] = 1;
+  std::vector<int> slot(size_t(p->Ks), -1);            // location -> (half index) * 2 + place in the half
+  std::vector<int> offs;
+  for (int kt = 0; kt < p->Kt; ++kt)
+    for (int kh = 0; kh < p->Kh; ++kh)
+      for (const Half& hf : halves) {
+        const int base = (kt * p->Kh + kh) * Kw;
+        const bool a = used[size_t(base + hf.tap0)], b = hf.tap1 >= 0 && used[size_t(base + hf.tap1)];
+        if (!a && !b) continue;
+        if (a) slot[size_t(base + hf.tap0)] = int(offs.size()) * 2;
+        if (b) slot[size_t(base + hf.tap1)] = int(offs.size()) * 2 + 1;
+        offs.push_back(((kt * L.img_h + kh) * L.img_w + hf.slot) * 16);
+      }
+  if (offs.size() % 2) offs.push_back(offs.back());    // the unused half of the last MMA reads the other half's window
+  L.n_pairs = int(offs.size()) / 2;
+  L.pair_off.assign(offs.begin(), offs.end());
+  L.wimg.assign(size_t(L.n_pairs) * 2 * L.n_pad * 8, 0);
+  const uint16_t* tiles = reinterpret_cast<const uint16_t*>(p->tiles.data());
+  for (int pr = 0; pr < p->P; ++pr)
+    for (int q = 0; q < p->Q; ++q)
+      for (int32_t e = p->group_ptr[size_t(pr) * p->Q + q]; e < p->group_ptr[size_t(pr) * p->Q + q + 1]; ++e) {
+        const int at = slot[p->pos_idx[size_t(e)]];
+        for (int i = 0; i < p->g_m && pr * p->g_m + i < p->M; ++i)
+          for (int j = 0; j < p->g_n && q * p->g_n + j < p->N; ++j) {
+            const int m = pr * p->g_m + i, c = q * p->g_n + j;
+            L.wimg[((size_t(at / 2) * (L.n_pad / 8) + m / 8) * 8 + m % 8) * 8 + (at % 2) * 4 + c] =
+                tiles[(size_t(e) * p->g_m + i) * p->g_n + j];
+          }
+      }
+  return true;
 }
 
 static uint64_t next_handle_id() {

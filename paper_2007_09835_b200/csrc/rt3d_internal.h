@@ -54,7 +54,13 @@ struct UmmaLayout {
 // sw-th column), so that consecutive outputs are consecutive voxels of an image and every kernel
 // location is a shifted window of one image.  K is walked in pairs of kernel locations (8 padded
 // channels each), one K=16 MMA per pair.
+//
+// Packed form (C_in <= 4, sw = 2): an image entry of 16 bytes holds four channels of TWO input columns, the two that one
+// pair of kernel columns reads, so that a K=16 MMA covers four kernel locations instead of two.  All input rows are staged
+// (an output row is sh image rows down), the producer composes the entries from 8-byte copies listed in `ops`.
 struct SmallCLayout {
+  bool packed = false;
+  std::vector<uint32_t> ops;         // packed: destination / 8 in the image | column << 16 | row << 22 | frame << 28
   int sh = 1, sw = 1;
   int n_pad = 0;                     // output channels rounded up to 16 (<= 256)
   int n_pairs = 0;
@@ -130,8 +136,8 @@ struct DeviceBlob {
   std::map<int, Umma> umma;          // keyed like the handle's layouts
   struct Sub { void* steps = nullptr; int32_t* step_ptr = nullptr; void* blocks = nullptr; bool ready = false; };
   std::map<int, Sub> sub;            // sub-tile kernel, keyed by n_tile
-  struct SmallC { void* wimg = nullptr; int32_t* pairs = nullptr; };
-  std::map<int, SmallC> smallc;      // small-C_in kernel: weight image and pair offsets, keyed by sh*16+sw
+  struct SmallC { void* base = nullptr; unsigned short* wimg = nullptr; int32_t* pairs = nullptr; uint32_t* ops = nullptr; };
+  std::map<int, SmallC> smallc;      // small-C_in kernel: weight image, window offsets and copies, keyed like the layouts
   struct F32 { void* base = nullptr; int32_t* entry_ptr = nullptr; int32_t* tile_ptr = nullptr; int32_t* counts = nullptr; uint32_t* entries = nullptr; float* tiles = nullptr; };
   F32 f32;                           // register-blocked fp32 kernel
   float* splitk = nullptr; size_t splitk_bytes = 0;            // split-K partial tiles (grown on demand)
@@ -160,7 +166,7 @@ struct rt3d_packed {
   std::mutex mu;                     // guards the lazily built members below
   std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by n_tile (+ 4096: the t-grouped order)
   std::map<int, rt3d::SubLayout> sub_layouts;     // keyed by n_tile
-  std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw, built on first use
+  std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw (+ 1024: packed), built on first use
   std::unique_ptr<rt3d::F32Layout> f32_layout;        // built on first use
   std::vector<rt3d::DeviceBlob*> blobs;
   // The last few calls made with this handle, ready to launch again (api.cu); the oldest one gives way.
@@ -182,7 +188,8 @@ bool umma_layout_possible(const rt3d_packed* p);
 const SubLayout* get_sub_layout(rt3d_packed* p, int n_tile);
 
 // Small-C_in layout (nullptr if the handle does not qualify: needs bf16, N <= 8, M <= 256).
-const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw);
+// `packed`: the form with two columns an entry (nullptr unless N <= 4, sw = 2 and the image fits its offsets).
+const SmallCLayout* get_smallc_layout(rt3d_packed* p, int sh, int sw, bool packed = false);
 
 // Layout of the register-blocked fp32 kernel (nullptr unless fp32 with group sizes that are multiples of four).
 bool f32_layout_possible(const rt3d_packed* p);

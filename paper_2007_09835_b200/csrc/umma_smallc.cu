@@ -13,7 +13,14 @@
 // bound by writing its output.  Kernel locations that no group keeps are not in the pair list.
 // The bias is one more MMA (a ones column times the bias as two bf16 terms): the kernel is bound by the
 // instruction count of its epilogue warps, and that removes a third of it.
-// With a spatial stride the input is staged as one image per stride phase (strided TMA boxes), so
+// Up to four channels and a column stride of 2 (the RGB first layers): the packed form (SmallCLayout) puts two input
+// columns into an entry and so four kernel locations into an MMA, 14 instead of 25 for 1x7x7.  An MMA reads 6 KB of shared
+// memory whatever its K slots hold, and the strided TMA boxes fetch one 16-byte piece at a time.  Two producer warps compose
+// the entries with 8-byte asynchronous copies, which also zero what lies outside the tensor or the channels.
+// 1x7x7 stride 2, 3 -> 45, 16 x 8 x 112^2: 41.4 -> 37.8 us; 3 -> 64, 16 x 16 x 224^2 (the separable network's): 112 -> 97.5.
+// With unit column stride a row is one contiguous box that TMA brings cheaply, and composing it costs more than the MMAs
+// saved: 3x3x3, 3 -> 64, 16 x 16 x 112^2 took 158 us instead of 130, so that stays with the boxes.
+// Otherwise, with a spatial stride, the input is staged as one image per stride phase (strided TMA boxes), so
 // that consecutive outputs are again consecutive voxels and every location a window of one image.
 //
 // Roles as in the main kernel: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..5
@@ -27,8 +34,10 @@ namespace {
 
 constexpr int kSmallCStages = 3;
 
-template <int kDummy>
-__global__ void __launch_bounds__(kThreadsUmma, 3)
+constexpr int kThreadsPacked = kThreadsUmma + 32;   // warp 6: second producer
+
+template <bool kPacked>
+__global__ void __launch_bounds__(kPacked ? kThreadsPacked : kThreadsUmma, 3)
 conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
                           const SmallCArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -50,18 +59,19 @@ conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid
   Barriers* bars = reinterpret_cast<Barriers*>(reinterpret_cast<unsigned char*>(pair_smem) +
                                                ((size_t(a.n_pairs) * 8 + 15) & ~size_t(15)));
   float* bias_s = align16_f32(bars + 1);
+  uint32_t* ops_s = reinterpret_cast<uint32_t*>(bias_s + a.n_pad);
   int32_t* err = a.sched + 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_per_frame = a.tiles_h * a.tiles_w;
   const int n_items = a.g.n * a.g.To * tiles_per_frame;
 
   if (threadIdx.x == 32) {                     // descriptor fetches overlap the rest of the set-up
-    tma_prefetch_map(&xmap);
+    if (!kPacked) tma_prefetch_map(&xmap);
     tma_prefetch_map(&ymap);
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < kSmallCStages; ++s) {
-      mbar_init(smem_u32(&bars->full[s]), 1);
+      mbar_init(smem_u32(&bars->full[s]), kPacked ? 64 : 1);
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -111,11 +121,58 @@ conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid
       bb[i] = __float2bfloat16_rn(val);
     }
   }
+  if (kPacked) {
+    for (int i = threadIdx.x; i < a.n_ops; i += blockDim.x) ops_s[i] = __ldg(a.ops + i);
+    // halves of entries that no copy writes
+    for (uint32_t i = threadIdx.x; i < kSmallCStages * halo_stride / 16; i += blockDim.x)
+      reinterpret_cast<uint4*>(gen + (halo_smem - base))[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
   // generic-proxy writes of the weight image must be visible to the tensor core (async proxy)
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
 
-  if (warp == 0) {
+  if (kPacked && (warp == 0 || warp == 6)) {
+    // Producers: the copies of a tile are dealt to 64 threads.  A tile's copies are waited for when the next tile's are
+    // issued, made visible to the tensor core and handed over.
+    if (a.n_pairs > 0) {
+      const int me = (warp == 6 ? 32 : 0) + lane, bytes = a.g.c * 2;
+      const char* x = static_cast<const char*>(a.x);
+      int stage = 0, full_stage = 0, in_flight = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      Walk4 k;
+      walk4_init(k, blockIdx.x, gridDim.x, a.tiles_w, a.tiles_h, a.g.To);
+      auto hand_over = [&]() {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(smem_u32(&bars->full[full_stage]));
+        if (++full_stage == kSmallCStages) full_stage = 0;
+        --in_flight;
+      };
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x, walk4_next(k)) {
+        if (!mbar_wait(smem_u32(&bars->empty[stage]), phase ^ 1u, bars, err, 11)) { ok = false; break; }
+        const int w0 = k.i0 * kSmallCTileW * a.g.sw - a.g.pw, h0 = k.i1 * kSmallCTileH * a.g.sh - a.g.ph, t0 = k.i2 * a.g.st - a.g.pt;
+        const uint32_t dst = halo_smem + stage * halo_stride;
+        const long long clip = (long long)k.i3 * a.g.t;
+#pragma unroll 4
+        for (int i = me; i < a.n_ops; i += 64) {
+          const uint32_t op = ops_s[i];
+          const int wi = w0 + int((op >> 16) & 63u), hi = h0 + int((op >> 22) & 63u), ti = t0 + int(op >> 28);
+          const bool in = unsigned(wi) < unsigned(a.g.w) && unsigned(hi) < unsigned(a.g.h) && unsigned(ti) < unsigned(a.g.t);
+          const char* src = in ? x + (((clip + ti) * a.g.h + hi) * a.g.w + wi) * 16 : x;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst + (op & 0xffffu) * 8u), "l"(src), "r"(in ? bytes : 0)
+                       : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (++stage == kSmallCStages) { stage = 0; phase ^= 1u; }
+        if (++in_flight == 2) {
+          asm volatile("cp.async.wait_group 1;" ::: "memory");
+          hand_over();
+        }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      while (ok && in_flight > 0) hand_over();
+    }
+  } else if (warp == 0) {
     if (lane == 0 && a.n_pairs > 0) {
       int stage = 0;
       uint32_t phase = 0;
@@ -142,7 +199,7 @@ conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = instr_desc_bf16(a.n_pad);
-      const uint32_t sbo_a = uint32_t(a.img_w) * 16u;             // next 8-voxel group = next image row
+      const uint32_t sbo_a = uint32_t(a.img_w) * 16u * uint32_t(kPacked ? a.g.sh : 1);   // next 8-voxel group = next output row
       const uint32_t lbo_b = uint32_t(a.n_pad) * 16u;             // second K half of the weight image
       int stage = 0;
       uint32_t phase = 0, j = 0;
@@ -220,20 +277,21 @@ conv3d_umma_smallc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid
 
 }  // namespace
 
-size_t smallc_smem_bytes(int n_pairs, int n_pad, int stage_bytes) {
+size_t smallc_smem_bytes(int n_pairs, int n_pad, int stage_bytes, int n_ops) {
   const size_t w = (size_t(n_pairs + 1) * 2 * n_pad * 16 + 128 + 127) & ~size_t(127);   // + bias operand and ones tile
   const size_t halo = (size_t(stage_bytes) + 127) & ~size_t(127);
-  return 1024 + 4 * kStoreWarpBytes + w + kSmallCStages * halo + ((size_t(n_pairs) * 8 + 15) & ~size_t(15)) + sizeof(Barriers) + 16 + size_t(n_pad) * 4;
+  return 1024 + 4 * kStoreWarpBytes + w + kSmallCStages * halo + ((size_t(n_pairs) * 8 + 15) & ~size_t(15)) + sizeof(Barriers) + 16 + size_t(n_pad) * 4 + size_t(n_ops) * 4;
 }
 
-cudaError_t launch_conv_umma_smallc(const SmallCArgs& a_in, const void* xmap, const void* ymap, int sm_count,
-                                    cudaStream_t stream) {
+template <bool kPacked>
+static cudaError_t launch_smallc_t(const SmallCArgs& a_in, const void* xmap, const void* ymap, int sm_count, cudaStream_t stream) {
+  constexpr int kThreads = kPacked ? kThreadsPacked : kThreadsUmma;
   SmallCArgs a = a_in;
   int cols = 32;
   while (cols < 2 * a.n_pad) cols *= 2;
   if (cols > 512) return cudaErrorInvalidValue;
   a.tmem_cols = cols;
-  const size_t smem = smallc_smem_bytes(a.n_pairs, a.n_pad, a.n_phases * a.phase_stride);
+  const size_t smem = smallc_smem_bytes(a.n_pairs, a.n_pad, a.n_phases * a.phase_stride, a.n_ops);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const long long n_items = (long long)a.g.n * a.g.To * a.tiles_h * a.tiles_w;
   if (n_items <= 0) return cudaSuccess;
@@ -245,10 +303,10 @@ cudaError_t launch_conv_umma_smallc(const SmallCArgs& a_in, const void* xmap, co
   const int dev_idx = current_device_index();
   if (dev_idx < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev_idx]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_smallc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_smallc_kernel<kPacked>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     // ask for the largest shared-memory carve-out: with the default one fewer CTAs fit an SM than the sizes allow
-    e = cudaFuncSetAttribute(conv3d_umma_smallc_kernel<0>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    e = cudaFuncSetAttribute(conv3d_umma_smallc_kernel<kPacked>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     attr_done[dev_idx] = true;
   }
@@ -261,9 +319,9 @@ cudaError_t launch_conv_umma_smallc(const SmallCArgs& a_in, const void* xmap, co
   static int regs_per_thread = 0;
   if (regs_per_thread == 0) {
     cudaFuncAttributes fa;
-    regs_per_thread = cudaFuncGetAttributes(&fa, conv3d_umma_smallc_kernel<0>) == cudaSuccess ? fa.numRegs : 128;
+    regs_per_thread = cudaFuncGetAttributes(&fa, conv3d_umma_smallc_kernel<kPacked>) == cudaSuccess ? fa.numRegs : 128;
   }
-  int per_sm = 65536 / (((regs_per_thread + 7) & ~7) * kThreadsUmma);
+  int per_sm = 65536 / (((regs_per_thread + 7) & ~7) * kThreads);
   const int by_smem = int((228 * 1024) / (smem + 1024));
   if (per_sm > by_smem) per_sm = by_smem;
   if (per_sm > 512 / cols) per_sm = 512 / cols;
@@ -271,8 +329,12 @@ cudaError_t launch_conv_umma_smallc(const SmallCArgs& a_in, const void* xmap, co
   if (per_sm < 1) per_sm = 1;
   const long long want = (long long)sm_count * per_sm;
   const int grid = int(n_items < want ? n_items : want);
-  LaunchSetup ls(dim3(grid), dim3(kThreadsUmma), smem, stream);
-  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_smallc_kernel<0>, xm, ym, a);
+  LaunchSetup ls(dim3(grid), dim3(kThreads), smem, stream);
+  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_smallc_kernel<kPacked>, xm, ym, a);
+}
+
+cudaError_t launch_conv_umma_smallc(const SmallCArgs& a, const void* xmap, const void* ymap, int sm_count, cudaStream_t stream) {
+  return a.ops ? launch_smallc_t<true>(a, xmap, ymap, sm_count, stream) : launch_smallc_t<false>(a, xmap, ymap, sm_count, stream);
 }
 
 }  // namespace rt3d
