@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "kept_blocks.h"
 #include "rt3d_internal.h"
 
 using namespace rt3d;
@@ -31,6 +32,26 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
 }
 template <typename T>
 cudaError_t dev_malloc(T** p, size_t bytes) { return dev_malloc(reinterpret_cast<void**>(p), bytes); }
+
+// Device memory of uploaded layouts.  A kept block may still be read by kernels that its last owner launched (cudaFree
+// would have waited for them), so taking one waits for the device.
+KeptBlocks& weight_blocks() {
+  static KeptBlocks* kept = new KeptBlocks([](void* p) { cudaFree(p); });
+  return *kept;
+}
+cudaError_t weight_malloc(void** p, size_t bytes) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if ((*p = weight_blocks().take(bytes, dev)) != nullptr) {
+    if ((e = cudaDeviceSynchronize()) == cudaSuccess) return e;
+    cudaFree(*p);
+    return e;
+  }
+  if ((e = dev_malloc(p, bytes)) == cudaSuccess) weight_blocks().note(*p, bytes, dev);
+  return e;
+}
+void weight_free(void* p) { weight_blocks().give(p); }
 
 // Planning mode of the calling thread (rt3d_plan_begin / rt3d_plan_end): compute calls do everything they would do
 // before their launch (choose the kernel, build and upload weight layouts, size the workspaces) and return.
@@ -276,13 +297,19 @@ class Upload {
     items_[n_++] = Item{reinterpret_cast<void**>(dst), v.data(), bytes, bytes_};
     bytes_ += (bytes + 16 + 255) & ~size_t(255);       // 256-byte aligned parts, readable 16 bytes on
   }
+  // A part that is not copied to.
+  template <typename T>
+  void reserve(T** dst, size_t bytes) {
+    items_[n_++] = Item{reinterpret_cast<void**>(dst), nullptr, 0, bytes_};
+    bytes_ += (bytes + 16 + 255) & ~size_t(255);
+  }
   // Allocates, copies and sets the pointers; *base owns the memory.  Nothing is kept on failure.
   rt3d_status run(void** base) {
-    if (dev_malloc(base, bytes_) != cudaSuccess) { *base = nullptr; return RT3D_ERR_ALLOC; }
+    if (weight_malloc(base, bytes_) != cudaSuccess) { *base = nullptr; return RT3D_ERR_ALLOC; }
     for (int i = 0; i < n_; ++i) {
       char* d = static_cast<char*>(*base) + items_[i].off;
       if (items_[i].bytes && cudaMemcpy(d, items_[i].src, items_[i].bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
-        cudaFree(*base);
+        weight_free(*base);
         *base = nullptr;
         return RT3D_ERR_CUDA;
       }
@@ -293,18 +320,22 @@ class Upload {
 
  private:
   struct Item { void** dst; const void* src; size_t bytes, off; };
-  Item items_[8];
+  Item items_[12];
   int n_ = 0;
   size_t bytes_ = 0;
 };
+
+void add_canonical(rt3d_packed* h, DeviceBlob* b, Upload& up) {
+  up.add(&b->group_ptr, h->group_ptr);
+  up.add(&b->pos_idx, h->pos_idx);
+  up.add(&b->tiles, h->tiles);
+}
 
 // Device copies of the canonical arrays: for the index-driven CUDA-core kernel, and to build the tensor-core layouts from.
 rt3d_status get_canonical_locked(rt3d_packed* h, DeviceBlob* b) {
   if (b->canonical) return RT3D_OK;
   Upload up;
-  up.add(&b->group_ptr, h->group_ptr);
-  up.add(&b->pos_idx, h->pos_idx);
-  up.add(&b->tiles, h->tiles);
+  add_canonical(h, b, up);
   return up.run(&b->canonical);
 }
 rt3d_status get_canonical(rt3d_packed* h, DeviceBlob* b) {
@@ -319,26 +350,24 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
     const size_t wbytes = L->steps.size() * size_t(L->n_tile) * kChunk * 2;
     // The canonical arrays go to the device once, a quarter to a third of the size of the zero-filled tiles, and a kernel
     // fills the tiles in there: 512 x 512 x 27 at 0.28 kept, 14 MB of tiles: 9 -> 1.6 ms with the allocation.
-    const rt3d_status cs = get_canonical_locked(h, blob);
-    if (cs != RT3D_OK) return cs;
-    if (!u.wtiles && dev_malloc(&u.wtiles, wbytes + 1024) != cudaSuccess) { u.wtiles = nullptr; return RT3D_ERR_ALLOC; }
+    // The first layout shares the allocation of the canonical arrays: a cudaMalloc and its cudaFree are 0.2 to 0.4 ms each.
+    const bool shared = !blob->canonical;
+    void** const base = shared ? &blob->canonical : &u.base;
     int32_t* slots = nullptr;
-    if (!u.base) {
-      Upload up;
-      up.add(&u.step_ptr, L->step_ptr);
-      up.add(&u.steps, L->steps);
-      up.add(&slots, L->slots);
-      if (L->t_groups) { up.add(&u.grp_ptr, L->grp_ptr); up.add(&u.grp_first, L->grp_first); }
-      const rt3d_status s = up.run(&u.base);
-      if (s != RT3D_OK) return s;
-      if (wbytes && (launch_fill_umma_tiles(blob->group_ptr, blob->pos_idx, blob->tiles, slots, h->M, h->N, h->Ks, h->g_m, h->g_n,
-                                            h->Q, h->P * h->Q, h->nnz, L->n_tile, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
-                     cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)) {
-        cudaFree(u.base);
-        u.base = nullptr;
-        return RT3D_ERR_CUDA;
-      }
-    }
+    Upload up;
+    up.reserve(&u.wtiles, wbytes + 1024);
+    if (shared) add_canonical(h, blob, up);
+    up.add(&u.step_ptr, L->step_ptr);
+    up.add(&u.steps, L->steps);
+    up.add(&slots, L->slots);
+    if (L->t_groups) { up.add(&u.grp_ptr, L->grp_ptr); up.add(&u.grp_first, L->grp_first); }
+    const rt3d_status s = up.run(base);
+    if (s != RT3D_OK) return s;
+    const auto fail = [&] { weight_free(*base); *base = nullptr; return RT3D_ERR_CUDA; };
+    if (wbytes && (launch_fill_umma_tiles(blob->group_ptr, blob->pos_idx, blob->tiles, slots, h->M, h->N, h->Ks, h->g_m, h->g_n,
+                                          h->Q, h->P * h->Q, h->nnz, L->n_tile, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
+                   cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess))
+      return fail();
     // 2-D map over the weight tiles: rows of 64 bf16 (128 bytes), one box = one [n_tile][64] tile
     const cuuint64_t rows = L->steps.empty() ? cuuint64_t(L->n_tile) : cuuint64_t(L->steps.size()) * L->n_tile;
     cuuint64_t dims[2] = {64, rows};
@@ -348,13 +377,13 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
     CUresult r = g_encode(reinterpret_cast<CUtensorMap*>(u.wmap), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, u.wtiles, dims,
                           strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return RT3D_ERR_CUDA;
+    if (r != CUDA_SUCCESS) return fail();
     if (L->n_tile % 16 == 0) {
       cuuint32_t box_half[2] = {64, cuuint32_t(L->n_tile / 2)};
       r = g_encode(reinterpret_cast<CUtensorMap*>(u.wmap_half), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, u.wtiles, dims,
                    strides, box_half, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (r != CUDA_SUCCESS) return RT3D_ERR_CUDA;
+      if (r != CUDA_SUCCESS) return fail();
     }
     u.ready = true;
   }
@@ -1286,15 +1315,13 @@ void rt3d_packed_free(rt3d_packed* p) {
   }
   for (DeviceBlob* b : p->blobs) {
     if (have_dev) cudaSetDevice(b->device);
-    cudaFree(b->canonical);
-    for (auto& kv : b->umma) {
-      cudaFree(kv.second.wtiles); cudaFree(kv.second.base);
-    }
+    weight_free(b->canonical);
+    for (auto& kv : b->umma) weight_free(kv.second.base);
     cudaFree(b->stage_x); cudaFree(b->stage_y); cudaFree(b->stage_bias);
     for (void* hs : b->host_streams) if (hs) cudaStreamDestroy(static_cast<cudaStream_t>(hs));
     for (void* he : b->host_events) if (he) cudaEventDestroy(static_cast<cudaEvent_t>(he));
-    for (auto& kv : b->smallc) cudaFree(kv.second.base);
-    cudaFree(b->f32.base);
+    for (auto& kv : b->smallc) weight_free(kv.second.base);
+    weight_free(b->f32.base);
     for (auto& kv : b->sub) { cudaFree(kv.second.steps); cudaFree(kv.second.step_ptr); cudaFree(kv.second.blocks); }
     cudaFree(b->splitk); cudaFree(b->splitk_cnt);
     delete b;

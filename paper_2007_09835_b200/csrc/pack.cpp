@@ -9,6 +9,7 @@
 #include <thread>
 #include <utility>
 
+#include "kept_blocks.h"
 #include "rt3d_internal.h"
 
 namespace rt3d {
@@ -16,9 +17,8 @@ namespace rt3d {
 uint16_t f32_to_bf16_bits(float f) {
   uint32_t u;
   std::memcpy(&u, &f, 4);
-  if ((u & 0x7F800000u) == 0x7F800000u && (u & 0x007FFFFFu)) return uint16_t((u >> 16) | 0x40u);
-  u += 0x7FFFu + ((u >> 16) & 1u);   // ties to even
-  return uint16_t(u >> 16);
+  const uint32_t rounded = u + 0x7FFFu + ((u >> 16) & 1u);          // ties to even
+  return uint16_t(((u & 0x7FFFFFFFu) > 0x7F800000u ? u | 0x400000u : rounded) >> 16);    // a NaN stays one
 }
 
 float bf16_bits_to_f32(uint16_t b) {
@@ -37,32 +37,65 @@ bool umma_layout_possible(const rt3d_packed* p) {
   return p->dtype == RT3D_BF16 && p->Kt <= 63 && p->Kh <= 63 && p->Kw <= 63 && ceil_div(p->N, kChunk) <= 4095;
 }
 
+// Never destroyed: handles may be freed while the process exits.
+static KeptBlocks& host_blocks() {
+  static KeptBlocks* kept = new KeptBlocks([](void* p) { delete[] static_cast<unsigned char*>(p); });
+  return *kept;
+}
+unsigned char* host_block(size_t bytes) {
+  if (void* p = host_blocks().take(bytes, -1)) return static_cast<unsigned char*>(p);
+  unsigned char* p = new unsigned char[bytes];
+  host_blocks().note(p, bytes, -1);
+  return p;
+}
+void host_block_free(unsigned char* p) { host_blocks().give(p); }
+
 static float tile_value(const rt3d_packed* p, int64_t e, int i, int j) {
   const int64_t o = (e * p->g_m + i) * p->g_n + j;
   if (p->dtype == RT3D_BF16) return bf16_bits_to_f32(reinterpret_cast<const uint16_t*>(p->tiles.data())[o]);
   return reinterpret_cast<const float*>(p->tiles.data())[o];
 }
 
-// Runs fn(i) for i in [0, n), on up to eight threads if each gets at least `grain` units of work in all.
-template <typename F>
-static void parallel_for(int n, int64_t work, int64_t grain, const F& fn) {
-  int threads = int(std::min<int64_t>(std::min<int64_t>(work / grain, n), std::min(8u, std::thread::hardware_concurrency())));
+// Runs first(i) for i in [0, n), then between() once, then, unless that said no, second(i) for i in [0, n): on up to eight
+// threads if each gets at least `grain` units of work in all.  The threads are started once for both passes (starting and
+// joining seven costs 0.25 ms).
+template <typename F, typename G, typename H>
+static void two_passes(int n, int64_t work, int64_t grain, const F& first, const G& between, const H& second) {
+  const int threads = int(std::min<int64_t>(std::min<int64_t>(work / grain, n), std::min(8u, std::thread::hardware_concurrency())));
   if (threads <= 1) {
-    for (int i = 0; i < n; ++i) fn(i);
+    for (int i = 0; i < n; ++i) first(i);
+    if (!between()) return;
+    for (int i = 0; i < n; ++i) second(i);
     return;
   }
-  std::atomic<int> next{0};
+  std::atomic<int> next[2] = {{0}, {0}}, done{0}, go{0};
   const int step = std::max(1, n / (threads * 8));       // pieces small enough to even out, large enough to be few
-  auto worker = [&] {
-    for (int i0 = next.fetch_add(step); i0 < n; i0 = next.fetch_add(step))
+  auto pass = [&](std::atomic<int>& at, const auto& fn) {
+    for (int i0 = at.fetch_add(step); i0 < n; i0 = at.fetch_add(step))
       for (int i = i0; i < std::min(n, i0 + step); ++i) fn(i);
   };
   std::vector<std::thread> pool;
+  pool.reserve(size_t(threads));
   try {
-    for (int t = 1; t < threads; ++t) pool.emplace_back(worker);
+    for (int t = 1; t < threads; ++t)
+      pool.emplace_back([&] {
+        pass(next[0], first);
+        done.fetch_add(1);
+        while (go.load() == 0) std::this_thread::yield();
+        if (go.load() == 1) pass(next[1], second);
+      });
   } catch (const std::system_error&) {                   // no more threads to be had: the others do the work
   }
-  worker();
+  pass(next[0], first);
+  while (done.load() < int(pool.size())) std::this_thread::yield();
+  try {
+    go = between() ? 1 : 2;
+  } catch (...) {
+    go = 2;
+    for (std::thread& t : pool) t.join();
+    throw;
+  }
+  if (go.load() == 1) pass(next[1], second);
   for (std::thread& t : pool) t.join();
 }
 
@@ -97,10 +130,12 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
     std::fill(slot.begin(), slot.end(), -1);
     for (int pr = p_lo; pr < p_hi; ++pr)
       for (int q = 0; q < p->Q; ++q) {
-        const int c_lo = q * p->g_n, c_hi = std::min(p->N, c_lo + p->g_n);
-        for (int32_t e = p->group_ptr[pr * p->Q + q]; e < p->group_ptr[pr * p->Q + q + 1]; ++e)
-          for (int ch = c_lo / kChunk; ch <= (c_hi - 1) / kChunk; ++ch)
-            slot[size_t(p->pos_idx[e]) * L.n_chunks + ch] = 0;
+        const int c_lo = q * p->g_n, c_hi = std::min(p->N, c_lo + p->g_n), n_chunks = L.n_chunks;
+        const uint16_t* const end = p->pos_idx.data() + p->group_ptr[size_t(pr) * p->Q + q + 1];
+        for (int ch = c_lo / kChunk; ch <= (c_hi - 1) / kChunk; ++ch) {
+          int32_t* const mark = slot.data() + ch;
+          for (const uint16_t* e = p->pos_idx.data() + p->group_ptr[size_t(pr) * p->Q + q]; e < end; ++e) mark[size_t(*e) * n_chunks] = 0;
+        }
       }
     const int32_t base = L.step_ptr[b];
     int32_t cnt = 0;
@@ -334,7 +369,7 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
         for (int32_t e = p->group_ptr[grp]; e < p->group_ptr[grp + 1]; ++e) at[p->pos_idx[e]] = e;
       }
   };
-  parallel_for(L.n_stages, work, grain, [&](int st) {
+  const auto count_entries = [&](int st) {
     std::vector<int32_t> kept;
     for (int s = 0; s < L.n_sets; ++s) {
       find_kept(st, s, kept);
@@ -348,11 +383,14 @@ const F32Layout* get_f32_layout(rt3d_packed* p) {
       L.entry_ptr[at + 1] = count[0] + count[1] + count[2];
       L.tile_ptr[at + 1] = 2 * count[0] + count[1] + count[2];
     }
-  });
-  for (size_t i = 0; i < n_lists; ++i) { L.entry_ptr[i + 1] += L.entry_ptr[i]; L.tile_ptr[i + 1] += L.tile_ptr[i]; }
-  L.entries.resize(size_t(L.entry_ptr[n_lists]));
-  L.tiles.allocate(size_t(L.tile_ptr[n_lists]) * 64);
-  parallel_for(L.n_stages, work, grain, [&](int st) {
+  };
+  const auto allocate = [&] {
+    for (size_t i = 0; i < n_lists; ++i) { L.entry_ptr[i + 1] += L.entry_ptr[i]; L.tile_ptr[i + 1] += L.tile_ptr[i]; }
+    L.entries.resize(size_t(L.entry_ptr[n_lists]));
+    L.tiles.allocate(size_t(L.tile_ptr[n_lists]) * 64);
+    return true;
+  };
+  two_passes(L.n_stages, work, grain, count_entries, allocate, [&](int st) {
     std::vector<int32_t> kept;
     for (int s = 0; s < L.n_sets; ++s) {
       find_kept(st, s, kept);
@@ -458,6 +496,8 @@ static uint64_t next_handle_id() {
   return next_id.fetch_add(1);
 }
 
+constexpr size_t kGatherGroup = 64;      // weights of a group that pass 2 gathers at once
+
 static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, int Kt, int Kh, int Kw,
                              int g_m, int g_n, int dtype, int is_dense, rt3d_packed** out) {
   if (!w || !out) return RT3D_ERR_INVALID_ARG;
@@ -478,73 +518,89 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
     const size_t esz = dtype == RT3D_BF16 ? 2 : 4;
     const size_t n_groups = size_t(h->P) * h->Q;
     h->group_ptr.resize(n_groups + 1);
-    // Both passes walk the weights and the mask in memory order, the Ks values of one kernel at a time, and are shared
-    // between threads by rows of groups.
+    // Both passes are shared between threads by groups, in memory order.
     const int64_t work = int64_t(M) * N * Ks, grain = int64_t(1) << 18;
-    // pass 1: group-level decisions with the uniformity check of the KGS definition
+    // pass 1: group-level decisions with the uniformity check of the KGS definition.  A kernel's bytes are nearly always
+    // those of the group's first kernel, so they are compared as a block, and value by value (any nonzero value keeps a
+    // weight) only where the blocks differ: 512 x 512 x 27 with 8 threads a millisecond of one thread -> 0.4.
     std::vector<uint8_t> keep(mask ? n_groups * Ks : 0);
     std::atomic<bool> uniform{true}, vanilla{true};
-    parallel_for(h->P, work, grain, [&](int pr) {
-      for (int q = 0; q < h->Q; ++q) {
-        const size_t grp = size_t(pr) * h->Q + q;
-        if (!mask) { h->group_ptr[grp + 1] = Ks; continue; }
-        uint8_t* kp = keep.data() + grp * Ks;
-        uint8_t differs = 0;
-        for (int i = 0; i < g_m && pr * g_m + i < M; ++i)
-          for (int j = 0; j < g_n && q * g_n + j < N; ++j) {
-            const uint8_t* row = mask + (int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks;
-            if (i == 0 && j == 0) {
-              for (int k = 0; k < Ks; ++k) kp[k] = row[k] != 0;
-            } else {
-              for (int k = 0; k < Ks; ++k) differs |= uint8_t(kp[k] ^ uint8_t(row[k] != 0));
-            }
-          }
-        if (differs) uniform = false;
-        int kept_here = 0;
-        for (int k = 0; k < Ks; ++k) kept_here += kp[k];
-        if (kept_here != 0 && kept_here != Ks) vanilla = false;
-        h->group_ptr[grp + 1] = kept_here;
+    const auto decide = [&](int grp) {
+      if (!mask) { h->group_ptr[size_t(grp) + 1] = Ks; return; }
+      const int pr = grp / h->Q, q = grp % h->Q, rows = std::min(g_m, M - pr * g_m), cols = std::min(g_n, N - q * g_n);
+      uint8_t* kp = keep.data() + size_t(grp) * Ks;
+      const uint8_t* first = mask + (int64_t(pr) * g_m * N + int64_t(q) * g_n) * Ks;
+      int kept_here = 0;
+      for (int k = 0; k < Ks; ++k) { kp[k] = first[k] != 0; kept_here += kp[k]; }
+      for (int i = 0; i < rows; ++i)
+        for (int j = 0; j < cols; ++j) {
+          const uint8_t* row = first + (int64_t(i) * N + j) * Ks;
+          if (std::memcmp(row, first, size_t(Ks)) == 0) continue;
+          for (int k = 0; k < Ks; ++k)
+            if (kp[k] != uint8_t(row[k] != 0)) uniform = false;
+        }
+      if (kept_here != 0 && kept_here != Ks && vanilla.load(std::memory_order_relaxed)) vanilla = false;   // written once
+      h->group_ptr[size_t(grp) + 1] = kept_here;
+    };
+    rt3d_status status = RT3D_OK;
+    const auto allocate = [&] {
+      if (!uniform) { status = RT3D_ERR_MASK_NOT_GROUP_UNIFORM; return false; }
+      int64_t nnz = 0;
+      for (size_t grp = 0; grp < n_groups; ++grp) {
+        nnz += h->group_ptr[grp + 1];
+        if (nnz > 0x7FFFFFFF) { status = RT3D_ERR_UNSUPPORTED; return false; }
+        h->group_ptr[grp + 1] = int32_t(nnz);
       }
-    });
-    if (!uniform) { delete h; return RT3D_ERR_MASK_NOT_GROUP_UNIFORM; }
-    int64_t nnz = 0;
-    for (size_t grp = 0; grp < n_groups; ++grp) {
-      nnz += h->group_ptr[grp + 1];
-      if (nnz > 0x7FFFFFFF) { delete h; return RT3D_ERR_UNSUPPORTED; }
-      h->group_ptr[grp + 1] = int32_t(nnz);
-    }
-    h->group_ptr[0] = 0;
-    h->nnz = nnz;
-    h->is_vanilla = vanilla;
-    h->pos_idx.resize(size_t(nnz));
-    h->tiles.allocate(size_t(nnz) * g_m * g_n * esz);
-    // pass 2: emit index and tiles
-    parallel_for(h->P, work, grain, [&](int pr) {
-      const int rows = std::min(g_m, M - pr * g_m);
-      for (int q = 0; q < h->Q; ++q) {
-        const size_t grp = size_t(pr) * h->Q + q;
-        const int32_t e0 = h->group_ptr[grp], n_e = h->group_ptr[grp + 1] - e0;
-        const int cols = std::min(g_n, N - q * g_n);
-        uint16_t* pos = h->pos_idx.data() + e0;
-        int n = 0;
-        for (int k = 0; k < Ks; ++k)
-          if (!mask || keep[grp * Ks + k]) pos[n++] = uint16_t(k);
-        unsigned char* out = h->tiles.data() + size_t(e0) * g_m * g_n * esz;
-        if (rows < g_m || cols < g_n) std::memset(out, 0, size_t(n_e) * g_m * g_n * esz);    // kernels that do not exist
-        for (int i = 0; i < rows; ++i)
-          for (int j = 0; j < cols; ++j) {
-            const float* row = w + (int64_t(pr * g_m + i) * N + (q * g_n + j)) * Ks;
-            const size_t at = size_t(i) * g_n + j, step = size_t(g_m) * g_n;
-            if (dtype == RT3D_BF16) {
-              uint16_t* o = reinterpret_cast<uint16_t*>(out) + at;
-              for (int e = 0; e < n_e; ++e) o[e * step] = f32_to_bf16_bits(row[pos[e]]);
-            } else {
-              float* o = reinterpret_cast<float*>(out) + at;
-              for (int e = 0; e < n_e; ++e) o[e * step] = row[pos[e]];
-            }
+      h->group_ptr[0] = 0;
+      h->nnz = nnz;
+      h->is_vanilla = vanilla;
+      h->pos_idx.resize(size_t(nnz));
+      h->tiles.allocate(size_t(nnz) * g_m * g_n * esz);
+      return true;
+    };
+    // pass 2: emit index and tiles.  A small whole group is gathered tile by tile, which writes in order and converts in
+    // vectors; otherwise kernel by kernel, which reads in order.
+    two_passes(int(n_groups), work, grain, decide, allocate, [&](int grp) {
+      const int pr = grp / h->Q, q = grp % h->Q, rows = std::min(g_m, M - pr * g_m), cols = std::min(g_n, N - q * g_n);
+      const int32_t e0 = h->group_ptr[size_t(grp)], n_e = h->group_ptr[size_t(grp) + 1] - e0;
+      const size_t step = size_t(g_m) * g_n;
+      uint16_t* pos = h->pos_idx.data() + e0;
+      int n = 0;
+      for (int k = 0; k < Ks; ++k)
+        if (!mask || keep[size_t(grp) * Ks + k]) pos[n++] = uint16_t(k);
+      unsigned char* out = h->tiles.data() + size_t(e0) * step * esz;
+      const float* base = w + (int64_t(pr) * g_m * N + int64_t(q) * g_n) * Ks;
+      if (rows == g_m && cols == g_n && step <= kGatherGroup) {
+        float v[kGatherGroup];
+        for (int e = 0; e < n_e; ++e, out += step * esz) {
+          const float* at = base + pos[e];
+          for (int i = 0; i < g_m; ++i)
+            for (int j = 0; j < g_n; ++j) v[i * g_n + j] = at[(int64_t(i) * N + j) * Ks];
+          if (dtype == RT3D_BF16) {
+            uint16_t b[kGatherGroup];
+            for (size_t i = 0; i < step; ++i) b[i] = f32_to_bf16_bits(v[i]);
+            std::memcpy(out, b, step * 2);
+          } else {
+            std::memcpy(out, v, step * 4);
           }
+        }
+        return;
       }
+      if (rows < g_m || cols < g_n) std::memset(out, 0, size_t(n_e) * step * esz);           // kernels that do not exist
+      for (int i = 0; i < rows; ++i)
+        for (int j = 0; j < cols; ++j) {
+          const float* row = base + (int64_t(i) * N + j) * Ks;
+          const size_t at = size_t(i) * g_n + j;
+          if (dtype == RT3D_BF16) {
+            uint16_t* o = reinterpret_cast<uint16_t*>(out) + at;
+            for (int e = 0; e < n_e; ++e) o[e * step] = f32_to_bf16_bits(row[pos[e]]);
+          } else {
+            float* o = reinterpret_cast<float*>(out) + at;
+            for (int e = 0; e < n_e; ++e) o[e * step] = row[pos[e]];
+          }
+        }
     });
+    if (status != RT3D_OK) { delete h; return status; }
   } catch (const std::bad_alloc&) {
     delete h;
     return RT3D_ERR_ALLOC;

@@ -86,17 +86,22 @@ struct SubLayout {
   int max_steps = 0;                 // longest bundle list
 };
 
+// Host memory of the packed weights: a block kept from a freed handle, or a new one (pack.cpp).
+unsigned char* host_block(size_t bytes);
+void host_block_free(unsigned char* p);
+
 // Bytes that are written once, without the zeros a vector would fill them with first.
 class RawBytes {
  public:
-  void allocate(size_t n) { data_.reset(new unsigned char[n]); size_ = n; }
+  void allocate(size_t n) { data_.reset(host_block(n)); size_ = n; }
   unsigned char* data() { return data_.get(); }
   const unsigned char* data() const { return data_.get(); }
   size_t size() const { return size_; }
   unsigned char operator[](size_t i) const { return data_[i]; }
 
  private:
-  std::unique_ptr<unsigned char[]> data_;
+  struct Free { void operator()(unsigned char* p) const { host_block_free(p); } };
+  std::unique_ptr<unsigned char[], Free> data_;
   size_t size_ = 0;
 };
 

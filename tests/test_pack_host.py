@@ -124,3 +124,30 @@ def test_concatenated_handles_hold_the_filters_one_after_the_other(dtype):
         with pytest.raises(rt3d.Rt3dError) as e:
             rt3d.rt3d_pack_concat(bad)
         assert e.value.status == rt3d.ERR_SHAPE
+
+
+def test_blocks_of_freed_handles_are_reused_safely():
+    """Layers of kept-block size, packed and freed by several threads at once, equal the ones packed first."""
+    import threading
+    sizes = [(256, 256, (3, 3, 3)), (250, 255, (3, 3, 3)), (512, 512, (1, 1, 3))]
+    layers = []
+    for i, (m, n, k) in enumerate(sizes):
+        spec = synth.ConvSpec("l", n, m, k, (1, 1, 1), (0, 0, 0))
+        layers.append(synth.make_layer(spec, 5, i, 4, 4, "bernoulli", 0.4))
+    def pack(i):
+        v = rt3d.rt3d_pack_kgs(layers[i]["w"], layers[i]["mask"], 4, 4, rt3d.RT3D_BF16).view()
+        return v["group_ptr"], v["pos_idx"], v["tiles"]
+    first = [pack(i) for i in range(len(sizes))]
+    wrong = []
+
+    def work(at):
+        for r in range(6):
+            i = (at + r) % len(sizes)
+            if not all(np.array_equal(a, b) for a, b in zip(pack(i), first[i])):
+                wrong.append(i)
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong

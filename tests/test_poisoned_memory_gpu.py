@@ -161,3 +161,25 @@ def test_forward_passes_with_poison_before_every_launch(which, batch, monkeypatc
         assert torch.equal(y, y0)
     assert state["launches"] >= 18
     assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+def test_weight_block_of_a_freed_handle_waits_for_its_kernels():
+    """A handle freed right behind its launch on a side stream: the next handle takes the memory only when the kernel is done."""
+    spec = synth.ConvSpec("kept", 256, 256, (3, 3, 3), (1, 1, 1), (1, 1, 1), True)
+    layers = [synth.make_layer(spec, 91, i, 4, 4, "bernoulli", 0.4) for i in range(2)]
+    xs = synth.make_input(910, (4, 4, 28, 28, 256))
+    xd = nets.to_device(xs)
+
+    def conv(i):
+        lay = nets.ConvLayer(spec, layers[i]["w"], layers[i]["bias"], layers[i]["mask"], 4, 4, torch.bfloat16)
+        y = lay.alloc_out(xd)
+        lay.fused(xd, y)
+        return y
+    ref = [conv(i).clone() for i in range(2)]
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    for r in range(6):
+        with torch.cuda.stream(stream):
+            y = [conv(i) for i in (r % 2, 1 - r % 2)]
+        stream.synchronize()
+        assert torch.equal(y[0], ref[r % 2]) and torch.equal(y[1], ref[1 - r % 2])
