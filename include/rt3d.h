@@ -13,8 +13,8 @@
  *   - Compute calls enqueue work on the given CUDA stream (a cudaStream_t passed as
  *     void*, NULL = default stream) and return without synchronising.  The first compute
  *     call that uses a handle on a device uploads the handle's device blobs (allocation +
- *     copy), and the first call of a shape that splits K grows the handle's scratch buffer;
- *     later calls allocate nothing.  rt3d_packed_prepare does the upload ahead of time.
+ *     copy), and the first call of a shape whose left-over tiles are split along K (tail split) grows the
+ *     handle's scratch buffer; later calls allocate nothing.  rt3d_packed_prepare does the upload ahead of time.
  *     That scratch belongs to the handle: two calls on the SAME handle whose kernels may overlap
  *     on the GPU (different streams) must be serialised by the caller.
  *   - Kernels are launched with programmatic stream serialisation: a kernel's set-up may overlap
@@ -378,7 +378,7 @@ int64_t rt3d_alloc_count(void);
 
 /* Planning mode of the calling thread.  Between rt3d_plan_begin and rt3d_plan_end every compute call of this
  * library (convolutions, fused pair, pool, add) validates its arguments, chooses its kernel, builds and uploads
- * the weight layout that kernel needs and sizes the K-split / tail-split workspace of the handle exactly as the
+ * the weight layout that kernel needs and sizes the tail-split workspace of the handle exactly as the
  * real call would, but launches nothing and touches no activation.  Running a network's sequence of calls once in
  * planning mode (same shapes, same parameters) therefore moves every allocation and upload out of the later real
  * calls: afterwards rt3d_alloc_count does not change while those calls run.  rt3d_last_plan reports the planned
@@ -398,7 +398,7 @@ void rt3d_plan_end(void);
  * every SM with the 32-bit pattern `value` (e.g. 0x7FC07FC0: two bf16 NaNs) and waits for it: a kernel launched next
  * that reads shared or tensor memory it did not write itself (padding multiplied by zero weights, say) then
  * produces NaNs instead of depending silently on what ran before it.  The partial-tile scratch of every handle's
- * K splits on the device is set to all ones (NaNs) as well.  Device work only; nothing else changes. */
+ * tail splits on the device is set to all ones (NaNs) as well.  Device work only; nothing else changes. */
 enum { RT3D_DEBUG_WAIT_CYCLES = 1, RT3D_DEBUG_DROP_LAST_LOAD = 2, RT3D_DEBUG_T_GROUPS = 3, RT3D_DEBUG_POISON = 4 };
 rt3d_status rt3d_debug_set(int what, long long value);
 /* Diagnostics.  RT3D_DEBUG_WAIT_SITE: after a synchronisation of the device, the number of the wait inside a
