@@ -14,14 +14,17 @@ namespace rt3d {
 namespace {
 
 constexpr int kNormThreads = 256;
-constexpr int kNormChunk = 2048;      // floats of one weight row that a block reduces at a time
+constexpr int kNormChunk = 2048;      // floats of one weight row that a block can reduce at a time
+constexpr int kNormRun = 1024;        // ... and that it takes where groups are short enough
 
 // One block takes a row p of kernel groups and a run of whole groups along the input channels, at most kNormChunk
 // floats of each of its g_m weight rows.  A weight row [N][Ks] is contiguous, so
 // every thread reads 16 bytes (VEC) or 4 of it and adds up the g_m rows at that place in registers, with the loads of
 // four rows in flight; shared memory then holds one value per (input channel, location), of which each output sums g_n.
 // The former kernel, one thread per output, read runs of Ks floats that began at odd addresses, one 4-byte load each.
-// 1024 x 512 x 27 fp32, 4x4 groups, the three calls of a step one after the other: 88 -> 26.9 us.
+// 1024 x 512 x 27 fp32, 4x4 groups, the three calls of a step one after the other: 88 -> 26.9 us, this one 12.7; with chunks
+// of 1024 instead of 2048 floats, one load round per thread and twice the blocks to even out the last wave, 11.0 (57 MB at
+// the measured copy rate: 8.7).
 template <int G, bool VEC>
 __global__ void __launch_bounds__(kNormThreads)
 group_norms_kernel(const float* __restrict__ w, int M, int N, int Ks, int g_m, int g_n, int Q, int q_run, int n_runs,
@@ -106,9 +109,9 @@ cudaError_t launch_group_norms(const float* w, int M, int N, int Ks, int g_m, in
     LaunchSetup ls(dim3(unsigned((total + 255) / 256)), dim3(256), 0, st);
     return cudaLaunchKernelEx(&ls.cfg, group_norms_wide_kernel<G>, w, M, N, Ks, g_m, g_n, Q, norms, total);
   }
-  // groups per block: a whole chunk, in steps of four so that every run starts on a 16-byte boundary of its row; at
-  // most a quarter of a chunk where fewer blocks than two per SM would run
-  int q_run = kNormChunk / (g_n * Ks);
+  // groups per block: a whole run, in steps of four so that every run starts on a 16-byte boundary of its row; at
+  // most a quarter of a run where fewer blocks than two per SM would run
+  int q_run = g_n * Ks < kNormRun ? kNormRun / (g_n * Ks) : 1;
   if ((long long)P * ((Q + q_run - 1) / q_run) < 2 * 148) q_run = (q_run + 3) / 4;
   if (q_run > 4) q_run &= ~3;
   const bool vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0 && ((long long)N * Ks) % 4 == 0 && (q_run * g_n * Ks) % 4 == 0;
@@ -144,37 +147,48 @@ constexpr int kMaskThreads = 256;
 constexpr int kMaskChunk = 4096;      // bytes of one mask row that a block expands at a time
 
 // The g_m mask rows of a row of kernel groups are the same N * Ks bytes: a block expands a chunk of them once into
-// shared memory (each decision goes to the g_n channels of its group) and writes it to every row in 16-byte stores.  A row
-// may start at any byte, so the words of a row that does not start on a 16-byte boundary are cut out of the staged chunk at
-// that row's shift (funnel shifts), and only a chunk's first and last partial word go out byte by byte.  Bound by its
-// instructions: one thread per mask byte paid two 64-bit divisions for each, and gathering the bytes of a word instead of
-// scattering the decisions still took 740 instructions a thread (1024 x 512 x 27: 9.7 us, scattering 7.3 us).
+// shared memory (each decision goes to the g_n channels of its group) and writes it to every row in 16-byte stores.  Chunks
+// are whole groups where a group fits one; 2^lg lanes take a group's locations, so that neither needs a division or a
+// test.  A row may start at any byte, so the words of a row that does not start on a 16-byte boundary are cut out of the
+// staged chunk at that row's shift (funnel shifts), and only a chunk's first and last partial word go out byte by byte;
+// rows with the same shift (row length a multiple of 16) share the words in registers.  Bound by its instructions:
+// 1024 x 512 x 27, 4x4: 9.7 us gathering the bytes of a word, 7.2 scattering with a division and a test per byte, 6.1 now.
 __global__ void __launch_bounds__(kMaskThreads)
-expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int n_chunks,
-                   uint8_t* __restrict__ mask) {
+expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int chunk, int n_chunks,
+                   int lg, uint8_t* __restrict__ mask) {
   pdl_entry();
   __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 12];      // [4] words of slack in front: shifts read from there
   uint8_t* bytes = reinterpret_cast<uint8_t*>(row_s + 4);
   const int p = blockIdx.x / n_chunks;
-  const long long row_len = (long long)N * Ks, c0 = (long long)(blockIdx.x - p * n_chunks) * kMaskChunk;
-  const int len = int(min((long long)kMaskChunk, row_len - c0));
+  const long long row_len = (long long)N * Ks, c0 = (long long)(blockIdx.x - p * n_chunks) * chunk;
+  const int len = int(min((long long)chunk, row_len - c0));
   // the groups that the chunk touches, their decisions a contiguous run; first: where the first of them starts
   const long long span = (long long)g_n * Ks;
-  const int q0 = int(c0 / span), q1 = int((c0 + len - 1) / span);
-  const int first = int(q0 * span - c0), n_dec = (q1 + 1 - q0) * Ks;
+  const int q0 = int(c0 / span), n_q = int((c0 + len - 1) / span) + 1 - q0;
+  const int first = int(q0 * span - c0);
   const uint8_t* g = gmask + ((long long)p * Q + q0) * Ks;
-  for (int i = threadIdx.x; i < n_dec; i += kMaskThreads) {
-    const uint8_t bit = __ldg(g + i);
-    const int q = i / Ks;
-    int o = first + q * int(span) + (i - q * Ks);
+  const int k0 = threadIdx.x & ((1 << lg) - 1);
+  const bool whole = first == 0 && n_q * span <= kMaskChunk;           // bytes beyond len are not written out
 #pragma unroll 4
-    for (int j = 0; j < g_n; ++j, o += Ks)
-      if (unsigned(o) < unsigned(len)) bytes[o] = bit;
-  }
+  for (int q = threadIdx.x >> lg; q < n_q; q += kMaskThreads >> lg)
+    for (int k = k0; k < Ks; k += 1 << lg) {
+      const uint8_t bit = __ldg(g + q * Ks + k);
+      int o = first + q * int(span) + k;
+      if (whole) {
+#pragma unroll 4
+        for (int j = 0; j < g_n; ++j, o += Ks) bytes[o] = bit;
+      } else {
+        for (int j = 0; j < g_n; ++j, o += Ks)
+          if (unsigned(o) < unsigned(len)) bytes[o] = bit;
+      }
+    }
   __syncthreads();
   const int rows = min(g_m, M - p * g_m);
-  for (int i = 0; i < rows; ++i) {
-    uint8_t* dst = mask + (long long)(p * g_m + i) * row_len + c0;
+  uint8_t* dst0 = mask + (long long)(p * g_m) * row_len + c0;
+  const bool same_shift = (row_len & 15) == 0;
+  for (int i0 = 0; i0 < rows; i0 += same_shift ? rows : 1) {
+    uint8_t* dst = dst0 + i0 * row_len;
+    const int n_rows = same_shift ? rows : 1;
     const int shift = int(reinterpret_cast<uintptr_t>(dst) & 15);    // dst is `shift` bytes into its first 16-byte word
     const int n_words = (shift + len + 15) / 16;
     for (int u = threadIdx.x; u < n_words; u += kMaskThreads) {
@@ -190,9 +204,12 @@ expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int 
           v.z = __funnelshift_r(row_s[w0 + 2], row_s[w0 + 3], sh);
           v.w = __funnelshift_r(row_s[w0 + 3], row_s[w0 + 4], sh);
         }
-        *reinterpret_cast<uint4*>(dst + o) = v;
+        uint8_t* at = dst + o;
+#pragma unroll 4
+        for (int i = 0; i < n_rows; ++i, at += row_len) *reinterpret_cast<uint4*>(at) = v;
       } else {
-        for (int b = max(o, 0); b < min(o + 16, len); ++b) dst[b] = bytes[b];
+        for (int i = 0; i < n_rows; ++i)
+          for (int b = max(o, 0); b < min(o + 16, len); ++b) dst[i * row_len + b] = bytes[b];
       }
     }
   }
@@ -234,9 +251,16 @@ rt3d_status rt3d_kgs_expand_mask(const uint8_t* group_mask, int M, int N, int Kt
   if (!group_mask || !mask || M <= 0 || N <= 0 || Kt <= 0 || Kh <= 0 || Kw <= 0 || g_m <= 0 || g_n <= 0) return RT3D_ERR_INVALID_ARG;
   const int Ks = Kt * Kh * Kw;
   const int Q = (N + g_n - 1) / g_n;
-  const int P = (M + g_m - 1) / g_m, n_chunks = int(((long long)N * Ks + kMaskChunk - 1) / kMaskChunk);
+  // whole groups per chunk, sixteen of them at a time so that chunks start on 16-byte boundaries of the row
+  const long long span = (long long)g_n * Ks;
+  int chunk = kMaskChunk;
+  if (span * 16 <= kMaskChunk) chunk = int(kMaskChunk / (span * 16) * (span * 16));
+  else if (span <= kMaskChunk) chunk = int(kMaskChunk / span * span);
+  const int P = (M + g_m - 1) / g_m, n_chunks = int(((long long)N * Ks + chunk - 1) / chunk);
+  int lg = 0;
+  while (lg < 5 && (1 << lg) < Ks) ++lg;
   LaunchSetup ls(dim3(unsigned((long long)P * n_chunks)), dim3(kMaskThreads), 0, static_cast<cudaStream_t>(stream));
-  const cudaError_t e = cudaLaunchKernelEx(&ls.cfg, expand_mask_kernel, group_mask, M, N, Ks, g_m, g_n, Q, n_chunks, mask);
+  const cudaError_t e = cudaLaunchKernelEx(&ls.cfg, expand_mask_kernel, group_mask, M, N, Ks, g_m, g_n, Q, chunk, n_chunks, lg, mask);
   return e == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
 }
 

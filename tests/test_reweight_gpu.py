@@ -68,7 +68,8 @@ def test_reweight_argument_errors():
 @pytest.mark.parametrize("M,N,k,g_m,g_n,byte", [
     (4, 4, (1, 1, 1), 4, 4, 0), (5, 3, (3, 1, 1), 4, 4, 1), (9, 37, (3, 3, 3), 8, 4, 3),      # rows at odd bytes, ragged groups
     (8, 152, (3, 3, 3), 4, 4, 0), (12, 151, (3, 3, 3), 4, 4, 5),                              # a mask chunk and a few bytes
-    (16, 76, (3, 3, 3), 4, 4, 0), (7, 80, (3, 3, 3), 8, 8, 2), (6, 20, (5, 7, 7), 4, 16, 0)])  # run ends; groups beyond a chunk
+    (16, 76, (3, 3, 3), 4, 4, 0), (7, 80, (3, 3, 3), 8, 8, 2), (6, 20, (5, 7, 7), 4, 16, 0),   # run ends; groups beyond a run
+    (5, 40, (5, 7, 7), 4, 32, 1), (8, 70, (5, 3, 5), 4, 4, 0)])                               # ... beyond a chunk; a few to a chunk
 def test_pruning_step_at_run_and_word_edges(M, N, k, g_m, g_n, byte):
     """Rows and buffers that start at any byte / float, runs and chunks that end inside a word, groups too long for a run."""
     rng = np.random.default_rng(M * 1000 + N)
