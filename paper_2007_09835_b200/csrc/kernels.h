@@ -27,7 +27,7 @@ cudaError_t launch_conv_simt(int dtype, const ConvGeom& g, const void* x, void* 
 // Register-blocked fp32 kernel (simt_conv_f32.cu).
 struct F32Args {
   ConvGeom g;
-  int bt, bh, bw;                     // output box of a block: at most (8 / sets) * 16 lanes' positions times vt * vh voxels
+  int bt, bh, bw;                     // output box of a block: at most 8 / (sets * parts) * 16 lanes' positions times vt * vh voxels
   int vt, vh;                         // a thread's voxels: vt along t times vh along h, bt / vt and bh / vh apart
   int tiles_t, tiles_h, tiles_w;
   int ht, hh, hw;                     // staged input box
@@ -45,12 +45,13 @@ struct F32Args {
   const float* bias;                  // or nullptr
   const float* residual;              // or nullptr, pitch rcs
   int rcs;
+  int parts;                          // warps that share a set and its voxels, each with a part of every list of entries
 };
-struct F32Plan { int voxels, sets; int bt, bh, bw, vt, vh; };
+struct F32Plan { int voxels, sets, parts; int bt, bh, bw, vt, vh; };
 struct F32Layout;
-// Candidate (voxels per thread, row sets per block, output box) for a call, best first (density = kept
+// Candidate (voxels per thread, row sets per block, parts, output box) for a call, best first (density = kept
 // share of the (group, location) places); conv_f32_fill says whether one's staging fits shared memory.
-constexpr int kF32MaxPlans = 16;
+constexpr int kF32MaxPlans = 40;
 int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]);
 bool conv_f32_fill(const F32Plan& plan, const F32Layout& L, F32Args* a);
 cudaError_t launch_conv_f32(const F32Args& a, const F32Plan& plan, cudaStream_t stream);

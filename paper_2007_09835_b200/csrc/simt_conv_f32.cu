@@ -18,6 +18,10 @@
 // 655 us instead of 524).  Measured, 0.4 of the places kept: 64 -> 128 channels, 3x3x3, 2 x 16 x 56 x 56 voxels 2475 ->
 // 524 us (7.2 -> 34 TFLOP/s kept); 16 -> 32 channels, 8 x 28 x 28 voxels 27.4 -> 9.6 us, half of it launch and latency.
 //
+// Small calls leave an SM too few warps, each a serial chain of entries, or too few voxels a thread.  There `parts` warps
+// share a set and its voxels, each takes its part of every list, and the first adds up the others' sums, in order, through
+// shared memory: the call of 8 x 28 x 28 voxels 10.1 -> 9.2 us, 64 -> 128 channels on 4 x 14 x 14 26 -> 20 us.
+//
 // Two buffers; the copies of stage s + 1 (cp.async) run while stage s is multiplied.
 #include <algorithm>
 #include <cmath>
@@ -38,6 +42,11 @@ typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 __device__ __forceinline__ float2 unpack2(f32x2 v) {
@@ -66,13 +75,14 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
 struct F32Smem {
   int tile_bytes, x_bytes, entry_bytes, buffer_bytes, total;
 };
-__host__ __device__ inline F32Smem f32_smem(int max_tiles, int max_entries, int quads, int voxels) {
+__host__ __device__ inline F32Smem f32_smem(int max_tiles, int max_entries, int quads, int voxels, int sum_bytes = 0) {
   F32Smem s;
   s.tile_bytes = max_tiles * 64;
   s.x_bytes = quads * voxels * 16;
   s.entry_bytes = ((max_entries + 1) * 4 + 15) & ~15;              // one past the end is read ahead
   s.buffer_bytes = s.tile_bytes + s.x_bytes + s.entry_bytes;
   s.total = 2 * s.buffer_bytes + kKoffMax * 4 + voxels * 4;
+  if (s.total < sum_bytes) s.total = sum_bytes;
   return s;
 }
 
@@ -105,7 +115,7 @@ __device__ __forceinline__ void run_list(int n, uint32_t& ep, uint32_t& wp, uint
   }
 }
 
-template <int V>
+template <int V, bool kParts>
 __global__ void __launch_bounds__(kThreadsF32, 2)
 conv3d_f32_kernel(const F32Args a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -116,8 +126,9 @@ conv3d_f32_kernel(const F32Args a) {
   int* koff_s = reinterpret_cast<int*>(smem + 2 * sm.buffer_bytes);        // kernel location -> byte offset in a plane
   int* vox_s = koff_s + kKoffMax;                                          // staged voxel -> input voxel, or -1
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int voxel_warps = (kThreadsF32 / 32) / a.sets;
-  const int set_local = warp / voxel_warps, vw = warp - set_local * voxel_warps;
+  const int parts = kParts ? a.parts : 1, part = kParts ? warp % parts : 0;
+  const int voxel_warps = (kThreadsF32 / 32) / a.sets / parts, slot = kParts ? warp / parts : warp;
+  const int set_local = slot / voxel_warps, vw = slot - set_local * voxel_warps;
   const int set0 = blockIdx.y * a.sets, n_here = min(a.sets, a.n_sets - set0);
 
   int tile = blockIdx.x;
@@ -204,11 +215,36 @@ conv3d_f32_kernel(const F32Args a) {
       uint32_t wp = b0 + uint32_t(__ldg(a.tile_ptr + i0 + set_local) - t0_) * 64u + (lane & 1) * 32;   // this lane's two outputs
       uint32_t ep = b0 + sm.tile_bytes + sm.x_bytes + (es - e0) * 4;
       const uint32_t x_lane = b0 + sm.tile_bytes + vox_off;
-      run_list<V, 0, 1>(n_both, ep, wp, x_lane, delta, acc);
-      run_list<V, 0, 0>(n_first, ep, wp, x_lane, delta, acc);
-      run_list<V, 1, 1>(n_e - n_both - n_first, ep, wp, x_lane, delta, acc);
+      if constexpr (!kParts) {
+        run_list<V, 0, 1>(n_both, ep, wp, x_lane, delta, acc);
+        run_list<V, 0, 0>(n_first, ep, wp, x_lane, delta, acc);
+        run_list<V, 1, 1>(n_e - n_both - n_first, ep, wp, x_lane, delta, acc);
+      } else {
+        const auto mine = [&](int n, int rows, auto run) {             // this warp's part of the next list
+          const int from = n * part / parts, to = n * (part + 1) / parts;
+          uint32_t ep_at = ep + from * 4, wp_at = wp + from * rows * 64;
+          run(to - from, ep_at, wp_at);
+          ep += n * 4;
+          wp += n * rows * 64;
+        };
+        mine(n_both, 2, [&](int n, uint32_t& e, uint32_t& w) { run_list<V, 0, 1>(n, e, w, x_lane, delta, acc); });
+        mine(n_first, 1, [&](int n, uint32_t& e, uint32_t& w) { run_list<V, 0, 0>(n, e, w, x_lane, delta, acc); });
+        mine(n_e - n_both - n_first, 1, [&](int n, uint32_t& e, uint32_t& w) { run_list<V, 1, 1>(n, e, w, x_lane, delta, acc); });
+      }
     }
     __syncthreads();
+  }
+
+  if (kParts) {                                      // the buffers are free: the other parts' sums, [part][register][lane]
+    f32x2* sums = reinterpret_cast<f32x2*>(smem) + (set_local * voxel_warps + vw) * (parts - 1) * (V * 128) + lane;
+    if (part > 0)
+#pragma unroll
+      for (int i = 0; i < 4 * V; ++i) sums[(part - 1) * (V * 128) + i * 32] = acc[i / (2 * V)][(i / 2) % V][i & 1];
+    __syncthreads();
+    if (part > 0) return;
+    for (int p = 0; p < parts - 1; ++p)
+#pragma unroll
+      for (int i = 0; i < 4 * V; ++i) acc[i / (2 * V)][(i / 2) % V][i & 1] = add2(acc[i / (2 * V)][(i / 2) % V][i & 1], sums[p * (V * 128) + i * 32]);
   }
 
   // bias, residual, ReLU; a pair of lanes writes the 16 bytes of a (voxel, row)
@@ -236,19 +272,21 @@ conv3d_f32_kernel(const F32Args a) {
   }
 }
 
-template <int V>
+template <int V, bool kParts>
 cudaError_t launch_t(const F32Args& a, dim3 grid, size_t smem, cudaStream_t stream) {
   static bool attr_done[kMaxDevices] = {};             // the attribute is per device
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_f32_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_f32_kernel<V, kParts>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
   LaunchSetup ls(grid, dim3(kThreadsF32), smem, stream);
-  return cudaLaunchKernelEx(&ls.cfg, conv3d_f32_kernel<V>, a);
+  return cudaLaunchKernelEx(&ls.cfg, conv3d_f32_kernel<V, kParts>, a);
 }
+
+int f32_sum_bytes(int voxels, int parts) { return (kThreadsF32 / 32) / parts * (parts - 1) * voxels * 1024; }
 
 int staged(int out, int kernel, int stride) { return kernel == 1 ? out : (out - 1) * stride + kernel; }
 
@@ -278,7 +316,7 @@ double choose_box_f32(const ConvGeom& g, int lanes, int voxels, double weight, F
 }  // namespace
 
 // Cycles of the busiest SM for every variant, fitted to timings on B200: an entry costs a scheduler 25 + V (4 + 10 h) with
-// four warps at work (h = tiles per entry) and a warp by itself 45 + V (12 + 30 h); a stage costs its copies and barriers.
+// four warps at work (h = tiles per entry) and a warp by itself 45 + V (12 + 30 h); a stage costs its copies and barriers, adding up the parts 220 V for each and 800.
 static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
   const int Ks = g.Kt * g.Kh * g.Kw, n_rows = ceil_div(g.M, 4), n_quads = ceil_div(g.c, 4), quads = f32_stage_quads(Ks);
   const int n_stages = ceil_div(n_quads, quads);
@@ -287,22 +325,25 @@ static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan
   const int n_sets = ceil_div(n_rows, 2);
   const double places = double(n_quads) * Ks, rows = n_rows > 1 ? 2.0 : 1.0;
   const double entries = places * (rows > 1.0 ? density * (2.0 - density) : density), hits = places * density * rows;
+  const double warps = double(g.n) * g.To * g.Ho * g.Wo * n_sets / 16.0;
   for (int V = 1; V <= 8; V *= 2)
-    for (int lg = 0; lg < 4; ++lg) {
-      const int sets = 1 << lg;
-      if (sets >= 2 * n_sets) continue;
-      F32Plan p{V, sets, 1, 1, 1, 1, 1};
-      if (choose_box_f32(g, (8 / sets) * 16, V, 0.1, &p) < 0) continue;
+    for (int lg = 0; lg < 16; ++lg) {
+      const int sets = 1 << (lg & 3), parts = 1 << (lg >> 2);
+      if (sets >= 2 * n_sets || sets * parts > 8) continue;
+      if (parts > 1 && (V == 8 || warps / V > 32.0 * sm_count)) continue;      // enough warps as it is
+      F32Plan p{V, sets, parts, 1, 1, 1, 1, 1};
+      if (choose_box_f32(g, 8 / (sets * parts) * 16, V, 0.1, &p) < 0) continue;
       const double boxes = double(g.n) * ceil_div(g.To, p.bt) * ceil_div(g.Ho, p.bh) * ceil_div(g.Wo, p.bw);
       const int halo = staged(p.bt, g.Kt, g.st) * staged(p.bh, g.Kh, g.sh) * staged(p.bw, g.Kw, g.sw);
       const double mean = double(quads) * Ks * density * 2 * sets;         // tiles of a stage
-      const F32Smem sm = f32_smem(int(mean * 1.2) + 1, quads * Ks * sets, quads, halo);
+      const F32Smem sm = f32_smem(int(mean * 1.2) + 1, quads * Ks * sets, quads, halo, f32_sum_bytes(V, parts));
       if (sm.total > 227 * 1024) continue;
       const int occ = 226 * 1024 / (sm.total + 1024) > 1 ? 2 : 1;
       const double per_sm = double(ceil_div64(int64_t(boxes) * ceil_div(n_sets, sets), sm_count));
       const double h = hits / entries, staging = double(n_stages) * (halo * quads * 32.0 + mean * 4 * 12.0) / 128.0;
-      const double busy = 2.0 * entries * (25.0 + V * (4.0 + 10.0 * h)) + staging;      // two warps a scheduler
-      const double lone = entries * (45.0 + V * (12.0 + 30.0 * h)) + staging + n_stages * 900.0 + 2500.0;
+      const double own = parts > 1 ? entries / parts + 1.5 * n_stages : entries, sum = parts > 1 ? 800.0 + 220.0 * V * (parts - 1) : 0.0;
+      const double busy = 2.0 * own * (25.0 + V * (4.0 + 10.0 * h)) + staging + sum;      // two warps a scheduler
+      const double lone = own * (45.0 + V * (12.0 + 30.0 * h)) + staging + sum + n_stages * 900.0 + 2500.0;
       double t = per_sm * busy;
       if (std::ceil(per_sm / occ) * lone > t) t = std::ceil(per_sm / occ) * lone;
       int at = n;
@@ -338,21 +379,21 @@ bool conv_f32_fill(const F32Plan& p, const F32Layout& L, F32Args* a) {
   a->ht = staged(p.bt, g.Kt, g.st); a->hh = staged(p.bh, g.Kh, g.sh); a->hw = staged(p.bw, g.Kw, g.sw);
   a->ht_step = g.Kt == 1 ? g.st : 1; a->hh_step = g.Kh == 1 ? g.sh : 1; a->hw_step = g.Kw == 1 ? g.sw : 1;
   a->n_sets = L.n_sets; a->n_stages = L.n_stages; a->quads = L.quads;
-  a->sets = p.sets;
+  a->sets = p.sets; a->parts = p.parts;
   const int lg = p.sets == 1 ? 0 : p.sets == 2 ? 1 : p.sets == 4 ? 2 : 3;
   a->max_entries = L.max_entries[lg]; a->max_tiles = L.max_tiles[lg];
-  return f32_smem(a->max_tiles, a->max_entries, a->quads, a->ht * a->hh * a->hw).total <= 227 * 1024 &&
+  return f32_smem(a->max_tiles, a->max_entries, a->quads, a->ht * a->hh * a->hw, f32_sum_bytes(p.voxels, p.parts)).total <= 227 * 1024 &&
          (long long)g.n * a->tiles_t * a->tiles_h * a->tiles_w < (1ll << 31) && ceil_div(L.n_sets, p.sets) <= 65535;
 }
 
 cudaError_t launch_conv_f32(const F32Args& a, const F32Plan& p, cudaStream_t stream) {
   const dim3 grid(unsigned(a.g.n * a.tiles_t * a.tiles_h * a.tiles_w), unsigned(ceil_div(a.n_sets, p.sets)));
-  const size_t smem = size_t(f32_smem(a.max_tiles, a.max_entries, a.quads, a.ht * a.hh * a.hw).total);
+  const size_t smem = size_t(f32_smem(a.max_tiles, a.max_entries, a.quads, a.ht * a.hh * a.hw, f32_sum_bytes(p.voxels, p.parts)).total);
   switch (p.voxels) {
-    case 1: return launch_t<1>(a, grid, smem, stream);
-    case 2: return launch_t<2>(a, grid, smem, stream);
-    case 4: return launch_t<4>(a, grid, smem, stream);
-    case 8: return launch_t<8>(a, grid, smem, stream);
+    case 1: return p.parts > 1 ? launch_t<1, true>(a, grid, smem, stream) : launch_t<1, false>(a, grid, smem, stream);
+    case 2: return p.parts > 1 ? launch_t<2, true>(a, grid, smem, stream) : launch_t<2, false>(a, grid, smem, stream);
+    case 4: return p.parts > 1 ? launch_t<4, true>(a, grid, smem, stream) : launch_t<4, false>(a, grid, smem, stream);
+    case 8: return launch_t<8, false>(a, grid, smem, stream);
   }
   return cudaErrorInvalidValue;
 }

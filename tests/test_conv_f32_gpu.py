@@ -24,6 +24,8 @@ pytestmark = pytest.mark.gpu
     ((1, 4, 20, 20), 12, 40, (1, 7, 7), (1, 2, 2), (4, 4), "bernoulli", 0.4),       # 49 locations
     ((1, 2, 6, 6), 64, 512, (3, 3, 3), (1, 1, 1), (8, 4), "vanilla_total", 200),    # whole groups: empty and full stages
     ((1, 2, 6, 6), 24, 40, (3, 3, 3), (1, 1, 1), (4, 4), "exact_total", 1),         # one place kept in all
+    ((1, 4, 14, 14), 61, 122, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.4),      # few voxels: warps that share them
+    ((1, 2, 7, 7), 128, 128, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.05),      # ... with parts of nearly empty lists
     ((4, 16, 40, 40), 16, 128, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.4)])    # several boxes per SM
 def test_fp32_kernel_matches_oracle(x, cin, cout, k, stride, group, kind, density):
     spec = synth.ConvSpec("f32", cin, cout, k, stride, tuple(v // 2 for v in k), True)
