@@ -2,7 +2,7 @@
 //
 // A pruning loop packs, uploads and frees a layer again and again, and most of that was memory management: the page faults
 // of a fresh 4 MB block (1 ms), cudaMalloc and cudaFree of 18 MB (0.45 and 0.55 ms).  512 x 512 x 27 at 0.28 kept, packed,
-// uploaded, read back and freed: 4.9 -> 2.6 ms.
+// uploaded, read back and freed: 4.9 -> 2.6 ms (2.0 since).
 // Bounds: at most kMost bytes in all, no block over half of that; a request that finds nothing that fits gives every kept
 // block of its kind back to the system first, so that blocks of sizes no longer asked for do not stay.
 #pragma once

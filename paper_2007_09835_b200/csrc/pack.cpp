@@ -14,13 +14,6 @@
 
 namespace rt3d {
 
-uint16_t f32_to_bf16_bits(float f) {
-  uint32_t u;
-  std::memcpy(&u, &f, 4);
-  const uint32_t rounded = u + 0x7FFFu + ((u >> 16) & 1u);          // ties to even
-  return uint16_t(((u & 0x7FFFFFFFu) > 0x7F800000u ? u | 0x400000u : rounded) >> 16);    // a NaN stays one
-}
-
 float bf16_bits_to_f32(uint16_t b) {
   uint32_t u = uint32_t(b) << 16;
   float f;
@@ -498,6 +491,30 @@ static uint64_t next_handle_id() {
 
 constexpr size_t kGatherGroup = 64;      // weights of a group that pass 2 gathers at once
 
+// The tiles of one whole group, location by location.  GM, GN: the group's size where it is known when compiling (0: not),
+// which turns the gather and the conversion into straight code (512 x 512 x 27, 4x4, eight threads: 1.25 -> 0.7 ms).
+template <int GM, int GN>
+static void gather_group(const float* base, int64_t row_len, int Ks, const uint16_t* pos, int n, int g_m_, int g_n_, int dtype,
+                         unsigned char* out) {
+  const int g_m = GM ? GM : g_m_, g_n = GN ? GN : g_n_, step = g_m * g_n;
+  float v[GM && GN ? GM * GN : kGatherGroup];
+  uint16_t b[GM && GN ? GM * GN : kGatherGroup];
+  for (int e = 0; e < n; ++e) {
+    for (int i = 0; i < g_m; ++i) {
+      const float* at = base + pos[e] + i * row_len;
+      for (int j = 0; j < g_n; ++j) v[i * g_n + j] = at[j * Ks];
+    }
+    if (dtype == RT3D_BF16) {
+      for (int i = 0; i < step; ++i) b[i] = f32_to_bf16_bits(v[i]);
+      std::memcpy(out, b, size_t(step) * 2);
+      out += size_t(step) * 2;
+    } else {
+      std::memcpy(out, v, size_t(step) * 4);
+      out += size_t(step) * 4;
+    }
+  }
+}
+
 static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, int Kt, int Kh, int Kw,
                              int g_m, int g_n, int dtype, int is_dense, rt3d_packed** out) {
   if (!w || !out) return RT3D_ERR_INVALID_ARG;
@@ -571,19 +588,9 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
       unsigned char* out = h->tiles.data() + size_t(e0) * step * esz;
       const float* base = w + (int64_t(pr) * g_m * N + int64_t(q) * g_n) * Ks;
       if (rows == g_m && cols == g_n && step <= kGatherGroup) {
-        float v[kGatherGroup];
-        for (int e = 0; e < n_e; ++e, out += step * esz) {
-          const float* at = base + pos[e];
-          for (int i = 0; i < g_m; ++i)
-            for (int j = 0; j < g_n; ++j) v[i * g_n + j] = at[(int64_t(i) * N + j) * Ks];
-          if (dtype == RT3D_BF16) {
-            uint16_t b[kGatherGroup];
-            for (size_t i = 0; i < step; ++i) b[i] = f32_to_bf16_bits(v[i]);
-            std::memcpy(out, b, step * 2);
-          } else {
-            std::memcpy(out, v, step * 4);
-          }
-        }
+        if (g_m == 4 && g_n == 4) gather_group<4, 4>(base, int64_t(N) * Ks, Ks, pos, n_e, 4, 4, dtype, out);
+        else if (g_n == 4) gather_group<0, 4>(base, int64_t(N) * Ks, Ks, pos, n_e, g_m, 4, dtype, out);
+        else gather_group<0, 0>(base, int64_t(N) * Ks, Ks, pos, n_e, g_m, g_n, dtype, out);
         return;
       }
       if (rows < g_m || cols < g_n) std::memset(out, 0, size_t(n_e) * step * esz);           // kernels that do not exist

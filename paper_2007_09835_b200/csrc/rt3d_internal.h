@@ -3,6 +3,7 @@
 
 #include <cstdint>
 #include <cstddef>
+#include <cstring>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -23,7 +24,13 @@ inline int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
 
 // Round-to-nearest-even float -> bfloat16 bits (NaN kept quiet), and back.
-uint16_t f32_to_bf16_bits(float f);
+// Inline: a function that the library exports is called through its linkage table, once per weight.
+inline uint16_t f32_to_bf16_bits(float f) {
+  uint32_t u;
+  std::memcpy(&u, &f, 4);
+  const uint32_t rounded = u + 0x7FFFu + ((u >> 16) & 1u);          // ties to even
+  return uint16_t(((u & 0x7FFFFFFFu) > 0x7F800000u ? u | 0x400000u : rounded) >> 16);    // a NaN stays one
+}
 float bf16_bits_to_f32(uint16_t b);
 
 // Encoded K step of the tensor-core path: which kernel location and which 64-channel chunk.
