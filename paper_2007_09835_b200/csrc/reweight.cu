@@ -17,6 +17,13 @@ constexpr int kNormThreads = 256;
 constexpr int kNormChunk = 2048;      // floats of one weight row that a block can reduce at a time
 constexpr int kNormRun = 1024;        // ... and that it takes where groups are short enough
 
+// log2 of the lanes that share the Ks locations of a group: the next power of two, at most a warp.
+int lanes_of(int Ks) {
+  int lg = 0;
+  while (lg < 5 && (1 << lg) < Ks) ++lg;
+  return lg;
+}
+
 // One block takes a row p of kernel groups and a run of whole groups along the input channels, at most kNormChunk
 // floats of each of its g_m weight rows.  A weight row [N][Ks] is contiguous, so
 // every thread reads 16 bytes (VEC) or 4 of it and adds up the g_m rows at that place in registers, with the loads of
@@ -24,11 +31,11 @@ constexpr int kNormRun = 1024;        // ... and that it takes where groups are 
 // The former kernel, one thread per output, read runs of Ks floats that began at odd addresses, one 4-byte load each.
 // 1024 x 512 x 27 fp32, 4x4 groups, the three calls of a step one after the other: 88 -> 26.9 us, this one 12.7; with chunks
 // of 1024 instead of 2048 floats, one load round per thread and twice the blocks to even out the last wave, 11.0 (57 MB at
-// the measured copy rate: 8.7).
+// the measured copy rate: 8.7); straight code for four rows and no divisions: 10.7.
 template <int G, bool VEC>
-__global__ void __launch_bounds__(kNormThreads)
+__global__ void __launch_bounds__(kNormThreads, 8)
 group_norms_kernel(const float* __restrict__ w, int M, int N, int Ks, int g_m, int g_n, int Q, int q_run, int n_runs,
-                   float* __restrict__ norms) {
+                   int lg, float* __restrict__ norms) {
   pdl_entry();
   __shared__ __align__(16) float part[kNormChunk];
   const int p = blockIdx.x / n_runs, q0 = (blockIdx.x - p * n_runs) * q_run;
@@ -38,7 +45,17 @@ group_norms_kernel(const float* __restrict__ w, int M, int N, int Ks, int g_m, i
   const float* base = w + (long long)m0 * row_len + (long long)q0 * g_n * Ks;
   const int len = int(min((long long)nq * g_n * Ks, row_len - (long long)q0 * g_n * Ks));   // missing channels add 0
   auto term = [](float v) { return G == 1 ? fabsf(v) : v * v; };
-  if (VEC) {
+  if (VEC && rows == 4) {
+    for (int o = threadIdx.x * 4; o < len; o += kNormThreads * 4) {
+      const float* at = base + o;
+      float4 v[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r, at += row_len) v[r] = __ldg(reinterpret_cast<const float4*>(at));
+      *reinterpret_cast<float4*>(part + o) =
+          make_float4(((term(v[0].x) + term(v[1].x)) + term(v[2].x)) + term(v[3].x), ((term(v[0].y) + term(v[1].y)) + term(v[2].y)) + term(v[3].y),
+                      ((term(v[0].z) + term(v[1].z)) + term(v[2].z)) + term(v[3].z), ((term(v[0].w) + term(v[1].w)) + term(v[2].w)) + term(v[3].w));
+    }
+  } else if (VEC) {
     for (int o = threadIdx.x * 4; o < len; o += kNormThreads * 4) {
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
       int i = 0;
@@ -72,13 +89,16 @@ group_norms_kernel(const float* __restrict__ w, int M, int N, int Ks, int g_m, i
   }
   __syncthreads();
   float* out = norms + ((long long)p * Q + q0) * Ks;
-  for (int r = threadIdx.x; r < nq * Ks; r += kNormThreads) {
-    const int q = r / Ks, k = r - q * Ks;
-    const float* src = part + q * g_n * Ks + k;
+  for (int q = threadIdx.x >> lg; q < nq; q += kNormThreads >> lg) {       // 2^lg lanes to a group: no division
     const int cols = min(g_n, N - (q0 + q) * g_n);
-    float s = 0.f;
-    for (int j = 0; j < cols; ++j) s += src[j * Ks];
-    out[r] = G == 1 ? s : sqrtf(s);
+    for (int k = threadIdx.x & ((1 << lg) - 1); k < Ks; k += 1 << lg) {
+      const float* src = part + q * g_n * Ks + k;
+      float s = 0.f;
+      if (cols == 4) s = ((src[0] + src[Ks]) + src[2 * Ks]) + src[3 * Ks];
+      else
+        for (int j = 0; j < cols; ++j) s += src[j * Ks];
+      out[q * Ks + k] = G == 1 ? s : sqrtf(s);
+    }
   }
 }
 
@@ -115,10 +135,10 @@ cudaError_t launch_group_norms(const float* w, int M, int N, int Ks, int g_m, in
   if ((long long)P * ((Q + q_run - 1) / q_run) < 2 * 148) q_run = (q_run + 3) / 4;
   if (q_run > 4) q_run &= ~3;
   const bool vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0 && ((long long)N * Ks) % 4 == 0 && (q_run * g_n * Ks) % 4 == 0;
-  const int n_runs = (Q + q_run - 1) / q_run;
+  const int n_runs = (Q + q_run - 1) / q_run, lg = lanes_of(Ks);
   LaunchSetup ls(dim3(unsigned((long long)P * n_runs)), dim3(kNormThreads), 0, st);
-  return vec ? cudaLaunchKernelEx(&ls.cfg, group_norms_kernel<G, true>, w, M, N, Ks, g_m, g_n, Q, q_run, n_runs, norms)
-             : cudaLaunchKernelEx(&ls.cfg, group_norms_kernel<G, false>, w, M, N, Ks, g_m, g_n, Q, q_run, n_runs, norms);
+  return vec ? cudaLaunchKernelEx(&ls.cfg, group_norms_kernel<G, true>, w, M, N, Ks, g_m, g_n, Q, q_run, n_runs, lg, norms)
+             : cudaLaunchKernelEx(&ls.cfg, group_norms_kernel<G, false>, w, M, N, Ks, g_m, g_n, Q, q_run, n_runs, lg, norms);
 }
 
 // Four norms per thread where the arrays allow it (VEC: 16-byte aligned floats, 4-byte aligned decisions).
@@ -152,10 +172,10 @@ constexpr int kMaskChunk = 4096;      // bytes of one mask row that a block expa
 // test.  A row may start at any byte, so the words of a row that does not start on a 16-byte boundary are cut out of the
 // staged chunk at that row's shift (funnel shifts), and only a chunk's first and last partial word go out byte by byte;
 // rows with the same shift (row length a multiple of 16) share the words in registers.  Bound by its instructions:
-// 1024 x 512 x 27, 4x4: 9.7 us gathering the bytes of a word, 7.2 scattering with a division and a test per byte, 6.1 now.
+// 1024 x 512 x 27, 4x4: 9.7 us gathering the bytes of a word, 7.2 scattering with a division and a test per byte, 5.6 now.
 __global__ void __launch_bounds__(kMaskThreads)
-expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int chunk, int n_chunks,
-                   int lg, uint8_t* __restrict__ mask) {
+expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int g_m, int g_n, int Q, int chunk, int q_chunk,
+                   int n_chunks, int lg, uint8_t* __restrict__ mask) {
   pdl_entry();
   __shared__ __align__(16) uint32_t row_s[kMaskChunk / 4 + 12];      // [4] words of slack in front: shifts read from there
   uint8_t* bytes = reinterpret_cast<uint8_t*>(row_s + 4);
@@ -164,11 +184,17 @@ expand_mask_kernel(const uint8_t* __restrict__ gmask, int M, int N, int Ks, int 
   const int len = int(min((long long)chunk, row_len - c0));
   // the groups that the chunk touches, their decisions a contiguous run; first: where the first of them starts
   const long long span = (long long)g_n * Ks;
-  const int q0 = int(c0 / span), n_q = int((c0 + len - 1) / span) + 1 - q0;
-  const int first = int(q0 * span - c0);
+  int q0 = int(blockIdx.x - p * n_chunks) * q_chunk, n_q, first = 0;    // q_chunk: whole groups in a chunk, or 0
+  if (q_chunk > 0) {
+    n_q = min(q_chunk, Q - q0);
+  } else {
+    q0 = int(c0 / span);
+    n_q = int((c0 + len - 1) / span) + 1 - q0;
+    first = int(q0 * span - c0);
+  }
   const uint8_t* g = gmask + ((long long)p * Q + q0) * Ks;
   const int k0 = threadIdx.x & ((1 << lg) - 1);
-  const bool whole = first == 0 && n_q * span <= kMaskChunk;           // bytes beyond len are not written out
+  const bool whole = q_chunk > 0;                                       // bytes beyond len are not written out
 #pragma unroll 4
   for (int q = threadIdx.x >> lg; q < n_q; q += kMaskThreads >> lg)
     for (int k = k0; k < Ks; k += 1 << lg) {
@@ -257,10 +283,9 @@ rt3d_status rt3d_kgs_expand_mask(const uint8_t* group_mask, int M, int N, int Kt
   if (span * 16 <= kMaskChunk) chunk = int(kMaskChunk / (span * 16) * (span * 16));
   else if (span <= kMaskChunk) chunk = int(kMaskChunk / span * span);
   const int P = (M + g_m - 1) / g_m, n_chunks = int(((long long)N * Ks + chunk - 1) / chunk);
-  int lg = 0;
-  while (lg < 5 && (1 << lg) < Ks) ++lg;
+  const int lg = lanes_of(Ks);
   LaunchSetup ls(dim3(unsigned((long long)P * n_chunks)), dim3(kMaskThreads), 0, static_cast<cudaStream_t>(stream));
-  const cudaError_t e = cudaLaunchKernelEx(&ls.cfg, expand_mask_kernel, group_mask, M, N, Ks, g_m, g_n, Q, chunk, n_chunks, lg, mask);
+  const cudaError_t e = cudaLaunchKernelEx(&ls.cfg, expand_mask_kernel, group_mask, M, N, Ks, g_m, g_n, Q, chunk, span <= kMaskChunk ? int(chunk / span) : 0, n_chunks, lg, mask);
   return e == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
 }
 
