@@ -461,6 +461,28 @@ TileBox choose_box_search(const ConvGeom& g, bool prefer_deep) {
   return best;
 }
 
+// Box inside one clip for the t-grouped variant where none of the boxes with the fewest tiles suits it: up to a sixteenth
+// more tiles, the fewest bytes from L2 (a group's input frames and its Kt weight tiles) over all tiles.  Returns their ratio to
+// what the fewest tiles with a box per step read; it is taken up to 0.8, for strided rows, where the larger boxes take the
+// copy engine longer, up to 0.68 (0.65 gained 15 % there, 0.71 lost 8 %), and up to 0.6 where it costs the bulk stores.  21 -> 33 channels 3x3x3 on 2 x 10 x 43 x 39 voxels, 286 tiles 10 frames
+// deep for 275 tiles of two clips: 37.4 -> 17.8 us; 17 -> 49 on 2 x 5 x 52 x 87 49.4 -> 24.2; 31 -> 238 on 23 x 7 x 37 x 83
+// 350 -> 275; 87 -> 154 on 6 x 12 x 90 x 17 147 -> 103.
+double choose_box_grouped(const ConvGeom& g, int n_tile, long long fewest, TileBox* out) {
+  double best = -1.0;
+  for (int bt = 2; bt <= g.To && bt <= kTileM && bt * g.st <= 256; ++bt)
+    for (int bh = 1; bh <= g.Ho && bt * bh <= kTileM && bh * g.sh <= 256; ++bh) {
+      int bw = kTileM / (bt * bh);
+      if (bw > g.Wo) bw = g.Wo;
+      if (bw * g.sw > 256) continue;
+      bw = ceil_div(g.Wo, ceil_div(g.Wo, bw));              // no wider than the columns need
+      const long long tiles = (long long)g.n * ceil_div(g.To, bt) * ceil_div(g.Ho, bh) * ceil_div(g.Wo, bw);
+      if (tiles * 16 > fewest * 17) continue;
+      const double cost = double(tiles) * (double(bt + g.Kt - 1) * bh * bw + g.Kt * 0.5 * n_tile);
+      if (best < 0 || cost < best) { best = cost; *out = TileBox{1, bt, bh, bw}; }
+    }
+  return best >= 0 ? best / (double(fewest) * g.Kt * (kTileM + 0.5 * n_tile)) : 2.0;
+}
+
 // Bundle width, number of K splits and kernel (single CTAs or CTA pairs) for a call.  Model, fitted to timings on B200:
 //  - A K step takes its tensor time or the time its operands need from L2, 65 bytes per clock and SM whatever the kernel
 //    (at 128 columns 32 KB for a CTA, 24 KB for one of a pair, 14 KB where the kt steps share an input tile): this bounds
@@ -982,7 +1004,7 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.pool_t = pl_t; a.pool_h = pl_h; a.pool_w = pl_w; a.sbw = sb[0]; a.sbh = sb[1];
   a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
   a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
-  const long long m_tiles = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
+  long long m_tiles = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
   UmmaPlan plan = pick_plan(w, g, m_tiles, d->sm_count);
   if (pooled) {                     // pooling lives in the TMA-store epilogue, which a K split does not use
     // A layer this small is faster split over K and pooled by a second launch: AUTO declines the fusion.
@@ -1021,6 +1043,19 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     }
     probe.n_tile = plan.n_tile; probe.n_bundles = ceil_div(w->M, plan.n_tile); probe.dense = dense_entry ? 1 : 0;
     use_ts = umma_pair_ts_supported(&probe, w->Ks * ceil_div(w->N, kChunk) * probe.n_bundles);
+    const double ratio = use_ts || pooled ? 2.0 : choose_box_grouped(g, plan.n_tile, m_tiles, &deep);
+    const bool rect2 = ratio < 1.0 && warp_block(deep.bw, deep.bh, deep.bt, deep.bn, sb2);
+    if (ratio <= (rect && !rect2 ? 0.6 : g.sh * g.sw > 1 ? 0.68 : 0.8)) {
+      probe.box = deep;
+      probe.sbw = sb2[0]; probe.sbh = sb2[1];
+      probe.tiles_n = g.n; probe.tiles_t = ceil_div(g.To, deep.bt);
+      probe.tiles_h = ceil_div(g.Ho, deep.bh); probe.tiles_w = ceil_div(g.Wo, deep.bw);
+      use_ts = umma_pair_ts_supported(&probe, w->Ks * ceil_div(w->N, kChunk) * probe.n_bundles);
+      if (use_ts) {
+        rect = rect2;
+        m_tiles = (long long)probe.tiles_n * probe.tiles_t * probe.tiles_h * probe.tiles_w;
+      }
+    }
     if (use_ts) {
       a.box = probe.box; a.sbw = probe.sbw; a.sbh = probe.sbh;
       a.tiles_n = probe.tiles_n; a.tiles_t = probe.tiles_t; a.tiles_h = probe.tiles_h; a.tiles_w = probe.tiles_w;

@@ -32,6 +32,7 @@ CASES = [
     (64, 128, (3, 3, 3), (1, 2, 2), (2, 8, 32, 32), (4, 4), "bernoulli", False, False),     # spatial stride
     (64, 64, (7, 1, 1), (2, 1, 1), (2, 16, 40, 40), (4, 4), "bernoulli", False, False),     # temporal stride 2: two phase tiles
     (64, 96, (5, 3, 3), (2, 1, 1), (2, 16, 20, 20), (4, 4), "bernoulli", False, True),      # the same, five taps, every tile split
+    (21, 33, (3, 3, 3), (1, 1, 1), (2, 10, 43, 39), (4, 4), "bernoulli", False, False),     # 286 deep boxes for 275 of two clips
 ]
 
 
