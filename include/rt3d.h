@@ -299,6 +299,17 @@ rt3d_status rt3d_maxpool3d(const rt3d_tensor* x, int kt, int kh, int kw, int st,
 /* y = a + b (optionally ReLU); equal extents and dtype; y may alias a or b. */
 rt3d_status rt3d_add_relu(const rt3d_tensor* a, const rt3d_tensor* b, int relu, rt3d_tensor* y, void* stream);
 
+/* rt3d_copy_f32 - n small copies of device memory in one launch: dst[i] = src[i], zeros where src is NULL.  `copies` is a HOST
+ * array that is read during the call.  No dst may overlap another dst or a src.  (Layers that run as one, see
+ * rt3d_pack_concat, bring their biases together with it; enqueued in front of the convolution it reads what the biases hold
+ * at that point of the stream.)  Errors: INVALID_ARG (no dst, count < 1, n < 1), CUDA. */
+typedef struct {
+  const float* src;      /* device, or NULL                                                      */
+  float*  dst;           /* device                                                               */
+  int32_t count;         /* values                                                               */
+} rt3d_copy;
+rt3d_status rt3d_copy_f32(const rt3d_copy* copies, int32_t n, void* stream);
+
 /*
  * Pruning step on the device (Section 4), the stage right before rt3d_pack_kgs.  All pointers DEVICE.
  * rt3d_kgs_group_norms: norms[p][q][k] = group-lasso norm of the weights of kernel group (p,q) at
@@ -324,9 +335,10 @@ rt3d_status rt3d_kgs_expand_mask(const uint8_t* group_mask, int M, int N, int Kt
  *   lane      index into `streams`: the stream the call goes to
  *   RECORD / WAIT  k[0] = slot: the slot takes the lane's work so far / the lane waits for what the slot took last
  * Calls:  SPARSE, DENSE (x, w, bias, p, y); FUSED (and r = residual or data NULL, k[0..2] = pool_t/h/w); PAIR (x, w, bias,
- * p, w2, bias2, p2, r, y); MAXPOOL (x, k[0..8] = kt kh kw st sh sw pt ph pw, y); ADD (x, r = second addend, k[0] = relu, y). */
+ * p, w2, bias2, p2, r, y); MAXPOOL (x, k[0..8] = kt kh kw st sh sw pt ph pw, y); ADD (x, r = second addend, k[0] = relu, y);
+ * COPY (x.data = HOST array of rt3d_copy, k[0] = its length). */
 enum { RT3D_CALL_SPARSE = 0, RT3D_CALL_DENSE = 1, RT3D_CALL_FUSED = 2, RT3D_CALL_PAIR = 3, RT3D_CALL_MAXPOOL = 4,
-       RT3D_CALL_ADD = 5, RT3D_CALL_RECORD = 6, RT3D_CALL_WAIT = 7 };
+       RT3D_CALL_ADD = 5, RT3D_CALL_RECORD = 6, RT3D_CALL_WAIT = 7, RT3D_CALL_COPY = 8 };
 #define RT3D_CALL_SLOTS 8
 typedef struct {
   int32_t kind, lane;

@@ -49,7 +49,12 @@ class Call(ctypes.Structure):
                 ("p", ConvParams), ("p2", ConvParams), ("k", ctypes.c_int32 * 9)]
 
 
-(CALL_SPARSE, CALL_DENSE, CALL_FUSED, CALL_PAIR, CALL_MAXPOOL, CALL_ADD, CALL_RECORD, CALL_WAIT), CALL_SLOTS = range(8), 8
+(CALL_SPARSE, CALL_DENSE, CALL_FUSED, CALL_PAIR, CALL_MAXPOOL, CALL_ADD, CALL_RECORD, CALL_WAIT, CALL_COPY) = range(9)
+CALL_SLOTS = 8
+
+
+class Copy(ctypes.Structure):
+    _fields_ = [("src", ctypes.c_void_p), ("dst", ctypes.c_void_p), ("count", ctypes.c_int32)]
 
 
 class Fusion(ctypes.Structure):
@@ -95,6 +100,7 @@ def _load():
     lib.rt3d_kgs_expand_mask.argtypes = [vp, i, i, i, i, i, i, i, vp, vp]
     lib.rt3d_run_calls.argtypes = [ctypes.POINTER(Call), ctypes.c_int32, ctypes.POINTER(vp), ctypes.c_int32,
                                    ctypes.POINTER(ctypes.c_int32)]
+    lib.rt3d_copy_f32.argtypes = [ctypes.POINTER(Copy), ctypes.c_int32, vp]
     lib.rt3d_maxpool3d.argtypes = [TP] + [i] * 9 + [TP, vp]
     lib.rt3d_add_relu.argtypes = [TP, TP, i, TP, vp]
     i64p = ctypes.POINTER(ctypes.c_int64)
@@ -374,6 +380,12 @@ class CallSequence:
             c.k[i] = int(v)
         self.calls.append(c)
 
+    def note_copies(self, stream, arr, copies):
+        c = Call(kind=CALL_COPY, lane=self._lane(stream), x=Tensor(ctypes.addressof(arr)))
+        c.k[0] = len(arr)
+        self.keep.append((arr, copies))
+        self.calls.append(c)
+
     def note_event(self, kind, stream, event):
         """Work recorded into / waited for through a torch event, on a torch stream."""
         if kind == CALL_RECORD:
@@ -479,6 +491,17 @@ def rt3d_add_relu(a: Tensor, b: Tensor, relu: bool, y: Tensor, stream=None):
     _check(_lib.rt3d_add_relu(ctypes.byref(a), ctypes.byref(b), int(bool(relu)), ctypes.byref(y),
                               _stream_ptr(stream)), "rt3d_add_relu")
     _note(CALL_ADD, stream, a, y, b, k=(bool(relu),))
+
+
+def rt3d_copy_f32(copies, stream=None):
+    """copies: (source, destination, first value, count) each, float32 device tensors: the source (zeros where it is None) goes to
+    the destination's values from `first` on."""
+    arr = (Copy * len(copies))(*(Copy(None if s is None else s.data_ptr(), d.data_ptr() + 4 * int(first), int(count))
+                                 for s, d, first, count in copies))
+    _check(_lib.rt3d_copy_f32(arr, len(arr), _stream_ptr(stream)), "rt3d_copy_f32")
+    seq = noting()
+    if seq is not None:
+        seq.note_copies(stream, arr, copies)
 
 
 def rt3d_kgs_group_norms(w, g_m: int, g_n: int, norm: int, norms, stream=None):

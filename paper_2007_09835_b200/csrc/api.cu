@@ -1401,6 +1401,19 @@ rt3d_status rt3d_add_relu(const rt3d_tensor* a, const rt3d_tensor* b, int relu, 
   return RT3D_OK;
 }
 
+rt3d_status rt3d_copy_f32(const rt3d_copy* copies, int32_t n, void* stream) {
+  if (!copies || n < 1) return RT3D_ERR_INVALID_ARG;
+  for (int32_t i = 0; i < n; ++i)
+    if (!copies[i].dst || copies[i].count < 1) return RT3D_ERR_INVALID_ARG;
+  if (t_plan_only) return RT3D_OK;
+  for (int32_t i = 0; i < n; i += kCopiesPerLaunch) {
+    if (launch_copy_f32(copies + i, std::min(n - i, kCopiesPerLaunch), static_cast<cudaStream_t>(stream)) != cudaSuccess)
+      return RT3D_ERR_CUDA;
+    g_launches.fetch_add(1);
+  }
+  return RT3D_OK;
+}
+
 rt3d_status rt3d_run_calls(const rt3d_call* calls, int32_t n, void* const* streams, int32_t n_streams, int32_t* failed) {
   if (failed) *failed = -1;
   if (!calls || n < 0 || !streams || n_streams < 1) return RT3D_ERR_INVALID_ARG;
@@ -1441,6 +1454,7 @@ rt3d_status rt3d_run_calls(const rt3d_call* calls, int32_t n, void* const* strea
           s = rt3d_maxpool3d(&c.x, c.k[0], c.k[1], c.k[2], c.k[3], c.k[4], c.k[5], c.k[6], c.k[7], c.k[8], &y, st);
           break;
         case RT3D_CALL_ADD: s = rt3d_add_relu(&c.x, &c.r, c.k[0], &y, st); break;
+        case RT3D_CALL_COPY: s = rt3d_copy_f32(static_cast<const rt3d_copy*>(c.x.data), c.k[0], st); break;
         case RT3D_CALL_RECORD:
         case RT3D_CALL_WAIT: {
           if (c.k[0] < 0 || c.k[0] >= RT3D_CALL_SLOTS) break;

@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "rt3d.h"
 #include "tile_consts.h"
 
 namespace rt3d {
@@ -60,6 +61,9 @@ cudaError_t launch_maxpool3d(int dtype, const void* x, int n, int t, int h, int 
                              int kt, int kh, int kw, int st, int sh, int sw, int pt, int ph, int pw,
                              void* y, int To, int Ho, int Wo, int ycs, cudaStream_t stream);
 
+// At most kCopiesPerLaunch copies (1.5 KB of the 4 KB that a kernel's arguments may take).
+constexpr int kCopiesPerLaunch = 64;
+cudaError_t launch_copy_f32(const rt3d_copy* copies, int n, cudaStream_t stream);
 cudaError_t launch_add_relu(int dtype, const void* a, int acs, const void* b, int bcs, void* y, int ycs,
                             int64_t voxels, int c, int relu, cudaStream_t stream);
 

@@ -9,6 +9,8 @@
 // register-blocked fp32 kernel (simt_conv_f32.cu) does: kernel groups that are not whole 4 x 4 tiles, mostly.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 #include "pdl.cuh"
 
@@ -387,7 +389,23 @@ __global__ void add_relu_bf16x8_kernel(const uint4* __restrict__ a, int acs8, co
   y[(long long)v * ycs8 + cc] = out;
 }
 
+// A few hundred values to a copy, one block each: the launch is all it costs (S3D: 26 copies before a forward pass of 830 us).
+// The descriptors travel as the kernel's argument, so nothing on the host has to outlive the call.
+struct CopyList { rt3d_copy at[kCopiesPerLaunch]; };
+__global__ void copy_f32_kernel(const __grid_constant__ CopyList list) {
+  pdl_entry();
+  const rt3d_copy& c = list.at[blockIdx.x];
+  for (int i = threadIdx.x; i < c.count; i += blockDim.x) c.dst[i] = c.src ? c.src[i] : 0.f;
+}
+
 }  // namespace
+
+cudaError_t launch_copy_f32(const rt3d_copy* copies, int n, cudaStream_t stream) {
+  CopyList list{};
+  std::copy(copies, copies + n, list.at);
+  LaunchSetup ls(dim3(unsigned(n)), dim3(256), 0, stream);
+  return cudaLaunchKernelEx(&ls.cfg, copy_f32_kernel, list);
+}
 
 cudaError_t launch_conv_simt(int dtype, const ConvGeom& g, const void* x, void* y, const int32_t* group_ptr,
                              const uint16_t* pos_idx, const void* tiles, const float* bias, int g_m, int g_n,

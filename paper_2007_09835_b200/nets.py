@@ -19,7 +19,7 @@ _pycall, _ADDRESS = B.pycall(), B.ADDRESS
 # The binding's compute functions as they are: calls go round them only while they are what the binding's module holds (a
 # tracer or a test that wraps them sees every call).
 _FUNCTIONS = {fn: getattr(B, fn) for fn in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_sparse_fused",
-                                            "rt3d_conv2plus1d_fused", "rt3d_maxpool3d", "rt3d_add_relu")}
+                                            "rt3d_conv2plus1d_fused", "rt3d_maxpool3d", "rt3d_add_relu", "rt3d_copy_f32")}
 
 
 def _unwrapped(*names) -> bool:
@@ -451,9 +451,10 @@ class S3DNet(_NotedForward):
         parts = [self.layers[sp.name] for sp in specs]
         made = self.__dict__.setdefault("_concats", {})
         key = tuple(sp.name for sp in specs)
-        now = [(p.packed, p.bias) for p in parts]
-        if key not in made or any(a is not c or b is not d for (a, b), (c, d) in zip(made[key][0], now)):
+        now = [(p.packed, bool(p.packed.handle), p.spec, p.bias is None) for p in parts]
+        if key not in made or made[key][0] != now:
             layer = None
+            specs = [p.spec for p in parts]
             if all(sp.relu == specs[0].relu and sp.stride == specs[0].stride and sp.pad == specs[0].pad for sp in specs) and \
                     len({p.dtype for p in parts}) == 1 and all(sp.cout % 8 == 0 for sp in specs):
                 try:
@@ -466,23 +467,43 @@ class S3DNet(_NotedForward):
                     layer.spec = dataclasses.replace(specs[0], name="+".join(key), cout=sum(sp.cout for sp in specs))
                     layer.dtype, layer.dense, layer.device = parts[0].dtype, parts[0].dense, parts[0].device
                     layer.packed = packed
-                    layer.bias = None if all(p.bias is None for p in parts) else torch.cat(
-                        [torch.zeros(sp.cout, device=p.device) if p.bias is None else p.bias for sp, p in zip(specs, parts)])
+                    layer.bias = None               # filled from the parts' biases by _merged at every pass
+                    if any(p.bias is not None for p in parts):
+                        layer.bias = torch.empty(layer.spec.cout, device=parts[0].device)
             made[key] = (now, layer)
         return made[key][1]
 
-    def _block(self, op, x, off, last, algo, stream, merge):
+    def _merged(self, stream):
+        """The merged convolutions by block name: (all three, None), (None, the two reductions) or neither.  Their biases are
+        brought together in one launch on the device: every pass, a captured one too, reads what the layers' biases hold."""
+        found, copies = {}, []
+        for i, op in enumerate(self.plan):
+            if not hasattr(op, "b0"):
+                continue
+            last = i + 1 == len(self.plan)
+            specs = (op.b1[0], op.b2[0]) if last else (op.b1[0], op.b2[0], op.b0)
+            layer = self._concat(specs)
+            found[op.name] = (None, layer) if last else (layer, None)
+            if layer is not None and layer.bias is not None:
+                first = 0
+                for part in (self.layers[sp.name] for sp in specs):
+                    copies.append((part.bias, layer.bias, first, part.spec.cout))
+                    first += part.spec.cout
+        if copies:
+            B.rt3d_copy_f32(copies, stream)
+        return found
+
+    def _block(self, op, x, off, algo, stream, merged):
         """One Inception block on channels [off, off + cin) of x; returns (output tensor, first channel of the output in it).
 
-        The three 1x1x1 convolutions that read the block's input run as one where the layers allow it (`merge`): a third of
+        The three 1x1x1 convolutions that read the block's input run as one where the layers allow it (`merged`): a third of
         the reads of x and of the launches.  It writes [b1 reduction | b2 reduction | b0] side by side, so the block's output
         then lies behind the reductions in one wide tensor, on a 128-byte boundary; the last block, whose output is the
         network's, merges the two reductions only."""
         n, t, h, w, _ = x.shape
         xd = B.channel_slice_desc(x, off, op.cin)
         r1, r2 = op.b1[0].cout, op.b2[0].cout
-        wide = self._concat((op.b1[0], op.b2[0], op.b0)) if merge and not last else None
-        both = self._concat((op.b1[0], op.b2[0])) if merge and last else None
+        wide, both = merged
         if wide is not None:
             start = -(-(r1 + r2) // 64) * 64                        # first channel of the output
             out = self.ws.get(op.name + ".wide", (n, t, h, w, start + -(-op.cout // 64) * 64), x.dtype, x.device)
@@ -547,9 +568,10 @@ class S3DNet(_NotedForward):
 
     def _forward(self, x, algo, keep, stream):
         c, off = self.plan[0].cin, 0
+        merged = self._merged(stream) if keep is None else {}
         for i, op in enumerate(self.plan):
             if hasattr(op, "b0"):                                   # Inception block
-                x, off = self._block(op, x, off, i + 1 == len(self.plan), algo, stream, keep is None)
+                x, off = self._block(op, x, off, algo, stream, merged.get(op.name, (None, None)))
                 c = op.cout
             elif hasattr(op, "cout"):
                 if off:                                             # behind a wide block

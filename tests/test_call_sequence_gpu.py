@@ -76,3 +76,24 @@ def test_layer_call_refuses_what_the_descriptor_refuses():
             lay(bad, torch.zeros_like(x))
     with pytest.raises(rt3d.Rt3dError):
         lay(x, x)                                                 # overlapping buffers
+
+
+def test_small_copies_in_one_launch():
+    """As many as a launch takes, one more, and lengths around a block's threads; values beside a destination stay."""
+    src = torch.randn(70 * 300, device="cuda")
+    dst = torch.full((70 * 301,), 7.0, device="cuda")
+    for n in (1, 64, 65, 70):
+        out, want, copies = dst.clone(), dst.clone(), []
+        for i in range(n):
+            count = (1, 255, 256, 257, 300)[i % 5]
+            s = None if i % 7 == 3 else src[300 * i: 300 * i + count]
+            copies.append((s, out, 301 * i, count))
+            want[301 * i: 301 * i + count] = 0 if s is None else s
+        launches = rt3d.rt3d_launch_count()
+        rt3d.rt3d_copy_f32(copies)
+        assert rt3d.rt3d_launch_count() - launches == -(-n // 64)
+        assert torch.equal(out, want)
+    for bad in ([], [(src, dst, 0, 0)]):
+        with pytest.raises(rt3d.Rt3dError) as e:
+            rt3d.rt3d_copy_f32(bad)
+        assert e.value.status == rt3d.ERR_INVALID_ARG

@@ -379,3 +379,49 @@ def test_c3d_batch1_graph_replays_give_the_same_bits(c3d):
         bad += 0 if torch.equal(y, y0) else 1
     assert bad == 0, f"{bad} of 1500 replays differ from the first"
     assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+# --------------------------------------------------------- S3D-shaped: the 1x1x1 convolutions of a block as one
+def merged_net(plan, layers):
+    net = nets.S3DNet(plan, device_layers(layers, synth.s3d_convs(plan)))
+    return net, len([op for op in plan if isinstance(op, synth.InceptionSpec)])
+
+
+def test_s3d_merged_forward_matches_reference(s3d):
+    """The pass that a user makes: nothing collects the layers' outputs, so the convolutions that read a block's input run
+    as one.  Held to the reference like the pass that keeps every output."""
+    plan, layers, x, rec, final = s3d
+    net, blocks = merged_net(plan, layers)
+    xd = nets.to_device(x)
+    for _ in range(2):                                    # the pass that is noted, and the noted one
+        y = nets.to_numpy(net.forward(xd), 1024)
+        assert y.shape == (1, 2, 7, 7, 1024)
+        assert rel_err(y, final) <= TOL_FREE
+    assert len(net._concats) == blocks and all(layer is not None for _, layer in net._concats.values())
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+def test_s3d_merged_forward_reads_the_biases_at_every_pass(s3d):
+    """A bias written in place counts from the next pass on, whether the pass is noted, replayed as a graph or neither,
+    and whether or not the tensor's version counter saw the write."""
+    plan, layers, x, rec, final = s3d
+    net, _ = merged_net(plan, layers)
+    xd = nets.to_device(x)
+    old = net.forward(xd).clone()
+    graph = nets.GraphedForward(net, xd)
+    blocks = [op for op in plan if isinstance(op, synth.InceptionSpec)]
+    rng = np.random.default_rng(3)
+    for i, op in enumerate((blocks[0], blocks[4], blocks[-1])):
+        for sp in (op.b0, op.b1[0], op.b2[0]):
+            new = torch.from_numpy(rng.normal(0, 0.3, sp.cout).astype(np.float32))
+            layers = {**layers, sp.name: {**layers[sp.name], "bias": new.numpy()}}
+            bias = net.layers[sp.name].bias
+            (bias.data if i == 1 else bias).copy_(new)
+        want = merged_net(plan, layers)[0].forward(xd)
+        assert not torch.equal(want, old)
+        assert torch.equal(net.forward(xd), want)
+        assert torch.equal(graph(), want)
+        unmerged = nets.to_numpy(net.forward(xd, keep={}), 1024)
+        assert rel_err(nets.to_numpy(want, 1024), unmerged) <= TOL_FREE
+        old = want.clone()
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
