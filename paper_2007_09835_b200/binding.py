@@ -9,7 +9,9 @@ from __future__ import annotations
 
 import contextlib
 import ctypes
+import itertools
 import os
+import sys
 import threading
 
 import numpy as np
@@ -199,15 +201,21 @@ class Packed:
         _check(_lib.rt3d_packed_prepare(self.handle), "rt3d_packed_prepare")
 
     def free(self):
+        global _last_free
         if self.handle:
-            _lib.rt3d_packed_free(self.handle)
-            self.handle = ctypes.c_void_p(None)
+            h, self.handle = self.handle, ctypes.c_void_p(None)
+            _last_free = next(_frees)           # before the memory goes: who notices looks at the handle again
+            _lib.rt3d_packed_free(h)
 
-    def __del__(self):
+    def __del__(self):                          # nobody holds it any more, so no sequence of calls does
         try:
-            self.free()
+            if self.handle:
+                _lib.rt3d_packed_free(self.handle)
         except Exception:
             pass
+
+
+_frees, _last_free = itertools.count(1), 0      # handles freed while somebody may hold them: a value of its own for each
 
 
 def _np_f32(a):
@@ -349,6 +357,7 @@ class CallSequence:
     def __init__(self, x_ptr: int, stream_ptr: int):
         self.x_ptr, self.calls, self.keep, self.lanes, self.slots = x_ptr, [], [], [stream_ptr], {}
         self.array = None
+        self.handles, self.biases, self.last_free = {}, {}, _last_free
 
     @contextlib.contextmanager
     def noting(self):
@@ -373,9 +382,10 @@ class CallSequence:
             if h is not None:
                 setattr(c, names[0], h.handle)
                 setattr(c, names[2], q)
+                self.handles[id(h)] = h
             if b is not None:
                 setattr(c, names[1], b.data_ptr())
-            self.keep.append((h, b))
+                self.biases[id(b)] = (b, getattr(c, names[1]))
         for i, v in enumerate(k):
             c.k[i] = int(v)
         self.calls.append(c)
@@ -383,6 +393,7 @@ class CallSequence:
     def note_copies(self, stream, arr, copies):
         c = Call(kind=CALL_COPY, lane=self._lane(stream), x=Tensor(ctypes.addressof(arr)))
         c.k[0] = len(arr)
+        self.biases.update((id(s), (s, a.src)) for a, (s, _, _, _) in zip(arr, copies) if s is not None)
         self.keep.append((arr, copies))
         self.calls.append(c)
 
@@ -395,11 +406,26 @@ class CallSequence:
         c.k[0] = self.slots[id(event)]
         self.calls.append(c)
 
-    def finish(self):
+    def finish(self, out, buffers):
+        """out: the tensor that the pass returns; buffers: its activation buffers, whose memory stays while the sequence does."""
         self.array = (Call * len(self.calls))(*self.calls)
+        self.keep.append([b.untyped_storage() for b in buffers])
+        held = [(out, out.data_ptr()), *self.biases.values()]
+        self.tensors = tuple(t for t, _ in held)
+        self.addresses = b"".join((p or 0).to_bytes(8, sys.byteorder) for _, p in held)
         self.inputs = [t for c in self.array for t in (c.x, c.r) if t.data == self.x_ptr]
         self.streams = (ctypes.c_void_p * len(self.lanes))(*self.lanes)
         self.calls = None
+
+    def holds(self) -> bool:
+        """Whether the handles are still there and the biases and the output where they were (their tensors may have been given
+        other memory since)."""
+        if self.last_free != _last_free:
+            seen = _last_free
+            if not all(h.handle for h in self.handles.values()):
+                return False
+            self.last_free = seen
+        return pycall().pointers_are(self.tensors, self.addresses)
 
     def run(self, x_ptr: int, stream_ptr: int) -> int:
         """Status of the run; the side streams are the ones of the first pass."""

@@ -165,6 +165,22 @@ PyObject* expand_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {   // addres
       reinterpret_cast<void*>(stream)));
 }
 
+// pointers_are(tensors, addresses): whether every tensor of a tuple still has its address of a bytes object (8 bytes each).
+PyObject* pointers_are(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (!want(n, 2)) return nullptr;
+  if (!PyTuple_Check(a[0]) || !PyBytes_Check(a[1]) || PyBytes_GET_SIZE(a[1]) != PyTuple_GET_SIZE(a[0]) * Py_ssize_t(sizeof(uintptr_t))) {
+    PyErr_SetString(PyExc_TypeError, "a tuple of tensors and their addresses");
+    return nullptr;
+  }
+  for (Py_ssize_t i = 0; i < PyTuple_GET_SIZE(a[0]); ++i) {
+    uintptr_t now, then;
+    if (!data_ptr(PyTuple_GET_ITEM(a[0], i), &now)) return nullptr;
+    __builtin_memcpy(&then, PyBytes_AS_STRING(a[1]) + i * sizeof(then), sizeof(then));
+    if (now != then) Py_RETURN_FALSE;
+  }
+  Py_RETURN_TRUE;
+}
+
 // conv(address, x, c_in, handle, bias, params, y, c_out, stream[, residual, (pool_t, pool_h, pool_w)]) -> status.
 // With the last two the address is rt3d_conv3d_sparse_fused's, else rt3d_conv3d_sparse's or _dense's.
 PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -221,6 +237,8 @@ PyMethodDef methods[] = {
     {"group_norms", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(group_norms)), METH_FASTCALL, ""},
     {"reweight", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(reweight)), METH_FASTCALL, ""},
     {"expand_mask", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(expand_mask)), METH_FASTCALL, ""},
+    {"pointers_are", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(pointers_are)), METH_FASTCALL,
+     "pointers_are(tensors, addresses) -> bool"},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

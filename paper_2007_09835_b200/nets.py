@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import contextlib
 import dataclasses
+import itertools
 
 import numpy as np
 import torch
@@ -45,7 +46,8 @@ def to_numpy(t: torch.Tensor, c: int) -> np.ndarray:
     return t[..., :c].float().cpu().numpy()
 
 
-_layer_changes = 0      # counts assignments to any layer's attributes: a noted sequence of calls holds from one to the next
+# The last assignment to any layer's attribute, a value of its own for each: a noted sequence of calls holds from one to the next.
+_changes, _layer_changes = itertools.count(1), 0
 
 
 class ConvLayer:
@@ -53,9 +55,9 @@ class ConvLayer:
 
     def __setattr__(self, name, value):
         global _layer_changes
-        _layer_changes += 1
         object.__setattr__(self, name, value)
         object.__setattr__(self, "_params", {})     # parameter structures by (ReLU, kernel family, zero padding, concurrent)
+        _layer_changes = next(_changes)
 
     def __init__(self, spec, w, bias, mask, g_m=4, g_n=4, dtype=torch.bfloat16, dense=False, device="cuda"):
         self.spec = spec
@@ -172,7 +174,8 @@ def _wait(stream, ev):
 class _NotedForward:
     """Base of the networks.  The calls of a forward pass are noted when an input of its shape is seen first, and issued
     by one library call from then on (R(2+1)D: 33 calls, 590 us of Python; S3D: 90 calls and 36 stream events, 1730 us).
-    Noted passes are dropped when a layer, a switch of the network or its set of buffers has changed since."""
+    Noted passes are dropped when a layer, the memory of a bias or of the output, a switch of the network or its set of
+    buffers has changed since."""
 
     _SWITCHES = ()          # attributes that decide which calls a pass makes
     _MOST = 8               # input shapes remembered
@@ -190,20 +193,22 @@ class _NotedForward:
         found = noted.get(key)
         if found is not None:
             seq, out, buffers, changes, layers, state = found
-            if changes == _layer_changes and layers == self._all_layers() and state == self._state() and ptr not in buffers:
+            if changes == _layer_changes and layers == self._all_layers() and state == self._state() and ptr not in buffers and \
+                    seq.holds():
                 status = seq.run(ptr, B.current_stream_ptr() if stream is None else int(stream))
                 if status == B.OK:
                     return out
             del noted[key]
         seq = B.CallSequence(ptr, B.current_stream_ptr() if stream is None else int(stream))
+        changes = _layer_changes
         with seq.noting():
             out = self._forward(x, algo, None, stream)
         buffers = {b.data_ptr(): b for b in self.ws.bufs.values()}      # kept alive as long as the noted calls
         if ptr not in buffers:
-            seq.finish()
+            seq.finish(out, buffers.values())
             if len(noted) >= self._MOST:
                 noted.pop(next(iter(noted)))
-            noted[key] = (seq, out, buffers, _layer_changes, self._all_layers(), self._state())
+            noted[key] = (seq, out, buffers, changes, self._all_layers(), self._state())
         return out
 
 
@@ -464,12 +469,12 @@ class S3DNet(_NotedForward):
                         raise
                 else:
                     layer = object.__new__(ConvLayer)
-                    layer.spec = dataclasses.replace(specs[0], name="+".join(key), cout=sum(sp.cout for sp in specs))
-                    layer.dtype, layer.dense, layer.device = parts[0].dtype, parts[0].dense, parts[0].device
-                    layer.packed = packed
-                    layer.bias = None               # filled from the parts' biases by _merged at every pass
-                    if any(p.bias is not None for p in parts):
-                        layer.bias = torch.empty(layer.spec.cout, device=parts[0].device)
+                    cout = sum(sp.cout for sp in specs)
+                    vars(layer).update(             # no assignment: what other passes have noted still holds
+                        spec=dataclasses.replace(specs[0], name="+".join(key), cout=cout), packed=packed, _params={},
+                        dtype=parts[0].dtype, dense=parts[0].dense, device=parts[0].device,
+                        # filled from the parts' biases by _merged at every pass
+                        bias=torch.empty(cout, device=parts[0].device) if any(p.bias is not None for p in parts) else None)
             made[key] = (now, layer)
         return made[key][1]
 

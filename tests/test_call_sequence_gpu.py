@@ -78,6 +78,59 @@ def test_layer_call_refuses_what_the_descriptor_refuses():
         lay(x, x)                                                 # overlapping buffers
 
 
+@pytest.mark.parametrize("name,clip", [("c3d", (16, 112, 112, 3)), ("r2plus1d", (4, 56, 56, 3)), ("s3d", (8, 96, 96, 3))])
+def test_noted_forward_follows_a_bias_whose_storage_was_replaced(name, clip):
+    net, _ = bench.build_network(name)
+    x = nets.to_device(synth.make_input(9, (2,) + clip))
+    before = net.forward(x).clone()
+    old = []                                                      # the old storages stay in use
+    for layer in net.layers.values():
+        old.append(layer.bias.data)
+        layer.bias.data = layer.bias.data + 0.25
+    changed = net.forward(x).clone()
+    assert not torch.equal(changed, before)
+    assert torch.equal(changed, net._forward(x, 0, None, None))
+    assert torch.equal(changed, net.forward(x))
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+@pytest.mark.parametrize("name,clip", [("c3d", (16, 112, 112, 3)), ("s3d", (8, 96, 96, 3))])
+def test_noted_forward_writes_the_tensor_that_it_returns(name, clip):
+    net, _ = bench.build_network(name)
+    x = nets.to_device(synth.make_input(9, (2,) + clip))
+    y = net.forward(x)
+    want, old = y.clone(), y.data                                 # the old storage stays in use
+    y.data = torch.zeros_like(y)
+    again = net.forward(x)
+    assert torch.equal(again, want)
+    assert again.data_ptr() == y.data_ptr() != old.data_ptr()
+
+
+@pytest.mark.parametrize("name,clip", [("c3d", (16, 112, 112, 3)), ("r2plus1d", (4, 56, 56, 3)), ("s3d", (8, 96, 96, 3))])
+def test_noted_forward_refuses_a_freed_layer(name, clip):
+    """A handle freed by hand is refused by the next pass, as a layer's own call refuses it; one that nobody uses, or that
+    went with its last reference, leaves the notes alone."""
+    net, _ = bench.build_network(name)
+    x = nets.to_device(synth.make_input(9, (1,) + clip))
+    want = net.forward(x).clone()
+    noted = list(net._noted.values())
+    spec = synth.ConvSpec("l", 16, 16, (1, 1, 1), (1, 1, 1), (0, 0, 0), True)
+    L = synth.make_layer(spec, 3, 0, 4, 4, "none", None)
+    for by_hand in (True, False):
+        other = rt3d.rt3d_pack_dense(L["w"], rt3d.RT3D_BF16)
+        if by_hand:
+            other.free()
+        del other
+        assert torch.equal(net.forward(x), want)
+        assert [a[0] for a in net._noted.values()] == [a[0] for a in noted]
+    list(net.layers.values())[-1].packed.free()
+    for _ in range(2):
+        with pytest.raises(rt3d.Rt3dError) as e:
+            net.forward(x)
+        assert e.value.status == rt3d.ERR_INVALID_ARG
+    torch.cuda.synchronize()
+
+
 def test_small_copies_in_one_launch():
     """As many as a launch takes, one more, and lengths around a block's threads; values beside a destination stay."""
     src = torch.randn(70 * 300, device="cuda")
