@@ -276,12 +276,12 @@ rt3d_status get_blob(rt3d_packed* h, DeviceBlob** out) {
   std::lock_guard<std::mutex> lock(h->mu);
   DeviceBlob* b = find_blob(h, dev);
   if (!b) {
-    b = new (std::nothrow) DeviceBlob;
-    if (!b) return RT3D_ERR_ALLOC;
-    b->device = dev;
-    h->blobs.push_back(b);
+    std::unique_ptr<DeviceBlob> made(new DeviceBlob);
+    made->device = dev;
+    h->blobs.reserve(h->blobs.size() + 1);
     std::lock_guard<std::mutex> reg(g_blobs_mu);
-    g_blobs.push_back(b);
+    g_blobs.push_back(made.get());
+    h->blobs.push_back(b = made.release());
   }
   *out = b;
   return RT3D_OK;
@@ -904,8 +904,8 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   return RT3D_OK;
 }
 
-rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
-                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz = nullptr) {
+rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
+                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz) {
   CallKey key;
   if (make_key(&key, x, wc, bias, p, y, fz ? fz->residual : nullptr, dense_entry ? 1 : 0)) {
     if (fz) { key.misc[2] = fz->pool_t; key.misc[3] = fz->pool_h; key.misc[4] = fz->pool_w; }
@@ -1114,7 +1114,7 @@ rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
 
 // Fused spatial -> temporal pair.  Argument errors first (as the two separate calls would report them), then
 // the eligibility screen of the one-kernel path.
-rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* wsc, const float* bias_s, const rt3d_conv_params* ps,
+rt3d_status conv2plus1d_body(const rt3d_tensor* x, const rt3d_packed* wsc, const float* bias_s, const rt3d_conv_params* ps,
                              const rt3d_packed* wtc, const float* bias_t, const rt3d_conv_params* pt,
                              const rt3d_tensor* res, rt3d_tensor* y, void* stream) {
   if (!wsc || !wtc || !ps || !pt || !y) return RT3D_ERR_INVALID_ARG;
@@ -1185,6 +1185,17 @@ rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* wsc, const
   });
 }
 
+// The two as the entry points call them: no exception leaves.
+rt3d_status conv_impl(const rt3d_tensor* x, const rt3d_packed* w, const float* bias, const rt3d_conv_params* p,
+                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz = nullptr) {
+  return c_entry([&] { return conv_body(x, w, bias, p, y, stream, dense_entry, fz); });
+}
+rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* ws, const float* bias_s, const rt3d_conv_params* ps,
+                             const rt3d_packed* wt, const float* bias_t, const rt3d_conv_params* pt,
+                             const rt3d_tensor* res, rt3d_tensor* y, void* stream) {
+  return c_entry([&] { return conv2plus1d_body(x, ws, bias_s, ps, wt, bias_t, pt, res, y, stream); });
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ entry point without allocation
@@ -1225,7 +1236,7 @@ rt3d_status rt3d_conv3d_host(const rt3d_tensor* x, rt3d_packed* w, const float* 
   rt3d_status s = make_geom(x, w, p, y, &g);
   if (s != RT3D_OK) return s;
   DeviceBlob* blob = nullptr;
-  if ((s = get_blob(w, &blob)) != RT3D_OK) return s;
+  if ((s = c_entry([&] { return get_blob(w, &blob); })) != RT3D_OK) return s;
   const size_t xb = size_t(tensor_span_bytes(x)), yb = size_t(tensor_span_bytes(y));
   {
     std::lock_guard<std::mutex> lock(w->mu);
@@ -1318,8 +1329,7 @@ rt3d_status rt3d_conv3d_host(const rt3d_tensor* x, rt3d_packed* w, const float* 
   return (cuda_ok && joined && synced) ? RT3D_OK : RT3D_ERR_CUDA;
 }
 
-rt3d_status rt3d_packed_prepare(rt3d_packed* p) {
-  if (!p) return RT3D_ERR_INVALID_ARG;
+static rt3d_status prepare_body(rt3d_packed* p) {
   DeviceState* d = nullptr;
   rt3d_status s = get_device_state(&d);
   if (s != RT3D_OK) return s;
@@ -1337,6 +1347,11 @@ rt3d_status rt3d_packed_prepare(rt3d_packed* p) {
   }
   for (int S = 2; S <= 8; ++S) umma_split_capacity(S, d->sm_count);      // what the K splits ask the runtime, once per device
   return cudaDeviceSynchronize() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
+}
+
+rt3d_status rt3d_packed_prepare(rt3d_packed* p) {
+  if (!p) return RT3D_ERR_INVALID_ARG;
+  return c_entry([&] { return prepare_body(p); });
 }
 
 void rt3d_packed_free(rt3d_packed* p) {
@@ -1464,7 +1479,8 @@ rt3d_status rt3d_run_calls(const rt3d_call* calls, int32_t n, void* const* strea
             for (Events& e : own.sets)
               if (e.device == dev) events = &e;
             if (!events) {
-              own.sets.emplace_back();
+              s = c_entry([&] { own.sets.emplace_back(); return RT3D_OK; });
+              if (s != RT3D_OK) break;
               events = &own.sets.back();
               events->device = dev;
             }

@@ -8,6 +8,7 @@
 #pragma once
 #include <cstddef>
 #include <mutex>
+#include <new>
 #include <unordered_map>
 #include <vector>
 
@@ -39,14 +40,19 @@ class KeptBlocks {
     for (void* g : gone) release_(g);
     return p;
   }
-  // Tells of a block that the caller allocated, so that give() knows its size.
-  void note(void* p, size_t bytes, int device) {
+  // Tells of a block that the caller allocated, so that give() knows its size; one that is not noted for want of memory is
+  // released there.
+  void note(void* p, size_t bytes, int device) noexcept {
     if (bytes < kSmallest || bytes > kMost / 2) return;
-    std::lock_guard<std::mutex> lock(mu_);
-    out_[p] = Block{p, bytes, device};
+    try {
+      std::lock_guard<std::mutex> lock(mu_);
+      kept_.reserve(out_.size() + kept_.size() + 1);      // room for all of them, so that give() allocates nothing
+      out_[p] = Block{p, bytes, device};
+    } catch (const std::bad_alloc&) {
+    }
   }
   // Keeps a block or releases it.
-  void give(void* p) {
+  void give(void* p) noexcept {
     if (!p) return;
     {
       std::lock_guard<std::mutex> lock(mu_);
@@ -67,7 +73,7 @@ class KeptBlocks {
  private:
   struct Block { void* p; size_t bytes; int device; };
   void drop_locked(std::vector<void*>& gone) {
-    for (const Block& b : kept_) gone.push_back(b.p);
+    for (const Block& b : kept_) gone.push_back(b.p);    // all of them, or none if it throws
     kept_.clear();
     total_ = 0;
   }

@@ -4,6 +4,8 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <new>
 #include <system_error>
 #include <thread>
@@ -51,7 +53,7 @@ static float tile_value(const rt3d_packed* p, int64_t e, int i, int j) {
 
 // Runs first(i) for i in [0, n), then between() once, then, unless that said no, second(i) for i in [0, n): on up to eight
 // threads if each gets at least `grain` units of work in all.  The threads are started once for both passes (starting and
-// joining seven costs 0.25 ms).
+// joining seven costs 0.25 ms).  What is thrown on any of them ends both passes early and is thrown again on this one.
 template <typename F, typename G, typename H>
 static void two_passes(int n, int64_t work, int64_t grain, const F& first, const G& between, const H& second) {
   const int threads = int(std::min<int64_t>(std::min<int64_t>(work / grain, n), std::min(8u, std::thread::hardware_concurrency())));
@@ -62,10 +64,21 @@ static void two_passes(int n, int64_t work, int64_t grain, const F& first, const
     return;
   }
   std::atomic<int> next[2] = {{0}, {0}}, done{0}, go{0};
+  std::atomic<bool> failed{false};
+  std::exception_ptr error;                              // of the thread that set `failed`; read after the join
   const int step = std::max(1, n / (threads * 8));       // pieces small enough to even out, large enough to be few
-  auto pass = [&](std::atomic<int>& at, const auto& fn) {
-    for (int i0 = at.fetch_add(step); i0 < n; i0 = at.fetch_add(step))
-      for (int i = i0; i < std::min(n, i0 + step); ++i) fn(i);
+  const auto guarded = [&](const auto& fn) {
+    try {
+      fn();
+    } catch (...) {
+      if (!failed.exchange(true)) error = std::current_exception();
+    }
+  };
+  const auto pass = [&](std::atomic<int>& at, const auto& fn) {
+    guarded([&] {
+      for (int i0 = at.fetch_add(step); i0 < n && !failed.load(std::memory_order_relaxed); i0 = at.fetch_add(step))
+        for (int i = i0; i < std::min(n, i0 + step); ++i) fn(i);
+    });
   };
   std::vector<std::thread> pool;
   pool.reserve(size_t(threads));
@@ -78,18 +91,16 @@ static void two_passes(int n, int64_t work, int64_t grain, const F& first, const
         if (go.load() == 1) pass(next[1], second);
       });
   } catch (const std::system_error&) {                   // no more threads to be had: the others do the work
+  } catch (const std::bad_alloc&) {
   }
   pass(next[0], first);
   while (done.load() < int(pool.size())) std::this_thread::yield();
-  try {
-    go = between() ? 1 : 2;
-  } catch (...) {
-    go = 2;
-    for (std::thread& t : pool) t.join();
-    throw;
-  }
-  if (go.load() == 1) pass(next[1], second);
+  bool on = false;
+  if (!failed) guarded([&] { on = between(); });
+  go = on ? 1 : 2;
+  if (on) pass(next[1], second);
   for (std::thread& t : pool) t.join();
+  if (error) std::rethrow_exception(error);
 }
 
 // For each bundle of n_tile output channels, list the (kernel location, 64-channel chunk)
@@ -524,10 +535,10 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
   if (dtype != RT3D_F32 && dtype != RT3D_BF16) return RT3D_ERR_INVALID_ARG;
   const int64_t Ks64 = int64_t(Kt) * Kh * Kw;
   if (Ks64 > 65535) return RT3D_ERR_INVALID_ARG;
-  rt3d_packed* h = new (std::nothrow) rt3d_packed;
-  if (!h) return RT3D_ERR_ALLOC;
-  h->id = next_handle_id();
-  try {
+  return c_entry([&] {
+    std::unique_ptr<rt3d_packed> owner(new rt3d_packed);
+    rt3d_packed* const h = owner.get();
+    h->id = next_handle_id();
     h->M = M; h->N = N; h->Kt = Kt; h->Kh = Kh; h->Kw = Kw; h->g_m = g_m; h->g_n = g_n;
     h->P = ceil_div(M, g_m); h->Q = ceil_div(N, g_n); h->Ks = int(Ks64);
     h->dtype = dtype; h->is_dense = is_dense;
@@ -607,13 +618,9 @@ static rt3d_status pack_impl(const float* w, const uint8_t* mask, int M, int N, 
           }
         }
     });
-    if (status != RT3D_OK) { delete h; return status; }
-  } catch (const std::bad_alloc&) {
-    delete h;
-    return RT3D_ERR_ALLOC;
-  }
-  *out = h;
-  return RT3D_OK;
+    if (status == RT3D_OK) *out = owner.release();
+    return status;
+  });
 }
 
 }  // namespace rt3d
@@ -646,10 +653,9 @@ rt3d_status rt3d_pack_concat(const rt3d_packed* const* parts, int n_parts, rt3d_
     bytes += int64_t(p->tiles.size());
   }
   if (nnz > 0x7FFFFFFF) return RT3D_ERR_UNSUPPORTED;
-  rt3d_packed* h = new (std::nothrow) rt3d_packed;
-  if (!h) return RT3D_ERR_ALLOC;
-  h->id = next_handle_id();
-  try {
+  return c_entry([&] {
+    std::unique_ptr<rt3d_packed> h(new rt3d_packed);
+    h->id = next_handle_id();
     const rt3d_packed* a = parts[0];
     h->N = a->N; h->Kt = a->Kt; h->Kh = a->Kh; h->Kw = a->Kw; h->g_m = a->g_m; h->g_n = a->g_n; h->Q = a->Q; h->Ks = a->Ks;
     h->dtype = a->dtype; h->is_dense = a->is_dense; h->is_vanilla = 1;
@@ -666,12 +672,9 @@ rt3d_status rt3d_pack_concat(const rt3d_packed* const* parts, int n_parts, rt3d_
       at += p->tiles.size();
       h->nnz += p->nnz;
     }
-  } catch (const std::bad_alloc&) {
-    delete h;
-    return RT3D_ERR_ALLOC;
-  }
-  *out = h;
-  return RT3D_OK;
+    *out = h.release();
+    return RT3D_OK;
+  });
 }
 
 rt3d_status rt3d_packed_view_get(const rt3d_packed* p, rt3d_packed_view* v) {
@@ -702,10 +705,10 @@ namespace {
 rt3d_status unpack_device_layout(const rt3d_packed* p, int n_tile, bool t_groups, float* w_out);
 }
 rt3d_status rt3d_unpack_device_layout(const rt3d_packed* p, int n_tile, float* w_out) {
-  return unpack_device_layout(p, n_tile, false, w_out);
+  return c_entry([&] { return unpack_device_layout(p, n_tile, false, w_out); });
 }
 rt3d_status rt3d_unpack_device_layout_tgroups(const rt3d_packed* p, int n_tile, float* w_out) {
-  return unpack_device_layout(p, n_tile, true, w_out);
+  return c_entry([&] { return unpack_device_layout(p, n_tile, true, w_out); });
 }
 namespace {
 rt3d_status unpack_device_layout(const rt3d_packed* p, int n_tile, bool t_groups, float* w_out) {
@@ -753,8 +756,9 @@ rt3d_status unpack_device_layout(const rt3d_packed* p, int n_tile, bool t_groups
 
 rt3d_status rt3d_unpack_sub_layout(const rt3d_packed* p, int n_tile, float* w_out) {
   if (!p || !w_out) return RT3D_ERR_INVALID_ARG;
-  const SubLayout* L = get_sub_layout(const_cast<rt3d_packed*>(p), n_tile);
-  if (!L) return RT3D_ERR_UNSUPPORTED;
+  const SubLayout* L = nullptr;
+  const rt3d_status built = c_entry([&] { L = get_sub_layout(const_cast<rt3d_packed*>(p), n_tile); return RT3D_OK; });
+  if (built != RT3D_OK || !L) return built != RT3D_OK ? built : RT3D_ERR_UNSUPPORTED;
   std::memset(w_out, 0, sizeof(float) * size_t(p->M) * p->N * p->Ks);
   for (int b = 0; b < L->n_bundles; ++b) {
     const int n_ranges = ceil_div(std::min(L->n_tile, p->M - b * L->n_tile), kSubRange);

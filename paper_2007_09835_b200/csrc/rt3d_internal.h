@@ -93,6 +93,17 @@ struct SubLayout {
   int max_steps = 0;                 // longest bundle list
 };
 
+// Runs the body of a C entry point.  No exception crosses it: what can be thrown in the library says that host memory or
+// another resource of the process could not be had.
+template <typename F>
+rt3d_status c_entry(const F& body) noexcept {
+  try {
+    return body();
+  } catch (...) {
+    return RT3D_ERR_ALLOC;
+  }
+}
+
 // Host memory of the packed weights: a block kept from a freed handle, or a new one (pack.cpp).
 unsigned char* host_block(size_t bytes);
 void host_block_free(unsigned char* p);
