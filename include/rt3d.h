@@ -173,7 +173,13 @@ rt3d_status rt3d_unpack_sub_layout(const rt3d_packed* p, int n_tile, float* w_ou
  * first compute call).  Call it before any stream capture.  Synchronises the device. */
 rt3d_status rt3d_packed_prepare(rt3d_packed* p);
 
+/* Frees a handle.  Waits for the device, as freeing device memory does.  Blocks of 256 KB to 32 MB are kept for the next
+ * handles, up to 64 MB of host memory and 64 MB of device memory (all devices together) in the process: the oldest go when
+ * others need the room, and all of them before the library reports that an allocation failed. */
 void rt3d_packed_free(rt3d_packed* p);
+
+/* Gives all kept blocks back to the system now.  May be called at any time from any thread. */
+void rt3d_release_kept(void);
 
 /*
  * rt3d_conv3d_sparse - the hot path: y = act(bias + conv3d(x, W (.) mask)), iterating only
@@ -385,7 +391,8 @@ rt3d_status rt3d_last_device_status(void* stream);
 /* Number of kernels this library has launched in this process (all devices). */
 int64_t rt3d_launch_count(void);
 
-/* Number of device allocations (cudaMalloc calls) this library has made in this process. */
+/* Number of device allocations (cudaMalloc calls) this library has made in this process; a layout that is uploaded into a
+ * kept block (rt3d_packed_free) makes none. */
 int64_t rt3d_alloc_count(void);
 
 /* Planning mode of the calling thread.  Between rt3d_plan_begin and rt3d_plan_end every compute call of this

@@ -93,6 +93,7 @@ def _load():
     lib.rt3d_packed_prepare.argtypes = [vp]
     lib.rt3d_packed_free.argtypes = [vp]
     lib.rt3d_packed_free.restype = None
+    lib.rt3d_release_kept.restype = None
     for name in ("rt3d_conv3d_sparse", "rt3d_conv3d_dense", "rt3d_conv3d_host", "rt3d_conv3d_sparse_noalloc"):
         getattr(lib, name).argtypes = [TP, vp, vp, CP, TP, vp]
     lib.rt3d_conv3d_sparse_fused.argtypes = [TP, vp, vp, CP, ctypes.POINTER(Fusion), TP, vp]
@@ -572,6 +573,11 @@ def rt3d_last_plan() -> dict:
 
 def rt3d_last_device_status(stream=None) -> int:
     return int(_lib.rt3d_last_device_status(_stream_ptr(stream)))
+
+
+def rt3d_release_kept():
+    """Gives the memory that is kept for the next handles back to the system (host and device)."""
+    _lib.rt3d_release_kept()
 
 
 def rt3d_launch_count() -> int:

@@ -25,33 +25,37 @@ namespace {
 std::atomic<int64_t> g_launches{0};
 std::atomic<int64_t> g_allocs{0};            // device allocations made by this library (rt3d_alloc_count)
 
-// Every device allocation of the library goes through here.
-cudaError_t dev_malloc(void** p, size_t bytes) {
-  g_allocs.fetch_add(1);
-  return cudaMalloc(p, bytes);
-}
-template <typename T>
-cudaError_t dev_malloc(T** p, size_t bytes) { return dev_malloc(reinterpret_cast<void**>(p), bytes); }
-
-// Device memory of uploaded layouts.  A kept block may still be read by kernels that its last owner launched (cudaFree
-// would have waited for them), so taking one waits for the device.
+// Device memory of uploaded layouts.  Never destroyed: handles may be freed while the process exits.
 KeptBlocks& weight_blocks() {
   static KeptBlocks* kept = new KeptBlocks([](void* p) { cudaFree(p); });
   return *kept;
 }
+
+// Every device allocation of the library goes through here.
+cudaError_t dev_malloc(void** p, size_t bytes) {
+  g_allocs.fetch_add(1);
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    weight_blocks().release_all();
+    g_allocs.fetch_add(1);
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+template <typename T>
+cudaError_t dev_malloc(T** p, size_t bytes) { return dev_malloc(reinterpret_cast<void**>(p), bytes); }
+
 cudaError_t weight_malloc(void** p, size_t bytes) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if ((*p = weight_blocks().take(bytes, dev)) != nullptr) {
-    if ((e = cudaDeviceSynchronize()) == cudaSuccess) return e;
-    cudaFree(*p);
-    return e;
-  }
+  if ((*p = weight_blocks().take(bytes, dev)) != nullptr) return cudaSuccess;
   if ((e = dev_malloc(p, bytes)) == cudaSuccess) weight_blocks().note(*p, bytes, dev);
   return e;
 }
-void weight_free(void* p) { weight_blocks().give(p); }
+// `idle`: the caller has waited for the kernels that may read the block, which cudaFree would do; only then is it kept.
+void weight_free(void* p, bool idle) { idle ? weight_blocks().give(p) : weight_blocks().drop(p); }
 
 // Planning mode of the calling thread (rt3d_plan_begin / rt3d_plan_end): compute calls do everything they would do
 // before their launch (choose the kernel, build and upload weight layouts, size the workspaces) and return.
@@ -309,7 +313,7 @@ class Upload {
     for (int i = 0; i < n_; ++i) {
       char* d = static_cast<char*>(*base) + items_[i].off;
       if (items_[i].bytes && cudaMemcpy(d, items_[i].src, items_[i].bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
-        weight_free(*base);
+        weight_free(*base, false);
         *base = nullptr;
         return RT3D_ERR_CUDA;
       }
@@ -363,7 +367,7 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
     if (L->t_groups) { up.add(&u.grp_ptr, L->grp_ptr); up.add(&u.grp_first, L->grp_first); }
     const rt3d_status s = up.run(base);
     if (s != RT3D_OK) return s;
-    const auto fail = [&] { weight_free(*base); *base = nullptr; return RT3D_ERR_CUDA; };
+    const auto fail = [&] { weight_free(*base, false); *base = nullptr; return RT3D_ERR_CUDA; };
     if (wbytes && (launch_fill_umma_tiles(blob->group_ptr, blob->pos_idx, blob->tiles, slots, h->M, h->N, h->Ks, h->g_m, h->g_n,
                                           h->Q, h->P * h->Q, h->nnz, L->n_tile, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
                    cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess))
@@ -1364,20 +1368,25 @@ void rt3d_packed_free(rt3d_packed* p) {
       g_blobs.erase(std::remove(g_blobs.begin(), g_blobs.end(), b), g_blobs.end());
   }
   for (DeviceBlob* b : p->blobs) {
-    if (have_dev) cudaSetDevice(b->device);
-    weight_free(b->canonical);
-    for (auto& kv : b->umma) weight_free(kv.second.base);
+    const bool idle = have_dev && cudaSetDevice(b->device) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+    weight_free(b->canonical, idle);
+    for (auto& kv : b->umma) weight_free(kv.second.base, idle);
     cudaFree(b->stage_x); cudaFree(b->stage_y); cudaFree(b->stage_bias);
     for (void* hs : b->host_streams) if (hs) cudaStreamDestroy(static_cast<cudaStream_t>(hs));
     for (void* he : b->host_events) if (he) cudaEventDestroy(static_cast<cudaEvent_t>(he));
-    for (auto& kv : b->smallc) weight_free(kv.second.base);
-    weight_free(b->f32.base);
+    for (auto& kv : b->smallc) weight_free(kv.second.base, idle);
+    weight_free(b->f32.base, idle);
     for (auto& kv : b->sub) { cudaFree(kv.second.steps); cudaFree(kv.second.step_ptr); cudaFree(kv.second.blocks); }
     cudaFree(b->splitk); cudaFree(b->splitk_cnt);
     delete b;
   }
   if (have_dev && cur >= 0) cudaSetDevice(cur);
   delete p;
+}
+
+void rt3d_release_kept(void) {
+  host_blocks_release();
+  weight_blocks().release_all();
 }
 
 rt3d_status rt3d_maxpool3d(const rt3d_tensor* x, int kt, int kh, int kw, int st, int sh, int sw, int pt, int ph,

@@ -39,11 +39,16 @@ static KeptBlocks& host_blocks() {
 }
 unsigned char* host_block(size_t bytes) {
   if (void* p = host_blocks().take(bytes, -1)) return static_cast<unsigned char*>(p);
-  unsigned char* p = new unsigned char[bytes];
+  unsigned char* p = new (std::nothrow) unsigned char[bytes];
+  if (!p) {
+    host_blocks().release_all();
+    p = new unsigned char[bytes];
+  }
   host_blocks().note(p, bytes, -1);
   return p;
 }
 void host_block_free(unsigned char* p) { host_blocks().give(p); }
+void host_blocks_release() { host_blocks().release_all(); }
 
 static float tile_value(const rt3d_packed* p, int64_t e, int i, int j) {
   const int64_t o = (e * p->g_m + i) * p->g_n + j;

@@ -107,6 +107,7 @@ rt3d_status c_entry(const F& body) noexcept {
 // Host memory of the packed weights: a block kept from a freed handle, or a new one (pack.cpp).
 unsigned char* host_block(size_t bytes);
 void host_block_free(unsigned char* p);
+void host_blocks_release();
 
 // Bytes that are written once, without the zeros a vector would fill them with first.
 class RawBytes {

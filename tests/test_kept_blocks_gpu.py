@@ -1,0 +1,80 @@
+"""Device memory kept from freed handles: taking it does not wait for the device, freeing does, and it can be given back."""
+import pytest
+import torch
+
+import rt3d_synth as synth
+import paper_2007_09835_b200 as rt3d
+from paper_2007_09835_b200 import binding as B
+from paper_2007_09835_b200 import nets
+
+pytestmark = pytest.mark.gpu
+
+SPEC = synth.ConvSpec("l", 256, 512, (3, 3, 3), (1, 1, 1), (1, 1, 1), True)
+
+
+@pytest.fixture(scope="module")
+def weights():
+    return synth.make_layer(SPEC, 3, 0, 4, 4, "bernoulli", 0.4)
+
+
+def layer(L):
+    return nets.ConvLayer(SPEC, L["w"], L["bias"], L["mask"], 4, 4, torch.bfloat16)
+
+
+def busy(stream):
+    """About a third of a second of work on a stream that nothing else waits for, and its end."""
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(600_000_000)
+        end = torch.cuda.Event()
+        end.record()
+    return end
+
+
+def test_first_call_into_a_kept_block_does_not_wait_for_the_device(weights):
+    x = nets.to_device(synth.make_input(1, (1, 4, 14, 14, 256)))
+    side = torch.cuda.Stream()
+    with B.concurrent_kernels():                          # plans whose blocks do not wait for one another
+        rt3d.rt3d_release_kept()
+        first = layer(weights)
+        y = first(x)
+        torch.cuda.synchronize()
+        del first
+        again, out = layer(weights), torch.zeros_like(y)
+        allocs = rt3d.rt3d_alloc_count()
+        end = busy(side)
+        again(x, out)
+        assert not end.query()                            # the call returned while the other stream was busy
+        assert rt3d.rt3d_alloc_count() == allocs          # and its weights went into the kept block
+        torch.cuda.synchronize()
+        assert torch.equal(out, y)
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+def test_free_waits_for_the_kernels_that_use_the_handle(weights):
+    x = nets.to_device(synth.make_input(1, (1, 4, 14, 14, 256)))
+    side, lay = torch.cuda.Stream(), layer(weights)
+    with B.concurrent_kernels():
+        want = lay(x)
+        y = torch.zeros_like(want)
+        torch.cuda.synchronize()
+        busy(side)
+        with torch.cuda.stream(side):
+            lay(x, y)
+            end = torch.cuda.Event()
+            end.record()
+        assert not end.query()
+        lay.packed.free()
+        assert end.query()
+    assert torch.equal(y, want)
+
+
+def test_kept_blocks_are_given_back(weights):
+    lay = layer(weights)
+    lay.packed.prepare()
+    rt3d.rt3d_release_kept()
+    torch.cuda.synchronize()
+    held = torch.cuda.mem_get_info()[0]
+    del lay
+    assert torch.cuda.mem_get_info()[0] == held           # kept
+    rt3d.rt3d_release_kept()
+    assert torch.cuda.mem_get_info()[0] > held
