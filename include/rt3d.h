@@ -14,7 +14,8 @@
  *     void*, NULL = default stream) and return without synchronising.  The first compute
  *     call that uses a handle on a device uploads the handle's device blobs (allocation +
  *     copy), and the first call of a shape whose left-over tiles are split along K (tail split) grows the
- *     handle's scratch buffer; later calls allocate nothing.  rt3d_packed_prepare does the upload ahead of time.
+ *     handle's scratch buffer; later calls allocate nothing.  Such a first call waits for its copies and fills, which go
+ *     through the legacy default stream (not for the device).  rt3d_packed_prepare does the upload ahead of time.
  *     That scratch belongs to the handle: two calls on the SAME handle whose kernels may overlap
  *     on the GPU (different streams) must be serialised by the caller.
  *   - Kernels are launched with programmatic stream serialisation: a kernel's set-up may overlap

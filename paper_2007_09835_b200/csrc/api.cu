@@ -90,6 +90,10 @@ struct DeviceState {
 std::mutex g_dev_mu;
 DeviceState g_dev[64];
 
+// Copies from pageable memory and fills go through the legacy stream and may return before they have reached the device, and
+// a caller's non-blocking stream does not wait for that stream: what a kernel reads has to be there before it is launched.
+cudaError_t uploads_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -104,7 +108,7 @@ rt3d_status get_device_state(DeviceState** out) {
     if (cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RT3D_ERR_CUDA;
     if (cudaDeviceGetAttribute(&d.cc_major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return RT3D_ERR_CUDA;
     if (dev_malloc(&d.sched, 256 * sizeof(int32_t)) != cudaSuccess) return RT3D_ERR_ALLOC;
-    if (cudaMemset(d.sched, 0, 256 * sizeof(int32_t)) != cudaSuccess) return RT3D_ERR_CUDA;
+    if (cudaMemset(d.sched, 0, 256 * sizeof(int32_t)) != cudaSuccess || uploads_done() != cudaSuccess) return RT3D_ERR_CUDA;
     if (!g_encode) {
       void* fn = nullptr;
       cudaDriverEntryPointQueryResult qres;
@@ -307,8 +311,9 @@ class Upload {
     items_[n_++] = Item{reinterpret_cast<void**>(dst), nullptr, 0, bytes_};
     bytes_ += (bytes + 16 + 255) & ~size_t(255);
   }
-  // Allocates, copies and sets the pointers; *base owns the memory.  Nothing is kept on failure.
-  rt3d_status run(void** base) {
+  // Allocates, copies and sets the pointers; *base owns the memory.  Nothing is kept on failure.  `wait`: returns when all of
+  // it is on the device (a caller that goes on in the legacy stream and waits for that needs no wait here).
+  rt3d_status run(void** base, bool wait = true) {
     if (weight_malloc(base, bytes_) != cudaSuccess) { *base = nullptr; return RT3D_ERR_ALLOC; }
     for (int i = 0; i < n_; ++i) {
       char* d = static_cast<char*>(*base) + items_[i].off;
@@ -318,6 +323,11 @@ class Upload {
         return RT3D_ERR_CUDA;
       }
       *items_[i].dst = d;
+    }
+    if (wait && uploads_done() != cudaSuccess) {
+      weight_free(*base, false);
+      *base = nullptr;
+      return RT3D_ERR_CUDA;
     }
     return RT3D_OK;
   }
@@ -365,12 +375,12 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
     up.add(&u.steps, L->steps);
     up.add(&slots, L->slots);
     if (L->t_groups) { up.add(&u.grp_ptr, L->grp_ptr); up.add(&u.grp_first, L->grp_first); }
-    const rt3d_status s = up.run(base);
+    const rt3d_status s = up.run(base, wbytes == 0);
     if (s != RT3D_OK) return s;
     const auto fail = [&] { weight_free(*base, false); *base = nullptr; return RT3D_ERR_CUDA; };
     if (wbytes && (launch_fill_umma_tiles(blob->group_ptr, blob->pos_idx, blob->tiles, slots, h->M, h->N, h->Ks, h->g_m, h->g_n,
                                           h->Q, h->P * h->Q, h->nnz, L->n_tile, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
-                   cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess))
+                   uploads_done() != cudaSuccess))
       return fail();
     // 2-D map over the weight tiles: rows of 64 bf16 (128 bytes), one box = one [n_tile][64] tile
     const cuuint64_t rows = L->steps.empty() ? cuuint64_t(L->n_tile) : cuuint64_t(L->steps.size()) * L->n_tile;
@@ -407,7 +417,8 @@ rt3d_status get_sub_blob(rt3d_packed* h, DeviceBlob* blob, const SubLayout* L, D
       return RT3D_ERR_ALLOC;
     if ((sbytes && cudaMemcpy(u.steps, L->steps.data(), sbytes, cudaMemcpyHostToDevice) != cudaSuccess) ||
         cudaMemcpy(u.step_ptr, L->step_ptr.data(), L->step_ptr.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        (bbytes && cudaMemcpy(u.blocks, L->payload.data(), bbytes, cudaMemcpyHostToDevice) != cudaSuccess))
+        (bbytes && cudaMemcpy(u.blocks, L->payload.data(), bbytes, cudaMemcpyHostToDevice) != cudaSuccess) ||
+        uploads_done() != cudaSuccess)
       return RT3D_ERR_CUDA;
     u.ready = true;
   }
@@ -756,7 +767,7 @@ rt3d_status ensure_splitk(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t
     cudaFree(blob->splitk_cnt);
     blob->splitk_cnt = nullptr; blob->splitk_cnt_bytes = 0;
     if (dev_malloc(&blob->splitk_cnt, cnt_bytes) != cudaSuccess) return RT3D_ERR_ALLOC;
-    if (cudaMemset(blob->splitk_cnt, 0, cnt_bytes) != cudaSuccess) return RT3D_ERR_CUDA;
+    if (cudaMemset(blob->splitk_cnt, 0, cnt_bytes) != cudaSuccess || uploads_done() != cudaSuccess) return RT3D_ERR_CUDA;
     blob->splitk_cnt_bytes = cnt_bytes;
   }
   return RT3D_OK;
@@ -1585,6 +1596,7 @@ rt3d_status rt3d_last_device_status(void* stream) {
       for (DeviceBlob* b : g_blobs)
         if (b->device == dev && b->splitk_cnt) cudaMemset(b->splitk_cnt, 0, b->splitk_cnt_bytes);
     }
+    uploads_done();
     return RT3D_ERR_TIMEOUT;
   }
   return RT3D_OK;
@@ -1690,7 +1702,7 @@ rt3d_status rt3d_debug_set(int what, long long value) {
     std::lock_guard<std::mutex> reg(g_blobs_mu);
     for (DeviceBlob* b : g_blobs)
       if (b->device == dev && b->splitk && cudaMemset(b->splitk, 0xFF, b->splitk_bytes) != cudaSuccess) return RT3D_ERR_CUDA;
-    return RT3D_OK;
+    return uploads_done() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
   }
   return RT3D_ERR_INVALID_ARG;
 }

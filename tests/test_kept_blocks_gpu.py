@@ -78,3 +78,25 @@ def test_kept_blocks_are_given_back(weights):
     assert torch.cuda.mem_get_info()[0] == held           # kept
     rt3d.rt3d_release_kept()
     assert torch.cuda.mem_get_info()[0] > held
+
+
+def test_flags_of_a_tail_split_are_clear_before_its_first_launch(weights):
+    """The scratch of a tail split is cleared through the default stream; on a stream that does not wait for that one, the call
+    has to."""
+    x = nets.to_device(synth.make_input(1, (1, 4, 14, 14, 256)))
+    want = layer(weights)(x, algo=B.ALGO_UMMA_PAIR)
+    plan = rt3d.rt3d_last_plan()
+    assert plan["tail_workers"] > 0, plan
+    lay, y, side = layer(weights), torch.zeros_like(want), torch.cuda.Stream()
+    with B.concurrent_kernels():
+        lay(x, y, algo=B.ALGO_UMMA_PAIR)                  # the same weight layout, no tail split
+    assert rt3d.rt3d_last_plan()["tail_workers"] == 0 and rt3d.rt3d_last_plan()["kernel"] == plan["kernel"]
+    y.zero_()
+    torch.cuda.synchronize()
+    end = busy(torch.cuda.default_stream())
+    with torch.cuda.stream(side):
+        lay(x, y, algo=B.ALGO_UMMA_PAIR)
+    assert end.query()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
