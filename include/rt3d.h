@@ -13,8 +13,8 @@
  *   - Compute calls enqueue work on the given CUDA stream (a cudaStream_t passed as
  *     void*, NULL = default stream) and return without synchronising.  The first compute
  *     call that uses a handle on a device uploads the handle's device blobs (allocation +
- *     copy), and the first call of a shape whose left-over tiles are split along K (tail split) grows the
- *     handle's scratch buffer; later calls allocate nothing.  Such a first call waits for its copies and fills, which go
+ *     copy), and the first call of a shape whose left-over tiles are split along K (tail split) may add a larger
+ *     scratch buffer to the handle (none goes before the handle does: captured graphs hold them); later calls allocate nothing.  Such a first call waits for its copies and fills, which go
  *     through the legacy default stream (not for the device).  rt3d_packed_prepare does the upload ahead of time.
  *     That scratch belongs to the handle: two calls on the SAME handle whose kernels may overlap
  *     on the GPU (different streams) must be serialised by the caller.

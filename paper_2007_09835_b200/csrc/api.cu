@@ -753,23 +753,27 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
   });
 }
 
-// Grows the handle's tail-split workspace on this device: `bytes` of partial tiles and `cnt_bytes` of
-// flags, which every kernel that uses them leaves zeroed.
-rt3d_status ensure_splitk(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t cnt_bytes) {
+// The handle's tail-split scratch on this device: at least `bytes` of partial tiles and `flag_bytes` of flags, which every
+// kernel that uses them leaves zeroed.  A larger one is at least twice the last, so that all of them take at most twice the
+// largest; none moves or goes before the handle does.
+rt3d_status get_tail(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t flag_bytes, DeviceBlob::Tail* out) {
   std::lock_guard<std::mutex> lock(w->mu);
-  if (blob->splitk_bytes < bytes) {
-    cudaFree(blob->splitk);
-    blob->splitk = nullptr; blob->splitk_bytes = 0;
-    if (dev_malloc(&blob->splitk, bytes) != cudaSuccess) return RT3D_ERR_ALLOC;
-    blob->splitk_bytes = bytes;
+  if (blob->tails.empty() || blob->tails.back().bytes < bytes || blob->tails.back().flag_bytes < flag_bytes) {
+    DeviceBlob::Tail t;
+    if (!blob->tails.empty()) { t.bytes = 2 * blob->tails.back().bytes; t.flag_bytes = 2 * blob->tails.back().flag_bytes; }
+    t.bytes = std::max(t.bytes, bytes);
+    t.flag_bytes = std::max(t.flag_bytes, flag_bytes);
+    std::lock_guard<std::mutex> reg(g_blobs_mu);               // others walk the lists of all handles
+    blob->tails.reserve(blob->tails.size() + 1);
+    if (dev_malloc(&t.partial, t.bytes) != cudaSuccess) return RT3D_ERR_ALLOC;
+    if (dev_malloc(&t.flags, t.flag_bytes) != cudaSuccess) { cudaFree(t.partial); return RT3D_ERR_ALLOC; }
+    if (cudaMemset(t.flags, 0, t.flag_bytes) != cudaSuccess || uploads_done() != cudaSuccess) {
+      cudaFree(t.partial); cudaFree(t.flags);
+      return RT3D_ERR_CUDA;
+    }
+    blob->tails.push_back(t);
   }
-  if (blob->splitk_cnt_bytes < cnt_bytes) {
-    cudaFree(blob->splitk_cnt);
-    blob->splitk_cnt = nullptr; blob->splitk_cnt_bytes = 0;
-    if (dev_malloc(&blob->splitk_cnt, cnt_bytes) != cudaSuccess) return RT3D_ERR_ALLOC;
-    if (cudaMemset(blob->splitk_cnt, 0, cnt_bytes) != cudaSuccess || uploads_done() != cudaSuccess) return RT3D_ERR_CUDA;
-    blob->splitk_cnt_bytes = cnt_bytes;
-  }
+  *out = blob->tails.back();
   return RT3D_OK;
 }
 
@@ -1111,18 +1115,17 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     if (!p->concurrent && (p->algo != RT3D_ALGO_AUTO || pairs >= d->sm_count / 2))
       umma_pair_tail_plan(&a, L->step_ptr.data(), d->sm_count, &tail_bytes, &flag_bytes, use_ts ? L->grp_ptr.data() : nullptr);
     if (a.tail_workers > 0) {
-      if ((s = ensure_splitk(w, blob, tail_bytes, flag_bytes)) != RT3D_OK) return s;
-      a.tail_scratch = blob->splitk; a.tail_flags = blob->splitk_cnt;
+      DeviceBlob::Tail t;
+      if ((s = get_tail(w, blob, tail_bytes, flag_bytes, &t)) != RT3D_OK) return s;
+      a.tail_scratch = t.partial; a.tail_flags = t.flags;
     }
   }
   const int sms = d->sm_count;
   const void* wmap = use_pair ? u->wmap_half : u->wmap;
   return submit(rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0},
                 [=](cudaStream_t st) {
-    UmmaArgs now = a;                              // a later call of another shape may have moved the handle's workspace
-    if (a.tail_workers > 0) { now.tail_scratch = blob->splitk; now.tail_flags = blob->splitk_cnt; }
     const void* ym = a.store_tma ? &ymap : nullptr;
-    return use_pair ? launch_conv_umma_pair(now, &xmap, wmap, ym, sms, st) : launch_conv_umma(now, &xmap, wmap, ym, sms, st);
+    return use_pair ? launch_conv_umma_pair(a, &xmap, wmap, ym, sms, st) : launch_conv_umma(a, &xmap, wmap, ym, sms, st);
   });
 }
 
@@ -1388,7 +1391,7 @@ void rt3d_packed_free(rt3d_packed* p) {
     for (auto& kv : b->smallc) weight_free(kv.second.base, idle);
     weight_free(b->f32.base, idle);
     for (auto& kv : b->sub) { cudaFree(kv.second.steps); cudaFree(kv.second.step_ptr); cudaFree(kv.second.blocks); }
-    cudaFree(b->splitk); cudaFree(b->splitk_cnt);
+    for (const DeviceBlob::Tail& t : b->tails) { cudaFree(t.partial); cudaFree(t.flags); }
     delete b;
   }
   if (have_dev && cur >= 0) cudaSetDevice(cur);
@@ -1594,7 +1597,8 @@ rt3d_status rt3d_last_device_status(void* stream) {
       cudaDeviceSynchronize();
       std::lock_guard<std::mutex> reg(g_blobs_mu);
       for (DeviceBlob* b : g_blobs)
-        if (b->device == dev && b->splitk_cnt) cudaMemset(b->splitk_cnt, 0, b->splitk_cnt_bytes);
+        if (b->device == dev)
+          for (const DeviceBlob::Tail& t : b->tails) cudaMemset(t.flags, 0, t.flag_bytes);
     }
     uploads_done();
     return RT3D_ERR_TIMEOUT;
@@ -1701,7 +1705,9 @@ rt3d_status rt3d_debug_set(int what, long long value) {
     if (cudaGetDevice(&dev) != cudaSuccess) return RT3D_ERR_CUDA;
     std::lock_guard<std::mutex> reg(g_blobs_mu);
     for (DeviceBlob* b : g_blobs)
-      if (b->device == dev && b->splitk && cudaMemset(b->splitk, 0xFF, b->splitk_bytes) != cudaSuccess) return RT3D_ERR_CUDA;
+      if (b->device == dev)
+        for (const DeviceBlob::Tail& t : b->tails)
+          if (cudaMemset(t.partial, 0xFF, t.bytes) != cudaSuccess) return RT3D_ERR_CUDA;
     return uploads_done() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
   }
   return RT3D_ERR_INVALID_ARG;

@@ -164,8 +164,10 @@ struct DeviceBlob {
   std::map<int, SmallC> smallc;      // small-C_in kernel: weight image, window offsets and copies, keyed like the layouts
   struct F32 { void* base = nullptr; int32_t* entry_ptr = nullptr; int32_t* tile_ptr = nullptr; int32_t* counts = nullptr; uint32_t* entries = nullptr; float* tiles = nullptr; };
   F32 f32;                           // register-blocked fp32 kernel
-  float* splitk = nullptr; size_t splitk_bytes = 0;            // split-K partial tiles (grown on demand)
-  int32_t* splitk_cnt = nullptr; size_t splitk_cnt_bytes = 0;  // split-K arrival counters, zero between launches
+  // Scratch of the CTA-pair kernel's tail splits: partial tiles, and flags that are zero between launches.  The last one is the
+  // largest; the others stay because captured graphs and prepared calls hold their addresses.
+  struct Tail { float* partial = nullptr; size_t bytes = 0; int32_t* flags = nullptr; size_t flag_bytes = 0; };
+  std::vector<Tail> tails;
   void* stage_x = nullptr; size_t stage_x_bytes = 0;   // staging for rt3d_conv3d_host
   void* stage_y = nullptr; size_t stage_y_bytes = 0;
   float* stage_bias = nullptr;

@@ -100,3 +100,29 @@ def test_flags_of_a_tail_split_are_clear_before_its_first_launch(weights):
     torch.cuda.synchronize()
     assert torch.equal(y, want)
     assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+def test_a_captured_tail_split_outlives_a_larger_one(weights):
+    """A call of another shape that needs more scratch leaves the scratch of a captured call in place."""
+    lay = layer(weights)
+    x, big = (nets.to_device(synth.make_input(1, s + (256,))) for s in ((1, 4, 14, 14), (1, 8, 28, 28)))
+    y = lay.alloc_out(x)
+    want = lay(x, algo=B.ALGO_UMMA_PAIR).clone()
+    workers = rt3d.rt3d_last_plan()["tail_workers"]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lay(x, y, algo=B.ALGO_UMMA_PAIR)
+    out = lay.alloc_out(big)
+    with B.concurrent_kernels():
+        lay(big, out, algo=B.ALGO_UMMA_PAIR)              # its weight layout, without a tail split
+    allocs = rt3d.rt3d_alloc_count()
+    lay(big, out, algo=B.ALGO_UMMA_PAIR)
+    assert rt3d.rt3d_last_plan()["tail_workers"] > workers > 0
+    assert rt3d.rt3d_alloc_count() == allocs + 2          # partial tiles and flags
+    first = out.clone()
+    for _ in range(3):
+        y.zero_()
+        graph.replay()
+        assert torch.equal(y, want)
+        assert torch.equal(lay(big, out, algo=B.ALGO_UMMA_PAIR), first)
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
