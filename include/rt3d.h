@@ -286,7 +286,7 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
 /*
  * rt3d_conv3d_host - end-to-end variant: x->data and y->data are HOST buffers (pinned
  * memory recommended), bias is HOST [M] or NULL.  Copies x to a library-owned device staging
- * buffer, runs rt3d_conv3d_sparse (or _dense for a dense handle) and copies y back; the work is
+ * buffer, runs rt3d_conv3d_sparse (or _dense for a dense handle) and copies y back, zeros in its padding channels; the work is
  * ordered after what `stream` holds on entry, and the call returns after the stream has been
  * synchronised.  Batches of at least two clips and 8 MiB go through in up to eight chunks of whole
  * clips (clips are independent), with the copies of neighbouring chunks on two internal streams, so

@@ -1266,11 +1266,18 @@ rt3d_status rt3d_conv3d_host(const rt3d_tensor* x, rt3d_packed* w, const float* 
     }
     if (blob->stage_y_bytes < yb) {
       cudaFree(blob->stage_y);
-      blob->stage_y = nullptr; blob->stage_y_bytes = 0;
+      blob->stage_y = nullptr; blob->stage_y_bytes = 0; blob->stage_y_pitch = 0;
       if (dev_malloc(&blob->stage_y, yb + 256) != cudaSuccess) return RT3D_ERR_ALLOC;
       blob->stage_y_bytes = yb;
-      // the padding channels, which no kernel writes, are copied out with the rest: not what the memory held before
-      if (cudaMemsetAsync(blob->stage_y, 0, yb + 256, static_cast<cudaStream_t>(stream)) != cudaSuccess) return RT3D_ERR_CUDA;
+      blob->stage_y_pitch = 0;
+    }
+    // The padding channels, which no kernel writes, are copied out with the rest: zeros, not what the memory held before or
+    // what a call of another pitch left there.
+    if (y->c_stride == w->M) {
+      blob->stage_y_pitch = 0;
+    } else if (blob->stage_y_pitch != y->c_stride) {
+      if (cudaMemsetAsync(blob->stage_y, 0, blob->stage_y_bytes, static_cast<cudaStream_t>(stream)) != cudaSuccess) return RT3D_ERR_CUDA;
+      blob->stage_y_pitch = y->c_stride;
     }
     if (!blob->stage_bias && dev_malloc(&blob->stage_bias, size_t(w->M) * 4) != cudaSuccess)
       return RT3D_ERR_ALLOC;

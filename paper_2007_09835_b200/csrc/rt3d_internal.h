@@ -170,6 +170,7 @@ struct DeviceBlob {
   std::vector<Tail> tails;
   void* stage_x = nullptr; size_t stage_x_bytes = 0;   // staging for rt3d_conv3d_host
   void* stage_y = nullptr; size_t stage_y_bytes = 0;
+  int stage_y_pitch = 0;                               // channel pitch at which stage_y's padding holds zeros, 0 = none
   float* stage_bias = nullptr;
   // rt3d_conv3d_host pipelines a large batch in chunks: copy-in and copy-out streams and events
   // (cudaStream_t / cudaEvent_t, created on first use)

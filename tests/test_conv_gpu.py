@@ -441,6 +441,23 @@ def test_conv3d_host_entry_point_pipelines_large_batches_in_chunks():
     check(yh[10:].float().numpy(), ref0, torch.bfloat16, "host path, last clip")
 
 
+def test_conv3d_host_entry_point_padding_channels_hold_zeros():
+    """Padding channels come back as zeros whatever pitch and batch the handle was called with before."""
+    spec = synth.ConvSpec("h", 16, 22, (1, 3, 3), (1, 1, 1), (0, 1, 1), True)
+    L = synth.make_layer(spec, 7, 11, 4, 4, "bernoulli", 0.4)
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.bfloat16)
+    bh = torch.from_numpy(L["bias"]).pin_memory()
+    for n, pitch in ((2, 40), (2, 24), (1, 40), (3, 40), (3, 64), (1, 24), (3, 24)):
+        x = synth.make_input(711 + n, (n, 2, 9, 9, 16))
+        want = lay(nets.to_device(x)).cpu()
+        xh = torch.from_numpy(x).to(torch.bfloat16).pin_memory()
+        yh = torch.full((n, 2, 9, 9, pitch), 55.0, dtype=torch.bfloat16).pin_memory()
+        rt3d.rt3d_conv3d_host(rt3d.tensor_desc(xh), lay.packed, bh, rt3d.tensor_desc(yh, 22), spec.stride, spec.pad, True)
+        assert torch.equal(yh[..., :22], want[..., :22]), (n, pitch)
+        assert not yh.view(-1, pitch)[:-1, 22:].any(), (n, pitch)     # the last voxel's padding is not copied
+        assert (yh.view(-1, pitch)[-1, 22:] == 55.0).all()
+
+
 def test_maxpool_and_add_relu_against_oracle():
     for dtype in (torch.bfloat16, torch.float32):
         for c, shape, pool in ((64, (2, 4, 8, 8), synth.PoolSpec("p", (2, 2, 2), (2, 2, 2), (0, 0, 0))),
