@@ -121,6 +121,16 @@ bool want(Py_ssize_t n, Py_ssize_t expected) {
   return n == expected;
 }
 
+// A library call with the interpreter released, as ctypes makes it: a launch may have to wait for room in its stream.
+template <typename F>
+PyObject* released(const F& call) {
+  rt3d_status s;
+  Py_BEGIN_ALLOW_THREADS
+  s = call();
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(long(s));
+}
+
 // The three calls of the pruning step, with the arguments of their binding functions behind the library's address.
 PyObject* group_norms(PyObject*, PyObject* const* a, Py_ssize_t n) {   // address, w, g_m, g_n, norm, norms, stream
   uintptr_t fn, w, norms, stream;
@@ -138,9 +148,11 @@ PyObject* group_norms(PyObject*, PyObject* const* a, Py_ssize_t n) {   // addres
   }
   Py_DECREF(shape);
   if (!ok) return nullptr;
-  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_group_norms)>(fn)(
-      reinterpret_cast<const float*>(w), e[0], e[1], e[2], e[3], e[4], v[0], v[1], v[2], reinterpret_cast<float*>(norms),
-      reinterpret_cast<void*>(stream)));
+  return released([&] {
+    return reinterpret_cast<decltype(&rt3d_kgs_group_norms)>(fn)(
+        reinterpret_cast<const float*>(w), e[0], e[1], e[2], e[3], e[4], v[0], v[1], v[2], reinterpret_cast<float*>(norms),
+        reinterpret_cast<void*>(stream));
+  });
 }
 
 PyObject* reweight(PyObject*, PyObject* const* a, Py_ssize_t n) {      // address, norms, count, eps, threshold, penalty, keep, stream
@@ -149,9 +161,11 @@ PyObject* reweight(PyObject*, PyObject* const* a, Py_ssize_t n) {      // addres
   const long long count = PyLong_AsLongLong(a[2]);
   const double eps = PyFloat_AsDouble(a[3]), threshold = PyFloat_AsDouble(a[4]);
   if (PyErr_Occurred() || !tensor_or_none(a[5], &penalty) || !tensor_or_none(a[6], &keep) || !stream_of(a[7], &stream)) return nullptr;
-  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_reweight)>(fn)(
-      reinterpret_cast<const float*>(norms), count, float(eps), float(threshold), reinterpret_cast<float*>(penalty),
-      reinterpret_cast<uint8_t*>(keep), reinterpret_cast<void*>(stream)));
+  return released([&] {
+    return reinterpret_cast<decltype(&rt3d_kgs_reweight)>(fn)(
+        reinterpret_cast<const float*>(norms), count, float(eps), float(threshold), reinterpret_cast<float*>(penalty),
+        reinterpret_cast<uint8_t*>(keep), reinterpret_cast<void*>(stream));
+  });
 }
 
 PyObject* expand_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {   // address, group mask, M, N, Kt, Kh, Kw, g_m, g_n, mask, stream
@@ -160,9 +174,11 @@ PyObject* expand_mask(PyObject*, PyObject* const* a, Py_ssize_t n) {   // addres
   if (!want(n, 11) || !as_pointer(a[0], &fn) || !data_ptr(a[1], &g) || !ints(a + 2, 7, v) || !data_ptr(a[9], &mask) ||
       !stream_of(a[10], &stream))
     return nullptr;
-  return PyLong_FromLong(reinterpret_cast<decltype(&rt3d_kgs_expand_mask)>(fn)(
-      reinterpret_cast<const uint8_t*>(g), v[0], v[1], v[2], v[3], v[4], v[5], v[6], reinterpret_cast<uint8_t*>(mask),
-      reinterpret_cast<void*>(stream)));
+  return released([&] {
+    return reinterpret_cast<decltype(&rt3d_kgs_expand_mask)>(fn)(
+        reinterpret_cast<const uint8_t*>(g), v[0], v[1], v[2], v[3], v[4], v[5], v[6], reinterpret_cast<uint8_t*>(mask),
+        reinterpret_cast<void*>(stream));
+  });
 }
 
 // pointers_are(tensors, addresses): whether every tensor of a tuple still has its address of a bytes object (8 bytes each).
@@ -219,15 +235,13 @@ PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   rt3d_conv_params params;
   __builtin_memcpy(&params, p.buf, sizeof(params));
   PyBuffer_Release(&p);
-  rt3d_status s;
-  Py_BEGIN_ALLOW_THREADS
-  const auto* w = reinterpret_cast<const rt3d_packed*>(handle);
-  const auto* b = reinterpret_cast<const float*>(bias);
-  void* st = reinterpret_cast<void*>(stream);
-  s = n == 11 ? reinterpret_cast<FusedFn>(fn)(&x, w, b, &params, &fz, &y, st)
-              : reinterpret_cast<ConvFn>(fn)(&x, w, b, &params, &y, st);
-  Py_END_ALLOW_THREADS
-  return PyLong_FromLong(long(s));
+  return released([&] {
+    const auto* w = reinterpret_cast<const rt3d_packed*>(handle);
+    const auto* b = reinterpret_cast<const float*>(bias);
+    void* st = reinterpret_cast<void*>(stream);
+    return n == 11 ? reinterpret_cast<FusedFn>(fn)(&x, w, b, &params, &fz, &y, st)
+                   : reinterpret_cast<ConvFn>(fn)(&x, w, b, &params, &y, st);
+  });
 }
 
 PyMethodDef methods[] = {

@@ -140,3 +140,30 @@ def test_channel_slice_descriptor():
         B.channel_slice_desc(t, 48, 24)             # runs past the pitch
     with pytest.raises(ValueError):
         B.channel_slice_desc(t[..., :32], 0, 8)     # not a dense tensor
+
+
+def test_pruning_calls_let_other_threads_run():
+    """A call that waits inside the library (here a C function that sleeps 0.3 s in its place) holds up no other thread."""
+    import ctypes
+    import threading
+    import time
+    sleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p).value
+
+    class Address:                                      # the first argument of each call is an address: the microseconds
+        shape = (4, 4, 1, 1, 1)
+
+        def data_ptr(self):
+            return 300_000
+
+    m, a = rt3d.pycall(), Address()
+    for call in (lambda: m.group_norms(sleep, a, 4, 4, 2, a, 0), lambda: m.reweight(sleep, a, 1, 1e-3, 0.0, None, None, 0),
+                 lambda: m.expand_mask(sleep, a, 4, 4, 1, 1, 1, 4, 4, a, 0)):
+        t = threading.Thread(target=call)
+        begun = time.monotonic()
+        t.start()
+        turns = 0
+        while t.is_alive() and time.monotonic() - begun < 5:
+            turns += 1
+            time.sleep(0.01)
+        t.join()
+        assert time.monotonic() - begun >= 0.29 and turns >= 5, turns
