@@ -12,6 +12,7 @@
 // RT3D_PDL=0 in the environment turns the launch attribute off (the device instructions are then no-ops).
 #pragma once
 
+#include <atomic>
 #include <cstdlib>
 #include <cuda_runtime.h>
 
@@ -33,6 +34,19 @@ inline int current_device_index() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
   return dev;
+}
+
+// SMs of the current device, or 0.
+inline int current_device_sms() {
+  static std::atomic<int> known[kMaxDevices];
+  const int dev = current_device_index();
+  if (dev < 0) return 0;
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
 }
 
 inline bool pdl_enabled() {

@@ -132,7 +132,7 @@ cudaError_t launch_group_norms(const float* w, int M, int N, int Ks, int g_m, in
   // groups per block: a whole run, in steps of four so that every run starts on a 16-byte boundary of its row; at
   // most a quarter of a run where fewer blocks than two per SM would run
   int q_run = g_n * Ks < kNormRun ? kNormRun / (g_n * Ks) : 1;
-  if ((long long)P * ((Q + q_run - 1) / q_run) < 2 * 148) q_run = (q_run + 3) / 4;
+  if ((long long)P * ((Q + q_run - 1) / q_run) < 2 * current_device_sms()) q_run = (q_run + 3) / 4;
   if (q_run > 4) q_run &= ~3;
   const bool vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0 && ((long long)N * Ks) % 4 == 0 && (q_run * g_n * Ks) % 4 == 0;
   const int n_runs = (Q + q_run - 1) / q_run, lg = lanes_of(Ks);
