@@ -98,6 +98,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn g_encode = nullptr;
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+ReplaceAddressFn g_replace_address = nullptr;
 
 rt3d_status get_device_state(DeviceState** out) {
   int dev = 0;
@@ -114,6 +116,10 @@ rt3d_status get_device_state(DeviceState** out) {
       cudaDriverEntryPointQueryResult qres;
       if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn)
         return RT3D_ERR_CUDA;
+      void* replace = nullptr;
+      if (cudaGetDriverEntryPoint("cuTensorMapReplaceAddress", &replace, cudaEnableDefault, &qres) != cudaSuccess || !replace)
+        return RT3D_ERR_CUDA;
+      g_replace_address = reinterpret_cast<ReplaceAddressFn>(replace);
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
     d.init = true;
@@ -186,20 +192,27 @@ std::atomic<int> g_plan_epoch{0};              // advanced by rt3d_debug_set: ca
 }  // namespace
 
 namespace rt3d {
-// Everything a convolution call is determined by.
+// Everything that a convolution call's plan is determined by: no address, so that a call on buffers the handle has not seen is
+// found like a repeated one.
 struct CallKey {
-  const void *x, *y, *res, *bias, *bias2;
   uint64_t w2;                                 // the second handle, by its id: its address may be another handle's later
   int32_t geo[24];                             // extents, pitches and dtypes of x, y and the residual
   int32_t p[20];                               // both convolutions' parameters
-  int32_t misc[6];                             // device, entry point, fused pool, epoch
+  int32_t misc[8];                             // device, entry point, fused pool, epoch, which of the two biases there are
 };
-// One call of a handle, ready to launch: a user runs a layer on the same few buffers again and again, and validating,
+// The memory that one call works on.
+struct CallBuffers {
+  const void* x;
+  void* y;
+  const void* res;
+  const float *bias, *bias2;
+};
+// One call of a handle, ready to launch on any buffers: a user runs a layer on the same few shapes again and again, and
 // choosing the kernel and encoding two or three tensor maps cost 1 to 2 us of the host's time for each call.
 struct PreparedCall {
   CallKey key;
   rt3d_plan_info info;
-  std::function<cudaError_t(cudaStream_t)> launch;
+  std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch;
 };
 }  // namespace rt3d
 
@@ -215,25 +228,36 @@ void put_params(const rt3d_conv_params* p, int32_t* at) {
   const int32_t v[10] = {p->st, p->sh, p->sw, p->pt, p->ph, p->pw, p->relu, p->algo, p->x_pad_zero, p->concurrent};
   memcpy(at, v, sizeof(v));
 }
-// False for arguments that the call will refuse anyway.
+// False for arguments that the call will refuse anyway, what depends on addresses (alignment, overlap) among them.
 bool make_key(CallKey* k, const rt3d_tensor* x, const rt3d_packed* w, const float* bias, const rt3d_conv_params* p,
               const rt3d_tensor* y, const rt3d_tensor* res, int entry) {
   int dev = 0;
-  if (!x || !w || !p || !y || cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (!x || !w || !p || !y || check_tensor(x) != RT3D_OK || check_tensor(y) != RT3D_OK || (res && check_tensor(res) != RT3D_OK) ||
+      check_alignment(x) != RT3D_OK || check_alignment(y) != RT3D_OK || (res && check_alignment(res) != RT3D_OK) ||
+      overlaps(x, y) || (res && overlaps(res, y)) || cudaGetDevice(&dev) != cudaSuccess)
+    return false;
   memset(k, 0, sizeof(*k));
-  k->x = x->data; k->y = y->data; k->bias = bias;
   put_tensor(x, k->geo);
   put_tensor(y, k->geo + 8);
-  if (res) { k->res = res->data; put_tensor(res, k->geo + 16); }
+  if (res) put_tensor(res, k->geo + 16);
   put_params(p, k->p);
-  k->misc[0] = dev; k->misc[1] = entry; k->misc[5] = g_plan_epoch.load();
+  k->misc[0] = dev; k->misc[1] = entry; k->misc[5] = g_plan_epoch.load(); k->misc[6] = bias != nullptr;
   return true;
 }
+
+// Tensor maps of a prepared call at the addresses of this one (nullptr: a map that the call has no use for).
+struct PlacedMaps {
+  CUtensorMap x, y;
+  bool ok;
+  PlacedMaps(const CUtensorMap& xmap, const void* xa, const CUtensorMap& ymap, void* ya) : x(xmap), y(ymap) {
+    ok = (!xa || g_replace_address(&x, const_cast<void*>(xa)) == CUDA_SUCCESS) && (!ya || g_replace_address(&y, ya) == CUDA_SUCCESS);
+  }
+};
 
 // Runs one call of a handle: from its prepared calls, or prepared now and kept.
 class Submit {
  public:
-  Submit(rt3d_packed* w, const CallKey& key, cudaStream_t st) : w_(w), key_(key), st_(st) {}
+  Submit(rt3d_packed* w, const CallKey& key, const CallBuffers& buffers, cudaStream_t st) : w_(w), key_(key), buffers_(buffers), st_(st) {}
   // true: the call was found and has been run (or only planned), with *status as its result
   bool again(rt3d_status* status) {
     std::shared_ptr<PreparedCall> c;
@@ -246,8 +270,9 @@ class Submit {
     *status = run(*c);
     return true;
   }
-  // A kernel launch chosen for this call.  `launch` must hold by value whatever it needs besides the handle's own memory.
-  rt3d_status operator()(const rt3d_plan_info& info, std::function<cudaError_t(cudaStream_t)> launch) {
+  // A kernel launch chosen for this call.  `launch` must hold by value whatever it needs besides the handle's own memory, and
+  // take the addresses of the tensors and biases from its argument.
+  rt3d_status operator()(const rt3d_plan_info& info, std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch) {
     auto c = std::make_shared<PreparedCall>(PreparedCall{key_, info, std::move(launch)});
     {
       std::lock_guard<std::mutex> lock(w_->mu);
@@ -261,12 +286,13 @@ class Submit {
   rt3d_status run(const PreparedCall& c) {
     t_last_plan = c.info;
     if (t_plan_only) return RT3D_OK;
-    if (c.launch(st_) != cudaSuccess) return RT3D_ERR_CUDA;
+    if (c.launch(buffers_, st_) != cudaSuccess) return RT3D_ERR_CUDA;
     g_launches.fetch_add(1);
     return RT3D_OK;
   }
   rt3d_packed* w_;
   const CallKey& key_;
+  const CallBuffers buffers_;
   cudaStream_t st_;
 };
 
@@ -743,13 +769,17 @@ rt3d_status launch_smallc(rt3d_packed* w, DeviceBlob* blob, const DeviceState* d
       g_encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, x->data, dims, strides, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return RT3D_ERR_CUDA;
-  CUtensorMap ymap;
+  CUtensorMap ymap{};
   const int sb[4] = {kSmallCTileW, 4, 1, 1};          // a warp owns 4 rows of 8 voxels of the 16 x 8 tile
   a.store_tma = encode_ymap(y, sb, pool_w, pool_h, 1, &ymap) ? 1 : 0;
   if (!a.store_tma && pool_h * pool_w > 1) return RT3D_ERR_UNSUPPORTED;
   const int sms = d->sm_count;
-  return submit(rt3d_plan_info{3, L->n_pad, 1, 0, pool_h * pool_w > 1 ? 1 : 0}, [=](cudaStream_t st) {
-    return launch_conv_umma_smallc(a, &xmap, a.store_tma ? &ymap : nullptr, sms, st);
+  return submit(rt3d_plan_info{3, L->n_pad, 1, 0, pool_h * pool_w > 1 ? 1 : 0}, [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, a.ops ? nullptr : c.x, ymap, a.store_tma ? c.y : nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    SmallCArgs now = a;
+    now.x = c.x; now.y = c.y; now.bias = c.bias; now.residual = c.res;
+    return launch_conv_umma_smallc(now, &m.x, a.store_tma ? &m.y : nullptr, sms, st);
   });
 }
 
@@ -827,7 +857,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = 0; a.debug_drop_last_load = 0;
   ConvGeom unit = g;                       // the staged block is a plain box of input voxels
-  CUtensorMap xmap, ymap;
+  CUtensorMap xmap, ymap{};
   if ((s = encode_xmap(x, unit, TileBox{1, h.ht, h.hh, h.hw}, &xmap)) != RT3D_OK) return s;
   int sb[4] = {1, 1, 1, 1};
   const bool rect = warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb);
@@ -836,8 +866,12 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   *launched = true;
   const int sms = d->sm_count;
   const void* wmap = u->wmap_half;
-  return submit(rt3d_plan_info{4, a.n_tile, 1, 0, 0}, [=](cudaStream_t st) {
-    return launch_conv_umma_halo(h, &xmap, wmap, h.u.store_tma ? &ymap : nullptr, sms, st);
+  return submit(rt3d_plan_info{4, a.n_tile, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, c.x, ymap, h.u.store_tma ? c.y : nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    HaloArgs now = h;
+    now.u.y = c.y; now.u.bias = c.bias; now.u.residual = c.res;
+    return launch_conv_umma_halo(now, &m.x, wmap, h.u.store_tma ? &m.y : nullptr, sms, st);
   });
 }
 
@@ -867,15 +901,19 @@ rt3d_status try_sub(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   a.steps = static_cast<const SubStep*>(u->steps); a.step_ptr = u->step_ptr; a.blocks = u->blocks;
   a.bias = bias; a.y = y->data; a.sched = d->sched;
   a.residual = res_data; a.rcs = res_pitch;
-  CUtensorMap xmap, ymap;
+  CUtensorMap xmap, ymap{};
   if ((s = encode_xmap(x, g, a.box, &xmap)) != RT3D_OK) return s;
   int sb[4] = {1, 1, 1, 1};
   const bool rect = warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb);
   a.store_tma = (rect && encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   *launched = true;
   const int sms = d->sm_count;
-  return submit(rt3d_plan_info{6, a.n_tile, 1, 0, 0}, [=](cudaStream_t st) {
-    return launch_conv_umma_sub(a, &xmap, a.store_tma ? &ymap : nullptr, sms, st);
+  return submit(rt3d_plan_info{6, a.n_tile, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, c.x, ymap, a.store_tma ? c.y : nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    SubArgs now = a;
+    now.y = c.y; now.bias = c.bias; now.residual = c.res;
+    return launch_conv_umma_sub(now, &m.x, a.store_tma ? &m.y : nullptr, sms, st);
   });
 }
 
@@ -918,7 +956,12 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
     a.bias = bias; a.residual = static_cast<const float*>(res_data); a.rcs = res_pitch;
     *launched = true;
     const F32Plan plan = plans[i];
-    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](cudaStream_t st) { return launch_conv_f32(a, plan, st); });
+    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+      F32Args now = a;
+      now.x = static_cast<const float*>(c.x); now.y = static_cast<float*>(c.y);
+      now.bias = c.bias; now.residual = static_cast<const float*>(c.res);
+      return launch_conv_f32(now, plan, st);
+    });
   }
   return RT3D_OK;
 }
@@ -926,10 +969,12 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
 rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
                       rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz) {
   CallKey key;
+  CallBuffers buffers{};
   if (make_key(&key, x, wc, bias, p, y, fz ? fz->residual : nullptr, dense_entry ? 1 : 0)) {
     if (fz) { key.misc[2] = fz->pool_t; key.misc[3] = fz->pool_h; key.misc[4] = fz->pool_w; }
+    buffers = CallBuffers{x->data, y->data, fz && fz->residual ? fz->residual->data : nullptr, bias, nullptr};
     rt3d_status found;
-    if (Submit(const_cast<rt3d_packed*>(wc), key, static_cast<cudaStream_t>(stream)).again(&found)) return found;
+    if (Submit(const_cast<rt3d_packed*>(wc), key, buffers, static_cast<cudaStream_t>(stream)).again(&found)) return found;
   }
   ConvGeom g;
   if (!y) return RT3D_ERR_INVALID_ARG;
@@ -964,7 +1009,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   if ((s = get_device_state(&d)) != RT3D_OK) return s;
   DeviceBlob* blob = nullptr;
   if ((s = get_blob(w, &blob)) != RT3D_OK) return s;
-  Submit submit(w, key, static_cast<cudaStream_t>(stream));
+  Submit submit(w, key, buffers, static_cast<cudaStream_t>(stream));
 
   const bool can_umma = umma_eligible(d, w, x, y, p);
   const bool can_simt = w->g_m <= kMaxGroupSimt && w->g_n <= kMaxGroupSimt;
@@ -980,11 +1025,9 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
     if (s != RT3D_OK || launched) return s;
     if ((s = get_canonical(w, blob)) != RT3D_OK) return s;
-    const void *xdata = x->data;
-    void* ydata = y->data;
-    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](cudaStream_t st) {
-      return launch_conv_simt(w->dtype, g, xdata, ydata, blob->group_ptr, blob->pos_idx, blob->tiles, bias, w->g_m, w->g_n,
-                              w->P, w->Q, dense_entry, res_data, res_pitch, st);
+    return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+      return launch_conv_simt(w->dtype, g, c.x, c.y, blob->group_ptr, blob->pos_idx, blob->tiles, c.bias, w->g_m, w->g_n,
+                              w->P, w->Q, dense_entry, c.res, res_pitch, st);
     });
   }
 
@@ -1102,7 +1145,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   }
   CUtensorMap xmap;
   if ((s = encode_xmap(x, g, a.box, &xmap, use_ts ? ((g.Kt - 1) / g.st) * g.st : 0)) != RT3D_OK) return s;
-  CUtensorMap ymap;
+  CUtensorMap ymap{};
   a.store_tma = (a.n_splits == 1 && rect && encode_ymap(y, sb, pl_w, pl_h, pl_t, &ymap)) ? 1 : 0;
   if (pooled && !a.store_tma) return RT3D_ERR_UNSUPPORTED;
   if (use_pair) {
@@ -1123,9 +1166,13 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   const int sms = d->sm_count;
   const void* wmap = use_pair ? u->wmap_half : u->wmap;
   return submit(rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0},
-                [=](cudaStream_t st) {
-    const void* ym = a.store_tma ? &ymap : nullptr;
-    return use_pair ? launch_conv_umma_pair(a, &xmap, wmap, ym, sms, st) : launch_conv_umma(a, &xmap, wmap, ym, sms, st);
+                [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, c.x, ymap, a.store_tma ? c.y : nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    UmmaArgs now = a;
+    now.y = c.y; now.bias = c.bias; now.residual = c.res;
+    const void* ym = a.store_tma ? &m.y : nullptr;
+    return use_pair ? launch_conv_umma_pair(now, &m.x, wmap, ym, sms, st) : launch_conv_umma(now, &m.x, wmap, ym, sms, st);
   });
 }
 
@@ -1137,11 +1184,13 @@ rt3d_status conv2plus1d_body(const rt3d_tensor* x, const rt3d_packed* wsc, const
                              const rt3d_tensor* res, rt3d_tensor* y, void* stream) {
   if (!wsc || !wtc || !ps || !pt || !y) return RT3D_ERR_INVALID_ARG;
   CallKey key;
+  CallBuffers buffers{};
   if (make_key(&key, x, wsc, bias_s, ps, y, res, 2)) {
-    key.w2 = wtc->id; key.bias2 = bias_t;
+    key.w2 = wtc->id; key.misc[7] = bias_t != nullptr;
     put_params(pt, key.p + 10);
+    buffers = CallBuffers{x->data, y->data, res ? res->data : nullptr, bias_s, bias_t};
     rt3d_status found;
-    if (Submit(const_cast<rt3d_packed*>(wsc), key, static_cast<cudaStream_t>(stream)).again(&found)) return found;
+    if (Submit(const_cast<rt3d_packed*>(wsc), key, buffers, static_cast<cudaStream_t>(stream)).again(&found)) return found;
   }
   ConvGeom g;
   rt3d_status s = make_geom(x, wsc, ps, nullptr, &g);
@@ -1198,8 +1247,12 @@ rt3d_status conv2plus1d_body(const rt3d_tensor* x, const rt3d_packed* wsc, const
   if ((s = encode_xmap(x, unit, TileBox{1, 1, a.hh, a.hw}, &xmap)) != RT3D_OK) return s;
   const int sms = d->sm_count;
   const void *m1 = u1->wmap_half, *m2 = u2->wmap_half;
-  return Submit(ws, key, static_cast<cudaStream_t>(stream))(rt3d_plan_info{5, a.n1, 1, 0, 0}, [=](cudaStream_t st) {
-    return launch_conv_umma_st(a, &xmap, m1, m2, sms, st);
+  return Submit(ws, key, buffers, static_cast<cudaStream_t>(stream))(rt3d_plan_info{5, a.n1, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, c.x, xmap, nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    StArgs now = a;
+    now.y = c.y; now.bias1 = c.bias; now.bias2 = c.bias2; now.residual = c.res;
+    return launch_conv_umma_st(now, &m.x, m1, m2, sms, st);
   });
 }
 

@@ -150,3 +150,92 @@ def test_small_copies_in_one_launch():
         with pytest.raises(rt3d.Rt3dError) as e:
             rt3d.rt3d_copy_f32(bad)
         assert e.value.status == rt3d.ERR_INVALID_ARG
+
+
+CALLS = [  # channels in and out, kernel, stride, extents, type, family, residual: every kernel that a call can be prepared for
+    (64, 64, (3, 3, 3), (1, 1, 1), (1, 4, 20, 20), torch.bfloat16, rt3d.ALGO_AUTO, True),
+    (64, 64, (3, 3, 3), (1, 1, 1), (1, 4, 20, 20), torch.bfloat16, rt3d.ALGO_UMMA, False),
+    (64, 96, (3, 3, 3), (1, 1, 1), (2, 4, 20, 20), torch.bfloat16, rt3d.ALGO_UMMA_PAIR, True),
+    (32, 64, (1, 3, 3), (1, 1, 1), (1, 4, 16, 16), torch.bfloat16, rt3d.ALGO_UMMA_HALO, True),
+    (64, 64, (3, 3, 3), (1, 1, 1), (1, 4, 12, 12), torch.bfloat16, rt3d.ALGO_UMMA_SUB, True),
+    (64, 40, (3, 3, 3), (1, 1, 1), (1, 4, 12, 12), torch.bfloat16, rt3d.ALGO_SIMT, True),
+    (3, 45, (1, 7, 7), (1, 2, 2), (1, 4, 32, 32), torch.bfloat16, rt3d.ALGO_AUTO, True),
+    (3, 64, (3, 3, 3), (1, 1, 1), (1, 4, 24, 24), torch.bfloat16, rt3d.ALGO_AUTO, True),
+    (24, 40, (3, 3, 3), (1, 1, 1), (1, 4, 12, 12), torch.float32, rt3d.ALGO_AUTO, True)]
+
+
+@pytest.mark.parametrize("cin,cout,k,stride,ext,dtype,algo,res", CALLS)
+def test_prepared_call_on_buffers_it_has_not_seen(cin, cout, k, stride, ext, dtype, algo, res):
+    """A call is prepared for its shapes, not for its buffers: new ones give the bits of a handle that has prepared nothing,
+    with and without a bias, and what depends on an address is refused as on a first call."""
+    spec = synth.ConvSpec("l", cin, cout, k, stride, tuple(a // 2 for a in k), True)
+    L = synth.make_layer(spec, 3, 0, 4, 4, "bernoulli", 0.5)
+    make = lambda: nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, dtype)
+
+    def call(lay, x, y, r):
+        return lay.fused(x, y, residual=r, algo=algo) if r is not None else lay(x, y, algo=algo)
+
+    def shifted(t, n=1):                                          # the same values 16 n bytes further on
+        flat = torch.zeros(t.numel() + 256, dtype=t.dtype, device="cuda")
+        at = n * 16 // t.element_size()
+        flat[at: at + t.numel()] = t.flatten()
+        return flat[at: at + t.numel()].view(t.shape)
+
+    lay = make()
+    for i in range(6):
+        x = shifted(nets.to_device(synth.make_input(i, ext + (cin,)), dtype), i)
+        y = shifted(torch.zeros(lay.out_shape(x), dtype=dtype, device="cuda"), 2 * i)
+        r = None
+        if res and i != 3:
+            r = shifted(torch.zeros_like(y), i + 1)
+            r[..., :cout] = torch.randn(r[..., :cout].shape, device="cuda")
+        want = torch.zeros_like(y)
+        other = make()
+        if i == 4:
+            lay.bias = other.bias = None
+        elif i == 5:
+            lay.bias = other.bias = torch.randn(cout, device="cuda")
+        call(other, x, want, r)
+        call(lay, x, y, r)
+        assert torch.equal(y, want), i
+    flat = torch.zeros(x.numel() + 64, dtype=dtype, device="cuda")
+    bad_x = flat[1: 1 + x.numel()].view(x.shape)                  # off the 16-byte boundary
+    flat = torch.zeros(y.numel() + 64, dtype=dtype, device="cuda")
+    bad_y = flat[1: 1 + y.numel()].view(y.shape)
+    both = torch.zeros(max(x.numel(), y.numel()), dtype=dtype, device="cuda")
+    over_x, over_y = both[: x.numel()].view(x.shape), both[: y.numel()].view(y.shape)
+    bad = [(bad_x, y, r), (x, bad_y, r), (over_x, over_y, r)]
+    if res:
+        bad += [(x, y, y), (x, y, bad_y)]
+    for args in bad:
+        launches = rt3d.rt3d_launch_count()
+        with pytest.raises(rt3d.Rt3dError) as e:
+            call(lay, *args)
+        assert e.value.status == rt3d.ERR_INVALID_ARG and rt3d.rt3d_launch_count() == launches
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+def test_prepared_pair_on_buffers_it_has_not_seen():
+    s = synth.ConvSpec("s", 64, 144, (1, 3, 3), (1, 1, 1), (0, 1, 1), True)
+    t = synth.ConvSpec("t", 144, 64, (3, 1, 1), (1, 1, 1), (1, 0, 0), True)
+    ls, lt = (synth.make_layer(sp, 3, i, 4, 4, "bernoulli", 0.4) for i, sp in enumerate((s, t)))
+    make = lambda: [nets.ConvLayer(sp, L["w"], L["bias"], L["mask"]) for sp, L in ((s, ls), (t, lt))]
+
+    def call(pair, x, y, r, biases=(True, True)):
+        rt3d.rt3d_conv2plus1d_fused(rt3d.tensor_desc(x), pair[0].packed, pair[0].bias if biases[0] else None, s.pad, True,
+                                    pair[1].packed, pair[1].bias if biases[1] else None, t.pad, True, rt3d.tensor_desc(y),
+                                    None if r is None else rt3d.tensor_desc(r))
+
+    pair = make()
+    for i in range(6):
+        x = nets.to_device(synth.make_input(i, (1, 4, 24, 24, 64)))
+        y, want = torch.zeros_like(x), torch.zeros_like(x)
+        r = torch.randn_like(x) if i % 2 else None
+        biases = (i != 4, i != 5)
+        call(make(), x, want, r, biases)
+        call(pair, x, y, r, biases)
+        assert torch.equal(y, want), i
+    assert rt3d.rt3d_last_plan()["kernel"] == 5
+    with pytest.raises(rt3d.Rt3dError):
+        call(pair, x, x, None)
+    assert rt3d.rt3d_last_device_status() == rt3d.OK
