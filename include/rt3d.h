@@ -51,7 +51,7 @@ typedef enum {
   RT3D_ERR_ALLOC = 5,                  /* host or device allocation failed                       */
   RT3D_ERR_CUDA = 6,                   /* a CUDA runtime / driver call failed                    */
   RT3D_ERR_TIMEOUT = 7,                /* a bounded device-side wait gave up (see rt3d_last_device_status) */
-  RT3D_ERR_WORKSPACE = 8,              /* rt3d_conv3d_sparse_noalloc: the call needs more than the fixed workspace */
+  RT3D_ERR_WORKSPACE = 8,              /* rt3d_conv3d_sparse_noalloc: the call exceeds that entry point's limit    */
   RT3D_ERR_NOT_PREPARED = 9            /* rt3d_conv3d_sparse_noalloc: handle was not prepared on this device */
 } rt3d_status;
 
@@ -276,7 +276,8 @@ rt3d_status rt3d_conv2plus1d_fused(const rt3d_tensor* x, const rt3d_packed* w_s,
  *     tile is 128 voxels x up to 256 channels and a K step is one kernel location x 64 input
  *     channels that some kernel group of the tile's channels keeps (the longest such list counts).  If S > 1 and (output tiles x S) partial tiles of 128 x n_tile floats exceed
  *     16 MiB, or there are more than 128 output tiles, the call is rejected with
- *     RT3D_ERR_WORKSPACE and nothing is launched (rt3d_conv3d_sparse has no such limit).
+ *     RT3D_ERR_WORKSPACE and nothing is launched (rt3d_conv3d_sparse has no such limit, and the split needs no
+ *     such memory: the limit stays because callers may rely on the refusal).
  *   - Results agree with rt3d_conv3d_sparse within the library's tolerance (the split count, and so
  *     the fp32 summation order, may differ); repeated calls give identical bits.
  */

@@ -1073,7 +1073,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     if (p->algo == RT3D_ALGO_AUTO && plan.n_splits > 1) return RT3D_ERR_UNSUPPORTED;
     plan.n_splits = 1;
   }
-  // CTA pairs: two tiles per MMA.  Worth it when every pair has work; forced by RT3D_ALGO_UMMA_PAIR.
+  // CTA pairs: two tiles per MMA.  Taken when every SM has a tile or the plan finds them faster; forced by RT3D_ALGO_UMMA_PAIR.
   bool use_pair = false;
   if (p->algo == RT3D_ALGO_UMMA_PAIR) {
     plan = UmmaPlan{default_n_tile(w->M), 1, true};
@@ -1086,7 +1086,8 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   }
   if (pooled && plan.n_tile % 32) return RT3D_ERR_UNSUPPORTED;      // pooled rows leave as whole 32-channel pieces
   // CTA pairs on bundles up to 128 wide with a kernel that is 2 or 3 deep: one deeper input tile per (kh, kw, chunk)
-  // (its box: among the boxes with as few tiles, one inside a single clip and as deep along t as possible)
+  // (its box: among the boxes with as few tiles, one inside a single clip and as deep along t as possible; where none suits,
+  // one inside a clip that reads less from L2 at up to a sixteenth more tiles: choose_box_grouped)
   bool use_ts = false;
   UmmaArgs probe = a;
   // (wide bundles: only kernels that are also wide in space; a 3x1x1 layer with 192-wide bundles lost 8 us of 43
@@ -1270,7 +1271,8 @@ rt3d_status conv2plus1d_impl(const rt3d_tensor* x, const rt3d_packed* ws, const 
 }  // namespace
 
 // ------------------------------------------------------------------ entry point without allocation
-// Size limit of rt3d_conv3d_sparse_noalloc's K split: output tiles and fp32 partial tiles of a call.
+// Size limit of rt3d_conv3d_sparse_noalloc's K split: output tiles and fp32 partial tiles of a call.  The split needs no such
+// memory; the limit is part of the interface, so that what was refused stays refused.
 #define RT3D_NOALLOC_PARTIAL_TILES 128                                   /* 128 x 256 fp32 each */
 #define RT3D_NOALLOC_PARTIAL_BYTES (RT3D_NOALLOC_PARTIAL_TILES * 128 * 256 * 4)   /* 16 MiB */
 

@@ -96,10 +96,10 @@ struct UmmaArgs {
   int sbw, sbh;                             // extents along w, h of the block of 32 voxels an epilogue warp owns
   int n_splits;                             // K splits per output tile (1 = none): the CTAs of one cluster
   int tail_workers;                         // CTA-pair kernel: pairs sharing the left-over items of the last round (0 = off)
-  float* tail_scratch;                      // device, [tail_workers][2 shares][2 CTAs][n_tile][128] fp32 partial tiles
-  int32_t* tail_flags;                      // device, [tail_workers][2][2][4 warps] "partial written" flags, zero between launches
+  float* tail_scratch;                      // device, [tail_workers][2 CTAs] fp32 partial tiles of 128 x n_tile
+  int32_t* tail_flags;                      // device, [tail_workers][2 CTAs][8 epilogue warps] "partial written" flags, zero between launches
   // CTA-pair kernel, t-grouped layout (ts != 0): steps that differ only in kt share one staged input tile that is
-  // Kt - 1 frames deeper (the xmap's box); needs temporal stride 1, one clip per box and bundles up to 128 wide.
+  // Kt - 1 frames deeper (the xmap's box), one tile per phase of the temporal stride (1 or 2); needs one clip per box.
   int ts;
   const int32_t* grp_ptr;                   // device, [n_bundles + 1]
   const int32_t* grp_first;                 // device, first step of each group + sentinel

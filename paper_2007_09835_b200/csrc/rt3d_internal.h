@@ -142,12 +142,12 @@ struct F32Layout {
 // Per-device copies of a handle's arrays.
 struct DeviceBlob {
   int device = -1;
-  void* canonical = nullptr;         // owns the canonical arrays (CUDA-core kernel), uploaded on its first use
+  void* canonical = nullptr;         // owns the canonical arrays and the first tensor-core layout built from them
   int32_t* group_ptr = nullptr;
   uint16_t* pos_idx = nullptr;
   void* tiles = nullptr;
   struct Umma {
-    void* base = nullptr;                       // owns the index arrays
+    void* base = nullptr;                       // owns the tiles and index arrays, unless they lie in `canonical`
     void* wtiles = nullptr;
     int32_t* step_ptr = nullptr;
     int32_t* steps = nullptr;

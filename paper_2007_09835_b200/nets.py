@@ -173,7 +173,8 @@ def _wait(stream, ev):
 
 class _NotedForward:
     """Base of the networks.  The calls of a forward pass are noted when an input of its shape is seen first, and issued
-    by one library call from then on (R(2+1)D: 33 calls, 590 us of Python; S3D: 90 calls and 36 stream events, 1730 us).
+    by one library call from then on (R(2+1)D: 33 calls, 590 us of Python; S3D with every convolution a call
+    of its own: 90 calls and 36 stream events, 1730 us).
     Noted passes are dropped when a layer, the memory of a bias or of the output, a switch of the network or its set of
     buffers has changed since."""
 

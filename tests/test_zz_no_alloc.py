@@ -3,11 +3,11 @@
 Who needs it: code that runs a layer from inside a real-time / latency-critical loop, or from a
 thread that must never block on the CUDA allocator (cudaMalloc synchronises the whole device), or
 in a process whose device memory is budgeted by another component.  Such a caller prepares the
-weights once up front and afterwards uses this entry point, whose K-split scratch is a fixed array
-inside the library.  The test calls it through the C ABI twice in a row and compares with the
+weights once up front and afterwards uses this entry point, whose K split exchanges its partial
+sums through shared memory.  The test calls it through the C ABI twice in a row and compares with the
 regular entry point and, for one case, with the CPU oracle; it checks that device memory does not move
-across the first call, that the K-split path through the fixed workspace really ran, and the two refusals
-(workspace too small, handle not prepared).
+across the first call, that the K-split path really ran, and the two refusals
+(beyond the size limit, handle not prepared).
 This file sorts last on purpose, so a run that stops at the first failure has already run
 every other test; it does not depend on any of them.
 """
@@ -49,7 +49,7 @@ def test_noalloc_matches_regular_entry_point_twice(shape, cin, cout, split):
     scale = float(y_ref.float().abs().max())
     assert scale > 0
     outs = []
-    for rep in range(2):                                # two calls in a row share the library's workspace
+    for rep in range(2):                                # two calls in a row give the same bits
         y = torch.full_like(y_ref, 123.0)
         torch.cuda.synchronize()
         free_before, allocs_before = torch.cuda.mem_get_info()[0], rt3d.rt3d_alloc_count()
@@ -72,7 +72,7 @@ def test_noalloc_matches_regular_entry_point_twice(shape, cin, cout, split):
 
 
 def test_noalloc_refuses_what_it_cannot_do():
-    # 26 output tiles x 5 splits x 128 KiB partial tiles = 16.25 MiB: more than the 16 MiB workspace
+    # 26 output tiles x 5 splits x 128 KiB partial tiles = 16.25 MiB: more than the 16 MiB limit
     spec, lay = _layer(1152, 512, (3, 3, 3), 7)
     x = nets.to_device(synth.make_input(802, (4, 2, 14, 14, 1152)))
     y = lay.alloc_out(x)
