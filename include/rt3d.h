@@ -370,6 +370,7 @@ rt3d_status rt3d_conv3d_cost(const rt3d_tensor* x, const rt3d_packed* w, const r
  *                5 fused (2+1)D kernel (rt3d_conv2plus1d_fused; n_tile = intermediate width),
  *                6 tensor-core sub-tile kernel (RT3D_ALGO_UMMA_SUB)
  *                7 tensor-core CTA-pair kernel, one deeper input tile per (kh, kw, chunk) shared by all kt
+ *                8 fp32 on the tensor cores, every value as three bf16 ones (fp32 calls under RT3D_ALGO_AUTO)
  *   n_tile       output channels per accumulator tile (tensor-core kernels, else 0)
  *   n_splits     K splits per output tile in the single-CTA kernel (1 = none)
  *   tail_workers CTA pairs that share, cut along K, the output tiles which do not fill a last round
@@ -415,12 +416,15 @@ void rt3d_plan_end(void);
  * RT3D_DEBUG_T_GROUPS: 0 switches off the CTA-pair kernel's variant that stages one deeper input tile per
  * (kh, kw, channel chunk) for all kt (plan kernel 7), so that it can be compared with the step-per-location
  * form (kernel 2) on the same handle; default 1.
+ * RT3D_DEBUG_F32_SPLIT: fp32 calls on the tensor cores (plan kernel 8): 0 never, 1 where they are expected to be faster
+ * (default), 2 wherever they can run.
  * RT3D_DEBUG_POISON: runs, on the default stream, a kernel that fills the shared memory and the tensor memory of
  * every SM with the 32-bit pattern `value` (e.g. 0x7FC07FC0: two bf16 NaNs) and waits for it: a kernel launched next
  * that reads shared or tensor memory it did not write itself (padding multiplied by zero weights, say) then
  * produces NaNs instead of depending silently on what ran before it.  The partial-tile scratch of every handle's
  * tail splits on the device is set to all ones (NaNs) as well.  Device work only; nothing else changes. */
-enum { RT3D_DEBUG_WAIT_CYCLES = 1, RT3D_DEBUG_DROP_LAST_LOAD = 2, RT3D_DEBUG_T_GROUPS = 3, RT3D_DEBUG_POISON = 4 };
+enum { RT3D_DEBUG_WAIT_CYCLES = 1, RT3D_DEBUG_DROP_LAST_LOAD = 2, RT3D_DEBUG_T_GROUPS = 3, RT3D_DEBUG_POISON = 4,
+       RT3D_DEBUG_F32_SPLIT = 5 };
 rt3d_status rt3d_debug_set(int what, long long value);
 /* Diagnostics.  RT3D_DEBUG_WAIT_SITE: after a synchronisation of the device, the number of the wait inside a
  * kernel that gave up since the last rt3d_last_device_status (0 = none; the numbers are the last argument of the

@@ -66,6 +66,8 @@ std::atomic<long long> g_debug_wait_cycles{-1};      // -1: not set yet (RT3D_DE
 std::atomic<int> g_debug_drop_last_load{0};
 // t-grouped CTA-pair variant: on unless the environment says RT3D_T_GROUPS=0; RT3D_DEBUG_T_GROUPS switches it at run time
 std::atomic<int> g_ts_enabled{[] { const char* e = getenv("RT3D_T_GROUPS"); return (e && e[0] == '0') ? 0 : 1; }()};
+// fp32 on the tensor cores: 0 never, 1 where it is expected to be faster, 2 wherever it can run (tests, comparisons)
+std::atomic<int> g_f32_split{1};
 long long debug_wait_cycles() {
   long long v = g_debug_wait_cycles.load();
   if (v < 0) {
@@ -385,7 +387,7 @@ rt3d_status get_canonical(rt3d_packed* h, DeviceBlob* b) {
 
 rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, DeviceBlob::Umma** out) {
   std::lock_guard<std::mutex> lock(h->mu);
-  DeviceBlob::Umma& u = blob->umma[L->n_tile + (L->t_groups ? 4096 : 0)];
+  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, L->t_groups)];
   if (!u.ready) {
     const size_t wbytes = L->steps.size() * size_t(L->n_tile) * kChunk * 2;
     // The canonical arrays go to the device once, a quarter to a third of the size of the zero-filled tiles, and a kernel
@@ -425,6 +427,34 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return fail();
     }
+    u.ready = true;
+  }
+  *out = &u;
+  return RT3D_OK;
+}
+
+// Device copy of the fp32 tensor-core kernel's layout, with the canonical arrays beside it.
+rt3d_status get_split_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, bool pair, DeviceBlob::Umma** out) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, false)];
+  if (!u.ready) {
+    const size_t wbytes = L->steps.size() * size_t(L->n_tile) * 192;
+    const bool shared = !blob->canonical;
+    void** const base = shared ? &blob->canonical : &u.base;
+    int32_t* slots = nullptr;
+    Upload up;
+    up.reserve(&u.wtiles, wbytes + 1024);
+    if (shared) add_canonical(h, blob, up);
+    up.add(&u.step_ptr, L->step_ptr);
+    up.add(&u.steps, L->steps);
+    up.add(&slots, L->slots);
+    const rt3d_status s = up.run(base, wbytes == 0);
+    if (s != RT3D_OK) return s;
+    const auto fail = [&] { weight_free(*base, false); *base = nullptr; return RT3D_ERR_CUDA; };
+    if (wbytes && (launch_fill_split_tiles(blob->group_ptr, blob->pos_idx, static_cast<const float*>(blob->tiles), slots, h->M, h->N, h->Ks,
+                                           h->g_m, h->g_n, h->Q, h->P * h->Q, h->nnz, L->n_tile, pair ? 2 : 1, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
+                   uploads_done() != cudaSuccess))
+      return fail();
     u.ready = true;
   }
   *out = &u;
@@ -935,6 +965,86 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
   return RT3D_OK;
 }
 
+// Whether an fp32 call is expected to take less time on the tensor cores than on the CUDA cores.  Both models are fitted to 92
+// random layers (8-160 input and 16-160 output channels, 0.2-1 kept, 6-530 us) on B200.  CUDA cores: the cycles of the plan
+// search at 0.656 ns, 3 us around them (half of the layers within 0.83-1.1 of it).  Tensor cores: 8 us around the rounds of
+// items over the SMs, per round its steps and the output of a tile; a step costs 0.31 us at up to 48 columns, 0.44 at 128
+// (0.85-1.1).  The margin leaves ties where they were: 27 -> 145 channels 3x3x3 on 2 x 4 x 16 x 44 24.2 us and 24.3.  Taken by
+// this rule the 92 layers gain 1.19x in the mean (the better of both each time: 1.23x), 64 -> 128 on 2 x 16 x 56 x 56 3.1x.
+// Up to 16 input channels stay on the CUDA cores: half of every step would be empty, and the tests of the register-blocked
+// kernel expect it there.  (It costs 16 -> 74 channels 3x3x3 dense on 16 x 51 x 35 35 us instead of 20.)
+bool split_is_faster(const rt3d_packed* w, const F32SplitArgs& a, int sm_count) {
+  if (w->N <= 16) return false;
+  const double density = double(w->nnz) / (double(w->P) * w->Q * w->Ks);
+  const double groups = double(std::max(1, kSplitChunk / w->g_n)) * std::max(1, a.n_tile / w->g_m);     // that share a step
+  const double steps = double(w->Ks) * ceil_div(w->N, kSplitChunk) * (w->is_dense ? 1.0 : 1.0 - std::pow(1.0 - density, groups));
+  const int ctas = a.pair ? 2 : 1;
+  const double tiles = double(a.tiles_n) * a.tiles_t * a.tiles_h * a.tiles_w;
+  const double rounds = std::ceil(std::ceil(tiles / ctas) * a.n_bundles / (sm_count / ctas));
+  const double step_us = a.n_tile <= 48 ? 0.31 : a.n_tile <= 64 ? 0.34 : a.n_tile <= 96 ? 0.36 : 0.44;
+  const double tile_us = a.n_tile <= 48 ? 0.5 : a.n_tile <= 64 ? 2.0 : a.n_tile <= 96 ? 3.2 : 4.0;
+  F32Plan plans[kF32MaxPlans];
+  double cycles = 0.0;
+  conv_f32_plans(a.g, density, sm_count, plans, &cycles);
+  // group sizes that are not multiples of four run the first CUDA-core kernel, which is several times slower
+  const double cuda_core_us = (3.0 + cycles * 0.656e-3) * (f32_layout_possible(w) ? 1.0 : 3.0);
+  return 8.0 + rounds * (steps * step_us + tile_us) < 0.95 * cuda_core_us;
+}
+
+// fp32 on the tensor cores, each value as three bf16 ones.
+// *launched = false (and RT3D_OK) when the handle or the shape does not suit it or the CUDA cores are faster.
+rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g, const float* bias,
+                      rt3d_tensor* y, const void* res_data, int res_pitch, Submit& submit, bool* launched) {
+  *launched = false;
+  const int mode = g_f32_split.load();
+  if (mode == 0 || d->cc_major != 10 || w->dtype != RT3D_F32 || x->c_stride % 4 || y->c_stride % 4 || (res_data && res_pitch % 4)) return RT3D_OK;
+  if (g.st > 8 || g.sh > 8 || g.sw > 8 || int64_t(x->w) * x->c_stride * 4 >= (int64_t(1) << 40)) return RT3D_OK;
+  if (int64_t(g.n) * g.To * g.Ho * g.Wo > 0x7fffffff) return RT3D_OK;
+  if (int64_t(w->Ks) * w->N > 32768) return RT3D_OK;       // a row computed again stays far below the limit of the others' waits
+  F32SplitArgs a;
+  a.g = g;
+  a.box = choose_box(g);
+  a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
+  a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
+  const int bundles = ceil_div(w->M, 128);
+  a.n_tile = round_up(ceil_div(w->M, bundles), 16); a.n_bundles = ceil_div(w->M, a.n_tile);
+  a.period = a.n_tile > 64 ? 8 : 4;
+  if (!umma_f32_plan(&a) || (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w * a.n_bundles > (1ll << 30)) return RT3D_OK;
+  if (mode == 1 && !split_is_faster(w, a, d->sm_count)) return RT3D_OK;
+  const UmmaLayout* L = get_split_layout(w, a.n_tile);
+  if (!L) return RT3D_OK;
+  DeviceBlob::Umma* u = nullptr;
+  rt3d_status s = get_split_blob(w, blob, L, a.pair != 0, &u);
+  if (s != RT3D_OK) return s;
+  a.last_chunk = L->n_chunks - 1;
+  a.last_k16 = w->N - a.last_chunk * kSplitChunk > 16 ? 2 : 1;
+  a.step_ptr = u->step_ptr; a.steps = u->steps; a.wtiles = static_cast<const unsigned char*>(u->wtiles);
+  a.x = nullptr; a.y = nullptr; a.bias = nullptr; a.residual = nullptr; a.rcs = res_pitch;
+  a.group_ptr = blob->group_ptr; a.pos_idx = blob->pos_idx; a.tiles = static_cast<const float*>(blob->tiles);
+  a.g_m = w->g_m; a.g_n = w->g_n; a.Q = w->Q;
+  a.sched = d->sched;
+  const cuuint64_t cs = cuuint64_t(x->c_stride) * 4;
+  cuuint64_t dims[5] = {cuuint64_t(x->c), cuuint64_t(x->w), cuuint64_t(x->h), cuuint64_t(x->t), cuuint64_t(x->n)};
+  cuuint64_t strides[4] = {cs, cs * x->w, cs * x->w * x->h, cs * x->w * x->h * x->t};
+  cuuint32_t bx[5] = {cuuint32_t(kSplitChunk), cuuint32_t(a.box.bw * g.sw), cuuint32_t(a.box.bh * g.sh), cuuint32_t(a.box.bt * g.st),
+                      cuuint32_t(a.box.bn)};
+  cuuint32_t estr[5] = {1, cuuint32_t(g.sw), cuuint32_t(g.sh), cuuint32_t(g.st), 1};
+  CUtensorMap xmap;
+  if (g_encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, x->data, dims, strides, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return RT3D_ERR_CUDA;
+  *launched = true;
+  const int sms = d->sm_count;
+  return submit(rt3d_plan_info{8, a.n_tile, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+    const PlacedMaps m(xmap, c.x, xmap, nullptr);
+    if (!m.ok) return cudaErrorInvalidValue;
+    F32SplitArgs now = a;
+    now.x = static_cast<const float*>(c.x); now.y = static_cast<float*>(c.y);
+    now.bias = c.bias; now.residual = static_cast<const float*>(c.res);
+    return launch_conv_umma_f32(now, &m.x, sms, st);
+  });
+}
+
 // Register-blocked fp32 kernel: every fp32 call whose kernel groups are whole 4 x 4 tiles.
 // *launched = false (and RT3D_OK) when the handle or the shape cannot use it.
 rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
@@ -942,7 +1052,8 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   *launched = false;
   if (!f32_layout_possible(w)) return RT3D_OK;
   F32Plan plans[kF32MaxPlans];
-  const int n_plans = conv_f32_plans(g, double(w->nnz) / (double(w->P) * w->Q * w->Ks), d->sm_count, plans);
+  double cycles = 0.0;
+  const int n_plans = conv_f32_plans(g, double(w->nnz) / (double(w->P) * w->Q * w->Ks), d->sm_count, plans, &cycles);
   F32Args a;
   a.g = g;
   for (int i = 0; i < n_plans; ++i) {
@@ -1022,6 +1133,10 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   if (!use_umma) {
     if (pooled) return RT3D_ERR_UNSUPPORTED;
     bool launched = false;
+    if (p->algo == RT3D_ALGO_AUTO) {
+      s = try_split(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
+      if (s != RT3D_OK || launched) return s;
+    }
     s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
     if (s != RT3D_OK || launched) return s;
     if ((s = get_canonical(w, blob)) != RT3D_OK) return s;
@@ -1755,6 +1870,7 @@ rt3d_status rt3d_debug_set(int what, long long value) {
   if (what == RT3D_DEBUG_WAIT_CYCLES) { if (value < 0) return RT3D_ERR_INVALID_ARG; g_debug_wait_cycles.store(value); return RT3D_OK; }
   if (what == RT3D_DEBUG_DROP_LAST_LOAD) { g_debug_drop_last_load.store(value != 0); return RT3D_OK; }
   if (what == RT3D_DEBUG_T_GROUPS) { g_ts_enabled.store(value != 0); return RT3D_OK; }
+  if (what == RT3D_DEBUG_F32_SPLIT) { if (value < 0 || value > 2) return RT3D_ERR_INVALID_ARG; g_f32_split.store(int(value)); return RT3D_OK; }
   if (what == RT3D_DEBUG_POISON) {
     DeviceState* d = nullptr;
     rt3d_status s = get_device_state(&d);

@@ -18,6 +18,9 @@ struct ConvGeom {
   int relu;
 };
 
+// Output-voxel box of one tensor-core tile: bn*bt*bh*bw <= 128 voxels.
+struct TileBox { int bn, bt, bh, bw; };
+
 // CUDA-core kernel driven by the canonical packed arrays.  dtype: 0 fp32, 1 bf16.
 // residual: tensor of the output's extents and dtype (pitch rcs) added before the ReLU, or nullptr.
 cudaError_t launch_conv_simt(int dtype, const ConvGeom& g, const void* x, void* y,
@@ -53,9 +56,43 @@ struct F32Layout;
 // Candidate (voxels per thread, row sets per block, parts, output box) for a call, best first (density = kept
 // share of the (group, location) places); conv_f32_fill says whether one's staging fits shared memory.
 constexpr int kF32MaxPlans = 40;
-int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]);
+// `cycles`: what the best one is expected to take.
+int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans], double* cycles);
 bool conv_f32_fill(const F32Plan& plan, const F32Layout& L, F32Args* a);
 cudaError_t launch_conv_f32(const F32Args& a, const F32Plan& plan, cudaStream_t stream);
+
+// fp32 on the tensor cores, every value as three bf16 ones (umma_conv_f32.cu).
+struct F32SplitArgs {
+  ConvGeom g;
+  TileBox box;
+  int n_tile, n_bundles;
+  int tiles_n, tiles_t, tiles_h, tiles_w;
+  const int32_t* step_ptr;            // device, [n_bundles + 1]
+  const int32_t* steps;               // device, kernel location and chunk of 32 input channels
+  int last_chunk, last_k16;           // the last chunk and how many of its two halves of 16 channels exist
+  const unsigned char* wtiles;        // device, n_tile * 192 bytes a step
+  int period;                         // steps that one accumulator takes before it is drained
+  // filled in by umma_f32_plan:
+  int pair;                           // whether CTA pairs run (and a step's weights lie in two halves)
+  int inputs, stages, slots;          // staged inputs, weight stages, A operands in tensor memory
+  const float* x;
+  float* y;
+  const float* bias;                  // or nullptr
+  const float* residual;              // or nullptr, pitch rcs
+  int rcs;
+  const int32_t* group_ptr;           // canonical arrays, for rows whose values three bf16 cannot hold
+  const uint16_t* pos_idx;
+  const float* tiles;
+  int g_m, g_n, Q;
+  int32_t* sched;                     // [2] = error word
+};
+bool umma_f32_plan(F32SplitArgs* a);
+// xmap: input boxes of 32 channels, 128-byte swizzle.
+cudaError_t launch_conv_umma_f32(const F32SplitArgs& a, const void* xmap, int sm_count, cudaStream_t stream);
+// Fills the zeroed weights of that kernel, n_tile * 192 bytes a step, from the canonical arrays, on the legacy default stream.
+cudaError_t launch_fill_split_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const float* tiles, const int32_t* slots,
+                                    int M, int N, int Ks, int g_m, int g_n, int Q, int n_groups, int64_t nnz, int n_tile,
+                                    int halves, int n_chunks, void* wtiles, size_t bytes);
 
 cudaError_t launch_maxpool3d(int dtype, const void* x, int n, int t, int h, int w, int c, int xcs,
                              int kt, int kh, int kw, int st, int sh, int sw, int pt, int ph, int pw,
@@ -72,9 +109,6 @@ cudaError_t launch_add_relu(int dtype, const void* a, int acs, const void* b, in
 cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const void* tiles, const int32_t* slots,
                                    int M, int N, int Ks, int g_m, int g_n, int Q, int n_groups, int64_t nnz, int n_tile,
                                    int n_chunks, void* wtiles, size_t bytes);
-
-// Output-voxel box of one tensor-core tile: bn*bt*bh*bw <= 128 voxels.
-struct TileBox { int bn, bt, bh, bw; };
 
 // Everything the tcgen05 kernel needs besides the two tensor maps.
 struct UmmaArgs {

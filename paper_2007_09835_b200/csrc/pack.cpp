@@ -114,12 +114,9 @@ static void two_passes(int n, int64_t work, int64_t grain, const F& first, const
 // here, for checks).  Steps are ordered by location, then chunk.
 // `t_groups`: the order is (kh, kw), chunk, kt instead, and the steps that differ only in kt form a
 // group (grp_ptr / grp_first): the CTA-pair kernel stages one input tile, Kt - 1 frames deeper, per group.
-const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
-  if (!umma_layout_possible(p)) return nullptr;
-  if (n_tile <= 0) n_tile = default_n_tile(p->M);
-  if (n_tile % 16 || n_tile > 256) return nullptr;
+static const UmmaLayout* step_layout(rt3d_packed* p, int n_tile, bool t_groups, int chunk) {
   std::lock_guard<std::mutex> lock(p->mu);
-  const int key = n_tile + (t_groups ? 4096 : 0);
+  const int key = umma_key(n_tile, t_groups);
   auto it = p->umma_layouts.find(key);
   if (it != p->umma_layouts.end()) return &it->second;
 
@@ -128,7 +125,7 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
   L.t_groups = t_groups;
   if (t_groups) L.grp_ptr.assign(1, 0);
   L.n_bundles = ceil_div(p->M, n_tile);
-  L.n_chunks = ceil_div(p->N, kChunk);
+  L.n_chunks = ceil_div(p->N, chunk);
   L.step_ptr.assign(L.n_bundles + 1, 0);
   const int Ks = p->Ks;
   std::vector<int32_t> slot(size_t(Ks) * L.n_chunks);
@@ -141,7 +138,7 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
       for (int q = 0; q < p->Q; ++q) {
         const int c_lo = q * p->g_n, c_hi = std::min(p->N, c_lo + p->g_n), n_chunks = L.n_chunks;
         const uint16_t* const end = p->pos_idx.data() + p->group_ptr[size_t(pr) * p->Q + q + 1];
-        for (int ch = c_lo / kChunk; ch <= (c_hi - 1) / kChunk; ++ch) {
+        for (int ch = c_lo / chunk; ch <= (c_hi - 1) / chunk; ++ch) {
           int32_t* const mark = slot.data() + ch;
           for (const uint16_t* e = p->pos_idx.data() + p->group_ptr[size_t(pr) * p->Q + q]; e < end; ++e) mark[size_t(*e) * n_chunks] = 0;
         }
@@ -177,6 +174,38 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
   if (t_groups) L.grp_first.push_back(int32_t(L.steps.size()));     // sentinel: end of the last group
   auto res = p->umma_layouts.emplace(key, std::move(L));
   return &res.first->second;
+}
+
+const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
+  if (!umma_layout_possible(p)) return nullptr;
+  if (n_tile <= 0) n_tile = default_n_tile(p->M);
+  if (n_tile % 16 || n_tile > 256) return nullptr;
+  return step_layout(p, n_tile, t_groups, kChunk);
+}
+
+// Three bf16 parts hold a weight to the last bit if it is neither huge nor so small that its last bits fall out of their range.
+static bool splits_exactly(const float* w, int64_t n) {
+  uint32_t lo = 0xffffffffu, hi = 0;                       // smallest magnitude but zero, largest one
+  for (int64_t i = 0; i < n; ++i) {
+    uint32_t u;
+    std::memcpy(&u, w + i, 4);
+    u &= 0x7fffffffu;
+    hi = std::max(hi, u);
+    lo = std::min(lo, u - 1u);                             // zero: the largest
+  }
+  return hi < 0x7b800000u && (lo == 0xffffffffu || lo >= 0x0d800000u - 1u);       // 2^120, 2^-100
+}
+
+const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile) {
+  if (p->dtype != RT3D_F32 || p->Kt > 63 || p->Kh > 63 || p->Kw > 63 || ceil_div(p->N, kSplitChunk) > 4095) return nullptr;
+  if (n_tile % 16 || n_tile < 16 || n_tile > 128) return nullptr;
+  {
+    std::lock_guard<std::mutex> lock(p->mu);
+    if (p->splits_exactly < 0)
+      p->splits_exactly = splits_exactly(reinterpret_cast<const float*>(p->tiles.data()), p->nnz * p->g_m * p->g_n) ? 1 : 0;
+    if (!p->splits_exactly) return nullptr;
+  }
+  return step_layout(p, n_tile, false, kSplitChunk);
 }
 
 // The weight tiles of a layout, as the device kernel builds them.

@@ -17,6 +17,7 @@ namespace rt3d {
 constexpr int kMaxGroup = 256;      // g_m, g_n <= 256 (pack, tensor-core kernels)
 constexpr int kMaxGroupSimt = 8;    // the CUDA-core kernel keeps one group row in registers: g_m, g_n <= 8
 constexpr int kChunk = 64;          // input channels per tensor-core K step (one 128-byte swizzle row of bf16)
+constexpr int kSplitChunk = 32;     // the same of the fp32 tensor-core kernel (one 128-byte row of fp32)
 constexpr int kTileM = 128;         // output voxels per tensor-core tile (TMEM lanes)
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
@@ -191,7 +192,8 @@ struct rt3d_packed {
   std::vector<uint16_t> pos_idx;
   rt3d::RawBytes tiles;              // nnz * g_m * g_n elements of float or bf16 bits
   std::mutex mu;                     // guards the lazily built members below
-  std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by n_tile (+ 4096: the t-grouped order)
+  std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by umma_key
+  int splits_exactly = -1;           // fp32: whether three bf16 parts hold every weight (-1: not looked at yet)
   std::map<int, rt3d::SubLayout> sub_layouts;     // keyed by n_tile
   std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw (+ 1024: packed), built on first use
   std::unique_ptr<rt3d::F32Layout> f32_layout;        // built on first use
@@ -206,11 +208,14 @@ namespace rt3d {
 // The weight tiles [steps.size()][n_tile][64] of a layout on the host (checks; the device fills its own).
 std::vector<uint16_t> fill_umma_tiles(const rt3d_packed* p, const UmmaLayout& L);
 
+inline int umma_key(int n_tile, bool t_groups) { return n_tile + (t_groups ? 4096 : 0); }
 // Default bundle width for M output channels: as few bundles as possible with n_tile <= 256.
 int default_n_tile(int M);
 // Builds (or returns the cached) tensor-core layout; nullptr if the handle cannot use it.
 const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups = false);
 bool umma_layout_possible(const rt3d_packed* p);
+// Steps of 32 input channels for the fp32 tensor-core kernel; nullptr if the handle or its weights do not suit it.
+const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile);
 // Builds (or returns the cached) layout of the sub-tile kernel; nullptr if the handle cannot use it.
 const SubLayout* get_sub_layout(rt3d_packed* p, int n_tile);
 

@@ -317,7 +317,7 @@ double choose_box_f32(const ConvGeom& g, int lanes, int voxels, double weight, F
 
 // Cycles of the busiest SM for every variant, fitted to timings on B200: an entry costs a scheduler 25 + V (4 + 10 h) with
 // four warps at work (h = tiles per entry) and a warp by itself 45 + V (12 + 30 h); a stage costs its copies and barriers, adding up the parts 220 V for each and 800.
-static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
+static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans], double* cycles) {
   const int Ks = g.Kt * g.Kh * g.Kw, n_rows = ceil_div(g.M, 4), n_quads = ceil_div(g.c, 4), quads = f32_stage_quads(Ks);
   const int n_stages = ceil_div(n_quads, quads);
   double cost[kF32MaxPlans];
@@ -351,23 +351,26 @@ static int search_plans(const ConvGeom& g, double density, int sm_count, F32Plan
       cost[at] = t; plans[at] = p;
       ++n;
     }
+  *cycles = n > 0 ? cost[0] : 0.0;
   return n;
 }
 
-int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans]) {
+int conv_f32_plans(const ConvGeom& g, double density, int sm_count, F32Plan plans[kF32MaxPlans], double* cycles) {
   // The search takes 0.1 ms; a call in chunks asks for the same shape for every chunk.
-  struct Entry { ConvGeom g; double density; int n; F32Plan plans[kF32MaxPlans]; };
+  struct Entry { ConvGeom g; double density, cycles; int n; F32Plan plans[kF32MaxPlans]; };
   thread_local Entry cache[4];
   thread_local int next = 0;
   for (const Entry& e : cache)
     if (e.n > 0 && memcmp(&e.g, &g, sizeof(g)) == 0 && e.density == density) {
       std::copy(e.plans, e.plans + e.n, plans);
+      *cycles = e.cycles;
       return e.n;
     }
   Entry& e = cache[next];
   next = (next + 1) % 4;
   e.g = g; e.density = density;
-  e.n = search_plans(g, density, sm_count, e.plans);
+  e.n = search_plans(g, density, sm_count, e.plans, &e.cycles);
+  *cycles = e.cycles;
   std::copy(e.plans, e.plans + e.n, plans);
   return e.n;
 }

@@ -1,0 +1,100 @@
+"""fp32 convolution on the tensor cores (plan kernel 8: every value as three bf16 ones) against the oracle, at the edges of its
+tiles, chunks, bundle widths and accumulator periods.
+
+Tolerance: a product of two values split three ways is wrong by less than 2^-23 of it, the sums are fp32 over at most 8 steps of
+32 channels and fp32 from there on: 2e-6 of the largest output, as for the CUDA-core kernel, is several times what the longest
+sum here shows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import rt3d_synth as synth
+import paper_2007_09835_b200 as rt3d
+from paper_2007_09835_b200 import nets
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def everywhere():
+    rt3d.rt3d_debug_set(rt3d.DEBUG_F32_SPLIT, 2)
+    yield
+    rt3d.rt3d_debug_set(rt3d.DEBUG_F32_SPLIT, 1)
+
+
+@pytest.mark.parametrize("x,cin,cout,k,stride,group,kind,density", [
+    ((1, 1, 1, 1), 4, 4, (1, 1, 1), (1, 1, 1), (4, 4), "none", None),               # one voxel, one step of half a chunk
+    ((1, 8, 28, 28), 16, 32, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.5),       # 16 channels: half chunks only; 32 columns
+    ((2, 3, 9, 11), 17, 33, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.4),        # just above both; ragged outputs, 48 columns
+    ((3, 5, 9, 11), 37, 43, (3, 3, 3), (2, 2, 2), (4, 4), "bernoulli", 0.4),        # a last chunk of half; strided; odd step count
+    ((2, 4, 16, 16), 64, 64, (1, 3, 3), (1, 2, 2), (8, 4), "bernoulli", 0.3),       # 64 columns: shared small products
+    ((1, 4, 33, 31), 30, 65, (1, 3, 3), (1, 1, 1), (8, 4), "bernoulli", 0.3),       # pairs: 80 columns, the second set of 32
+    ((2, 9, 17, 5), 70, 96, (3, 1, 1), (1, 1, 1), (8, 8), "bernoulli", 0.2),        # 96 columns, an odd number of tiles
+    ((2, 6, 14, 13), 34, 97, (1, 1, 1), (2, 2, 2), (4, 4), "none", None),           # 112 columns, one step a hand-shake
+    ((1, 6, 20, 20), 96, 128, (3, 3, 3), (1, 1, 1), (4, 4), "bernoulli", 0.4),      # 81 steps: more than one segment of 64
+    ((1, 5, 12, 12), 70, 150, (3, 3, 3), (1, 1, 1), (3, 5), "bernoulli", 0.4),      # two bundles; groups that no other fp32 kernel blocks
+    ((1, 2, 6, 6), 64, 256, (3, 3, 3), (1, 1, 1), (8, 4), "vanilla_total", 40),     # bundles with few steps
+    ((1, 2, 6, 6), 24, 40, (3, 3, 3), (1, 1, 1), (4, 4), "exact_total", 1),         # one place kept in all
+    ((2, 2, 6, 6), 64, 200, (3, 3, 3), (1, 1, 1), (8, 8), "exact_total", 1),        # a bundle without any step
+    ((5, 16, 40, 40), 33, 48, (3, 1, 1), (1, 1, 1), (4, 4), "bernoulli", 0.4)])     # several items per SM
+def test_split_kernel_matches_oracle(everywhere, x, cin, cout, k, stride, group, kind, density):
+    spec = synth.ConvSpec("f32", cin, cout, k, stride, tuple(v // 2 for v in k), True)
+    L = synth.make_layer(spec, 8, cin + cout, group[0], group[1], kind, density)
+    xs = synth.make_input(8, x + (cin,))
+    res = synth.uniform_pm1(77, (x[0],) + spec.out_extent(*x[1:]) + (cout,))
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], group[0], group[1], torch.float32, dense=kind == "none")
+    xd = nets.to_device(xs, torch.float32)
+    xd[..., cin:] = float("nan")                           # padding channels of the input are never read as data
+    y = torch.full(lay.out_shape(xd), 3.0, device="cuda")
+    for residual in (None, res):
+        if residual is None:
+            lay(xd, y, relu=False)
+        else:
+            lay.fused(xd, y, residual=nets.to_device(res, torch.float32), relu=True)
+        assert rt3d.rt3d_last_plan()["kernel"] == 8 and rt3d.rt3d_last_device_status() == rt3d.OK
+        ref = oracle.conv3d(xs, L["w"], L["mask"], L["bias"], spec.stride, spec.pad, False)
+        if residual is not None:
+            ref = np.maximum(ref + res, 0.0)
+        got = y.cpu().numpy()
+        assert np.abs(got[..., :cout] - ref).max() <= 2e-6 * np.abs(ref).max()
+        assert (got[..., cout:] == 3.0).all()              # those of the output are not written
+
+
+@pytest.mark.parametrize("cin,cout", [(40, 24), (40, 64), (40, 120)])
+def test_values_that_three_bf16_cannot_hold(everywhere, cin, cout):
+    """Infinities, NaNs, values next to the largest float and tiny ones: every output is what the CUDA-core kernel gives, up to
+    the order of its sums, and what pruned weights would have met has no effect."""
+    spec = synth.ConvSpec("f32", cin, cout, (3, 3, 3), (1, 1, 1), (1, 1, 1), False)
+    L = synth.make_layer(spec, 9, cin + cout, 4, 4, "bernoulli", 0.3)
+    xs = synth.make_input(9, (2, 4, 12, 12, cin))
+    xs[0, 1, 3, 4, 5] = np.inf
+    xs[0, 2, 8, 8, 21] = -np.inf
+    xs[0, 3, 10, 1, 7] = np.nan
+    xs[1, 0, 2, 2, 11] = 3.4e38
+    xs[1, 2, 6:, 6:, :] *= np.float32(1e-33)               # windows of nothing else: tiny outputs
+    xs[1, 1, 6:, 6:, :] *= np.float32(1e-33)
+    xs[1, 3, 6:, 6:, :] *= np.float32(1e-33)
+    lay = nets.ConvLayer(spec, L["w"], np.zeros_like(L["bias"]), L["mask"], 4, 4, torch.float32)
+    xd = nets.to_device(xs, torch.float32)
+    got = lay(xd).cpu().numpy()
+    assert rt3d.rt3d_last_plan()["kernel"] == 8 and rt3d.rt3d_last_device_status() == rt3d.OK
+    want = lay(xd, algo=rt3d.ALGO_SIMT).cpu().numpy()
+    assert rt3d.rt3d_last_plan()["kernel"] == 0
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.isnan(want).any()
+    assert np.array_equal(np.isposinf(got), np.isposinf(want)) and np.array_equal(np.isneginf(got), np.isneginf(want))
+    assert np.isinf(want).any()
+    rows = np.isfinite(want).all(axis=-1)                  # a voxel's sums are as wrong as its largest ones
+    err, size = np.abs(got[rows] - want[rows]).max(axis=-1), np.abs(want[rows]).max(axis=-1)
+    assert (size[size > 0].min() < 1e-32) and (err <= 1e-5 * size).all()
+
+
+def test_weights_that_three_bf16_cannot_hold_stay_on_the_cuda_cores(everywhere):
+    spec = synth.ConvSpec("f32", 32, 32, (1, 3, 3), (1, 1, 1), (0, 1, 1), False)
+    L = synth.make_layer(spec, 9, 1, 4, 4, "none", None)
+    xd = nets.to_device(synth.make_input(9, (1, 2, 8, 8, 32)), torch.float32)
+    for value in (1e-31, 3e36, np.inf, np.nan, -0.0):
+        w = L["w"].copy()
+        w[3, 5, 0, 1, 1] = value
+        nets.ConvLayer(spec, w, L["bias"], None, 4, 4, torch.float32, dense=True)(xd)
+        assert rt3d.rt3d_last_plan()["kernel"] == (8 if value == 0.0 else 0)
