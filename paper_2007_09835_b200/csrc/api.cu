@@ -837,6 +837,15 @@ rt3d_status get_tail(rt3d_packed* w, DeviceBlob* blob, size_t bytes, size_t flag
   return RT3D_OK;
 }
 
+// Whether the epilogue's pieces are turned in shared memory (umma_common.cuh: epilogue_row_turned): those that load a residual
+// and those that box stores cannot take.  Measured over 110 random layers, in favour of turning: with a residual, 1.05-1.57x
+// from 64 columns on (24 -> 466 channels 3x1x1 on 19 x 8 x 46 x 13 126 -> 80 us), 0.86-1.19x below (30 -> 20 14.8 -> 17.3); without one
+// 1.04-1.2x from 64 columns and nine steps on (110 -> 138 1x3x3 on 7 x 12 x 29 x 88 86 -> 71), 0.78-0.94x below (58 -> 18 3x1x1
+// 14.8 -> 19.0, 150 -> 398 in three steps 40 -> 45), where a tile waits for its last piece.
+bool turn_pieces(int n_tile, int steps, bool box_stores, bool residual) {
+  return n_tile >= 64 && (residual || (!box_stores && steps >= 9));
+}
+
 // Resident-weight kernel for thin stride-1 layers: used when the layer qualifies and (unless forced) has
 // at least one tile per SM.  *launched = false (and RT3D_OK) when the caller should take another kernel.
 rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g,
@@ -893,6 +902,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   const bool rect = warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb);
   a.sbw = sb[0]; a.sbh = sb[1];
   a.store_tma = (rect && encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
+  a.turned = turn_pieces(a.n_tile, h.n_steps, a.store_tma != 0, res_data != nullptr) ? 1 : 0;
   *launched = true;
   const int sms = d->sm_count;
   const void* wmap = u->wmap_half;
@@ -1264,6 +1274,8 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   CUtensorMap ymap{};
   a.store_tma = (a.n_splits == 1 && rect && encode_ymap(y, sb, pl_w, pl_h, pl_t, &ymap)) ? 1 : 0;
   if (pooled && !a.store_tma) return RT3D_ERR_UNSUPPORTED;
+  a.turned = use_pair && !pooled &&
+             turn_pieces(a.n_tile, dense_entry ? a.steps_dense : int(L->steps.size()) / a.n_bundles, a.store_tma != 0, res_data != nullptr) ? 1 : 0;
   if (use_pair) {
     // items that do not fill a last round of CTA pairs are cut along K and shared
     // (its CTA pairs wait for one another, which needs the whole grid resident at once: not used when the caller
@@ -1277,6 +1289,9 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
       DeviceBlob::Tail t;
       if ((s = get_tail(w, blob, tail_bytes, flag_bytes, &t)) != RT3D_OK) return s;
       a.tail_scratch = t.partial; a.tail_flags = t.flags;
+      // up to a round and a half: the shared tiles, which are not turned, and one more each; it is their latency that counts
+      // (83 -> 150 channels with a residual on 3 x 13 x 23 x 19, 76 items: 30.9 us, turned 31.2)
+      if (pairs * 4 < d->sm_count * 3) a.turned = 0;
     }
   }
   const int sms = d->sm_count;
@@ -1850,6 +1865,7 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
   a.tail_workers = 0; a.tail_scratch = nullptr; a.tail_flags = nullptr;
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = 0; a.debug_drop_last_load = 0;
+  a.turned = 0;
   a.store_tma = (a.n_splits == 1 && warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb) &&
                  encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   if (launch_conv_umma(a, &xmap, u->wmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;

@@ -126,6 +126,7 @@ struct UmmaArgs {
   int store_tma;                            // 1: epilogue stores go through shared memory + TMA (needs ymap)
   const void* residual;                     // device bf16 tensor of the output's extents added before the ReLU, or nullptr
   int rcs;                                  // its channel pitch
+  int turned;                               // 1: epilogue pieces go through shared memory (epilogue_row_turned); CTA pairs, without a fused pool
   int pool_t, pool_h, pool_w;               // fused max-pool window (1,1,1 = none); needs store_tma, ymap over the pooled tensor
   int sbw, sbh;                             // extents along w, h of the block of 32 voxels an epilogue warp owns
   int n_splits;                             // K splits per output tile (1 = none): the CTAs of one cluster

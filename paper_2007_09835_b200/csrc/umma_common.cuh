@@ -220,6 +220,22 @@ __device__ __forceinline__ uint32_t cvt_relu_bf16x2(float x, float y) {
   return d;
 }
 
+// Eight channels, of which `left` exist.  A row's last 16-byte unit may hold fewer: 8, 4 and 2 bytes as needed, the padding
+// behind them is left alone.  (Channel by channel, the 13 two-byte stores of a thread's second piece made the 45 outputs of the
+// R(2+1)D stem cost twice what 48 do: 74 -> 38 us.)
+__device__ __forceinline__ void store_unit(__nv_bfloat16* d, const uint4& o, int left) {
+  if (left >= 8) {
+    *reinterpret_cast<uint4*>(d) = o;
+  } else {
+    if (left & 4) *reinterpret_cast<uint2*>(d) = make_uint2(o.x, o.y);
+    if (left & 2) *reinterpret_cast<uint32_t*>(d + (left & 4)) = (left & 4) ? o.z : o.x;
+    if (left & 1) {
+      const uint32_t w = (left & 4) ? ((left & 2) ? o.w : o.z) : ((left & 2) ? o.y : o.x);
+      *reinterpret_cast<uint16_t*>(d + (left & 6)) = uint16_t(w);
+    }
+  }
+}
+
 template <int NC>
 __device__ __forceinline__ void epilogue_cols(const uint32_t* v, const float* bias_s, int relu,
                                               __nv_bfloat16* dst, int valid, const __nv_bfloat16* res, int res_avail) {
@@ -262,21 +278,7 @@ __device__ __forceinline__ void epilogue_cols(const uint32_t* v, const float* bi
 #pragma unroll
       for (int e = 0; e < 4; ++e) po[e] = __floats2bfloat162_rn(f[8 * q + 2 * e], f[8 * q + 2 * e + 1]);
     }
-    // A row's last 16-byte unit may hold fewer than eight channels: 8, 4 and 2 bytes as needed, the padding behind them is
-    // left alone.  (Channel by channel, the 13 two-byte stores of a thread's second piece made the 45 outputs of the
-    // R(2+1)D stem cost twice what 48 do: 74 -> 38 us.)
-    const int left = valid - 8 * q;
-    if (left >= 8) {
-      reinterpret_cast<uint4*>(dst)[q] = o;
-    } else {
-      __nv_bfloat16* d = dst + 8 * q;
-      if (left & 4) *reinterpret_cast<uint2*>(d) = make_uint2(o.x, o.y);
-      if (left & 2) *reinterpret_cast<uint32_t*>(d + (left & 4)) = (left & 4) ? o.z : o.x;
-      if (left & 1) {
-        const uint32_t w = (left & 4) ? ((left & 2) ? o.w : o.z) : ((left & 2) ? o.y : o.x);
-        *reinterpret_cast<uint16_t*>(d + (left & 6)) = uint16_t(w);
-      }
-    }
+    store_unit(dst + 8 * q, o, valid - 8 * q);
   }
 }
 
@@ -306,6 +308,92 @@ __device__ __forceinline__ void add_partials(uint32_t (&v)[32], bool wide, int c
       v[4 * q + 2] = __float_as_uint((__uint_as_float(v[4 * q + 2]) + t0[q].z) + t1[q].z);
       v[4 * q + 3] = __float_as_uint((__uint_as_float(v[4 * q + 3]) + t0[q].w) + t1[q].w);
     }
+  }
+}
+
+// ------------------------------------------------------------------------------ turning pieces
+// A piece is 32 channels of an epilogue warp's 32 voxels, 64 bytes a voxel.  A thread has one voxel's accumulators, but a load
+// or store in which every lane has its own voxel touches 32 lines.  So the residual's pieces are loaded, and the output's
+// stored where no box store can take them, with four lanes to a voxel (eight lines), and go through a buffer in shared memory
+// (2 KB a warp, 16-byte units exchanged by the row so that neither side's banks collide) on the way from and to the thread.
+struct Turn {
+  uint32_t smem;              // this warp's buffer
+  long long at[4];            // the voxels that this lane loads and stores for: rows 8 i + lane / 4; -1: none
+};
+__device__ __forceinline__ void turn_to(Turn& t, long long vox, bool in_range, int lane) {
+  const long long mine = in_range ? vox : -1;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) t.at[i] = __shfl_sync(0xffffffffu, mine, i * 8 + (lane >> 2));
+}
+__device__ __forceinline__ uint32_t turn_unit(const Turn& t, uint32_t row, uint32_t unit) {
+  return t.smem + row * 64u + ((unit ^ ((row >> 1) & 3u)) << 4);
+}
+// This lane's part of a residual piece, channels from m0 on, M in all: on its way while the piece's accumulators are read.
+__device__ __forceinline__ void residual_load(uint4 (&rv)[4], const Turn& t, const __nv_bfloat16* res, int rcs, int m0, int M, int lane) {
+  const int m = m0 + (lane & 3) * 8;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    rv[i] = (t.at[i] >= 0 && m < M) ? __ldg(reinterpret_cast<const uint4*>(res + t.at[i] * rcs + m)) : make_uint4(0u, 0u, 0u, 0u);
+}
+// The piece through the buffer to the threads that own its rows, added to their sums.  Of the last unit only the channels
+// that exist count (`left` from m0 on): whatever the residual's padding holds must not reach the output's.
+__device__ __forceinline__ void residual_add(float (&f)[32], const uint4* rv, const Turn& t, int left, int lane) {
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(turn_unit(t, i * 8u + (uint32_t(lane) >> 2), uint32_t(lane) & 3u)),
+                 "r"(rv[i].x), "r"(rv[i].y), "r"(rv[i].z), "r"(rv[i].w) : "memory");
+  __syncwarp();
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) {
+    uint32_t w[4];
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                 : "r"(turn_unit(t, uint32_t(lane), k)) : "memory");
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int c = 8 * int(k) + 2 * e;
+      f[c] += c < left ? __uint_as_float(w[e] << 16) : 0.f;
+      f[c + 1] += c + 1 < left ? __uint_as_float(w[e] & 0xffff0000u) : 0.f;
+    }
+  }
+}
+// A whole piece of a tile without box stores: bias, residual, ReLU, bf16, turned and stored.
+__device__ __forceinline__ void epilogue_piece_turned(const uint32_t* v, const float* bias_s, int relu, __nv_bfloat16* y, int ycs, int m0, int M,
+                                                      int lane, const Turn& t, const uint4* rv) {
+  float f[32];
+  if (bias_s != nullptr) {                                            // nullptr: the bias is in the accumulator already
+    const float4* b4 = reinterpret_cast<const float4*>(bias_s);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float4 b = b4[k];
+      f[4 * k] = __uint_as_float(v[4 * k]) + b.x; f[4 * k + 1] = __uint_as_float(v[4 * k + 1]) + b.y;
+      f[4 * k + 2] = __uint_as_float(v[4 * k + 2]) + b.z; f[4 * k + 3] = __uint_as_float(v[4 * k + 3]) + b.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) f[q] = __uint_as_float(v[q]);
+  }
+  __syncwarp();                                                       // the last piece's units have been read
+  if (rv != nullptr) residual_add(f, rv, t, M - m0, lane);
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) {                                  // this row's units: no other thread reads or writes them
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float x0 = f[8 * k + 2 * e], x1 = f[8 * k + 2 * e + 1];
+      if (relu) o[e] = cvt_relu_bf16x2(x0, x1);
+      else *reinterpret_cast<__nv_bfloat162*>(&o[e]) = __floats2bfloat162_rn(x0, x1);
+    }
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(turn_unit(t, uint32_t(lane), k)), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])
+                 : "memory");
+  }
+  __syncwarp();
+  const int m = m0 + (lane & 3) * 8;
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i) {
+    uint4 o;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w)
+                 : "r"(turn_unit(t, i * 8u + (uint32_t(lane) >> 2), uint32_t(lane) & 3u)) : "memory");
+    if (t.at[i] >= 0 && m < M) store_unit(y + t.at[i] * ycs + m, o, M - m);
   }
 }
 
@@ -406,7 +494,7 @@ __device__ __forceinline__ void epilogue_bar_sync(int n_threads) {
 // channels [m0, m0+32) x the warp's 32 voxels.
 __device__ __forceinline__ void epilogue_piece_tma(const uint32_t* v, const float* bias_s, int relu, int m0, int lane,
                                                    TmaStore& ts, const __nv_bfloat16* res, int res_avail,
-                                                   const PoolLanes* pool) {
+                                                   const PoolLanes* pool, Turn* turned = nullptr, const uint4* rv = nullptr) {
   float f[32];
   if (bias_s != nullptr) {                                            // nullptr: the bias is in the accumulator already
     const float4* b4 = reinterpret_cast<const float4*>(bias_s);      // 16-byte aligned by construction
@@ -434,6 +522,16 @@ __device__ __forceinline__ void epilogue_piece_tma(const uint32_t* v, const floa
         }
       }
     }
+  }
+  const uint32_t buf = ts.smem + (ts.piece % ts.bufs) * kStoreStageBytes;
+  if (turned != nullptr) {                         // the buffer serves the residual first
+    if (lane == 0) {
+      if (ts.bufs == 1) tma_store_wait_read_0();
+      else tma_store_wait_read_1();
+    }
+    __syncwarp();
+    turned->smem = buf;
+    residual_add(f, rv, *turned, res_avail, lane);
   }
   uint4 o[4];
   __nv_bfloat162* po = reinterpret_cast<__nv_bfloat162*>(o);
@@ -476,8 +574,7 @@ __device__ __forceinline__ void epilogue_piece_tma(const uint32_t* v, const floa
     writer = pool->writer;
     out_row = pool->out_row;
   }
-  const uint32_t buf = ts.smem + (ts.piece % ts.bufs) * kStoreStageBytes;
-  if (lane == 0) {                                 // the store issued ts.bufs pieces ago has read this buffer
+  if (turned == nullptr && lane == 0) {            // the store issued ts.bufs pieces ago has read this buffer
     if (ts.bufs == 1) tma_store_wait_read_0();
     else tma_store_wait_read_1();
   }
@@ -525,6 +622,38 @@ __device__ __forceinline__ void epilogue_row_tma(uint32_t taddr, int n_cols, boo
       if (warp_rows_valid) epilogue_piece_tma(v, bias_s ? bias_s + m0 : nullptr, relu, m0, lane, ts, res, res_left - col, pool);
     } else if (in_range) {
       epilogue_cols<16>(v, bias_s ? bias_s + m0 : nullptr, relu, dst + col, M - m0, res, res_left - col);
+    }
+  }
+}
+
+// The same for tiles of which a CTA does several one after the other: whole pieces are turned, the residual's on their way in,
+// the output's on their way out where there are no box stores.  A piece takes a little longer, but the SM's load and store unit
+// a quarter of the time, which is what such tiles were bound by.
+__device__ __forceinline__ void epilogue_row_turned(uint32_t taddr, int n_cols, bool has_acc, bool warp_rows_valid, bool in_range,
+                                                    const float* bias_s, int relu, __nv_bfloat16* y, int ycs, long long vox, int m_base,
+                                                    int M, int lane, TmaStore& ts, bool store_tma, Turn& t, const __nv_bfloat16* res,
+                                                    int rcs, int col0, int col_step, uint32_t acc2_off = 0) {
+  turn_to(t, vox, in_range, lane);
+  for (int col = col0; col < n_cols; col += col_step) {
+    const int m0 = m_base + col;
+    if (m0 >= M) break;
+    uint32_t v[32];
+    const bool wide = col + 32 <= n_cols;
+    uint4 rv[4];
+    if (wide && res) residual_load(rv, t, res, rcs, m0, M, lane);
+    if (has_acc) {
+      tmem_ld_acc(taddr + col, wide, acc2_off, v);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 32; ++q) v[q] = 0u;
+    }
+    const float* bs = bias_s + m0;
+    if (!wide) {
+      if (in_range) epilogue_cols<16>(v, bs, relu, y + vox * ycs + m0, M - m0, res ? res + vox * rcs + m0 : nullptr, M - m0);
+    } else if (!store_tma) {
+      epilogue_piece_turned(v, bs, relu, y, ycs, m0, M, lane, t, res ? rv : nullptr);
+    } else if (warp_rows_valid) {
+      epilogue_piece_tma(v, bs, relu, m0, lane, ts, nullptr, M - m0, nullptr, res ? &t : nullptr, rv);
     }
   }
 }

@@ -68,7 +68,8 @@ __device__ __forceinline__ void walk_next(TileWalk& k, const UmmaArgs& a) {
   k.in += k.dn + c;               // beyond tiles_n: the dummy second tile of an odd count (all voxels out of range)
 }
 
-template <bool kDense>
+// kTurn: the epilogue turns its pieces in shared memory (h.u.turned).
+template <bool kDense, bool kTurn>
 __global__ void __launch_bounds__(kThreadsHalo, 1)
 conv3d_umma_halo_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap_half,
                         const __grid_constant__ CUtensorMap ymap, const HaloArgs h, const int tmem_cols) {
@@ -211,6 +212,8 @@ conv3d_umma_halo_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
     __nv_bfloat16* yb = static_cast<__nv_bfloat16*>(a.y);
     const __nv_bfloat16* rb = static_cast<const __nv_bfloat16*>(a.residual);
     TmaStore ts{&ymap, store_smem + uint32_t(warp - 2) * kStoreWarpBytes, 0, 0, 0, 0, 0u};
+    [[maybe_unused]] Turn turn;
+    turn.smem = ts.smem;
     int r0 = quad * 32;
     const int bw_0 = r0 % a.box.bw; r0 /= a.box.bw;
     const int bh_0 = r0 % a.box.bh; r0 /= a.box.bh;
@@ -230,7 +233,10 @@ conv3d_umma_halo_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
       const __nv_bfloat16* res_row = (rb != nullptr && in_range) ? rb + vox * a.rcs : nullptr;
       __nv_bfloat16* dst = yb + vox * a.g.ycs;
       ts.c1 = w0 + bw_0; ts.c2 = h0 + bh_0; ts.c3 = t0 + bt_0; ts.c4 = k.in;
-      for (int col = half * 32; col < a.n_tile && col < a.g.M; col += 64) {
+      if constexpr (kTurn)
+        epilogue_row_turned(taddr, a.n_tile, h.n_steps > 0, quad * 32 < box_rows, in_range, bias_s, a.g.relu, yb, a.g.ycs, vox, 0, a.g.M,
+                            lane, ts, a.store_tma != 0, turn, rb, a.rcs, half * 32, 64);
+      for (int col = half * 32; !kTurn && col < a.n_tile && col < a.g.M; col += 64) {
         uint32_t v[32];
         const bool wide = col + 32 <= a.n_tile;
         if (h.n_steps > 0) {
@@ -274,21 +280,21 @@ size_t halo_smem_bytes(const HaloArgs& h) {
          8 * kStoreWarpBytes + sizeof(HaloBars) + size_t(h.u.n_tile) * 4 + 16;
 }
 
-template <bool kDense>
+template <bool kDense, bool kTurn>
 cudaError_t launch_halo_t(const HaloArgs& h, const CUtensorMap& xm, const CUtensorMap& wm, const CUtensorMap& ym,
                           int sm_count, int cols, size_t smem, long long n_items, cudaStream_t stream) {
   static bool attr_done[kMaxDevices] = {};             // the attributes are per device
   const int dev_idx = current_device_index();
   if (dev_idx < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev_idx]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_halo_kernel<kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_halo_kernel<kDense, kTurn>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev_idx] = true;
   }
   long long clusters = sm_count / 2;
   if (clusters > n_items) clusters = n_items;
   LaunchSetup ls(dim3(unsigned(2 * clusters)), dim3(kThreadsHalo), smem, stream, 2);
-  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_halo_kernel<kDense>, xm, wm, ym, h, cols);
+  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_halo_kernel<kDense, kTurn>, xm, wm, ym, h, cols);
 }
 
 }  // namespace
@@ -357,8 +363,11 @@ cudaError_t launch_conv_umma_halo(const HaloArgs& h, const void* xmap, const voi
   memcpy(&xm, xmap, sizeof(CUtensorMap));
   memcpy(&wm, wmap_half, sizeof(CUtensorMap));
   memcpy(&ym, ymap ? ymap : xmap, sizeof(CUtensorMap));
-  return a.dense ? launch_halo_t<true>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream)
-                 : launch_halo_t<false>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream);
+  if (a.turned)
+    return a.dense ? launch_halo_t<true, true>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream)
+                   : launch_halo_t<false, true>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream);
+  return a.dense ? launch_halo_t<true, false>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream)
+                 : launch_halo_t<false, false>(h, xm, wm, ym, sm_count, cols, smem, n_items, stream);
 }
 
 }  // namespace rt3d

@@ -66,7 +66,9 @@ constexpr int kTsTable = 2048;
 // tiles of the up to Kt steps (kt = 0 .. Kt-1 at one (kh, kw, chunk)) that read it, each through a descriptor that
 // starts kt frames into the tile: a third as many input bytes per step cross from L2, so more steps are in flight
 // in the same shared memory (a 64 -> 128 channel 3x3x3 layer was bound by that, at 387 clocks per step against 256).
-template <bool kDense, int kCps, bool kTS, bool kDual>
+// kTurn: the epilogue of a whole tile turns its pieces in shared memory (a.turned); a variant of its own, because the code
+// of both in one kernel cost layers that use neither 0.5 to 1 %.
+template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn>
 __global__ void __launch_bounds__(kThreadsPair, 1)
 conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap_half,
                         const __grid_constant__ CUtensorMap ymap, const UmmaArgs a, const int stages, const int tmem_cols) {
@@ -403,6 +405,8 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
     // two sets: each warp of a quadrant uses one of the quadrant's two staging buffers
     TmaStore ts{&ymap, store_smem + uint32_t(quad) * kStoreWarpBytes + uint32_t(set) * kStoreStageBytes, 0, 0, 0, 0, 0u,
                 1u};
+    [[maybe_unused]] Turn turn;
+    turn.smem = ts.smem;
     const PoolLanes pool_lanes = make_pool_lanes(a.pool_w, a.pool_h, a.pool_t, a.sbw, a.sbh, lane);
     const PoolLanes* pool = (a.pool_t * a.pool_h * a.pool_w > 1) ? &pool_lanes : nullptr;
     int r0 = quad * 32;                        // coordinates of the warp's first row inside the box
@@ -496,7 +500,11 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
         }
         continue;
       }
-      if (a.store_tma) {
+      if constexpr (kTurn) {
+        ts.c1 = c.w0 + bw_0; ts.c2 = c.h0 + bh_0; ts.c3 = c.t0 + bt_0; ts.c4 = c.n0 + bn_0;
+        epilogue_row_turned(taddr, a.n_tile, nsteps > 0, quad * 32 < box_rows, in_range, bias_s, a.g.relu, yb, a.g.ycs, vox, m_base, a.g.M,
+                            lane, ts, a.store_tma != 0, turn, rb, a.rcs, col0, col_step, acc2);
+      } else if (a.store_tma) {
         ts.c1 = (c.w0 + bw_0) / a.pool_w; ts.c2 = (c.h0 + bh_0) / a.pool_h; ts.c3 = (c.t0 + bt_0) / a.pool_t; ts.c4 = c.n0 + bn_0;
         epilogue_row_tma(taddr, a.n_tile, nsteps > 0, quad * 32 < box_rows, in_range, bias_s, a.g.relu,
                          yb + vox * a.g.ycs + m_base, m_base, a.g.M, lane, ts, res, res_left, pool, nullptr, nullptr, 0, 0,
@@ -563,13 +571,13 @@ size_t pair_smem_bytes_ts(const UmmaArgs& a) {
          16 + size_t(a.n_tile) * a.n_bundles * 4 + (3 * size_t(a.ts_table) + 16) * 4;
 }
 
-template <bool kDense, int kCps, bool kTS, bool kDual>
+template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn>
 cudaError_t prepare_pair_t() {
   static bool attr_done[kMaxDevices] = {};             // the attribute is per device
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, kTurn>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -596,12 +604,12 @@ int pair_max_clusters_t(int sm_count, size_t smem) {
   if (dev < 0) return sm_count / 2;
   int& max_clusters = max_clusters_dev[dev];
   if (max_clusters == 0) {
-    if (prepare_pair_t<kDense, kCps, kTS, kDual>() != cudaSuccess) return sm_count / 2;
+    if (prepare_pair_t<kDense, kCps, kTS, kDual, false>() != cudaSuccess) return sm_count / 2;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pair_launch_config(cfg, attr, unsigned(sm_count & ~1), smem, nullptr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual>, &cfg) != cudaSuccess || n <= 0) n = sm_count / 2;
+    if (cudaOccupancyMaxActiveClusters(&n, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, false>, &cfg) != cudaSuccess || n <= 0) n = sm_count / 2;
     max_clusters = n;
   }
   return max_clusters < sm_count / 2 ? max_clusters : sm_count / 2;
@@ -639,13 +647,14 @@ template <bool kDense, int kCps, bool kTS, bool kDual>
 cudaError_t launch_pair_t(const UmmaArgs& a, const CUtensorMap& xm, const CUtensorMap& wm, const CUtensorMap& ym,
                           int sm_count, int stages,
                           int cols, size_t smem, long long n_items, cudaStream_t stream) {
-  cudaError_t e = prepare_pair_t<kDense, kCps, kTS, kDual>();
+  cudaError_t e = a.turned ? prepare_pair_t<kDense, kCps, kTS, kDual, true>() : prepare_pair_t<kDense, kCps, kTS, kDual, false>();
   if (e != cudaSuccess) return e;
   long long clusters = pair_max_clusters_t<kDense, kCps, kTS, kDual>(sm_count, smem);
   const long long want = n_items > a.tail_workers ? n_items : a.tail_workers;
   if (clusters > want) clusters = want;
   LaunchSetup ls(dim3(unsigned(2 * clusters)), dim3(kThreadsPair), smem, stream, 2);
-  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual>, xm, wm, ym, a, stages, cols);
+  return cudaLaunchKernelEx(&ls.cfg, a.turned ? conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, true> : conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, false>,
+                            xm, wm, ym, a, stages, cols);
 }
 
 }  // namespace
