@@ -418,13 +418,15 @@ void rt3d_plan_end(void);
  * form (kernel 2) on the same handle; default 1.
  * RT3D_DEBUG_F32_SPLIT: fp32 calls on the tensor cores (plan kernel 8): 0 never, 1 where they are expected to be faster
  * (default), 2 wherever they can run.
+ * RT3D_DEBUG_NARROW: 0 switches off the K steps of 32 input channels that the step-list tensor-core kernels take for layers
+ * of up to 32 (64 otherwise); default 1.
  * RT3D_DEBUG_POISON: runs, on the default stream, a kernel that fills the shared memory and the tensor memory of
  * every SM with the 32-bit pattern `value` (e.g. 0x7FC07FC0: two bf16 NaNs) and waits for it: a kernel launched next
  * that reads shared or tensor memory it did not write itself (padding multiplied by zero weights, say) then
  * produces NaNs instead of depending silently on what ran before it.  The partial-tile scratch of every handle's
  * tail splits on the device is set to all ones (NaNs) as well.  Device work only; nothing else changes. */
 enum { RT3D_DEBUG_WAIT_CYCLES = 1, RT3D_DEBUG_DROP_LAST_LOAD = 2, RT3D_DEBUG_T_GROUPS = 3, RT3D_DEBUG_POISON = 4,
-       RT3D_DEBUG_F32_SPLIT = 5 };
+       RT3D_DEBUG_F32_SPLIT = 5, RT3D_DEBUG_NARROW = 6 };
 rt3d_status rt3d_debug_set(int what, long long value);
 /* Diagnostics.  RT3D_DEBUG_WAIT_SITE: after a synchronisation of the device, the number of the wait inside a
  * kernel that gave up since the last rt3d_last_device_status (0 = none; the numbers are the last argument of the

@@ -588,7 +588,7 @@ def rt3d_alloc_count() -> int:
     return int(_lib.rt3d_alloc_count())
 
 
-DEBUG_WAIT_CYCLES, DEBUG_DROP_LAST_LOAD, DEBUG_T_GROUPS, DEBUG_POISON, DEBUG_F32_SPLIT = 1, 2, 3, 4, 5
+DEBUG_WAIT_CYCLES, DEBUG_DROP_LAST_LOAD, DEBUG_T_GROUPS, DEBUG_POISON, DEBUG_F32_SPLIT, DEBUG_NARROW = 1, 2, 3, 4, 5, 6
 
 
 def rt3d_debug_get(what: int) -> int:

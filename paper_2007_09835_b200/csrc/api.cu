@@ -66,6 +66,8 @@ std::atomic<long long> g_debug_wait_cycles{-1};      // -1: not set yet (RT3D_DE
 std::atomic<int> g_debug_drop_last_load{0};
 // t-grouped CTA-pair variant: on unless the environment says RT3D_T_GROUPS=0; RT3D_DEBUG_T_GROUPS switches it at run time
 std::atomic<int> g_ts_enabled{[] { const char* e = getenv("RT3D_T_GROUPS"); return (e && e[0] == '0') ? 0 : 1; }()};
+// steps of 32 input channels (kNarrowChunk): RT3D_DEBUG_NARROW switches them off and on
+std::atomic<int> g_narrow_enabled{1};
 // fp32 on the tensor cores: 0 never, 1 where it is expected to be faster, 2 wherever it can run (tests, comparisons)
 std::atomic<int> g_f32_split{1};
 long long debug_wait_cycles() {
@@ -387,9 +389,9 @@ rt3d_status get_canonical(rt3d_packed* h, DeviceBlob* b) {
 
 rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, DeviceBlob::Umma** out) {
   std::lock_guard<std::mutex> lock(h->mu);
-  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, L->t_groups)];
+  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, L->t_groups, L->chunk != kChunk)];
   if (!u.ready) {
-    const size_t wbytes = L->steps.size() * size_t(L->n_tile) * kChunk * 2;
+    const size_t wbytes = L->steps.size() * size_t(L->n_tile) * L->chunk * 2;
     // The canonical arrays go to the device once, a quarter to a third of the size of the zero-filled tiles, and a kernel
     // fills the tiles in there: 512 x 512 x 27 at 0.28 kept, 14 MB of tiles: 9 -> 1.6 ms with the allocation.
     // The first layout shares the allocation of the canonical arrays: a cudaMalloc and its cudaFree are 0.2 to 0.4 ms each.
@@ -407,23 +409,24 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
     if (s != RT3D_OK) return s;
     const auto fail = [&] { weight_free(*base, false); *base = nullptr; return RT3D_ERR_CUDA; };
     if (wbytes && (launch_fill_umma_tiles(blob->group_ptr, blob->pos_idx, blob->tiles, slots, h->M, h->N, h->Ks, h->g_m, h->g_n,
-                                          h->Q, h->P * h->Q, h->nnz, L->n_tile, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
+                                          h->Q, h->P * h->Q, h->nnz, L->n_tile, L->chunk, L->n_chunks, u.wtiles, wbytes) != cudaSuccess ||
                    uploads_done() != cudaSuccess))
       return fail();
-    // 2-D map over the weight tiles: rows of 64 bf16 (128 bytes), one box = one [n_tile][64] tile
+    // 2-D map over the weight tiles: rows of a chunk's channels, one box = one tile
     const cuuint64_t rows = L->steps.empty() ? cuuint64_t(L->n_tile) : cuuint64_t(L->steps.size()) * L->n_tile;
-    cuuint64_t dims[2] = {64, rows};
-    cuuint64_t strides[1] = {128};
-    cuuint32_t box[2] = {64, cuuint32_t(L->n_tile)};
+    const CUtensorMapSwizzle swizzle = L->chunk == kChunk ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    cuuint64_t dims[2] = {cuuint64_t(L->chunk), rows};
+    cuuint64_t strides[1] = {cuuint64_t(L->chunk) * 2};
+    cuuint32_t box[2] = {cuuint32_t(L->chunk), cuuint32_t(L->n_tile)};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = g_encode(reinterpret_cast<CUtensorMap*>(u.wmap), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, u.wtiles, dims,
-                          strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                          strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail();
     if (L->n_tile % 16 == 0) {
-      cuuint32_t box_half[2] = {64, cuuint32_t(L->n_tile / 2)};
+      cuuint32_t box_half[2] = {cuuint32_t(L->chunk), cuuint32_t(L->n_tile / 2)};
       r = g_encode(reinterpret_cast<CUtensorMap*>(u.wmap_half), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, u.wtiles, dims,
-                   strides, box_half, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   strides, box_half, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return fail();
     }
@@ -436,7 +439,7 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
 // Device copy of the fp32 tensor-core kernel's layout, with the canonical arrays beside it.
 rt3d_status get_split_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, bool pair, DeviceBlob::Umma** out) {
   std::lock_guard<std::mutex> lock(h->mu);
-  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, false)];
+  DeviceBlob::Umma& u = blob->umma[umma_key(L->n_tile, false, false)];
   if (!u.ready) {
     const size_t wbytes = L->steps.size() * size_t(L->n_tile) * 192;
     const bool shared = !blob->canonical;
@@ -566,8 +569,17 @@ double choose_box_grouped(const ConvGeom& g, int n_tile, long long fewest, TileB
 // are tall enough for whole steps to vanish; a narrower bundle that matches the group height can win there.
 struct UmmaPlan { int n_tile, n_splits; bool pair; };
 
+// Whether the step-list kernels take a layer in steps of 32 input channels, half the bytes, MMAs and weights of one of 64: layers
+// of up to 32.  19 -> 489 channels 3x3x3 on 12 x 6 x 111 x 11 198 -> 120 us, 21 -> 164 on 18 x 16 x 75 x 15 152 -> 114, 17 -> 196 on
+// 3 x 3 x 63 x 44 38 -> 26, single steps and small calls 1.0-1.1x.  With more channels, where three steps of 32 would replace two
+// of 64, they lose: the copy engine takes rows at a rate, not bytes (77 -> 186 28.4 -> 31.7, 470 -> 182 33 -> 46, 265 -> 511 51 -> 63).
+bool narrow_steps(const rt3d_packed* w) { return w->N <= kNarrowChunk && g_narrow_enabled.load(); }
+
 UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_count) {
   const int M = w->M;
+  // Of a full step's bytes and MMAs; its hand-shake is the same.  (With few steps the output counts, and a bundle is no wider for
+  // it: 24 -> 347 1x3x3 on 14 x 4 x 7 x 7 at 64 columns 6.3 us, at 176 7.6.)
+  const double part = narrow_steps(w) && w->Ks > 12 ? 0.5 : 1.0;
   const int widest = default_n_tile(M);
   const bool tall = w->g_m >= 16 && !w->is_dense;
   UmmaPlan best{widest, 1, false};
@@ -593,7 +605,7 @@ UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_
       steps = items < sm_count ? double(L->max_steps) : double(L->steps.size()) / bundles;
     }
     constexpr double kByteNs = 1.0 / (65.0 * 1.85);
-    const double step_ns = std::max({1.08 * n, (kTileM * 128.0 + 128.0 * n) * kByteNs, 204.0});
+    const double step_ns = std::max({part * 1.08 * n, part * (kTileM * 128.0 + 128.0 * n) * kByteNs, 204.0});
     for (int S = 1; S <= 8; ++S) {
       const int capacity = umma_split_capacity(S, sm_count);
       if (capacity == 0 || (S > 1 && (steps / S < 4 || items >= 2LL * sm_count))) continue;
@@ -605,7 +617,7 @@ UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_
     if (umma_pair_supported(n, bundles) && (n == widest || (n & (n - 1)) == 0)) {
       const bool ts = g.Kt >= 2 && g.Kt <= 8 && g.st == 1 && g.To >= 4 && (n <= 128 || g.Kh * g.Kw >= 4);
       const double a_bytes = kTileM * 128.0 * (ts ? 1.25 / g.Kt : 1.0);
-      const double pair_ns = std::max({(n <= 128 ? 1.3 : 1.1) * n, (a_bytes + 64.0 * n) * kByteNs, 165.0});
+      const double pair_ns = std::max({part * (n <= 128 ? 1.3 : 1.1) * n, part * (a_bytes + 64.0 * n) * kByteNs, 165.0});
       // a last round that is not full is shared out along K where the items are long enough
       const double rounds = double((m_tiles + 1) / 2 * bundles) / (sm_count / 2);
       const double whole = std::ceil(rounds) * steps * pair_ns, shared = 5000.0 + rounds * steps * pair_ns;
@@ -628,17 +640,17 @@ bool umma_eligible(const DeviceState* d, const rt3d_packed* w, const rt3d_tensor
 }
 
 // `extra_t`: frames added to the box along t (the t-grouped CTA-pair variant stages Kt - 1 more; temporal stride 1).
-rt3d_status encode_xmap(const rt3d_tensor* x, const ConvGeom& g, const TileBox& box, CUtensorMap* map, int extra_t = 0) {
+rt3d_status encode_xmap(const rt3d_tensor* x, const ConvGeom& g, const TileBox& box, CUtensorMap* map, int extra_t = 0, int chunk = kChunk) {
   const cuuint64_t cs = cuuint64_t(x->c_stride) * 2;
   cuuint64_t dims[5] = {cuuint64_t(x->c), cuuint64_t(x->w), cuuint64_t(x->h), cuuint64_t(x->t), cuuint64_t(x->n)};
   cuuint64_t strides[4] = {cs, cs * x->w, cs * x->w * x->h, cs * x->w * x->h * x->t};
   // with a traversal stride s the engine loads ceil(box / s) elements, so a box of b outputs spans b*s inputs
-  cuuint32_t bx[5] = {64, cuuint32_t(box.bw * g.sw), cuuint32_t(box.bh * g.sh), cuuint32_t(box.bt * g.st + extra_t),
+  cuuint32_t bx[5] = {cuuint32_t(chunk), cuuint32_t(box.bw * g.sw), cuuint32_t(box.bh * g.sh), cuuint32_t(box.bt * g.st + extra_t),
                       cuuint32_t(box.bn)};
   cuuint32_t estr[5] = {1, cuuint32_t(g.sw), cuuint32_t(g.sh), cuuint32_t(g.st), 1};
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, x->data, dims, strides, bx, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, chunk == kChunk ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? RT3D_OK : RT3D_ERR_CUDA;
 }
 
@@ -903,6 +915,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   a.sbw = sb[0]; a.sbh = sb[1];
   a.store_tma = (rect && encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   a.turned = turn_pieces(a.n_tile, h.n_steps, a.store_tma != 0, res_data != nullptr) ? 1 : 0;
+  a.narrow = 0;
   *launched = true;
   const int sms = d->sm_count;
   const void* wmap = u->wmap_half;
@@ -1214,6 +1227,9 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   // (its box: among the boxes with as few tiles, one inside a single clip and as deep along t as possible; where none suits,
   // one inside a clip that reads less from L2 at up to a sixteenth more tiles: choose_box_grouped)
   bool use_ts = false;
+  // (few steps on single CTAs wait for their first tiles and for their output: in the S3D-shaped forward, whose branches have
+  // 16 to 32 channels there, 772 us as a graph, 778 in steps of 32)
+  a.narrow = narrow_steps(w) && (use_pair || w->Ks > 12) ? 1 : 0;
   UmmaArgs probe = a;
   // (wide bundles: only kernels that are also wide in space; a 3x1x1 layer with 192-wide bundles lost 8 us of 43
   // inside the S3D-shaped forward with it, while 3x3x3 layers gain 1-4 %)
@@ -1229,7 +1245,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
       probe.tiles_n = ceil_div(g.n, deep.bn); probe.tiles_t = ceil_div(g.To, deep.bt);
       probe.tiles_h = ceil_div(g.Ho, deep.bh); probe.tiles_w = ceil_div(g.Wo, deep.bw);
     }
-    probe.n_tile = plan.n_tile; probe.n_bundles = ceil_div(w->M, plan.n_tile); probe.dense = dense_entry ? 1 : 0;
+    probe.n_tile = plan.n_tile; probe.n_bundles = ceil_div(w->M, plan.n_tile); probe.dense = dense_entry && !a.narrow ? 1 : 0;
     use_ts = umma_pair_ts_supported(&probe, w->Ks * ceil_div(w->N, kChunk) * probe.n_bundles);
     const double ratio = use_ts || pooled ? 2.0 : choose_box_grouped(g, plan.n_tile, m_tiles, &deep);
     const bool rect2 = ratio < 1.0 && warp_block(deep.bw, deep.bh, deep.bt, deep.bn, sb2);
@@ -1250,12 +1266,12 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
       for (int i = 0; i < 4; ++i) sb[i] = sb2[i];
     }
   }
-  const UmmaLayout* L = get_umma_layout(w, plan.n_tile, use_ts);
+  const UmmaLayout* L = get_umma_layout(w, plan.n_tile, use_ts, a.narrow != 0);
   if (!L) return RT3D_ERR_UNSUPPORTED;
   DeviceBlob::Umma* u = nullptr;
   if ((s = get_umma_blob(w, blob, L, &u)) != RT3D_OK) return s;
   a.n_tile = L->n_tile; a.n_bundles = L->n_bundles; a.n_chunks = L->n_chunks;
-  a.dense = dense_entry ? 1 : 0;
+  a.dense = dense_entry && !a.narrow ? 1 : 0;
   a.steps_dense = w->Ks * L->n_chunks;
   a.step_ptr = u->step_ptr; a.steps = u->steps;
   a.bias = bias; a.y = y->data; a.sched = d->sched;
@@ -1270,12 +1286,12 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     a.ts_phases = probe.ts_phases;
   }
   CUtensorMap xmap;
-  if ((s = encode_xmap(x, g, a.box, &xmap, use_ts ? ((g.Kt - 1) / g.st) * g.st : 0)) != RT3D_OK) return s;
+  if ((s = encode_xmap(x, g, a.box, &xmap, use_ts ? ((g.Kt - 1) / g.st) * g.st : 0, L->chunk)) != RT3D_OK) return s;
   CUtensorMap ymap{};
   a.store_tma = (a.n_splits == 1 && rect && encode_ymap(y, sb, pl_w, pl_h, pl_t, &ymap)) ? 1 : 0;
   if (pooled && !a.store_tma) return RT3D_ERR_UNSUPPORTED;
   a.turned = use_pair && !pooled &&
-             turn_pieces(a.n_tile, dense_entry ? a.steps_dense : int(L->steps.size()) / a.n_bundles, a.store_tma != 0, res_data != nullptr) ? 1 : 0;
+             turn_pieces(a.n_tile, int(L->steps.size()) / a.n_bundles * L->chunk / kChunk, a.store_tma != 0, res_data != nullptr) ? 1 : 0;
   if (use_pair) {
     // items that do not fill a last round of CTA pairs are cut along K and shared
     // (its CTA pairs wait for one another, which needs the whole grid resident at once: not used when the caller
@@ -1865,7 +1881,7 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
   a.tail_workers = 0; a.tail_scratch = nullptr; a.tail_flags = nullptr;
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = 0; a.debug_drop_last_load = 0;
-  a.turned = 0;
+  a.turned = a.narrow = 0;
   a.store_tma = (a.n_splits == 1 && warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb) &&
                  encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   if (launch_conv_umma(a, &xmap, u->wmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;
@@ -1886,6 +1902,7 @@ rt3d_status rt3d_debug_set(int what, long long value) {
   if (what == RT3D_DEBUG_WAIT_CYCLES) { if (value < 0) return RT3D_ERR_INVALID_ARG; g_debug_wait_cycles.store(value); return RT3D_OK; }
   if (what == RT3D_DEBUG_DROP_LAST_LOAD) { g_debug_drop_last_load.store(value != 0); return RT3D_OK; }
   if (what == RT3D_DEBUG_T_GROUPS) { g_ts_enabled.store(value != 0); return RT3D_OK; }
+  if (what == RT3D_DEBUG_NARROW) { g_narrow_enabled.store(value != 0); return RT3D_OK; }
   if (what == RT3D_DEBUG_F32_SPLIT) { if (value < 0 || value > 2) return RT3D_ERR_INVALID_ARG; g_f32_split.store(int(value)); return RT3D_OK; }
   if (what == RT3D_DEBUG_POISON) {
     DeviceState* d = nullptr;

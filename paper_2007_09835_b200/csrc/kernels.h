@@ -104,17 +104,18 @@ cudaError_t launch_copy_f32(const rt3d_copy* copies, int n, cudaStream_t stream)
 cudaError_t launch_add_relu(int dtype, const void* a, int acs, const void* b, int bcs, void* y, int ycs,
                             int64_t voxels, int c, int relu, cudaStream_t stream);
 
-// Fills the zeroed tiles [steps][n_tile][64] of a tensor-core layout from the canonical arrays (layout.cu), on the legacy
+// Fills the zeroed tiles [steps][n_tile][chunk] of a tensor-core layout from the canonical arrays (layout.cu), on the legacy
 // default stream.
 cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const void* tiles, const int32_t* slots,
                                    int M, int N, int Ks, int g_m, int g_n, int Q, int n_groups, int64_t nnz, int n_tile,
-                                   int n_chunks, void* wtiles, size_t bytes);
+                                   int chunk, int n_chunks, void* wtiles, size_t bytes);
 
 // Everything the tcgen05 kernel needs besides the two tensor maps.
 struct UmmaArgs {
   ConvGeom g;
   TileBox box;
   int n_tile, n_bundles, n_chunks;
+  int narrow;                               // 1: steps of 32 input channels instead of 64 (index-driven path only)
   int tiles_n, tiles_t, tiles_h, tiles_w;   // number of boxes along each axis
   int dense;                                // 1: steps are computed, not read
   int steps_dense;                          // Ks * n_chunks (dense only)

@@ -26,7 +26,7 @@ __device__ __forceinline__ int group_of(const int32_t* group_ptr, int n_groups, 
 __global__ void __launch_bounds__(256)
 fill_umma_tiles_kernel(const int32_t* __restrict__ group_ptr, const uint16_t* __restrict__ pos_idx,
                        const uint16_t* __restrict__ tiles, const int32_t* __restrict__ slots, int M, int N, int Ks,
-                       int g_m, int g_n, int Q, int n_groups, int nnz, int n_tile, int n_chunks, uint16_t* __restrict__ wtiles) {
+                       int g_m, int g_n, int Q, int n_groups, int nnz, int n_tile, int chunk_bits, int n_chunks, uint16_t* __restrict__ wtiles) {
   const int lane = threadIdx.x & 31, size = g_m * g_n;
   for (long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < nnz; e += (long long)gridDim.x * (blockDim.x >> 5)) {
     const int lo = group_of(group_ptr, n_groups, e);
@@ -36,8 +36,8 @@ fill_umma_tiles_kernel(const int32_t* __restrict__ group_ptr, const uint16_t* __
       const int i = v / g_n, m = p * g_m + i, c = q * g_n + (v - i * g_n);
       if (m >= M || c >= N) continue;
       const int b = m / n_tile;
-      const long long s = __ldg(slots + ((long long)b * Ks + k) * n_chunks + (c >> 6));
-      wtiles[(s * n_tile + (m - b * n_tile)) * 64 + (c & 63)] = src[v];
+      const long long s = __ldg(slots + ((long long)b * Ks + k) * n_chunks + (c >> chunk_bits));
+      wtiles[((s * n_tile + (m - b * n_tile)) << chunk_bits) + (c & ((1 << chunk_bits) - 1))] = src[v];
     }
   }
 }
@@ -85,12 +85,12 @@ cudaError_t launch_fill_split_tiles(const int32_t* group_ptr, const uint16_t* po
 
 cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const void* tiles, const int32_t* slots,
                                    int M, int N, int Ks, int g_m, int g_n, int Q, int n_groups, int64_t nnz, int n_tile,
-                                   int n_chunks, void* wtiles, size_t bytes) {
+                                   int chunk, int n_chunks, void* wtiles, size_t bytes) {
   cudaError_t e = cudaMemsetAsync(wtiles, 0, bytes, cudaStreamLegacy);
   if (e != cudaSuccess || nnz == 0) return e;
   const int64_t blocks = (nnz + 7) / 8;
   fill_umma_tiles_kernel<<<unsigned(blocks < 65536 ? blocks : 65536), 256, 0, cudaStreamLegacy>>>(
-      group_ptr, pos_idx, static_cast<const uint16_t*>(tiles), slots, M, N, Ks, g_m, g_n, Q, n_groups, int(nnz), n_tile, n_chunks,
+      group_ptr, pos_idx, static_cast<const uint16_t*>(tiles), slots, M, N, Ks, g_m, g_n, Q, n_groups, int(nnz), n_tile, chunk == 32 ? 5 : 6, n_chunks,
       static_cast<uint16_t*>(wtiles));
   return cudaGetLastError();
 }

@@ -116,13 +116,14 @@ static void two_passes(int n, int64_t work, int64_t grain, const F& first, const
 // group (grp_ptr / grp_first): the CTA-pair kernel stages one input tile, Kt - 1 frames deeper, per group.
 static const UmmaLayout* step_layout(rt3d_packed* p, int n_tile, bool t_groups, int chunk) {
   std::lock_guard<std::mutex> lock(p->mu);
-  const int key = umma_key(n_tile, t_groups);
+  const int key = umma_key(n_tile, t_groups, p->dtype == RT3D_BF16 && chunk != kChunk);
   auto it = p->umma_layouts.find(key);
   if (it != p->umma_layouts.end()) return &it->second;
 
   UmmaLayout L;
   L.n_tile = n_tile;
   L.t_groups = t_groups;
+  L.chunk = chunk;
   if (t_groups) L.grp_ptr.assign(1, 0);
   L.n_bundles = ceil_div(p->M, n_tile);
   L.n_chunks = ceil_div(p->N, chunk);
@@ -176,11 +177,11 @@ static const UmmaLayout* step_layout(rt3d_packed* p, int n_tile, bool t_groups, 
   return &res.first->second;
 }
 
-const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups) {
-  if (!umma_layout_possible(p)) return nullptr;
+const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups, bool narrow) {
+  if (!umma_layout_possible(p) || (narrow && ceil_div(p->N, kNarrowChunk) > 4095)) return nullptr;
   if (n_tile <= 0) n_tile = default_n_tile(p->M);
   if (n_tile % 16 || n_tile > 256) return nullptr;
-  return step_layout(p, n_tile, t_groups, kChunk);
+  return step_layout(p, n_tile, t_groups, narrow ? kNarrowChunk : kChunk);
 }
 
 // Three bf16 parts hold a weight to the last bit if it is neither huge nor so small that its last bits fall out of their range.

@@ -17,6 +17,7 @@ namespace rt3d {
 constexpr int kMaxGroup = 256;      // g_m, g_n <= 256 (pack, tensor-core kernels)
 constexpr int kMaxGroupSimt = 8;    // the CUDA-core kernel keeps one group row in registers: g_m, g_n <= 8
 constexpr int kChunk = 64;          // input channels per tensor-core K step (one 128-byte swizzle row of bf16)
+constexpr int kNarrowChunk = 32;    // the same for layers of up to 32
 constexpr int kSplitChunk = 32;     // the same of the fp32 tensor-core kernel (one 128-byte row of fp32)
 constexpr int kTileM = 128;         // output voxels per tensor-core tile (TMEM lanes)
 
@@ -47,7 +48,8 @@ inline void decode_step(int32_t s, int& kt, int& kh, int& kw, int& chunk) {
 struct UmmaLayout {
   int n_tile = 0;                    // multiple of 16, <= 256
   int n_bundles = 0;                 // ceil(M / n_tile)
-  int n_chunks = 0;                  // ceil(N / 64)
+  int chunk = kChunk;                // input channels of a step
+  int n_chunks = 0;                  // ceil(N / chunk)
   std::vector<int32_t> step_ptr;     // [n_bundles + 1] offsets into steps / weight tiles
   std::vector<int32_t> steps;        // encoded (kt,kh,kw,chunk), only non-empty steps of each bundle
   std::vector<int32_t> slots;        // [n_bundles][Ks][n_chunks] index of that (location, chunk)'s step, -1 if it has none
@@ -208,11 +210,11 @@ namespace rt3d {
 // The weight tiles [steps.size()][n_tile][64] of a layout on the host (checks; the device fills its own).
 std::vector<uint16_t> fill_umma_tiles(const rt3d_packed* p, const UmmaLayout& L);
 
-inline int umma_key(int n_tile, bool t_groups) { return n_tile + (t_groups ? 4096 : 0); }
+inline int umma_key(int n_tile, bool t_groups, bool narrow) { return n_tile + (t_groups ? 4096 : 0) + (narrow ? 8192 : 0); }
 // Default bundle width for M output channels: as few bundles as possible with n_tile <= 256.
 int default_n_tile(int M);
 // Builds (or returns the cached) tensor-core layout; nullptr if the handle cannot use it.
-const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups = false);
+const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups = false, bool narrow = false);
 bool umma_layout_possible(const rt3d_packed* p);
 // Steps of 32 input channels for the fp32 tensor-core kernel; nullptr if the handle or its weights do not suit it.
 const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile);

@@ -148,6 +148,22 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   return d;
 }
 
+// The same for tiles of 64-byte rows, 64-byte swizzle, 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
+  return uint64_t((addr & 0x3FFFFu) >> 4) | uint64_t(1) << 16 | uint64_t(512 >> 4) << 32 | uint64_t(1) << 46 | uint64_t(4) << 61;
+}
+// K steps of the step-list kernels: 64 input channels, or 32 (narrow) for layers that have no more.
+template <bool kNarrow>
+struct StepShape {
+  static constexpr int channels = kNarrow ? 32 : 64, k16 = channels / 16;
+  static constexpr uint32_t row = channels * 2, a_bytes = 128 * row;
+};
+template <bool kNarrow>
+__device__ __forceinline__ uint64_t smem_desc_step(uint32_t addr) {
+  if constexpr (kNarrow) return smem_desc_sw64(addr);
+  else return smem_desc_sw128(addr);
+}
+
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t instr_desc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);

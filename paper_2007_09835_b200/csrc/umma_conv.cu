@@ -67,15 +67,16 @@ __device__ __forceinline__ void item_steps(const UmmaArgs& a, const ItemCoord& c
 // layer.
 constexpr int kThreadsSingle = 320;
 
-template <bool kDense, int kCps>
+template <bool kDense, int kCps, bool kNarrow>
 __global__ void __launch_bounds__(kThreadsSingle, 1)
 conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
                    const __grid_constant__ CUtensorMap ymap, const UmmaArgs a, const int stages, const int tmem_cols) {
+  using Step = StepShape<kNarrow>;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;            // operand tiles need 1024-byte alignment
-  const uint32_t b_bytes = uint32_t(a.n_tile) * 128u;
-  const uint32_t chunk_bytes = kABytes + b_bytes;
+  const uint32_t b_bytes = uint32_t(a.n_tile) * Step::row;
+  const uint32_t chunk_bytes = Step::a_bytes + b_bytes;
   const uint32_t stage_bytes = kCps * chunk_bytes;
   const uint32_t store_smem = tiles_base + uint32_t(stages) * stage_bytes;     // 4 warps x 2 staging buffers
   Barriers* bars = reinterpret_cast<Barriers*>(smem_raw + (tiles_base - raw) + size_t(stages) * stage_bytes +
@@ -154,7 +155,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      const uint32_t tx_bytes = uint32_t(box_rows) * 128u + b_bytes;
+      const uint32_t tx_bytes = uint32_t(box_rows) * Step::row + b_bytes;
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const bool first_item = item == int(blockIdx.x);                // decoded before the dependency wait
         const ItemCoord c = first_item ? pre_c : decode_item(a, item, n_mtiles);
@@ -177,7 +178,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
           for (int q = 0; q < kCps; ++q) {
             if (q >= nload) break;
             if (kDense) {
-              c_ch[q] = ch * 64; c_w[q] = wq + kw; c_h[q] = hq + kh; c_t[q] = tq + kt;
+              c_ch[q] = ch * Step::channels; c_w[q] = wq + kw; c_h[q] = hq + kh; c_t[q] = tq + kt;
               if (++ch == a.n_chunks) { ch = 0; if (++kw == a.g.Kw) { kw = 0; if (++kh == a.g.Kh) { kh = 0; ++kt; } } }
             } else {
               int enc;
@@ -189,7 +190,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
                 enc = __ldg(a.steps + s_begin + i + q);
               }
               c_t[q] = tq + ((enc >> 24) & 63); c_h[q] = hq + ((enc >> 18) & 63); c_w[q] = wq + ((enc >> 12) & 63);
-              c_ch[q] = (enc & 4095) * 64;
+              c_ch[q] = (enc & 4095) * Step::channels;
             }
           }
           const uint32_t full = smem_u32(&bars->full[stage]);
@@ -204,7 +205,7 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
             if (q >= nload) break;
             const uint32_t a_dst = s_dst + q * chunk_bytes;
             tma_load_5d(a_dst, &xmap, full, c_ch[q], c_w[q], c_h[q], c_t[q], c.n0);
-            tma_load_2d(a_dst + kABytes, &wmap, full, 0, wrow);
+            tma_load_2d(a_dst + Step::a_bytes, &wmap, full, 0, wrow);
             wrow += a.n_tile;
           }
           if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -244,10 +245,10 @@ conv3d_umma_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         for (int q = 0; q < kCps; ++q) {
           if (q >= nload) break;
           const uint32_t a_addr = tiles_base + stage * stage_bytes + q * chunk_bytes;
-          const uint64_t adesc = smem_desc_sw128(a_addr);
-          const uint64_t bdesc = smem_desc_sw128(a_addr + kABytes);
+          const uint64_t adesc = smem_desc_step<kNarrow>(a_addr);
+          const uint64_t bdesc = smem_desc_step<kNarrow>(a_addr + Step::a_bytes);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)    // 4 x K=16 per 64-channel chunk: +32 bytes = +2 in descriptor units
+          for (int kk = 0; kk < Step::k16; ++kk)    // K=16 at a time: +32 bytes = +2 in descriptor units
             if (elected) umma_bf16(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, (i | q | kk) ? 1u : 0u);
         }
         if (elected) umma_commit(smem_u32(&bars->empty[stage]));
@@ -391,19 +392,19 @@ int pick_stages(int n_tile) {
   return s > kMaxStages ? kMaxStages : s;
 }
 
-template <bool kDense, int kCps>
+template <bool kDense, int kCps, bool kNarrow>
 cudaError_t launch_single_t(const UmmaArgs& a, const CUtensorMap& xm, const CUtensorMap& wm, const CUtensorMap& ym, int grid,
                             size_t smem, int stages, int cols, cudaStream_t stream) {
   static bool attr_done[kMaxDevices] = {};             // the attribute is per device
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_kernel<kDense, kCps>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_kernel<kDense, kCps, kNarrow>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
   LaunchSetup ls(dim3(grid), dim3(kThreadsSingle), smem, stream, unsigned(a.n_splits));
-  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_kernel<kDense, kCps>, xm, wm, ym, a, stages, cols);
+  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_kernel<kDense, kCps, kNarrow>, xm, wm, ym, a, stages, cols);
 }
 
 }  // namespace
@@ -421,8 +422,8 @@ int umma_split_capacity(int n_splits, int sm_count) {
     int n = 0;
     LaunchSetup ls(dim3(unsigned(sm_count / n_splits * n_splits)), dim3(kThreadsSingle), smem, nullptr, unsigned(n_splits));
     ls.cfg.numAttrs = 1;                                               // the cluster dimension alone
-    if (cudaFuncSetAttribute(conv3d_umma_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, conv3d_umma_kernel<false, 2>, &ls.cfg) != cudaSuccess)
+    if (cudaFuncSetAttribute(conv3d_umma_kernel<false, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, conv3d_umma_kernel<false, 2, false>, &ls.cfg) != cudaSuccess)
       n = 0;
     v = n * n_splits + 1;
     known[dev][n_splits].store(v);
@@ -444,7 +445,7 @@ cudaError_t launch_conv_umma(const UmmaArgs& a, const void* xmap, const void* wm
   int cols = 32;
   while (cols < 2 * a.n_tile) cols *= 2;
   if (cols > 512) return cudaErrorInvalidValue;
-  if (a.n_splits < 1 || a.n_splits > kMaxSplits) return cudaErrorInvalidValue;
+  if ((a.narrow && a.dense) || a.n_splits < 1 || a.n_splits > kMaxSplits) return cudaErrorInvalidValue;
   const long long n_items = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w * a.n_bundles * a.n_splits;
   if (n_items <= 0) return cudaSuccess;
   if (n_items > (1ll << 30)) return cudaErrorInvalidValue;
@@ -455,10 +456,17 @@ cudaError_t launch_conv_umma(const UmmaArgs& a, const void* xmap, const void* wm
   memcpy(&wm, wmap, sizeof(CUtensorMap));
   memcpy(&ym, ymap ? ymap : xmap, sizeof(CUtensorMap));
   const bool two = pick_cps_single(a.n_tile) == 2;
-  if (a.dense) return two ? launch_single_t<true, 2>(a, xm, wm, ym, grid, smem, stages, cols, stream)
-                          : launch_single_t<true, 1>(a, xm, wm, ym, grid, smem, stages, cols, stream);
-  return two ? launch_single_t<false, 2>(a, xm, wm, ym, grid, smem, stages, cols, stream)
-             : launch_single_t<false, 1>(a, xm, wm, ym, grid, smem, stages, cols, stream);
+  if (a.narrow) {
+    // A stage holds as many steps, of half the bytes, and there are up to twice as many: at eight stages the ring still holds
+    // the 512 n_tile bytes of a K split's share (8 x (8192 + 64 n_tile) and more).
+    const int more = 2 * stages < kMaxStages ? 2 * stages : kMaxStages;
+    return two ? launch_single_t<false, 2, true>(a, xm, wm, ym, grid, smem, more, cols, stream)
+               : launch_single_t<false, 1, true>(a, xm, wm, ym, grid, smem, more, cols, stream);
+  }
+  if (a.dense) return two ? launch_single_t<true, 2, false>(a, xm, wm, ym, grid, smem, stages, cols, stream)
+                          : launch_single_t<true, 1, false>(a, xm, wm, ym, grid, smem, stages, cols, stream);
+  return two ? launch_single_t<false, 2, false>(a, xm, wm, ym, grid, smem, stages, cols, stream)
+             : launch_single_t<false, 1, false>(a, xm, wm, ym, grid, smem, stages, cols, stream);
 }
 
 }  // namespace rt3d

@@ -68,16 +68,18 @@ constexpr int kTsTable = 2048;
 // in the same shared memory (a 64 -> 128 channel 3x3x3 layer was bound by that, at 387 clocks per step against 256).
 // kTurn: the epilogue of a whole tile turns its pieces in shared memory (a.turned); a variant of its own, because the code
 // of both in one kernel cost layers that use neither 0.5 to 1 %.
-template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn>
+// kNarrow: steps of 32 input channels.
+template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn, bool kNarrow>
 __global__ void __launch_bounds__(kThreadsPair, 1)
 conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap_half,
                         const __grid_constant__ CUtensorMap ymap, const UmmaArgs a, const int stages, const int tmem_cols) {
+  using Step = StepShape<kNarrow>;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
   const int n_half = a.n_tile / 2;
-  const uint32_t b_bytes = uint32_t(n_half) * 128u;             // this CTA's half of the B tile
-  const uint32_t chunk_bytes = kABytes + b_bytes;
+  const uint32_t b_bytes = uint32_t(n_half) * Step::row;           // this CTA's half of the B tile
+  const uint32_t chunk_bytes = Step::a_bytes + b_bytes;
   const uint32_t ts_a_slot = (uint32_t(a.ts_a_bytes) + 1023u) & ~1023u;
   const uint32_t ts_a_all = ts_a_slot * uint32_t(a.ts_phases);       // one deeper tile per phase of the temporal stride
   const uint32_t stage_bytes = kTS ? ts_a_all + uint32_t(a.g.Kt) * b_bytes : kCps * chunk_bytes;
@@ -215,7 +217,7 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      const uint32_t tx_chunk_both = 2u * (uint32_t(box_rows) * 128u + b_bytes);
+      const uint32_t tx_chunk_both = 2u * (uint32_t(box_rows) * Step::row + b_bytes);
       const int n_work = tw->n_full + tw->n_seg;
       for (int wi = 0; kTS && wi < n_work && ok; ++wi) {
         const Work wk = get_work(tw, wi, cluster_id, n_clusters);
@@ -250,7 +252,7 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
           if (leader) mbar_expect_tx(full_local, 2u * (uint32_t(a.ts_phases * a.ts_a_bytes) + uint32_t(ns) * b_bytes));
           // tile r: the frames t * st + r (traversal stride st along t), so that tap kt = q * st + r is its rows from frame q on
           for (int r = 0; r < a.ts_phases; ++r)
-            tma_load_5d_pair(s_dst + uint32_t(r) * ts_a_slot, &xmap, full_leader, ch * 64, wq + kw, hq + kh, tq + r, c.n0);
+            tma_load_5d_pair(s_dst + uint32_t(r) * ts_a_slot, &xmap, full_leader, ch * Step::channels, wq + kw, hq + kh, tq + r, c.n0);
           const int wrow = s0 * a.n_tile + int(rank) * n_half;
           for (int q = 0; q < ns; ++q)
             tma_load_2d_pair(s_dst + ts_a_all + uint32_t(q) * b_bytes, &wmap_half, full_leader, 0, wrow + q * a.n_tile);
@@ -278,12 +280,12 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
           for (int q = 0; q < kCps; ++q) {
             if (q >= nload) break;
             if (kDense) {
-              c_ch[q] = ch * 64; c_w[q] = wq + kw; c_h[q] = hq + kh; c_t[q] = tq + kt;
+              c_ch[q] = ch * Step::channels; c_w[q] = wq + kw; c_h[q] = hq + kh; c_t[q] = tq + kt;
               if (++ch == a.n_chunks) { ch = 0; if (++kw == a.g.Kw) { kw = 0; if (++kh == a.g.Kh) { kh = 0; ++kt; } } }
             } else {
               const int enc = __ldg(a.steps + s_begin + i + q);
               c_t[q] = tq + ((enc >> 24) & 63); c_h[q] = hq + ((enc >> 18) & 63); c_w[q] = wq + ((enc >> 12) & 63);
-              c_ch[q] = (enc & 4095) * 64;
+              c_ch[q] = (enc & 4095) * Step::channels;
             }
           }
           const uint32_t full_local = smem_u32(&bars->full[stage]);
@@ -296,7 +298,7 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
             if (q >= nload) break;
             const uint32_t a_dst = s_dst + q * chunk_bytes;
             tma_load_5d_pair(a_dst, &xmap, full_leader, c_ch[q], c_w[q], c_h[q], c_t[q], c.n0);
-            tma_load_2d_pair(a_dst + kABytes, &wmap_half, full_leader, 0, wrow);
+            tma_load_2d_pair(a_dst + Step::a_bytes, &wmap_half, full_leader, 0, wrow);
             wrow += a.n_tile;
           }
           if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -337,10 +339,10 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
             for (int q = 0; q < ns; ++q) {
               // computed steps (temporal stride 1 only): kt = q.  Every instruction in this loop shows in the time of
               // a 128-wide layer (four more ALU operations per step cost 6 %).
-              const uint64_t adesc = smem_desc_sw128(s_base + (kDense ? uint32_t(q) * uint32_t(a.ts_frame_bytes) : aoff_s[s0 + q]));
-              const uint64_t bdesc = smem_desc_sw128(s_base + ts_a_all + uint32_t(q) * b_bytes);
+              const uint64_t adesc = smem_desc_step<kNarrow>(s_base + (kDense ? uint32_t(q) * uint32_t(a.ts_frame_bytes) : aoff_s[s0 + q]));
+              const uint64_t bdesc = smem_desc_step<kNarrow>(s_base + ts_a_all + uint32_t(q) * b_bytes);
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
+              for (int kk = 0; kk < Step::k16; ++kk)
                 umma_bf16_pair(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, (!fresh | q | kk) ? 1u : 0u);
             }
             fresh = false;
@@ -374,10 +376,10 @@ conv3d_umma_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_c
             for (int q = 0; q < kCps; ++q) {
               if (q >= nload) break;
               const uint32_t a_addr = tiles_base + stage * stage_bytes + q * chunk_bytes;
-              const uint64_t adesc = smem_desc_sw128(a_addr);
-              const uint64_t bdesc = smem_desc_sw128(a_addr + kABytes);
+              const uint64_t adesc = smem_desc_step<kNarrow>(a_addr);
+              const uint64_t bdesc = smem_desc_step<kNarrow>(a_addr + Step::a_bytes);
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
+              for (int kk = 0; kk < Step::k16; ++kk)
                 umma_bf16_pair(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, (!fresh | q | kk) ? 1u : 0u);
             }
             fresh = false;
@@ -556,7 +558,7 @@ size_t pair_smem_bytes(int n_tile, int n_bundles) {
 
 // t-grouped variant: a stage = one deeper input tile + Kt weight half-tiles; the tables come after the bias.
 size_t ts_stage_bytes(const UmmaArgs& a) {
-  return size_t(a.ts_phases) * ((size_t(a.ts_a_bytes) + 1023) & ~size_t(1023)) + size_t(a.g.Kt) * size_t(a.n_tile / 2) * 128;
+  return size_t(a.ts_phases) * ((size_t(a.ts_a_bytes) + 1023) & ~size_t(1023)) + size_t(a.g.Kt) * size_t(a.n_tile / 2) * (a.narrow ? 64 : 128);
 }
 int pick_stages_pair_ts(const UmmaArgs& a) {
   const size_t fixed = 1024 + 4 * kStoreWarpBytes + sizeof(Barriers) + sizeof(TailWork) + 16 +
@@ -571,13 +573,13 @@ size_t pair_smem_bytes_ts(const UmmaArgs& a) {
          16 + size_t(a.n_tile) * a.n_bundles * 4 + (3 * size_t(a.ts_table) + 16) * 4;
 }
 
-template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn>
+template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn, bool kNarrow>
 cudaError_t prepare_pair_t() {
   static bool attr_done[kMaxDevices] = {};             // the attribute is per device
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, kTurn>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, kTurn, kNarrow>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -604,12 +606,12 @@ int pair_max_clusters_t(int sm_count, size_t smem) {
   if (dev < 0) return sm_count / 2;
   int& max_clusters = max_clusters_dev[dev];
   if (max_clusters == 0) {
-    if (prepare_pair_t<kDense, kCps, kTS, kDual, false>() != cudaSuccess) return sm_count / 2;
+    if (prepare_pair_t<kDense, kCps, kTS, kDual, false, false>() != cudaSuccess) return sm_count / 2;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     pair_launch_config(cfg, attr, unsigned(sm_count & ~1), smem, nullptr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, false>, &cfg) != cudaSuccess || n <= 0) n = sm_count / 2;
+    if (cudaOccupancyMaxActiveClusters(&n, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, false, false>, &cfg) != cudaSuccess || n <= 0) n = sm_count / 2;
     max_clusters = n;
   }
   return max_clusters < sm_count / 2 ? max_clusters : sm_count / 2;
@@ -643,18 +645,29 @@ int pair_max_clusters_ts(const UmmaArgs& a, int sm_count) {
 #undef RT3D_CALL
 }
 
+template <bool kDense, int kCps, bool kTS, bool kDual, bool kTurn, bool kNarrow>
+cudaError_t launch_pair_on(const UmmaArgs& a, const CUtensorMap& xm, const CUtensorMap& wm, const CUtensorMap& ym, int stages, int cols,
+                           LaunchSetup& ls) {
+  const cudaError_t e = prepare_pair_t<kDense, kCps, kTS, kDual, kTurn, kNarrow>();
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&ls.cfg, conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, kTurn, kNarrow>, xm, wm, ym, a, stages, cols);
+}
+
 template <bool kDense, int kCps, bool kTS, bool kDual>
 cudaError_t launch_pair_t(const UmmaArgs& a, const CUtensorMap& xm, const CUtensorMap& wm, const CUtensorMap& ym,
                           int sm_count, int stages,
                           int cols, size_t smem, long long n_items, cudaStream_t stream) {
-  cudaError_t e = a.turned ? prepare_pair_t<kDense, kCps, kTS, kDual, true>() : prepare_pair_t<kDense, kCps, kTS, kDual, false>();
-  if (e != cudaSuccess) return e;
   long long clusters = pair_max_clusters_t<kDense, kCps, kTS, kDual>(sm_count, smem);
   const long long want = n_items > a.tail_workers ? n_items : a.tail_workers;
   if (clusters > want) clusters = want;
   LaunchSetup ls(dim3(unsigned(2 * clusters)), dim3(kThreadsPair), smem, stream, 2);
-  return cudaLaunchKernelEx(&ls.cfg, a.turned ? conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, true> : conv3d_umma_pair_kernel<kDense, kCps, kTS, kDual, false>,
-                            xm, wm, ym, a, stages, cols);
+  if constexpr (!kDense) {
+    if (a.narrow)                                      // twice as many steps of half the bytes in a stage
+      return a.turned ? launch_pair_on<false, 2 * kCps, kTS, kDual, true, true>(a, xm, wm, ym, stages, cols, ls)
+                      : launch_pair_on<false, 2 * kCps, kTS, kDual, false, true>(a, xm, wm, ym, stages, cols, ls);
+  }
+  return a.turned ? launch_pair_on<kDense, kCps, kTS, kDual, true, false>(a, xm, wm, ym, stages, cols, ls)
+                  : launch_pair_on<kDense, kCps, kTS, kDual, false, false>(a, xm, wm, ym, stages, cols, ls);
 }
 
 }  // namespace
@@ -674,7 +687,7 @@ bool umma_pair_ts_supported(UmmaArgs* a, int total_steps) {
   t.ts_phases = a->g.st;
   const int frames = a->box.bt + (a->g.Kt - 1) / a->g.st;          // per phase tile (the deepest phase; the others load as many)
   if (frames * a->g.st > 256 || total_steps > kTsTable) return false;
-  t.ts_frame_bytes = a->box.bh * a->box.bw * 128;
+  t.ts_frame_bytes = a->box.bh * a->box.bw * (a->narrow ? 64 : 128);
   t.ts_a_bytes = frames * t.ts_frame_bytes;
   t.ts_table = a->dense ? 0 : (total_steps + 3) & ~3;
   // it has to fit with at least as many steps in flight as the step-per-location form has
@@ -701,12 +714,12 @@ void umma_pair_tail_plan(UmmaArgs* a, const int32_t* step_ptr_host, int sm_count
   const long long rounds = n_items / clusters;
   const int n_tail = int(n_items - rounds * clusters);
   if (n_tail == 0 || n_tail > kMaxTail) return;
-  const int cps = a->ts ? a->g.Kt : pick_cps(a->n_tile);   // steps per unit of the split, about
+  const int cps = a->ts ? a->g.Kt : pick_cps(a->n_tile) * (a->narrow ? 2 : 1);   // steps per unit of the split, about
   long long total = 0, g_min = 1 << 30, g_max = 0;
   for (int t = 0; t < n_tail; ++t) {
     const int b = int((rounds * clusters + t) / pairs_per_bundle);
     const int ns = a->dense ? a->steps_dense : step_ptr_host[b + 1] - step_ptr_host[b];
-    if (ns < 8) return;                                   // nothing worth cutting
+    if (ns < (a->narrow ? 16 : 8)) return;                                   // nothing worth cutting
     long long g = (ns + cps - 1) / cps;
     if (a->ts) g = a->dense ? (long long)a->g.Kh * a->g.Kw * a->n_chunks : grp_ptr_host[b + 1] - grp_ptr_host[b];
     total += g;
@@ -722,7 +735,7 @@ void umma_pair_tail_plan(UmmaArgs* a, const int32_t* step_ptr_host, int sm_count
   // Storing the shares and the owner's fix-up (the eight epilogue warps pulling the other shares through registers) are taken
   // to cost as much as this many K steps.  Measured with it: 54 steps an item gain (128 -> 256 at 8 x 8 x 28 x 28, 57.5 -> 54.9
   // us); 27 steps, 256 wide, lose: 111 items with 37 left over take 28.2 us split, 147 in two whole rounds 24.0.
-  const long long fixup_groups = (12 + cps - 1) / cps;
+  const long long fixup_groups = ((a->narrow ? 24 : 12) + cps - 1) / cps;
   if (range + fixup_groups >= g_max) return;
   a->tail_workers = int(workers);
   // per pair: one share (the first segment of its range) x two CTAs; one flag per epilogue warp
@@ -732,7 +745,7 @@ void umma_pair_tail_plan(UmmaArgs* a, const int32_t* step_ptr_host, int sm_count
 
 cudaError_t launch_conv_umma_pair(const UmmaArgs& a, const void* xmap, const void* wmap_half, const void* ymap,
                                   int sm_count, cudaStream_t stream) {
-  if (!umma_pair_supported(a.n_tile, a.n_bundles) || a.n_splits != 1) return cudaErrorInvalidValue;
+  if (!umma_pair_supported(a.n_tile, a.n_bundles) || a.n_splits != 1 || (a.narrow && a.dense)) return cudaErrorInvalidValue;
   if (a.tail_workers > 0 && (a.tail_scratch == nullptr || a.tail_flags == nullptr)) return cudaErrorInvalidValue;
   const int stages = a.ts ? pick_stages_pair_ts(a) : pick_stages_pair(a.n_tile);
   const size_t smem = a.ts ? pair_smem_bytes_ts(a) : pair_smem_bytes(a.n_tile, a.n_bundles);
