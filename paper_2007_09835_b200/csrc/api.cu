@@ -274,11 +274,17 @@ class Submit {
     *status = run(*c);
     return true;
   }
+  bool keep = true;                            // whether the chosen launch is kept for later calls
+  // Whether the call goes into a graph that is being captured: nothing can be allocated or uploaded then.
+  bool captured() const {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    return !t_plan_only && st_ != nullptr && cudaStreamIsCapturing(st_, &status) == cudaSuccess && status != cudaStreamCaptureStatusNone;
+  }
   // A kernel launch chosen for this call.  `launch` must hold by value whatever it needs besides the handle's own memory, and
   // take the addresses of the tensors and biases from its argument.
   rt3d_status operator()(const rt3d_plan_info& info, std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch) {
     auto c = std::make_shared<PreparedCall>(PreparedCall{key_, info, std::move(launch)});
-    {
+    if (keep) {
       std::lock_guard<std::mutex> lock(w_->mu);
       if (w_->calls.size() < kPreparedCalls) w_->calls.push_back(c);
       else w_->calls[w_->next_call++ % kPreparedCalls] = c;
@@ -436,6 +442,12 @@ rt3d_status get_umma_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L,
   return RT3D_OK;
 }
 
+bool umma_blob_ready(rt3d_packed* h, DeviceBlob* blob, int key) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  const auto it = blob->umma.find(key);
+  return it != blob->umma.end() && it->second.ready;
+}
+
 // Device copy of the fp32 tensor-core kernel's layout, with the canonical arrays beside it.
 rt3d_status get_split_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, bool pair, DeviceBlob::Umma** out) {
   std::lock_guard<std::mutex> lock(h->mu);
@@ -575,11 +587,11 @@ struct UmmaPlan { int n_tile, n_splits; bool pair; };
 // of 64, they lose: the copy engine takes rows at a rate, not bytes (77 -> 186 28.4 -> 31.7, 470 -> 182 33 -> 46, 265 -> 511 51 -> 63).
 bool narrow_steps(const rt3d_packed* w) { return w->N <= kNarrowChunk && g_narrow_enabled.load(); }
 
-UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_count) {
+UmmaPlan pick_plan(rt3d_packed* w, const ConvGeom& g, long long m_tiles, int sm_count, bool narrow) {
   const int M = w->M;
   // Of a full step's bytes and MMAs; its hand-shake is the same.  (With few steps the output counts, and a bundle is no wider for
   // it: 24 -> 347 1x3x3 on 14 x 4 x 7 x 7 at 64 columns 6.3 us, at 176 7.6.)
-  const double part = narrow_steps(w) && w->Ks > 12 ? 0.5 : 1.0;
+  const double part = narrow && w->Ks > 12 ? 0.5 : 1.0;
   const int widest = default_n_tile(M);
   const bool tall = w->g_m >= 16 && !w->is_dense;
   UmmaPlan best{widest, 1, false};
@@ -988,6 +1000,14 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
   return RT3D_OK;
 }
 
+constexpr int kSplitFewest = 16;                           // input channels up to which no fp32 call goes to the tensor cores
+
+// A row computed again stays far below the limit of the others' waits.
+bool split_channels_fit(const rt3d_packed* w) { return int64_t(w->Ks) * w->N <= 32768; }
+
+// Bundle width there: as few bundles of up to 128 channels as there can be.
+int split_n_tile(int M) { return round_up(ceil_div(M, ceil_div(M, 128)), 16); }
+
 // Whether an fp32 call is expected to take less time on the tensor cores than on the CUDA cores.  Both models are fitted to 92
 // random layers (8-160 input and 16-160 output channels, 0.2-1 kept, 6-530 us) on B200.  CUDA cores: the cycles of the plan
 // search at 0.656 ns, 3 us around them (half of the layers within 0.83-1.1 of it).  Tensor cores: 8 us around the rounds of
@@ -997,7 +1017,7 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
 // Up to 16 input channels stay on the CUDA cores: half of every step would be empty, and the tests of the register-blocked
 // kernel expect it there.  (It costs 16 -> 74 channels 3x3x3 dense on 16 x 51 x 35 35 us instead of 20.)
 bool split_is_faster(const rt3d_packed* w, const F32SplitArgs& a, int sm_count) {
-  if (w->N <= 16) return false;
+  if (w->N <= kSplitFewest) return false;
   const double density = double(w->nnz) / (double(w->P) * w->Q * w->Ks);
   const double groups = double(std::max(1, kSplitChunk / w->g_n)) * std::max(1, a.n_tile / w->g_m);     // that share a step
   const double steps = double(w->Ks) * ceil_div(w->N, kSplitChunk) * (w->is_dense ? 1.0 : 1.0 - std::pow(1.0 - density, groups));
@@ -1023,19 +1043,22 @@ rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt
   if (mode == 0 || d->cc_major != 10 || w->dtype != RT3D_F32 || x->c_stride % 4 || y->c_stride % 4 || (res_data && res_pitch % 4)) return RT3D_OK;
   if (g.st > 8 || g.sh > 8 || g.sw > 8 || int64_t(x->w) * x->c_stride * 4 >= (int64_t(1) << 40)) return RT3D_OK;
   if (int64_t(g.n) * g.To * g.Ho * g.Wo > 0x7fffffff) return RT3D_OK;
-  if (int64_t(w->Ks) * w->N > 32768) return RT3D_OK;       // a row computed again stays far below the limit of the others' waits
+  if (!split_channels_fit(w)) return RT3D_OK;
   F32SplitArgs a;
   a.g = g;
   a.box = choose_box(g);
   a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
   a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
-  const int bundles = ceil_div(w->M, 128);
-  a.n_tile = round_up(ceil_div(w->M, bundles), 16); a.n_bundles = ceil_div(w->M, a.n_tile);
+  a.n_tile = split_n_tile(w->M); a.n_bundles = ceil_div(w->M, a.n_tile);
   a.period = a.n_tile > 64 ? 8 : 4;
   if (!umma_f32_plan(&a) || (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w * a.n_bundles > (1ll << 30)) return RT3D_OK;
   if (mode == 1 && !split_is_faster(w, a, d->sm_count)) return RT3D_OK;
   const UmmaLayout* L = get_split_layout(w, a.n_tile);
   if (!L) return RT3D_OK;
+  if (submit.captured() && !umma_blob_ready(w, blob, umma_key(L->n_tile, false, false))) {
+    submit.keep = false;                                   // the CUDA cores' layout may be there
+    return RT3D_OK;
+  }
   DeviceBlob::Umma* u = nullptr;
   rt3d_status s = get_split_blob(w, blob, L, a.pair != 0, &u);
   if (s != RT3D_OK) return s;
@@ -1100,8 +1123,9 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   return RT3D_OK;
 }
 
+// `narrow`: whether the step-list kernels may take steps of 32 channels.
 rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
-                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz) {
+                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz, bool narrow = true) {
   CallKey key;
   CallBuffers buffers{};
   if (make_key(&key, x, wc, bias, p, y, fz ? fz->residual : nullptr, dense_entry ? 1 : 0)) {
@@ -1144,6 +1168,8 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   DeviceBlob* blob = nullptr;
   if ((s = get_blob(w, &blob)) != RT3D_OK) return s;
   Submit submit(w, key, buffers, static_cast<cudaStream_t>(stream));
+  submit.keep = narrow;
+  narrow = narrow && narrow_steps(w);
 
   const bool can_umma = umma_eligible(d, w, x, y, p);
   const bool can_simt = w->g_m <= kMaxGroupSimt && w->g_n <= kMaxGroupSimt;
@@ -1205,7 +1231,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
   a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
   long long m_tiles = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
-  UmmaPlan plan = pick_plan(w, g, m_tiles, d->sm_count);
+  UmmaPlan plan = pick_plan(w, g, m_tiles, d->sm_count, narrow);
   if (pooled) {                     // pooling lives in the TMA-store epilogue, which a K split does not use
     // A layer this small is faster split over K and pooled by a second launch: AUTO declines the fusion.
     if (p->algo == RT3D_ALGO_AUTO && plan.n_splits > 1) return RT3D_ERR_UNSUPPORTED;
@@ -1229,7 +1255,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   bool use_ts = false;
   // (few steps on single CTAs wait for their first tiles and for their output: in the S3D-shaped forward, whose branches have
   // 16 to 32 channels there, 772 us as a graph, 778 in steps of 32)
-  a.narrow = narrow_steps(w) && (use_pair || w->Ks > 12) ? 1 : 0;
+  a.narrow = narrow && (use_pair || w->Ks > 12) ? 1 : 0;
   UmmaArgs probe = a;
   // (wide bundles: only kernels that are also wide in space; a 3x1x1 layer with 192-wide bundles lost 8 us of 43
   // inside the S3D-shaped forward with it, while 3x3x3 layers gain 1-4 %)
@@ -1268,6 +1294,9 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   }
   const UmmaLayout* L = get_umma_layout(w, plan.n_tile, use_ts, a.narrow != 0);
   if (!L) return RT3D_ERR_UNSUPPORTED;
+  // rt3d_packed_prepare uploads the steps of 64, which rt3d_conv3d_sparse_noalloc reads too
+  if (narrow && submit.captured() && !umma_blob_ready(w, blob, umma_key(L->n_tile, use_ts, a.narrow != 0)))
+    return conv_body(x, wc, bias, p, y, stream, dense_entry, fz, false);
   DeviceBlob::Umma* u = nullptr;
   if ((s = get_umma_blob(w, blob, L, &u)) != RT3D_OK) return s;
   a.n_tile = L->n_tile; a.n_bundles = L->n_bundles; a.n_chunks = L->n_chunks;
@@ -1570,6 +1599,13 @@ static rt3d_status prepare_body(rt3d_packed* p) {
     if ((s = get_f32_blob(p, blob, L, &u)) != RT3D_OK) return s;
   } else if ((s = get_canonical(p, blob)) != RT3D_OK) {
     return s;
+  }
+  F32SplitArgs split;
+  split.n_tile = split_n_tile(p->M); split.n_bundles = ceil_div(p->M, split.n_tile);
+  if (d->cc_major == 10 && p->dtype == RT3D_F32 && p->N > kSplitFewest && split_channels_fit(p) && g_f32_split.load() && umma_f32_plan(&split)) {
+    DeviceBlob::Umma* u = nullptr;
+    const UmmaLayout* L = get_split_layout(p, split.n_tile);
+    if (L && (s = get_split_blob(p, blob, L, split.pair != 0, &u)) != RT3D_OK) return s;
   }
   for (int S = 2; S <= 8; ++S) umma_split_capacity(S, d->sm_count);      // what the K splits ask the runtime, once per device
   return cudaDeviceSynchronize() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
