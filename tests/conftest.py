@@ -1,4 +1,5 @@
 """Shared pytest configuration: registers the `gpu` marker and puts the repo root on sys.path."""
+import gc
 import os
 import sys
 
@@ -9,3 +10,10 @@ if ROOT not in sys.path:
 
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: test needs a CUDA device (run with -m gpu on a B200)")
+
+
+def pytest_runtest_setup(item):
+    """Handles that earlier tests left in reference cycles (a `pytest.raises` keeps the frames it caught) are freed here.  A free
+    waits for the device, and inside a test of what waits for it and what does not, a collection changes the answer."""
+    if item.get_closest_marker("gpu"):
+        gc.collect()
