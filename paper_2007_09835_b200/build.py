@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librt3d.so")
 SOURCES = ["api.cu", "pack.cpp", "layout.cu", "simt_kernels.cu", "simt_conv_f32.cu", "umma_conv.cu", "umma_conv_pair.cu", "umma_conv_halo.cu", "umma_conv_st.cu", "umma_conv_sub.cu", "umma_smallc.cu", "umma_conv_f32.cu", "reweight.cu", "debug_poison.cu"]
-HEADERS = ["kernels.h", "rt3d_internal.h", "umma_common.cuh", "umma_pair.cuh", "pdl.cuh", "tile_consts.h", "kept_blocks.h"]
+HEADERS = ["kernels.h", "rt3d_internal.h", "umma_common.cuh", "umma_pair.cuh", "pdl.cuh", "tile_consts.h", "kept_blocks.h", "f32_split_plan.h"]
 PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))   # extension module of the binding
 MICROBENCH = os.path.join(HERE, "rt3d_microbench")       # stand-alone instruction-rate microbenchmarks
 

@@ -26,6 +26,7 @@
 // with fp32 FMAs from the packed arrays, skipping what is pruned, by the threads that drain them.
 #include <algorithm>
 
+#include "f32_split_plan.h"
 #include "kernels.h"
 #include "pdl.cuh"
 #include "rt3d_internal.h"
@@ -36,11 +37,9 @@ namespace {
 
 constexpr int kThreadsSplit = 640;
 constexpr int kDrainThreads = 256;
-constexpr int kSplitSlots = 4;                          // most A operands in tensor memory
-constexpr int kSplitInputs = 8;                         // most staged inputs
-constexpr uint32_t kSlotCols = 48;                      // three parts of 32 channels, two to a column
+constexpr uint32_t kSlotCols = kSplitSlotCols;
 constexpr int kSplitSegment = 64;                       // steps after which a shared accumulator of small products is drained
-constexpr uint32_t kDrainStage = 32 * 64;               // bytes with which a drain warp turns 32 voxels x 16 channels
+constexpr uint32_t kDrainStage = kSplitDrainStage;
 
 struct __align__(8) SplitBars {
   Barriers b;                                           // full: weights; empty: MMAs done; tmem_*: the two xh wh accumulators
@@ -49,6 +48,7 @@ struct __align__(8) SplitBars {
   unsigned long long a_full[kSplitSlots];               // A operands (of a pair: and the weights) of both CTAs
   unsigned long long small_empty;                       // the small products' accumulator, where it is shared
 };
+static_assert(sizeof(SplitBars) == kSplitBarBytes && kABytes == kSplitInputBytes, "f32_split_plan.h");
 
 struct SplitItem { int bundle, n0, t0, h0, w0; };
 // `ctas`: tiles of an item, `rank`: which of them.
@@ -160,7 +160,7 @@ __device__ __noinline__ void exact_row(const F32SplitArgs& a, const float* bias_
 //   kSmall: two buffers for xh wh, one [order 2^-8 | order 2^-16], four MMAs
 //   kNone: two buffers for xh wh, one for all small products, six MMAs
 // kPair: CTA pairs.
-enum { kNone, kSmall, kAll };
+constexpr int kNone = kSplitNone, kSmall = kSplitSmall, kAll = kSplitAll;
 template <int NH, int kSub, int kMode, bool kPair>
 __global__ void __launch_bounds__(kThreadsSplit, 1)
 conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ F32SplitArgs a) {
@@ -562,25 +562,6 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
   }
 }
 
-// Variant for a bundle width: columns that a drain thread holds, steps per hand-shake, how the accumulators lie, CTA pairs.
-// Up to 64 columns single CTAs win with three or four MMAs a slice, above that pairs do: half of the weights' traffic in shared
-// memory, and the MMAs are as wide as they take to issue.  64 -> 128 channels 3x3x3 on 2 x 16 x 56 x 56: pairs 168 us, single
-// CTAs 192; 88 -> 41 on 2 x 14 x 59 x 12: 65 and 56.  Two steps per hand-shake where tensor memory holds two such A operands
-// (64 -> 32 on 2 x 16 x 56 x 56 149 -> 117 us).
-struct SplitVariant { int nh, sub, mode; bool pair; };
-SplitVariant split_variant(int n_tile) {
-  if (n_tile <= 32) return {16, 2, kAll, false};
-  if (n_tile <= 48) return {32, 2, kAll, false};
-  if (n_tile <= 64) return {32, 2, kSmall, false};
-  if (n_tile <= 96) return {48, 2, kNone, true};
-  return {64, 1, kNone, true};
-}
-
-size_t split_smem_bytes(const F32SplitArgs& a, const SplitVariant& v) {
-  return 1024 + size_t(v.sub) * (size_t(a.inputs) * kABytes + size_t(a.stages) * a.n_tile * (v.pair ? 96 : 192)) + 8 * kDrainStage +
-         sizeof(SplitBars) + 16 + size_t(a.n_tile) * a.n_bundles * 4;
-}
-
 template <int NH, int kSub, int kMode, bool kPair>
 cudaError_t launch_split_t(const F32SplitArgs& a, const CUtensorMap& xm, int grid, size_t smem, cudaStream_t stream) {
   static bool attr_done[kMaxDevices] = {};             // the attribute is per device
@@ -598,20 +579,19 @@ cudaError_t launch_split_t(const F32SplitArgs& a, const CUtensorMap& xm, int gri
 }  // namespace
 
 bool umma_f32_plan(F32SplitArgs* a) {
-  if (a->n_tile % 16 || a->n_tile < 16 || a->n_tile > 128) return false;
-  const SplitVariant v = split_variant(a->n_tile);
-  a->pair = v.pair ? 1 : 0;
-  a->slots = std::min(kSplitSlots, (512 - (v.mode == kAll ? 6 : v.mode == kSmall ? 4 : 3) * a->n_tile) / (v.sub * int(kSlotCols)));
-  a->stages = a->slots + 2;
-  for (a->inputs = kSplitInputs; a->inputs >= 3; --a->inputs)
-    if (split_smem_bytes(*a, v) <= 227 * 1024) return true;
-  return false;
+  SplitRing r;
+  if (!split_ring(a->n_tile, a->n_bundles, &r)) return false;
+  a->pair = split_variant(a->n_tile).pair ? 1 : 0;
+  a->inputs = r.inputs; a->stages = r.stages; a->slots = r.slots;
+  return true;
 }
 
 cudaError_t launch_conv_umma_f32(const F32SplitArgs& a, const void* xmap, int sm_count, cudaStream_t stream) {
   const SplitVariant v = split_variant(a.n_tile);
-  const size_t smem = split_smem_bytes(a, v);
-  if (smem > 227 * 1024 || a.stages <= a.slots || a.slots < 2 || a.period < 2 || a.period % 2 || kSplitSegment % a.period) return cudaErrorInvalidValue;
+  const SplitRing ring = {a.inputs, a.stages, a.slots};
+  const size_t smem = split_smem_bytes(a.n_tile, a.n_bundles, ring);
+  if (smem > kSplitSmem || a.inputs < 2 || a.inputs > kSplitInputs || a.stages > kMaxStages || !split_inputs_ordered(ring)) return cudaErrorInvalidValue;
+  if (a.stages <= a.slots || a.slots < 2 || a.slots > kSplitSlots || a.period < 2 || a.period % 2 || kSplitSegment % a.period) return cudaErrorInvalidValue;
   const int ctas = v.pair ? 2 : 1;
   const long long items = ((long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w + ctas - 1) / ctas * a.n_bundles;
   if (items <= 0) return cudaSuccess;

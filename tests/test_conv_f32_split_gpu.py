@@ -98,3 +98,23 @@ def test_weights_that_three_bf16_cannot_hold_stay_on_the_cuda_cores(everywhere):
         w[3, 5, 0, 1, 1] = value
         nets.ConvLayer(spec, w, L["bias"], None, 4, 4, torch.float32, dense=True)(xd)
         assert rt3d.rt3d_last_plan()["kernel"] == (8 if value == 0.0 else 0)
+
+
+@pytest.mark.parametrize("cin,cout,k,x", [
+    (64, 64, (3, 3, 3), (2, 8, 40, 40)), (64, 16, (3, 3, 3), (2, 8, 40, 40)), (96, 90, (3, 3, 3), (2, 8, 40, 40)),
+    (20, 3000, (1, 1, 1), (1, 2, 6, 6)), (20, 7680, (1, 1, 1), (1, 2, 6, 6))])           # biases that leave three weight stages, two inputs
+def test_inputs_that_arrive_late(everywhere, cin, cout, k, x):
+    """Boxes from memory beside boxes in the padding, which take no load at all: with nothing in L2 every pass gives the same bits,
+    and what the CUDA cores give up to the order of the sums."""
+    spec = synth.ConvSpec("f32", cin, cout, k, (1, 1, 1), tuple(v // 2 for v in k), False)
+    L = synth.make_layer(spec, 8, cin + cout, 4, 4, "bernoulli", 0.4)
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.float32)
+    xd = nets.to_device(synth.make_input(8, x + (cin,)), torch.float32)
+    want = lay(xd, algo=rt3d.ALGO_SIMT)
+    flush = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    first = lay(xd)
+    assert rt3d.rt3d_last_plan()["kernel"] == 8
+    assert float((first - want).abs().max()) <= 2e-6 * float(want.abs().max())
+    for i in range(5):
+        flush.fill_(i)
+        assert torch.equal(lay(xd), first) and rt3d.rt3d_last_device_status() == rt3d.OK
