@@ -184,7 +184,8 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups, boo
   return step_layout(p, n_tile, t_groups, narrow ? kNarrowChunk : kChunk);
 }
 
-// Three bf16 parts hold a weight to the last bit if it is neither huge nor so small that its last bits fall out of their range.
+// Whether every weight is zero or lies in [2^-100, 2^64): three bf16 parts hold it to the last bit then, and with the inputs' scale
+// of 2^24 inputs below 2^24 in magnitude keep every sum of the fp32 tensor-core kernel in range.
 static bool splits_exactly(const float* w, int64_t n) {
   uint32_t lo = 0xffffffffu, hi = 0;                       // smallest magnitude but zero, largest one
   for (int64_t i = 0; i < n; ++i) {
@@ -194,7 +195,7 @@ static bool splits_exactly(const float* w, int64_t n) {
     hi = std::max(hi, u);
     lo = std::min(lo, u - 1u);                             // zero: the largest
   }
-  return hi < 0x7b800000u && (lo == 0xffffffffu || lo >= 0x0d800000u - 1u);       // 2^120, 2^-100
+  return hi < 0x5f800000u && (lo == 0xffffffffu || lo >= 0x0d800000u - 1u);       // 2^64, 2^-100
 }
 
 const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile) {

@@ -20,10 +20,12 @@
 // and the arithmetic of a step, 0.31 us each.  Errors against 64 bits, relative, CUDA cores and here: 3.3e-7 and 1.2e-7 for
 // that layer, 6.0e-8 and 4.3e-8 for 44 channels 1x1x1; smaller here in all of 90 random layers that the dispatch sends here.
 //
-// What the split cannot hold is found in the result: an infinity or NaN in x, or a magnitude whose rounding to bf16
-// overflows, makes xm or xl a NaN and with them the voxel's whole row (NaN times a pruned weight's zero is NaN too); x below
-// 2^-110, whose last bits no bf16 holds, can only matter where the result is tiny.  Rows with such results are computed again
-// with fp32 FMAs from the packed arrays, skipping what is pruned, by the threads that drain them.
+// Range: x is split as 2^24 x, which leaves the parts of the smallest denormal (2^-149) normal bf16 numbers; the sums are
+// scaled back, exactly, as they are stored.  Weights are split as they are; handles with magnitudes outside of [2^-100, 2^64)
+// stay on the CUDA cores, so all parts are exact, and what a product of parts loses to underflow is below 2^-172.  What is too
+// large is found in the result: an infinity or NaN in x, or |x| from 2^103 on, makes the parts infinite or NaN and with them the
+// voxel's whole row (NaN times a pruned weight's zero is NaN too), and so do sums from 2^103 on.  Rows with such results are
+// computed again with fp32 FMAs from the packed arrays, skipping what is pruned, by the threads that drain them.
 #include <algorithm>
 
 #include "f32_split_plan.h"
@@ -119,12 +121,31 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
   return d;
 }
-// The three parts of two neighbouring channels.
+constexpr float kUp = 16777216.f, kDown = 1.f / 16777216.f;             // 2^24: see the head of the file
+struct Float2 { unsigned long long bits; };              // two floats for the instructions that work on both
+__device__ __forceinline__ Float2 float2_of(float a, float b) {
+  Float2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d.bits) : "f"(a), "f"(b));
+  return d;
+}
+// Two values rounded to bf16, and what is left of them (exact).
+__device__ __forceinline__ uint32_t take_bf16x2(Float2& x) {
+  float x0, x1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x.bits));
+  const uint32_t h = pack_bf16x2(x0, x1);
+  const Float2 taken = float2_of(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), minus = float2_of(-1.f, -1.f);
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x.bits) : "l"(taken.bits), "l"(minus.bits), "l"(x.bits));
+  return h;
+}
+// The three parts of two neighbouring channels.  Instructions on pairs: the splitting warps' arithmetic is what up to 48 columns
+// wait for (64 -> 32 channels 3x3x3 on 2 x 16 x 56 x 56 111.7 us, one value at a time 114.2).
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
-  h = pack_bf16x2(x0, x1);
-  const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);          // exact
-  m = pack_bf16x2(r0, r1);
-  l = pack_bf16x2(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+  Float2 x = float2_of(x0, x1);
+  const Float2 up = float2_of(kUp, kUp);
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(x.bits) : "l"(x.bits), "l"(up.bits));
+  h = take_bf16x2(x);
+  m = take_bf16x2(x);
+  l = take_bf16x2(x);
 }
 
 // One output channel of one voxel in fp32, in the order of the packed arrays.
@@ -476,9 +497,7 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
       int at[4];                                           // the voxels whose channels this lane stores
 #pragma unroll
       for (int it = 0; it < 4; ++it) at[it] = __shfl_sync(0xffffffffu, vox, it * 8 + (lane >> 2));
-      uint32_t low[4], high[4];                            // smallest (zero aside) and largest magnitude, in four chains
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { low[q] = 0xffffffffu; high[q] = 0u; }
+      uint32_t high[4] = {0u, 0u, 0u, 0u};                 // largest magnitude, in four chains
 #pragma unroll
       for (int k = 0; k < NH / 16; ++k) {
         if (16 * k >= n_here) break;
@@ -489,11 +508,7 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
         for (uint32_t q = 0; q < 4; ++q) {
           const float* v = sum + 16 * k + 4 * q;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const uint32_t u = __float_as_uint(v[e]) & 0x7fffffffu;
-            high[e] = max(high[e], u);
-            low[e] = min(low[e], u - 1u);                  // zero: the largest
-          }
+          for (int e = 0; e < 4; ++e) high[e] = max(high[e], __float_as_uint(v[e]) & 0x7fffffffu);
           asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
                        ::"r"(mine + uint32_t(lane) * 64u + ((q ^ ((uint32_t(lane) >> 1) & 3u)) << 4)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
         }
@@ -506,7 +521,8 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
           const uint32_t r8 = uint32_t(it) * 8u + (uint32_t(lane) >> 2);
           asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o[it][0]), "=f"(o[it][1]), "=f"(o[it][2]), "=f"(o[it][3])
                        : "r"(mine + r8 * 64u + (((uint32_t(lane) & 3u) ^ ((r8 >> 1) & 3u)) << 4)));
-          o[it][0] += b.x; o[it][1] += b.y; o[it][2] += b.z; o[it][3] += b.w;
+          o[it][0] = fmaf(o[it][0], kDown, b.x); o[it][1] = fmaf(o[it][1], kDown, b.y);
+          o[it][2] = fmaf(o[it][2], kDown, b.z); o[it][3] = fmaf(o[it][3], kDown, b.w);
         }
         if (a.residual != nullptr) {
 #pragma unroll
@@ -538,9 +554,8 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
         }
       }
       __syncwarp();
-      // infinite, NaN or close to it, or below 2^-80: see the head of the file
-      const bool odd = max(max(high[0], high[1]), max(high[2], high[3])) >= 0x7f000000u ||
-                       min(min(low[0], low[1]), min(low[2], low[3])) < 0x17800000u - 1u;
+      // infinite, NaN or close to it: see the head of the file
+      const bool odd = max(max(high[0], high[1]), max(high[2], high[3])) >= 0x7f000000u;
       if (odd && in_range) exact_row(a, bias_s, m0, m0 + n_here, nn, to, ho, wo);
       __syncwarp();
     }

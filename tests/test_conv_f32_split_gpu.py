@@ -118,3 +118,22 @@ def test_inputs_that_arrive_late(everywhere, cin, cout, k, x):
     for i in range(5):
         flush.fill_(i)
         assert torch.equal(lay(xd), first) and rt3d.rt3d_last_device_status() == rt3d.OK
+
+
+@pytest.mark.parametrize("cin,cout", [(40, 24), (40, 120)])
+@pytest.mark.parametrize("x_exp,w_exp", [(-115, 0), (-120, 0), (-130, 0), (-140, 0), (-147, 0), (-120, 40), (-128, 60), (-140, 60),
+                                         (-149, 63), (-60, -75), (60, 0), (90, 4), (120, 0), (-130, 100), (-136, 119)])
+def test_magnitudes_at_both_ends_of_the_range(everywhere, cin, cout, x_exp, w_exp):
+    """Inputs down to the smallest denormal and weights up to the largest: against sums in 64 bits, with the error of ordinary
+    magnitudes and that of a few roundings of a denormal result.  Handles whose weights do not fit run on the CUDA cores."""
+    spec = synth.ConvSpec("f32", cin, cout, (1, 3, 3), (1, 1, 1), (0, 1, 1), False)
+    L = synth.make_layer(spec, 9, cin + cout, 4, 4, "bernoulli", 0.4)
+    w = np.ldexp(L["w"] / np.float32(np.abs(L["w"]).max()), w_exp).astype(np.float32)
+    x = np.ldexp(synth.make_input(9, (1, 2, 8, 8, cin)), x_exp + 1).astype(np.float32)
+    lay = nets.ConvLayer(spec, w, np.zeros_like(L["bias"]), L["mask"], 4, 4, torch.float32)
+    got = lay(nets.to_device(x, torch.float32)).cpu().numpy()[..., :cout].astype(np.float64)
+    assert rt3d.rt3d_last_plan()["kernel"] == (8 if w_exp < 64 else 0) and rt3d.rt3d_last_device_status() == rt3d.OK
+    xp = np.pad(x.astype(np.float64), ((0, 0), (0, 0), (1, 1), (1, 1), (0, 0)))
+    wm = (w * L["mask"]).astype(np.float64)
+    ref = sum(xp[:, :, a:a + 8, b:b + 8] @ wm[:, :, 0, a, b].T for a in range(3) for b in range(3))
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max() + 40 * 9 * 2.0 ** -150
