@@ -1002,8 +1002,16 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
 
 constexpr int kSplitFewest = 16;                           // input channels up to which no fp32 call goes to the tensor cores
 
-// A row computed again stays far below the limit of the others' waits.
-bool split_channels_fit(const rt3d_packed* w) { return int64_t(w->Ks) * w->N <= 32768; }
+// What a drain warp does again for a tile whose rows are all infinite or NaN, while the other roles wait for it: for every four
+// output channels (fewer where a kernel group ends), every entry that their groups may have, four input channels at a time.
+// Handles with more than kSplitAgain stay on the CUDA cores.  606 -> 128 channels 3x3x3 at 1 x 1 groups, 0.9 kept, just below it:
+// 361 ms for a tile of NaNs, a sixth of what the waits allow (4 x 4 groups never come near: 59 ms at 1212 channels).
+constexpr int64_t kSplitAgain = 1 << 20;
+int64_t split_again(const rt3d_packed* w) {
+  const int64_t passes = w->g_m % 4 == 0 ? 16 : w->g_m == 1 ? 64 : 32;       // over a warp's columns, at most 64
+  return passes * w->Q * w->Ks * ceil_div(w->g_n, 4);
+}
+bool split_rows_bounded(const rt3d_packed* w) { return split_again(w) <= kSplitAgain && int64_t(w->Ks) * w->N <= 32768; }
 
 // Bundle width there: as few bundles of up to 128 channels as there can be.
 int split_n_tile(int M) { return round_up(ceil_div(M, ceil_div(M, 128)), 16); }
@@ -1043,7 +1051,7 @@ rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt
   if (mode == 0 || d->cc_major != 10 || w->dtype != RT3D_F32 || x->c_stride % 4 || y->c_stride % 4 || (res_data && res_pitch % 4)) return RT3D_OK;
   if (g.st > 8 || g.sh > 8 || g.sw > 8 || int64_t(x->w) * x->c_stride * 4 >= (int64_t(1) << 40)) return RT3D_OK;
   if (int64_t(g.n) * g.To * g.Ho * g.Wo > 0x7fffffff) return RT3D_OK;
-  if (!split_channels_fit(w)) return RT3D_OK;
+  if (!split_rows_bounded(w)) return RT3D_OK;
   F32SplitArgs a;
   a.g = g;
   a.box = choose_box(g);
@@ -1068,6 +1076,7 @@ rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt
   a.x = nullptr; a.y = nullptr; a.bias = nullptr; a.residual = nullptr; a.rcs = res_pitch;
   a.group_ptr = blob->group_ptr; a.pos_idx = blob->pos_idx; a.tiles = static_cast<const float*>(blob->tiles);
   a.g_m = w->g_m; a.g_n = w->g_n; a.Q = w->Q;
+  a.again = int(split_again(w));
   a.sched = d->sched;
   const cuuint64_t cs = cuuint64_t(x->c_stride) * 4;
   cuuint64_t dims[5] = {cuuint64_t(x->c), cuuint64_t(x->w), cuuint64_t(x->h), cuuint64_t(x->t), cuuint64_t(x->n)};
@@ -1602,7 +1611,7 @@ static rt3d_status prepare_body(rt3d_packed* p) {
   }
   F32SplitArgs split;
   split.n_tile = split_n_tile(p->M); split.n_bundles = ceil_div(p->M, split.n_tile);
-  if (d->cc_major == 10 && p->dtype == RT3D_F32 && p->N > kSplitFewest && split_channels_fit(p) && g_f32_split.load() && umma_f32_plan(&split)) {
+  if (d->cc_major == 10 && p->dtype == RT3D_F32 && p->N > kSplitFewest && split_rows_bounded(p) && g_f32_split.load() && umma_f32_plan(&split)) {
     DeviceBlob::Umma* u = nullptr;
     const UmmaLayout* L = get_split_layout(p, split.n_tile);
     if (L && (s = get_split_blob(p, blob, L, split.pair != 0, &u)) != RT3D_OK) return s;

@@ -84,6 +84,7 @@ struct F32SplitArgs {
   const uint16_t* pos_idx;
   const float* tiles;
   int g_m, g_n, Q;
+  int again;                          // products of an entry and a quad of channels that a drain warp may have to do again for a tile
   int32_t* sched;                     // [2] = error word
 };
 bool umma_f32_plan(F32SplitArgs* a);

@@ -40,6 +40,7 @@ namespace {
 constexpr int kThreadsSplit = 640;
 constexpr int kDrainThreads = 256;
 constexpr uint32_t kSlotCols = kSplitSlotCols;
+constexpr long long kAgainClocks = 2048;                // allowed to a drain warp for each of the products in F32SplitArgs::again
 constexpr int kSplitSegment = 64;                       // steps after which a shared accumulator of small products is drained
 constexpr uint32_t kDrainStage = kSplitDrainStage;
 
@@ -148,29 +149,100 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t
   l = take_bf16x2(x);
 }
 
-// One output channel of one voxel in fp32, in the order of the packed arrays.
-__device__ float exact_output(const F32SplitArgs& a, int m, int nn, int ti0, int hi0, int wi0) {
+// J consecutive values: one; four at a multiple of 16 bytes; or (kRagged) four of which `left`, at least one, exist, and zeros.
+constexpr int kOne = 1, kFour = 4, kRagged = 0;
+template <int J>
+__device__ __forceinline__ float4 load_some(const float* p, int left) {
+  if (J == kFour) return __ldg(reinterpret_cast<const float4*>(p));
+  if (J == kOne) return make_float4(__ldg(p), 0.f, 0.f, 0.f);
+  const float v[4] = {__ldg(p), __ldg(p + min(1, left - 1)), __ldg(p + min(2, left - 1)), __ldg(p + min(3, left - 1))};
+  return make_float4(v[0], left > 1 ? v[1] : 0.f, left > 2 ? v[2] : 0.f, left > 3 ? v[3] : 0.f);
+}
+// Adds two packed entries' products over J input channels to the sums of C output channels (of which n exist).  x: where an entry
+// meets the input, nullptr: nowhere.  No branches, so that the loads are on their way together: entries that meet nothing add
+// zeros, channels that do not exist repeat the last one.
+template <int C, int J>
+__device__ __forceinline__ void add_entries(float (&s)[4], const float* const (&x)[2], const float* somewhere, const float* const (&w)[2], int g_n, int n, int left) {
+  float4 v[2], t[2][C];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    v[u] = load_some<J>(x[u] != nullptr ? x[u] : somewhere, left);
+#pragma unroll
+    for (int c = 0; c < C; ++c) t[u][c] = load_some<J>(w[u] + min(c, n - 1) * g_n, left);
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const bool there = x[u] != nullptr;
+    const float4 f = make_float4(there ? v[u].x : 0.f, there ? v[u].y : 0.f, there ? v[u].z : 0.f, there ? v[u].w : 0.f);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      s[c] = fmaf(t[u][c].x, f.x, s[c]);
+      if (J != kOne) s[c] = fmaf(t[u][c].w, f.w, fmaf(t[u][c].z, f.z, fmaf(t[u][c].y, f.y, s[c])));
+    }
+  }
+}
+// n <= C output channels of one voxel from channel m on, all in one kernel group, in fp32 from the packed arrays.
+template <int C>
+__device__ __forceinline__ void exact_outputs(float (&s)[4], const F32SplitArgs& a, int m, int n, int nn, int ti0, int hi0, int wi0) {
   const ConvGeom& g = a.g;
   const int p = m / a.g_m, i = m - p * a.g_m;
-  float s = 0.f;
-  for (int q = 0; q < a.Q; ++q)
-    for (int e = __ldg(a.group_ptr + p * a.Q + q); e < __ldg(a.group_ptr + p * a.Q + q + 1); ++e) {
-      const int k = __ldg(a.pos_idx + e), kw = k % g.Kw, kh = (k / g.Kw) % g.Kh, kt = k / (g.Kw * g.Kh);
-      const int ti = ti0 + kt, hi = hi0 + kh, wi = wi0 + kw;
-      if (unsigned(ti) >= unsigned(g.t) || unsigned(hi) >= unsigned(g.h) || unsigned(wi) >= unsigned(g.w)) continue;
-      const float* xp = a.x + ((((long long)nn * g.t + ti) * g.h + hi) * g.w + wi) * g.xcs + q * a.g_n;
-      const float* wp = a.tiles + ((long long)e * a.g_m + i) * a.g_n;
-      for (int j = 0; j < a.g_n && q * a.g_n + j < g.c; ++j) s = fmaf(__ldg(wp + j), xp[j], s);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) s[c] = 0.f;
+  int e = __ldg(a.group_ptr + p * a.Q);
+  for (int q = 0; q < a.Q; ++q) {
+    const int e1 = __ldg(a.group_ptr + p * a.Q + q + 1), real = min(a.g_n, g.c - q * a.g_n);         // padding channels hold anything
+    for (; e < e1; e += 2) {
+      const float *x[2], *w[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int at = min(e + u, e1 - 1), k = __ldg(a.pos_idx + at), row = k / g.Kw, kt = row / g.Kh;
+        const int ti = ti0 + kt, hi = hi0 + row - kt * g.Kh, wi = wi0 + k - row * g.Kw;
+        const bool there = e + u < e1 && unsigned(ti) < unsigned(g.t) && unsigned(hi) < unsigned(g.h) && unsigned(wi) < unsigned(g.w);
+        x[u] = there ? a.x + ((((long long)nn * g.t + ti) * g.h + hi) * g.w + wi) * g.xcs + q * a.g_n : nullptr;
+        w[u] = a.tiles + ((long long)at * a.g_m + i) * a.g_n;
+      }
+      for (int j = 0; j < real; j += 4) {
+        if (real - j == 1) add_entries<C, kOne>(s, x, a.x, w, a.g_n, n, 1);
+        else if (a.g_n % 4 == 0 && real - j >= 4) add_entries<C, kFour>(s, x, a.x, w, a.g_n, n, 4);
+        else add_entries<C, kRagged>(s, x, a.x, w, a.g_n, n, real - j);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (x[u] != nullptr) x[u] += 4;
+          w[u] += 4;
+        }
+      }
     }
-  return s;
+    e = e1;
+  }
 }
-__device__ __noinline__ void exact_row(const F32SplitArgs& a, const float* bias_s, int m0, int m1, int nn, int to, int ho, int wo) {
+// The output channels [m0, m0 + n) of the voxels (one a lane) that `odd` names, shared out over the warp in fours: a single odd
+// voxel takes as long as one of its channel quads, a warp of them as long as all of its quads after one another.  Bound by the
+// latency of the loads: 700 to 1000 clocks for each entry and quad.  64 -> 128 channels 3x3x3 on 2 x 16 x 56 x 56, 0.4 kept: 0.57 ms
+// with one NaN in the input, 10.5 ms with nothing else (a voxel's channels one after the other on one lane: 8.5 and 70 ms; the CUDA
+// cores take 0.57 for any input).  Four entries at a time were no faster, and their registers cost finite inputs 1 %.  The other roles wait meanwhile: their limit grows by F32SplitArgs::again.
+__device__ __noinline__ void exact_rows(const F32SplitArgs& a, const float* bias_s, int m0, int n, uint32_t odd, int lane, int vox) {
   const ConvGeom& g = a.g;
-  const long long vox = (((long long)nn * g.To + to) * g.Ho + ho) * g.Wo + wo;
-  for (int m = m0; m < m1; ++m) {
-    float s = exact_output(a, m, nn, to * g.st - g.pt, ho * g.sh - g.ph, wo * g.sw - g.pw) + bias_s[m];
-    if (a.residual) s += a.residual[vox * a.rcs + m];
-    a.y[vox * g.ycs + m] = g.relu ? fmaxf(s, 0.f) : s;
+  const int n_odd = __popc(odd), items = n_odd * ((n + 3) / 4);
+  for (int first = 0; first < items; first += 32) {
+    const int item = min(first + lane, items - 1), quad = item / n_odd, from = __fns(odd, 0, item - quad * n_odd + 1);
+    const int at = __shfl_sync(0xffffffffu, vox, from), line = at / g.Wo, frame = line / g.Ho, nn = frame / g.To;
+    const int wi = (at - line * g.Wo) * g.sw - g.pw, hi = (line - frame * g.Ho) * g.sh - g.ph, ti = (frame - nn * g.To) * g.st - g.pt;
+    const int m1 = m0 + min(n, 4 * quad + 4);
+    for (int m = m0 + 4 * quad; m < m1 && first + lane < items;) {
+      const int here = min(m1, (m / a.g_m + 1) * a.g_m) - m;             // that lie in one group
+      float r[4];
+      if (here == 1) exact_outputs<1>(r, a, m, here, nn, ti, hi, wi);
+      else exact_outputs<4>(r, a, m, here, nn, ti, hi, wi);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (c >= here) break;
+        float s = r[c] + bias_s[m + c];
+        if (a.residual) s += a.residual[(long long)at * a.rcs + m + c];
+        a.y[(long long)at * g.ycs + m + c] = g.relu ? fmaxf(s, 0.f) : s;
+      }
+      m += here;
+    }
+    __syncwarp();
   }
 }
 
@@ -221,7 +293,7 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
     }
     mbar_init(smem_u32(&sb->small_empty), 8 * kCtas);
     bars->abort_flag = 0;
-    bars->wait_limit = kWaitCycles;
+    bars->wait_limit = kWaitCycles + a.again * kAgainClocks;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -555,9 +627,8 @@ conv3d_umma_f32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_co
       }
       __syncwarp();
       // infinite, NaN or close to it: see the head of the file
-      const bool odd = max(max(high[0], high[1]), max(high[2], high[3])) >= 0x7f000000u;
-      if (odd && in_range) exact_row(a, bias_s, m0, m0 + n_here, nn, to, ho, wo);
-      __syncwarp();
+      const uint32_t odd = __ballot_sync(0xffffffffu, in_range && max(max(high[0], high[1]), max(high[2], high[3])) >= 0x7f000000u);
+      if (odd) exact_rows(a, bias_s, m0, n_here, odd, lane, vox);
     }
   }
 

@@ -137,3 +137,45 @@ def test_magnitudes_at_both_ends_of_the_range(everywhere, cin, cout, x_exp, w_ex
     wm = (w * L["mask"]).astype(np.float64)
     ref = sum(xp[:, :, a:a + 8, b:b + 8] @ wm[:, :, 0, a, b].T for a in range(3) for b in range(3))
     assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max() + 40 * 9 * 2.0 ** -150
+
+
+@pytest.mark.parametrize("cin,cout,group,share", [
+    (64, 128, (4, 4), 1.0), (40, 90, (8, 8), 1.0), (37, 51, (3, 5), 1.0), (33, 64, (1, 1), 0.5), (70, 24, (8, 3), 0.5), (30, 100, (8, 6), 1.0),
+    (606, 128, (1, 1), 1.0)])                              # the last: as much as a warp may have to do again for a tile
+def test_tiles_of_rows_that_are_computed_again(everywhere, cin, cout, group, share):
+    """An input of infinities and NaNs: every row is computed again, by whichever lanes, as the CUDA cores do it, with a residual
+    and ragged channels, and the roles that wait for it do not give up."""
+    spec = synth.ConvSpec("f32", cin, cout, (3, 3, 3) if cin > 600 else (1, 3, 3), (1, 1, 1), (1, 1, 1) if cin > 600 else (0, 1, 1), False)
+    L = synth.make_layer(spec, 9, cin + cout, group[0], group[1], "bernoulli", 0.9 if cin > 600 else 0.3)
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], group[0], group[1], torch.float32)
+    xd = nets.to_device(synth.make_input(9, (2, 2, 10, 10, cin)), torch.float32)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    hit = torch.rand(xd.shape, device="cuda", generator=gen) < 0.002 * share
+    xd[hit] = float("inf")
+    xd[:, :, 5:] = torch.where(torch.rand(xd[:, :, 5:].shape, device="cuda", generator=gen) < share, xd[:, :, 5:] * 1e37, xd[:, :, 5:])
+    xd[0, 1, 2, 3, 4] = float("nan")
+    xd[..., cin:] = float("nan")
+    res = torch.rand(lay.out_shape(xd), device="cuda", generator=gen)
+    got, want = torch.full(lay.out_shape(xd), 3.0, device="cuda"), torch.full(lay.out_shape(xd), 3.0, device="cuda")
+    lay.fused(xd, got, residual=res, relu=False)
+    assert rt3d.rt3d_last_plan()["kernel"] == 8 and rt3d.rt3d_last_device_status() == rt3d.OK
+    rt3d.rt3d_debug_set(rt3d.DEBUG_F32_SPLIT, 0)
+    lay.fused(xd, want, residual=res, relu=False)
+    assert rt3d.rt3d_last_plan()["kernel"] == 0
+    assert (got[..., cout:] == 3.0).all()
+    got, want = got[..., :cout].double(), want[..., :cout].double()
+    assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isposinf(), want.isposinf()) and torch.equal(got.isneginf(), want.isneginf())
+    rows = want.isfinite().all(dim=-1)
+    assert (rows.any() or cin > 600) and (~want.isfinite()).any()
+    if rows.any():
+        err, size = (got[rows] - want[rows]).abs().amax(dim=-1), want[rows].abs().amax(dim=-1)
+        assert (err <= 1e-5 * size).all()
+
+
+def test_layers_with_more_to_compute_again_stay_on_the_cuda_cores(everywhere):
+    spec = synth.ConvSpec("f32", 608, 16, (3, 3, 3), (1, 1, 1), (1, 1, 1), False)
+    x = torch.zeros((1, 1, 4, 4, 608), device="cuda")
+    for group, kernel in (((1, 1), 0), ((2, 1), 8), ((4, 4), 8)):
+        L = synth.make_layer(spec, 9, 1, group[0], group[1], "bernoulli", 0.05)
+        nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], group[0], group[1], torch.float32)(x)
+        assert rt3d.rt3d_last_plan()["kernel"] == kernel
