@@ -3,6 +3,7 @@
 // Pure host code: no CUDA calls, usable without a GPU.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <exception>
 #include <memory>
@@ -198,14 +199,38 @@ static bool splits_exactly(const float* w, int64_t n) {
   return hi < 0x5f800000u && (lo == 0xffffffffu || lo >= 0x0d800000u - 1u);       // 2^64, 2^-100
 }
 
+// Whether an output channel's weights lean to one side: their sum is more than half of the sum of their magnitudes, and more than
+// weights of both signs would show by chance.  The tensor core cuts addends off, always towards zero, which averages out in sums of
+// both signs and adds up in sums of one.  Errors against 64 bits over the CUDA cores', inputs of one sign: at most 0.81 on 300 random
+// layers with weights N(0, s^2), at most 1.1 on nine layers with N(s / 4, s^2), and up to 4.4 with weights of one sign.
+static bool leans_to_one_side(const rt3d_packed* p) {
+  const float* tiles = reinterpret_cast<const float*>(p->tiles.data());
+  const int g_m = p->g_m, g_n = p->g_n;
+  for (int pr = 0; pr < p->P; ++pr) {
+    const int64_t first = p->group_ptr[size_t(pr) * p->Q], end = p->group_ptr[size_t(pr + 1) * p->Q];
+    const double chance = 25.0 / double(std::max<int64_t>(1, (end - first) * g_n));        // (5 standard deviations)^2
+    for (int i = 0; i < g_m; ++i) {
+      double sum = 0.0, size = 0.0;
+      for (int64_t e = first; e < end; ++e) {
+        const float* w = tiles + (e * g_m + i) * g_n;
+        float s = 0.f, a = 0.f;
+        for (int j = 0; j < g_n; ++j) { s += w[j]; a += std::fabs(w[j]); }
+        sum += s; size += a;
+      }
+      if (std::fabs(sum) > 0.5 * size && sum * sum > chance * size * size) return true;
+    }
+  }
+  return false;
+}
+
 const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile) {
   if (p->dtype != RT3D_F32 || p->Kt > 63 || p->Kh > 63 || p->Kw > 63 || ceil_div(p->N, kSplitChunk) > 4095) return nullptr;
   if (n_tile % 16 || n_tile < 16 || n_tile > 128) return nullptr;
   {
     std::lock_guard<std::mutex> lock(p->mu);
-    if (p->splits_exactly < 0)
-      p->splits_exactly = splits_exactly(reinterpret_cast<const float*>(p->tiles.data()), p->nnz * p->g_m * p->g_n) ? 1 : 0;
-    if (!p->splits_exactly) return nullptr;
+    if (p->splits_well < 0)
+      p->splits_well = splits_exactly(reinterpret_cast<const float*>(p->tiles.data()), p->nnz * p->g_m * p->g_n) && !leans_to_one_side(p) ? 1 : 0;
+    if (!p->splits_well) return nullptr;
   }
   return step_layout(p, n_tile, false, kSplitChunk);
 }

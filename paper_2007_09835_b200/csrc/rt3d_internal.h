@@ -195,7 +195,7 @@ struct rt3d_packed {
   rt3d::RawBytes tiles;              // nnz * g_m * g_n elements of float or bf16 bits
   std::mutex mu;                     // guards the lazily built members below
   std::map<int, rt3d::UmmaLayout> umma_layouts;   // keyed by umma_key
-  int splits_exactly = -1;           // fp32: whether three bf16 parts hold every weight (-1: not looked at yet)
+  int splits_well = -1;              // fp32: whether three bf16 parts hold every weight and sums lose nothing (-1: not looked at yet)
   std::map<int, rt3d::SubLayout> sub_layouts;     // keyed by n_tile
   std::map<int, rt3d::SmallCLayout> smallc_layouts;   // keyed by sh*16+sw (+ 1024: packed), built on first use
   std::unique_ptr<rt3d::F32Layout> f32_layout;        // built on first use
