@@ -448,6 +448,29 @@ bool umma_blob_ready(rt3d_packed* h, DeviceBlob* blob, int key) {
   return it != blob->umma.end() && it->second.ready;
 }
 
+// A step-list layout that is on the device, the widest with whole pieces of 32 columns where there is one; nullptr: none.
+const UmmaLayout* present_umma_layout(rt3d_packed* h, DeviceBlob* blob) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  const UmmaLayout* best = nullptr;
+  for (const auto& kv : blob->umma) {
+    const auto it = h->umma_layouts.find(kv.first);
+    if (!kv.second.ready || it == h->umma_layouts.end()) continue;
+    const auto rank = [](const UmmaLayout& L) { return (L.n_tile % 32 == 0 ? 512 : 0) + L.n_tile; };
+    if (!best || rank(it->second) > rank(*best)) best = &it->second;
+  }
+  return best;
+}
+
+// Whether a handle's layouts for the CUDA cores are on the device: the canonical arrays, the register-blocked kernel's.
+bool canonical_ready(rt3d_packed* h, DeviceBlob* blob) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  return blob->canonical != nullptr;
+}
+bool f32_blob_ready(rt3d_packed* h, DeviceBlob* blob) {
+  std::lock_guard<std::mutex> lock(h->mu);
+  return blob->f32.base != nullptr;
+}
+
 // Device copy of the fp32 tensor-core kernel's layout, with the canonical arrays beside it.
 rt3d_status get_split_blob(rt3d_packed* h, DeviceBlob* blob, const UmmaLayout* L, bool pair, DeviceBlob::Umma** out) {
   std::lock_guard<std::mutex> lock(h->mu);
@@ -1043,9 +1066,10 @@ bool split_is_faster(const rt3d_packed* w, const F32SplitArgs& a, int sm_count) 
 }
 
 // fp32 on the tensor cores, each value as three bf16 ones.
-// *launched = false (and RT3D_OK) when the handle or the shape does not suit it or the CUDA cores are faster.
+// *launched = false (and RT3D_OK) when the handle or the shape does not suit it, the CUDA cores are faster (unless `anyway`: what
+// they need is not there), or the call is being captured and the layout is not on the device.
 rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d_tensor* x, const ConvGeom& g, const float* bias,
-                      rt3d_tensor* y, const void* res_data, int res_pitch, Submit& submit, bool* launched) {
+                      rt3d_tensor* y, const void* res_data, int res_pitch, bool anyway, Submit& submit, bool* launched) {
   *launched = false;
   const int mode = g_f32_split.load();
   if (mode == 0 || d->cc_major != 10 || w->dtype != RT3D_F32 || x->c_stride % 4 || y->c_stride % 4 || (res_data && res_pitch % 4)) return RT3D_OK;
@@ -1064,11 +1088,14 @@ rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt
   // leave 0.93 on wide bundles and 1.01 up to 64 columns.  With more than 48 steps the CUDA cores' sums are long too.
   a.period = a.n_tile > 64 && w->Ks * ceil_div(w->N, kSplitChunk) > 48 ? 8 : 4;
   if (!umma_f32_plan(&a) || (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w * a.n_bundles > (1ll << 30)) return RT3D_OK;
-  if (mode == 1 && !split_is_faster(w, a, d->sm_count)) return RT3D_OK;
+  if (mode == 1 && !split_is_faster(w, a, d->sm_count)) {
+    if (!anyway) return RT3D_OK;
+    submit.keep = false;
+  }
   const UmmaLayout* L = get_split_layout(w, a.n_tile);
   if (!L) return RT3D_OK;
   if (submit.captured() && !umma_blob_ready(w, blob, umma_key(L->n_tile, false, false))) {
-    submit.keep = false;                                   // the CUDA cores' layout may be there
+    submit.keep = false;                                   // one of the CUDA cores' layouts may be there
     return RT3D_OK;
   }
   DeviceBlob::Umma* u = nullptr;
@@ -1136,9 +1163,12 @@ rt3d_status try_f32(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3d
   return RT3D_OK;
 }
 
-// `narrow`: whether the step-list kernels may take steps of 32 channels.
+// Which layouts the step-list kernels may choose from: all; those of steps of 64 channels; one that is on the device.  The others are
+// for calls that are being captured, which cannot upload the layout that they would choose, on handles of up to 32 channels: theirs
+// come in steps of 32 or 64, so that earlier calls and rt3d_packed_prepare may have left a layout of either kind.
+enum class StepLists { kAll, kWide, kPresent };
 rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* bias, const rt3d_conv_params* p,
-                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz, bool narrow = true) {
+                      rt3d_tensor* y, void* stream, bool dense_entry, const rt3d_fusion* fz, StepLists lists = StepLists::kAll) {
   CallKey key;
   CallBuffers buffers{};
   if (make_key(&key, x, wc, bias, p, y, fz ? fz->residual : nullptr, dense_entry ? 1 : 0)) {
@@ -1181,8 +1211,8 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   DeviceBlob* blob = nullptr;
   if ((s = get_blob(w, &blob)) != RT3D_OK) return s;
   Submit submit(w, key, buffers, static_cast<cudaStream_t>(stream));
-  submit.keep = narrow;
-  narrow = narrow && narrow_steps(w);
+  submit.keep = lists == StepLists::kAll;
+  const bool narrow = lists == StepLists::kAll && narrow_steps(w);
 
   const bool can_umma = umma_eligible(d, w, x, y, p);
   const bool can_simt = w->g_m <= kMaxGroupSimt && w->g_n <= kMaxGroupSimt;
@@ -1194,12 +1224,16 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   const bool use_umma = want_umma || (p->algo == RT3D_ALGO_AUTO && can_umma);
   if (!use_umma) {
     if (pooled) return RT3D_ERR_UNSUPPORTED;
+    // a call that is being captured takes what is there: after a call on the tensor cores that is their layout and the canonical
+    // arrays, after one on the CUDA cores the register-blocked kernel's layout or the canonical arrays
+    const bool without = submit.captured() && f32_layout_possible(w) && !f32_blob_ready(w, blob);
     bool launched = false;
     if (p->algo == RT3D_ALGO_AUTO) {
-      s = try_split(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
+      s = try_split(w, blob, d, x, g, bias, y, res_data, res_pitch, without, submit, &launched);
       if (s != RT3D_OK || launched) return s;
     }
-    s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
+    if (without && canonical_ready(w, blob)) submit.keep = false;
+    else s = try_f32(w, blob, d, x, g, bias, y, res_data, res_pitch, submit, &launched);
     if (s != RT3D_OK || launched) return s;
     if ((s = get_canonical(w, blob)) != RT3D_OK) return s;
     return submit(rt3d_plan_info{0, 0, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
@@ -1244,7 +1278,8 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   a.tiles_n = ceil_div(g.n, a.box.bn); a.tiles_t = ceil_div(g.To, a.box.bt);
   a.tiles_h = ceil_div(g.Ho, a.box.bh); a.tiles_w = ceil_div(g.Wo, a.box.bw);
   long long m_tiles = (long long)a.tiles_n * a.tiles_t * a.tiles_h * a.tiles_w;
-  UmmaPlan plan = pick_plan(w, g, m_tiles, d->sm_count, narrow);
+  const UmmaLayout* present = lists == StepLists::kPresent ? present_umma_layout(w, blob) : nullptr;
+  UmmaPlan plan = present ? UmmaPlan{present->n_tile, 1, false} : pick_plan(w, g, m_tiles, d->sm_count, narrow);
   if (pooled) {                     // pooling lives in the TMA-store epilogue, which a K split does not use
     // A layer this small is faster split over K and pooled by a second launch: AUTO declines the fusion.
     if (p->algo == RT3D_ALGO_AUTO && plan.n_splits > 1) return RT3D_ERR_UNSUPPORTED;
@@ -1253,10 +1288,10 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   // CTA pairs: two tiles per MMA.  Taken when every SM has a tile or the plan finds them faster; forced by RT3D_ALGO_UMMA_PAIR.
   bool use_pair = false;
   if (p->algo == RT3D_ALGO_UMMA_PAIR) {
-    plan = UmmaPlan{default_n_tile(w->M), 1, true};
+    plan = UmmaPlan{present ? present->n_tile : default_n_tile(w->M), 1, true};
     if (!umma_pair_supported(plan.n_tile, ceil_div(w->M, plan.n_tile))) return RT3D_ERR_UNSUPPORTED;
     use_pair = true;
-  } else if (p->algo == RT3D_ALGO_AUTO && plan.n_splits == 1 &&
+  } else if (p->algo == RT3D_ALGO_AUTO && plan.n_splits == 1 && !present &&
              umma_pair_supported(plan.n_tile, ceil_div(w->M, plan.n_tile)) &&
              (plan.pair || m_tiles * ceil_div(w->M, plan.n_tile) >= d->sm_count)) {
     use_pair = true;
@@ -1268,11 +1303,11 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   bool use_ts = false;
   // (few steps on single CTAs wait for their first tiles and for their output: in the S3D-shaped forward, whose branches have
   // 16 to 32 channels there, 772 us as a graph, 778 in steps of 32)
-  a.narrow = narrow && (use_pair || w->Ks > 12) ? 1 : 0;
+  a.narrow = present ? present->chunk != kChunk : narrow && (use_pair || w->Ks > 12);
   UmmaArgs probe = a;
   // (wide bundles: only kernels that are also wide in space; a 3x1x1 layer with 192-wide bundles lost 8 us of 43
   // inside the S3D-shaped forward with it, while 3x3x3 layers gain 1-4 %)
-  if (use_pair && g_ts_enabled.load() && g.st <= 2 && g.Kt >= 2 && g.Kt <= 8 && (plan.n_tile <= 128 || g.Kh * g.Kw >= 4)) {
+  if (use_pair && !present && g_ts_enabled.load() && g.st <= 2 && g.Kt >= 2 && g.Kt <= 8 && (plan.n_tile <= 128 || g.Kh * g.Kw >= 4)) {
     int sb2[4] = {1, 1, 1, 1};
     TileBox deep = a.box;
     const bool ok2 = pooled ? choose_box_pool(g, pl_w, pl_h, pl_t, &deep, sb2, true)
@@ -1305,15 +1340,16 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
       for (int i = 0; i < 4; ++i) sb[i] = sb2[i];
     }
   }
-  const UmmaLayout* L = get_umma_layout(w, plan.n_tile, use_ts, a.narrow != 0);
+  const UmmaLayout* L = present ? present : get_umma_layout(w, plan.n_tile, use_ts, a.narrow != 0);
   if (!L) return RT3D_ERR_UNSUPPORTED;
-  // rt3d_packed_prepare uploads the steps of 64, which rt3d_conv3d_sparse_noalloc reads too
-  if (narrow && submit.captured() && !umma_blob_ready(w, blob, umma_key(L->n_tile, use_ts, a.narrow != 0)))
-    return conv_body(x, wc, bias, p, y, stream, dense_entry, fz, false);
+  if (!present && narrow_steps(w) && submit.captured() && !umma_blob_ready(w, blob, umma_key(L->n_tile, use_ts, a.narrow != 0))) {
+    if (narrow) return conv_body(x, wc, bias, p, y, stream, dense_entry, fz, StepLists::kWide);
+    if (present_umma_layout(w, blob)) return conv_body(x, wc, bias, p, y, stream, dense_entry, fz, StepLists::kPresent);
+  }
   DeviceBlob::Umma* u = nullptr;
   if ((s = get_umma_blob(w, blob, L, &u)) != RT3D_OK) return s;
   a.n_tile = L->n_tile; a.n_bundles = L->n_bundles; a.n_chunks = L->n_chunks;
-  a.dense = dense_entry && !a.narrow ? 1 : 0;
+  a.dense = dense_entry && !a.narrow && L->t_groups == use_ts ? 1 : 0;       // computed steps come in the layout's own order
   a.steps_dense = w->Ks * L->n_chunks;
   a.step_ptr = u->step_ptr; a.steps = u->steps;
   a.bias = bias; a.y = y->data; a.sched = d->sched;
@@ -1341,7 +1377,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
     size_t tail_bytes = 0, flag_bytes = 0;
     // (nor for AUTO when there are fewer items than pairs: what it would gain there, the cluster split gains with less)
     const long long pairs = (m_tiles + 1) / 2 * L->n_bundles;
-    if (!p->concurrent && (p->algo != RT3D_ALGO_AUTO || pairs >= d->sm_count / 2))
+    if (!p->concurrent && !present && (p->algo != RT3D_ALGO_AUTO || pairs >= d->sm_count / 2))
       umma_pair_tail_plan(&a, L->step_ptr.data(), d->sm_count, &tail_bytes, &flag_bytes, use_ts ? L->grp_ptr.data() : nullptr);
     if (a.tail_workers > 0) {
       DeviceBlob::Tail t;
@@ -1425,6 +1461,12 @@ rt3d_status conv2plus1d_body(const rt3d_tensor* x, const rt3d_packed* wsc, const
   if (!umma_st_plan(&a, L1->steps.data(), L2->steps.data())) return RT3D_ERR_UNSUPPORTED;
   DeviceBlob *blob1 = nullptr, *blob2 = nullptr;
   if ((s = get_blob(ws, &blob1)) != RT3D_OK || (s = get_blob(wt, &blob2)) != RT3D_OK) return s;
+  // a pair that is being captured and whose layers have left their steps of 32 channels only: two calls take those
+  Submit submit(ws, key, buffers, static_cast<cudaStream_t>(stream));
+  const auto elsewhere = [](rt3d_packed* h, DeviceBlob* b, const UmmaLayout* L) {
+    return narrow_steps(h) && !umma_blob_ready(h, b, umma_key(L->n_tile, false, false)) && present_umma_layout(h, b);
+  };
+  if (submit.captured() && (elsewhere(ws, blob1, L1) || elsewhere(wt, blob2, L2))) return RT3D_ERR_UNSUPPORTED;
   DeviceBlob::Umma *u1 = nullptr, *u2 = nullptr;
   if ((s = get_umma_blob(ws, blob1, L1, &u1)) != RT3D_OK || (s = get_umma_blob(wt, blob2, L2, &u2)) != RT3D_OK) return s;
   a.M2 = wt->M; a.ycs = y->c_stride; a.relu2 = pt->relu ? 1 : 0;
@@ -1436,7 +1478,7 @@ rt3d_status conv2plus1d_body(const rt3d_tensor* x, const rt3d_packed* wsc, const
   if ((s = encode_xmap(x, unit, TileBox{1, 1, a.hh, a.hw}, &xmap)) != RT3D_OK) return s;
   const int sms = d->sm_count;
   const void *m1 = u1->wmap_half, *m2 = u2->wmap_half;
-  return Submit(ws, key, buffers, static_cast<cudaStream_t>(stream))(rt3d_plan_info{5, a.n1, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+  return submit(rt3d_plan_info{5, a.n1, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
     const PlacedMaps m(xmap, c.x, xmap, nullptr);
     if (!m.ok) return cudaErrorInvalidValue;
     StArgs now = a;
@@ -1890,14 +1932,15 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
   {
     std::lock_guard<std::mutex> lock(w->mu);
     blob = find_blob(w, dev);
-    if (blob) {
-      auto it = blob->umma.find(n_tile);
-      if (it != blob->umma.end() && it->second.ready) u = &it->second;
+    // steps of 64, which rt3d_packed_prepare uploads, or the steps of 32 of an earlier call
+    for (const int key : {umma_key(n_tile, false, false), umma_key(n_tile, false, true)}) {
+      if (!blob || u) break;
+      const auto it = blob->umma.find(key);
+      const auto li = w->umma_layouts.find(key);
+      if (it != blob->umma.end() && it->second.ready && li != w->umma_layouts.end()) { u = &it->second; L = &li->second; }
     }
-    auto li = w->umma_layouts.find(n_tile);
-    if (li != w->umma_layouts.end()) L = &li->second;
   }
-  if (!blob || !u || !L) return RT3D_ERR_NOT_PREPARED;
+  if (!u) return RT3D_ERR_NOT_PREPARED;
 
   UmmaArgs a;
   a.g = g;
@@ -1923,14 +1966,14 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
   if (a.n_splits > 1 && (tiles * a.n_splits * kTileM * L->n_tile * 4LL > RT3D_NOALLOC_PARTIAL_BYTES || tiles > RT3D_NOALLOC_PARTIAL_TILES))
     return RT3D_ERR_WORKSPACE;
   CUtensorMap xmap;
-  if ((s = encode_xmap(x, g, a.box, &xmap)) != RT3D_OK) return s;
+  if ((s = encode_xmap(x, g, a.box, &xmap, 0, L->chunk)) != RT3D_OK) return s;
   CUtensorMap ymap;
   int sb[4];
   a.pool_t = a.pool_h = a.pool_w = 1; a.sbw = a.sbh = 1;
   a.tail_workers = 0; a.tail_scratch = nullptr; a.tail_flags = nullptr;
   a.ts = 0; a.grp_ptr = nullptr; a.grp_first = nullptr; a.ts_a_bytes = 0; a.ts_frame_bytes = 0; a.ts_table = 0; a.ts_phases = 1;
   a.wait_cycles = 0; a.debug_drop_last_load = 0;
-  a.turned = a.narrow = 0;
+  a.turned = 0; a.narrow = L->chunk != kChunk;
   a.store_tma = (a.n_splits == 1 && warp_block(a.box.bw, a.box.bh, a.box.bt, a.box.bn, sb) &&
                  encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   if (launch_conv_umma(a, &xmap, u->wmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;

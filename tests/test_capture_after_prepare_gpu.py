@@ -59,3 +59,89 @@ def test_narrow_layer_after_prepare():
     assert captured == plan
     assert float((got - want).abs().max()) <= 2 ** -7 * float(want.abs().max())       # the same products in the same order
     assert torch.equal(lay(x), want)
+
+
+def _restrided(lay, stride):
+    """The same handle as a layer of another stride."""
+    other = object.__new__(nets.ConvLayer)
+    other.__dict__.update(lay.__dict__)
+    s = lay.spec
+    other.spec = synth.ConvSpec(s.name, s.cin, s.cout, s.k, stride, s.pad, s.relu)
+    return other
+
+
+@pytest.mark.parametrize("group,stride,kernel", [((4, 4), (1, 1, 1), 8), ((4, 4), (1, 1, 9), 0), ((3, 5), (1, 1, 9), 0)])
+def test_fp32_call_after_one_on_the_tensor_cores(group, stride, kernel):
+    """Only the tensor cores' layout and the canonical arrays are there; alone the captured call would run on the CUDA cores.  (A
+    stride of nine is more than the tensor-core kernel takes, groups of 3 x 5 need no layout of their own on the CUDA cores.)"""
+    spec = synth.ConvSpec("c", 64, 128, (3, 3, 3), (1, 1, 1), (1, 1, 1), True)
+    L = synth.make_layer(spec, 15, 192, group[0], group[1], "bernoulli", 0.4)
+    warm, lay = [nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], group[0], group[1], torch.float32) for _ in range(2)]
+    x = nets.to_device(synth.make_input(15, (2, 8, 28, 28, 64)), torch.float32)
+    small = nets.to_device(synth.make_input(15, (1, 1, 4, 4, 64)), torch.float32)
+    want = _restrided(warm, stride)(small)
+    assert rt3d.rt3d_last_plan()["kernel"] == 0
+    lay(x)
+    assert rt3d.rt3d_last_plan()["kernel"] == 8
+    got, plan = _captured(_restrided(lay, stride), small)
+    assert plan["kernel"] == kernel and float((got - want).abs().max()) <= 2e-6 * float(want.abs().max())
+    again = _restrided(lay, stride)(small)                 # with no capture it uploads what it would rather have
+    assert rt3d.rt3d_last_plan()["kernel"] == 0 and torch.equal(again, want)
+
+
+@pytest.mark.parametrize("cin,cout,k,large,small", [
+    (24, 64, (1, 3, 3), (8, 8, 28, 28), (1, 2, 9, 9)),                              # steps of 32 on CTA pairs, then single CTAs with few steps
+    (24, 64, (3, 3, 3), (8, 8, 28, 28), (1, 2, 9, 9)),                              # ... ordered for shared input tiles, then a K split
+    (30, 200, (3, 3, 3), (1, 2, 7, 7), (8, 8, 28, 28)),                             # the other way round
+    (30, 350, (1, 3, 3), (14, 4, 7, 7), (8, 8, 28, 28)), (30, 350, (1, 3, 3), (8, 8, 28, 28), (1, 1, 7, 7))])
+@pytest.mark.parametrize("dense", [False, True])
+def test_narrow_layer_after_a_call_of_another_shape(cin, cout, k, large, small, dense):
+    spec = synth.ConvSpec("c", cin, cout, k, (1, 1, 1), tuple(v // 2 for v in k), True)
+    L = synth.make_layer(spec, 15, cin + cout, 4, 4, "none" if dense else "bernoulli", None if dense else 0.4)
+    warm, lay = [nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.bfloat16, dense=dense) for _ in range(2)]
+    first = nets.to_device(synth.make_input(15, large + (cin,)), torch.bfloat16)
+    x = nets.to_device(synth.make_input(16, small + (cin,)), torch.bfloat16)
+    want = warm(x)
+    lay(first)
+    got, _ = _captured(lay, x)
+    assert float((got - want).abs().max()) <= 2 ** -7 * float(want.abs().max())
+    assert torch.equal(lay(x), want)                       # what served the capture is not kept
+
+
+def test_call_without_allocation_after_one_in_steps_of_32():
+    warm, lay = _layers(torch.bfloat16, 24, 64, (3, 3, 3), (1, 1, 1))
+    x = nets.to_device(synth.make_input(15, (2, 8, 28, 28, 24)), torch.bfloat16)
+    y, want = lay.alloc_out(x), warm(x)
+    rt3d.rt3d_debug_set(rt3d.DEBUG_T_GROUPS, 0)
+    try:
+        lay(x)
+    finally:
+        rt3d.rt3d_debug_set(rt3d.DEBUG_T_GROUPS, 1)
+    allocs = rt3d.rt3d_alloc_count()
+    rt3d.rt3d_conv3d_sparse_noalloc(rt3d.tensor_desc(x, 24), lay.packed, lay.bias, rt3d.tensor_desc(y, 64), (1, 1, 1), (1, 1, 1), True)
+    assert rt3d.rt3d_alloc_count() == allocs and rt3d.rt3d_last_device_status() == rt3d.OK
+    assert float((y - want).abs().max()) <= 2 ** -7 * float(want.abs().max())
+
+
+def test_fused_pair_whose_layers_ran_in_steps_of_32():
+    """The fused kernel wants steps of 64: it declines, as it does for other pairs, and the two calls are served."""
+    s_warm, s = _layers(torch.bfloat16, 24, 32, (1, 3, 3), (1, 1, 1))
+    t_warm, t = _layers(torch.bfloat16, 32, 48, (3, 1, 1), (1, 1, 1))
+    x = nets.to_device(synth.make_input(15, (8, 8, 18, 18, 24)), torch.bfloat16)
+    want = t_warm(s_warm(x))
+    mid = s(x)
+    y = t(mid)
+    y.zero_()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        try:
+            rt3d.rt3d_conv2plus1d_fused(rt3d.tensor_desc(x, 24), s.packed, s.bias, s.spec.pad, True, t.packed, t.bias, t.spec.pad, True,
+                                        rt3d.tensor_desc(y, 48))
+            declined = False
+        except rt3d.Rt3dError as e:
+            declined = e.status == rt3d.ERR_UNSUPPORTED
+            t(s(x, mid), y)
+    graph.replay()
+    assert declined and rt3d.rt3d_last_device_status() == rt3d.OK
+    assert float((y - want).abs().max()) <= 2 ** -7 * float(want.abs().max())
