@@ -185,42 +185,40 @@ const UmmaLayout* get_umma_layout(rt3d_packed* p, int n_tile, bool t_groups, boo
   return step_layout(p, n_tile, t_groups, narrow ? kNarrowChunk : kChunk);
 }
 
-// Whether every weight is zero or lies in [2^-100, 2^64): three bf16 parts hold it to the last bit then, and with the inputs' scale
-// of 2^24 inputs below 2^24 in magnitude keep every sum of the fp32 tensor-core kernel in range.
-static bool splits_exactly(const float* w, int64_t n) {
-  uint32_t lo = 0xffffffffu, hi = 0;                       // smallest magnitude but zero, largest one
-  for (int64_t i = 0; i < n; ++i) {
-    uint32_t u;
-    std::memcpy(&u, w + i, 4);
-    u &= 0x7fffffffu;
-    hi = std::max(hi, u);
-    lo = std::min(lo, u - 1u);                             // zero: the largest
-  }
-  return hi < 0x5f800000u && (lo == 0xffffffffu || lo >= 0x0d800000u - 1u);       // 2^64, 2^-100
-}
-
-// Whether an output channel's weights lean to one side: their sum is more than half of the sum of their magnitudes, and more than
-// weights of both signs would show by chance.  The tensor core cuts addends off, always towards zero, which averages out in sums of
-// both signs and adds up in sums of one.  Errors against 64 bits over the CUDA cores', inputs of one sign: at most 0.81 on 300 random
-// layers with weights N(0, s^2), at most 1.1 on nine layers with N(s / 4, s^2), and up to 4.4 with weights of one sign.
-static bool leans_to_one_side(const rt3d_packed* p) {
+// Whether the fp32 tensor-core kernel suits the weights:
+//  - Each is zero or lies in [2^-100, 2^64): three bf16 parts hold it to the last bit then, and with the inputs' scale of 2^24 inputs
+//    below 2^24 in magnitude keep every sum in range.
+//  - No output channel's weights lean to one side: their sum more than half of the sum of their magnitudes, and more than weights of
+//    both signs would show by chance.  The tensor core cuts addends off, always towards zero, which averages out in sums of both
+//    signs and adds up in sums of one.  Errors against 64 bits over the CUDA cores', inputs of one sign: at most 0.81 on 300 random
+//    layers with weights N(0, s^2), at most 1.1 on nine layers with N(s / 4, s^2), and up to 4.4 with weights of one sign.
+static bool splits_well(const rt3d_packed* p) {
   const float* tiles = reinterpret_cast<const float*>(p->tiles.data());
-  const int g_m = p->g_m, g_n = p->g_n;
+  const int g_m = p->g_m, g_n = p->g_n, size = g_m * g_n;
+  std::vector<float> sums(2 * size_t(size));
   for (int pr = 0; pr < p->P; ++pr) {
     const int64_t first = p->group_ptr[size_t(pr) * p->Q], end = p->group_ptr[size_t(pr + 1) * p->Q];
-    const double chance = 25.0 / double(std::max<int64_t>(1, (end - first) * g_n));        // (5 standard deviations)^2
-    for (int i = 0; i < g_m; ++i) {
-      double sum = 0.0, size = 0.0;
-      for (int64_t e = first; e < end; ++e) {
-        const float* w = tiles + (e * g_m + i) * g_n;
-        float s = 0.f, a = 0.f;
-        for (int j = 0; j < g_n; ++j) { s += w[j]; a += std::fabs(w[j]); }
-        sum += s; size += a;
+    float *const sum = sums.data(), *const mag = sum + size;       // of every place of a group, over the row's entries
+    std::fill(sums.begin(), sums.end(), 0.f);
+    int outside = 0;
+    for (int64_t e = first; e < end; ++e) {
+      const float* w = tiles + e * size;
+      for (int v = 0; v < size; ++v) {
+        const float m = std::fabs(w[v]);
+        sum[v] += w[v];
+        mag[v] += m;
+        outside |= (int(m < 0x1p-100f) & int(m > 0.f)) | int(!(m < 0x1p64f));          // (NaNs are)
       }
-      if (std::fabs(sum) > 0.5 * size && sum * sum > chance * size * size) return true;
+    }
+    if (outside) return false;
+    const double chance = 25.0 / double(std::max<int64_t>(1, (end - first) * g_n));            // (five standard deviations)^2
+    for (int i = 0; i < g_m; ++i) {
+      double s = 0.0, m = 0.0;
+      for (int k = 0; k < g_n; ++k) { s += sum[i * g_n + k]; m += mag[i * g_n + k]; }
+      if (std::fabs(s) > 0.5 * m && s * s > chance * m * m) return false;
     }
   }
-  return false;
+  return true;
 }
 
 const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile) {
@@ -229,7 +227,7 @@ const UmmaLayout* get_split_layout(rt3d_packed* p, int n_tile) {
   {
     std::lock_guard<std::mutex> lock(p->mu);
     if (p->splits_well < 0)
-      p->splits_well = splits_exactly(reinterpret_cast<const float*>(p->tiles.data()), p->nnz * p->g_m * p->g_n) && !leans_to_one_side(p) ? 1 : 0;
+      p->splits_well = splits_well(p) ? 1 : 0;
     if (!p->splits_well) return nullptr;
   }
   return step_layout(p, n_tile, false, kSplitChunk);

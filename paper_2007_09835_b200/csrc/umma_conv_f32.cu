@@ -19,7 +19,7 @@
 // 1.58 of the 1.64 PFLOP/s that cuBLAS reaches; the register-blocked FMAs of 0.4 of the places take 528), below that the hand-shakes
 // and the arithmetic of a step, 0.31 us each.  Errors against 64 bits, relative, CUDA cores and here: 3.3e-7 and 1.2e-7 for
 // that layer, 6.0e-8 and 4.3e-8 for 44 channels 1x1x1; at most 0.81 of the CUDA cores' in 300 random layers that the dispatch sends
-// here, with weights of both signs.  Layers whose weights lean to one side do not come here (pack.cpp: leans_to_one_side).
+// here, with weights of both signs.  Layers whose weights lean to one side do not come here (pack.cpp: splits_well).
 //
 // Range: x is split as 2^24 x, which leaves the parts of the smallest denormal (2^-149) normal bf16 numbers; the sums are
 // scaled back, exactly, as they are stored.  Weights are split as they are; handles with magnitudes outside of [2^-100, 2^64)
