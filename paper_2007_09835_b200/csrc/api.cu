@@ -40,6 +40,7 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
     weight_blocks().release_all();
     g_allocs.fetch_add(1);
     e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();      // the caller's answer, not that of the next launch
   }
   return e;
 }
@@ -1100,6 +1101,10 @@ rt3d_status try_split(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt
   }
   DeviceBlob::Umma* u = nullptr;
   rt3d_status s = get_split_blob(w, blob, L, a.pair != 0, &u);
+  if (s == RT3D_ERR_ALLOC) {                               // the CUDA cores' layout is a fraction of this one's size
+    submit.keep = false;
+    return RT3D_OK;
+  }
   if (s != RT3D_OK) return s;
   a.last_chunk = L->n_chunks - 1;
   a.last_k16 = w->N - a.last_chunk * kSplitChunk > 16 ? 2 : 1;
@@ -1660,7 +1665,8 @@ static rt3d_status prepare_body(rt3d_packed* p) {
   if (d->cc_major == 10 && p->dtype == RT3D_F32 && p->N > kSplitFewest && split_rows_bounded(p) && g_f32_split.load() && umma_f32_plan(&split)) {
     DeviceBlob::Umma* u = nullptr;
     const UmmaLayout* L = get_split_layout(p, split.n_tile);
-    if (L && (s = get_split_blob(p, blob, L, split.pair != 0, &u)) != RT3D_OK) return s;
+    // without the device memory for it calls run on the CUDA cores
+    if (L && (s = get_split_blob(p, blob, L, split.pair != 0, &u)) != RT3D_OK && s != RT3D_ERR_ALLOC) return s;
   }
   for (int S = 2; S <= 8; ++S) umma_split_capacity(S, d->sm_count);      // what the K splits ask the runtime, once per device
   return cudaDeviceSynchronize() == cudaSuccess ? RT3D_OK : RT3D_ERR_CUDA;
