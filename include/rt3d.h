@@ -433,8 +433,11 @@ enum { RT3D_DEBUG_WAIT_CYCLES = 1, RT3D_DEBUG_DROP_LAST_LOAD = 2, RT3D_DEBUG_T_G
 rt3d_status rt3d_debug_set(int what, long long value);
 /* Diagnostics.  RT3D_DEBUG_WAIT_SITE: after a synchronisation of the device, the number of the wait inside a
  * kernel that gave up since the last rt3d_last_device_status (0 = none; the numbers are the last argument of the
- * kernels' bounded waits in the sources); -1 on error.  Does not clear the word. */
-enum { RT3D_DEBUG_WAIT_SITE = 1 };
+ * kernels' bounded waits in the sources); -1 on error.  Does not clear the word.
+ * Of the calling thread's last call, beside rt3d_last_plan: RT3D_DEBUG_STEP_CHANNELS: input channels of a K step of the
+ * step-list and resident-weight bf16 kernels (64 or 32; 0 for the other kernels); RT3D_DEBUG_TURNED: 1 if their epilogue turned
+ * its pieces in shared memory. */
+enum { RT3D_DEBUG_WAIT_SITE = 1, RT3D_DEBUG_STEP_CHANNELS = 2, RT3D_DEBUG_TURNED = 3 };
 long long rt3d_debug_get(int what);
 
 const char* rt3d_status_string(rt3d_status s);

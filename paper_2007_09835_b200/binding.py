@@ -597,7 +597,7 @@ def rt3d_debug_get(what: int) -> int:
     return int(_lib.rt3d_debug_get(int(what)))
 
 
-DEBUG_WAIT_SITE = 1
+DEBUG_WAIT_SITE, DEBUG_STEP_CHANNELS, DEBUG_TURNED = 1, 2, 3
 
 
 def rt3d_debug_set(what: int, value: int):

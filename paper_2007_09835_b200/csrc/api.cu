@@ -191,7 +191,13 @@ bool overlaps(const rt3d_tensor* a, const rt3d_tensor* b) {
 }
 
 // ------------------------------------------------------------------------ prepared calls
-thread_local rt3d_plan_info t_last_plan = {-1, 0, 0, 0, 0};
+// What a caller may ask about the last call, and what tests ask besides (rt3d_debug_get).
+struct LastPlan {
+  rt3d_plan_info info;
+  int step_channels, turned;
+  LastPlan(const rt3d_plan_info& i, int step = 0, int turn = 0) : info(i), step_channels(step), turned(turn) {}
+};
+thread_local LastPlan t_last_plan = rt3d_plan_info{-1, 0, 0, 0, 0};
 std::atomic<int> g_plan_epoch{0};              // advanced by rt3d_debug_set: calls prepared before it are prepared again
 
 }  // namespace
@@ -216,7 +222,7 @@ struct CallBuffers {
 // choosing the kernel and encoding two or three tensor maps cost 1 to 2 us of the host's time for each call.
 struct PreparedCall {
   CallKey key;
-  rt3d_plan_info info;
+  LastPlan plan;
   std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch;
 };
 }  // namespace rt3d
@@ -283,8 +289,8 @@ class Submit {
   }
   // A kernel launch chosen for this call.  `launch` must hold by value whatever it needs besides the handle's own memory, and
   // take the addresses of the tensors and biases from its argument.
-  rt3d_status operator()(const rt3d_plan_info& info, std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch) {
-    auto c = std::make_shared<PreparedCall>(PreparedCall{key_, info, std::move(launch)});
+  rt3d_status operator()(const LastPlan& plan, std::function<cudaError_t(const CallBuffers&, cudaStream_t)> launch) {
+    auto c = std::make_shared<PreparedCall>(PreparedCall{key_, plan, std::move(launch)});
     if (keep) {
       std::lock_guard<std::mutex> lock(w_->mu);
       if (w_->calls.size() < kPreparedCalls) w_->calls.push_back(c);
@@ -295,7 +301,7 @@ class Submit {
 
  private:
   rt3d_status run(const PreparedCall& c) {
-    t_last_plan = c.info;
+    t_last_plan = c.plan;
     if (t_plan_only) return RT3D_OK;
     if (c.launch(buffers_, st_) != cudaSuccess) return RT3D_ERR_CUDA;
     g_launches.fetch_add(1);
@@ -955,7 +961,7 @@ rt3d_status try_halo(rt3d_packed* w, DeviceBlob* blob, DeviceState* d, const rt3
   *launched = true;
   const int sms = d->sm_count;
   const void* wmap = u->wmap_half;
-  return submit(rt3d_plan_info{4, a.n_tile, 1, 0, 0}, [=](const CallBuffers& c, cudaStream_t st) {
+  return submit(LastPlan({4, a.n_tile, 1, 0, 0}, kChunk, a.turned), [=](const CallBuffers& c, cudaStream_t st) {
     const PlacedMaps m(xmap, c.x, ymap, h.u.store_tma ? c.y : nullptr);
     if (!m.ok) return cudaErrorInvalidValue;
     HaloArgs now = h;
@@ -1395,7 +1401,7 @@ rt3d_status conv_body(const rt3d_tensor* x, const rt3d_packed* wc, const float* 
   }
   const int sms = d->sm_count;
   const void* wmap = use_pair ? u->wmap_half : u->wmap;
-  return submit(rt3d_plan_info{use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0},
+  return submit(LastPlan({use_pair ? (use_ts ? 7 : 2) : 1, a.n_tile, a.n_splits, a.tail_workers, pooled ? 1 : 0}, L->chunk, a.turned),
                 [=](const CallBuffers& c, cudaStream_t st) {
     const PlacedMaps m(xmap, c.x, ymap, a.store_tma ? c.y : nullptr);
     if (!m.ok) return cudaErrorInvalidValue;
@@ -1871,12 +1877,14 @@ rt3d_status rt3d_conv3d_query_algo(const rt3d_tensor* x, const rt3d_packed* w, c
 }
 
 rt3d_status rt3d_last_plan(rt3d_plan_info* info) {
-  if (!info || t_last_plan.kernel < 0) return RT3D_ERR_INVALID_ARG;
-  *info = t_last_plan;
+  if (!info || t_last_plan.info.kernel < 0) return RT3D_ERR_INVALID_ARG;
+  *info = t_last_plan.info;
   return RT3D_OK;
 }
 
 long long rt3d_debug_get(int what) {
+  if (what == RT3D_DEBUG_STEP_CHANNELS) return t_last_plan.step_channels;
+  if (what == RT3D_DEBUG_TURNED) return t_last_plan.turned;
   if (what != RT3D_DEBUG_WAIT_SITE) return -1;
   DeviceState* d = nullptr;
   if (get_device_state(&d) != RT3D_OK) return -1;
@@ -1984,7 +1992,7 @@ rt3d_status rt3d_conv3d_sparse_noalloc(const rt3d_tensor* x, const rt3d_packed* 
                  encode_ymap(y, sb, 1, 1, 1, &ymap)) ? 1 : 0;
   if (launch_conv_umma(a, &xmap, u->wmap, a.store_tma ? &ymap : nullptr, d->sm_count, st) != cudaSuccess) return RT3D_ERR_CUDA;
   g_launches.fetch_add(1);
-  t_last_plan = rt3d_plan_info{1, a.n_tile, a.n_splits, 0, 0};
+  t_last_plan = LastPlan({1, a.n_tile, a.n_splits, 0, 0}, L->chunk);
   return RT3D_OK;
 }
 

@@ -53,10 +53,10 @@ def test_narrow_layer_after_prepare():
     x = nets.to_device(synth.make_input(15, (8, 8, 56, 56, 24)), torch.bfloat16)
     want = warm(x)
     plan = rt3d.rt3d_last_plan()
-    assert plan["kernel"] == 2 and plan["tail_workers"] == 0
+    assert plan["kernel"] == 2 and plan["tail_workers"] == 0 and rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == 32
     lay.packed.prepare()                                   # steps of 64 channels
     got, captured = _captured(lay, x)
-    assert captured == plan
+    assert captured == plan and rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == 64
     assert float((got - want).abs().max()) <= 2 ** -7 * float(want.abs().max())       # the same products in the same order
     assert torch.equal(lay(x), want)
 
@@ -102,10 +102,13 @@ def test_narrow_layer_after_a_call_of_another_shape(cin, cout, k, large, small, 
     first = nets.to_device(synth.make_input(15, large + (cin,)), torch.bfloat16)
     x = nets.to_device(synth.make_input(16, small + (cin,)), torch.bfloat16)
     want = warm(x)
+    wanted = rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS)
     lay(first)
+    there = rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS)
     got, _ = _captured(lay, x)
+    assert rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == there
     assert float((got - want).abs().max()) <= 2 ** -7 * float(want.abs().max())
-    assert torch.equal(lay(x), want)                       # what served the capture is not kept
+    assert torch.equal(lay(x), want) and rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == wanted       # what served the capture is not kept
 
 
 def test_call_without_allocation_after_one_in_steps_of_32():
@@ -119,6 +122,7 @@ def test_call_without_allocation_after_one_in_steps_of_32():
         rt3d.rt3d_debug_set(rt3d.DEBUG_T_GROUPS, 1)
     allocs = rt3d.rt3d_alloc_count()
     rt3d.rt3d_conv3d_sparse_noalloc(rt3d.tensor_desc(x, 24), lay.packed, lay.bias, rt3d.tensor_desc(y, 64), (1, 1, 1), (1, 1, 1), True)
+    assert rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == 32
     assert rt3d.rt3d_alloc_count() == allocs and rt3d.rt3d_last_device_status() == rt3d.OK
     assert float((y - want).abs().max()) <= 2 ** -7 * float(want.abs().max())
 

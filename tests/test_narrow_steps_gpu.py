@@ -43,6 +43,8 @@ def test_steps_of_32_channels(x, cin, cout, k, stride, kind, algo):
             finally:
                 rt3d.rt3d_debug_set(rt3d.DEBUG_NARROW, 1)
             assert rt3d.rt3d_last_device_status() == rt3d.OK
+            few = algo == SINGLE and k[0] * k[1] * k[2] <= 12          # few locations on single CTAs: steps of 64
+            assert rt3d.rt3d_debug_get(rt3d.DEBUG_STEP_CHANNELS) == (32 if narrow and not few else 64)
             out[narrow] = nets.to_numpy(y, cout)
         ref = np.maximum(conv + (res if residual else 0), 0)
         assert np.abs(out[1] - ref).max() <= 2e-2 * np.abs(ref).max()

@@ -42,8 +42,37 @@ def test_turned_pieces(x, cin, cout, k, stride, algo, residual):
                                       True, residual=rt3d.tensor_desc(res, cout) if residual else None, algo=algo)
     assert rt3d.rt3d_last_device_status() == rt3d.OK
     assert rt3d.rt3d_last_plan()["kernel"] == 4 if algo == rt3d.ALGO_UMMA_HALO else rt3d.rt3d_last_plan()["kernel"] in (2, 7)
-    assert rt3d.rt3d_last_plan()["tail_workers"] == 0
+    assert rt3d.rt3d_last_plan()["tail_workers"] == 0 and rt3d.rt3d_debug_get(rt3d.DEBUG_TURNED) == 1
     got = y.float().cpu().numpy()
     assert np.abs(got[..., :cout] - ref).max() <= 2e-2 * np.abs(ref).max()
     unit = (cout + 7) // 8 * 8                             # box stores may zero the rest of a row's last 16-byte unit
     assert (got[..., unit:] == 55.0).all()
+
+
+@pytest.mark.parametrize("cin,cout,k", [(64, 128, (3, 3, 3)), (83, 150, (3, 3, 3))])
+def test_turned_tiles_beside_a_tail_split(cin, cout, k):
+    """Whole rounds of tiles, which are turned, and a last one that is shared out along K, which is not."""
+    spec = synth.ConvSpec("t", cin, cout, k, (1, 1, 1), (1, 1, 1), True)
+    L = synth.make_layer(spec, 12, cin + cout, 4, 4, "bernoulli", 0.5)
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.bfloat16)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for clips in range(8, 64):                             # 100 tiles a clip: look for a count with a shared last round
+        x = (clips, 8, 40, 40)
+        xd = torch.zeros(x + (nets.pitch_for(cin, torch.bfloat16),), dtype=torch.bfloat16, device="cuda")
+        y = lay.alloc_out(xd)
+        with rt3d.planning():
+            lay.fused(xd, y, residual=y.new_zeros(y.shape))
+        plan = rt3d.rt3d_last_plan()
+        if plan["tail_workers"] > 0 and rt3d.rt3d_debug_get(rt3d.DEBUG_TURNED) == 1:
+            break
+    assert plan["tail_workers"] > 0 and plan["kernel"] in (2, 7) and clips * 100 > sms
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    xd[..., :cin] = (torch.rand(x + (cin,), device="cuda", generator=gen) * 2 - 1).bfloat16()
+    res = torch.full_like(y, float("nan"))
+    res[..., :cout] = (torch.rand(y.shape[:4] + (cout,), device="cuda", generator=gen) * 2 - 1).bfloat16()
+    rt3d.rt3d_conv3d_sparse_fused(rt3d.tensor_desc(xd, cin), lay.packed, lay.bias, rt3d.tensor_desc(y, cout), spec.stride, spec.pad, True,
+                                  residual=rt3d.tensor_desc(res, cout))
+    assert rt3d.rt3d_last_plan() == plan and rt3d.rt3d_last_device_status() == rt3d.OK and rt3d.rt3d_debug_get(rt3d.DEBUG_TURNED) == 1
+    want = torch.relu(lay(xd, relu=False, algo=rt3d.ALGO_SIMT)[..., :cout].float() + res[..., :cout].float())
+    got = y[..., :cout].float()
+    assert float((got - want).abs().max()) <= 2e-2 * float(want.abs().max())
