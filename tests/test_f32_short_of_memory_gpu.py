@@ -21,6 +21,7 @@ def test_layout_of_the_tensor_cores_does_not_fit():
     assert rt3d.rt3d_last_plan()["kernel"] == 8
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
+    rt3d.rt3d_release_kept()                               # blocks of freed handles, which would hold it
     room = torch.cuda.mem_get_info()[0] - (40 << 20)       # 9 MB for each of the two layouts beside it fit, the 50 MB that it comes with do not
     hold = torch.empty(room, dtype=torch.uint8, device="cuda")
     try:
