@@ -1030,7 +1030,11 @@ rt3d_status get_f32_blob(rt3d_packed* h, DeviceBlob* blob, const F32Layout* L, D
   return RT3D_OK;
 }
 
-constexpr int kSplitFewest = 16;                           // input channels up to which no fp32 call goes to the tensor cores
+// Up to 16 input channels half of every step is empty, and the CUDA cores skip what is pruned: only unpruned layers of more than 32
+// outputs go to the tensor cores.  Over 130 random layers of 8 to 16 channels, of those that split_is_faster would send: unpruned
+// ones of more than 32 outputs 1.02 to 3.5 times faster there (15 -> 118 3x3x3 on 3 x 12 x 56 x 31 77.6 -> 23.7 us), of up to 32
+// 0.74 to 1.6, pruned ones 0.89 to 1.5.
+bool split_fills_steps(const rt3d_packed* w) { return w->N > 16 || (w->M > 32 && w->nnz == int64_t(w->P) * w->Q * w->Ks); }
 
 // What a drain warp does again for a tile whose rows are all infinite or NaN, while the other roles wait for it: for every four
 // output channels (fewer where a kernel group ends), every entry that their groups may have, four input channels at a time.
@@ -1052,10 +1056,8 @@ int split_n_tile(int M) { return round_up(ceil_div(M, ceil_div(M, 128)), 16); }
 // items over the SMs, per round its steps and the output of a tile; a step costs 0.31 us at up to 48 columns, 0.44 at 128
 // (0.85-1.1).  The margin leaves ties where they were: 27 -> 145 channels 3x3x3 on 2 x 4 x 16 x 44 24.2 us and 24.3.  Taken by
 // this rule the 92 layers gain 1.19x in the mean (the better of both each time: 1.23x), 64 -> 128 on 2 x 16 x 56 x 56 3.1x.
-// Up to 16 input channels stay on the CUDA cores: half of every step would be empty, and the tests of the register-blocked
-// kernel expect it there.  (It costs 16 -> 74 channels 3x3x3 dense on 16 x 51 x 35 35 us instead of 20.)
 bool split_is_faster(const rt3d_packed* w, const F32SplitArgs& a, int sm_count) {
-  if (w->N <= kSplitFewest) return false;
+  if (!split_fills_steps(w)) return false;
   const double density = double(w->nnz) / (double(w->P) * w->Q * w->Ks);
   const double groups = double(std::max(1, kSplitChunk / w->g_n)) * std::max(1, a.n_tile / w->g_m);     // that share a step
   const double steps = double(w->Ks) * ceil_div(w->N, kSplitChunk) * (w->is_dense ? 1.0 : 1.0 - std::pow(1.0 - density, groups));
@@ -1668,7 +1670,7 @@ static rt3d_status prepare_body(rt3d_packed* p) {
   }
   F32SplitArgs split;
   split.n_tile = split_n_tile(p->M); split.n_bundles = ceil_div(p->M, split.n_tile);
-  if (d->cc_major == 10 && p->dtype == RT3D_F32 && p->N > kSplitFewest && split_rows_bounded(p) && g_f32_split.load() && umma_f32_plan(&split)) {
+  if (d->cc_major == 10 && p->dtype == RT3D_F32 && split_fills_steps(p) && split_rows_bounded(p) && g_f32_split.load() && umma_f32_plan(&split)) {
     DeviceBlob::Umma* u = nullptr;
     const UmmaLayout* L = get_split_layout(p, split.n_tile);
     // without the device memory for it calls run on the CUDA cores

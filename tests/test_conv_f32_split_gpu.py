@@ -179,3 +179,16 @@ def test_layers_with_more_to_compute_again_stay_on_the_cuda_cores(everywhere):
         L = synth.make_layer(spec, 9, 1, group[0], group[1], "bernoulli", 0.05)
         nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], group[0], group[1], torch.float32)(x)
         assert rt3d.rt3d_last_plan()["kernel"] == kernel
+
+
+@pytest.mark.parametrize("cin,cout,density,kernel", [(15, 118, None, 8), (16, 118, 0.9, 0), (17, 118, 0.9, 8)])
+def test_layers_of_up_to_16_channels(cin, cout, density, kernel):
+    """Half of a step is empty: the dispatch sends unpruned ones, and the results are the CUDA cores' up to the order of the sums."""
+    spec = synth.ConvSpec("f32", cin, cout, (3, 3, 3), (1, 1, 1), (1, 1, 1), True)
+    L = synth.make_layer(spec, 8, cin, 4, 4, "bernoulli" if density else "none", density)
+    lay = nets.ConvLayer(spec, L["w"], L["bias"], L["mask"], 4, 4, torch.float32, dense=density is None)
+    x = nets.to_device(synth.make_input(8, (3, 12, 28, 31, cin)), torch.float32)
+    got = lay(x)
+    assert rt3d.rt3d_last_plan()["kernel"] == kernel and rt3d.rt3d_last_device_status() == rt3d.OK
+    want = lay(x, algo=rt3d.ALGO_SIMT)
+    assert float((got - want).abs().max()) <= 2e-6 * float(want.abs().max())
