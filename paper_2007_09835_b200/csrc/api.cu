@@ -40,8 +40,8 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
     weight_blocks().release_all();
     g_allocs.fetch_add(1);
     e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation) cudaGetLastError();      // the caller's answer, not that of the next launch
   }
+  if (e != cudaSuccess) cudaGetLastError();                      // this call's answer, not that of the next one that asks
   return e;
 }
 template <typename T>

@@ -70,6 +70,16 @@ fill_split_tiles_kernel(const int32_t* __restrict__ group_ptr, const uint16_t* _
   }
 }
 
+// Returns this launch's own error: the runtime's last one may be an earlier call's, a caller's among them.
+template <typename... P, typename... A>
+cudaError_t launch_fill(void (*kernel)(P...), int64_t blocks, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks < 65536 ? blocks : 65536));
+  cfg.blockDim = dim3(256);
+  cfg.stream = cudaStreamLegacy;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 }  // namespace
 
 cudaError_t launch_fill_split_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const float* tiles, const int32_t* slots,
@@ -78,9 +88,8 @@ cudaError_t launch_fill_split_tiles(const int32_t* group_ptr, const uint16_t* po
   cudaError_t e = cudaMemsetAsync(wtiles, 0, bytes, cudaStreamLegacy);
   if (e != cudaSuccess || nnz == 0) return e;
   const int64_t blocks = (nnz + 7) / 8;
-  fill_split_tiles_kernel<<<unsigned(blocks < 65536 ? blocks : 65536), 256, 0, cudaStreamLegacy>>>(
-      group_ptr, pos_idx, tiles, slots, M, N, Ks, g_m, g_n, Q, n_groups, int(nnz), n_tile, halves, n_chunks, static_cast<__nv_bfloat16*>(wtiles));
-  return cudaGetLastError();
+  return launch_fill(fill_split_tiles_kernel, blocks, group_ptr, pos_idx, tiles, slots, M, N, Ks, g_m, g_n, Q, n_groups, int(nnz), n_tile, halves,
+                     n_chunks, static_cast<__nv_bfloat16*>(wtiles));
 }
 
 cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos_idx, const void* tiles, const int32_t* slots,
@@ -89,10 +98,8 @@ cudaError_t launch_fill_umma_tiles(const int32_t* group_ptr, const uint16_t* pos
   cudaError_t e = cudaMemsetAsync(wtiles, 0, bytes, cudaStreamLegacy);
   if (e != cudaSuccess || nnz == 0) return e;
   const int64_t blocks = (nnz + 7) / 8;
-  fill_umma_tiles_kernel<<<unsigned(blocks < 65536 ? blocks : 65536), 256, 0, cudaStreamLegacy>>>(
-      group_ptr, pos_idx, static_cast<const uint16_t*>(tiles), slots, M, N, Ks, g_m, g_n, Q, n_groups, int(nnz), n_tile, chunk == 32 ? 5 : 6, n_chunks,
-      static_cast<uint16_t*>(wtiles));
-  return cudaGetLastError();
+  return launch_fill(fill_umma_tiles_kernel, blocks, group_ptr, pos_idx, static_cast<const uint16_t*>(tiles), slots, M, N, Ks, g_m, g_n, Q, n_groups,
+                     int(nnz), n_tile, chunk == 32 ? 5 : 6, n_chunks, static_cast<uint16_t*>(wtiles));
 }
 
 }  // namespace rt3d
